@@ -325,7 +325,7 @@ constexpr int64_t kSurrogateParams = 30 * 256 + 256 + 256 * 256 + 256 + 256 + 1;
 struct Surrogate {
     void *buf = nullptr;   // one allocation holding everything below
     float *w = nullptr, *m = nullptr, *v = nullptr, *g = nullptr, *mean = nullptr, *std = nullptr;
-    __nv_bfloat16 *wb = nullptr, *w2t = nullptr;
+    __nv_bfloat16 *wb = nullptr;
     int64_t step = 0;
     bool ready = false;
     ~Surrogate();
