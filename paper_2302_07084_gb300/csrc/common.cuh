@@ -45,6 +45,16 @@ __host__ __device__ __forceinline__ u32x4 philox10(u32x4 c, uint32_t k0, uint32_
     return c;
 }
 
+// acc += a b on two packed floats, each one rounding (fma.rn.f32x2, sm_100 and
+// later): half the issue slots of two scalar FMAs.
+#ifdef __CUDACC__
+__device__ __forceinline__ void f2_add_prod(float2 &acc, float2 a, float2 b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;"
+        : "+l"(reinterpret_cast<uint64_t &>(acc))
+        : "l"(reinterpret_cast<const uint64_t &>(a)), "l"(reinterpret_cast<const uint64_t &>(b)));
+}
+#endif
+
 // Error state shared by host code of the library.
 struct Status {
     int code = 0;

@@ -4,12 +4,13 @@
 //
 // For each label l: minimise 1/2 |w|^2 + C sum_i log(1 + exp(-y_il w.x_i)),
 // y in {-1, +1}, x with a constant-1 bias feature; `iters` Newton steps from
-// w = 0, all labels at once:
+// w = 0, all labels at once, four launches a step:
 //   margins   Z = X W                                  (right_multiply)
-//   weights   r = C (sigma(yz) - 1) y, D = C sigma (1 - sigma)
-//   gradient  G = W + X^T R                            (row blocks, FP32, summed in FP64)
-//   Hessians  H_l = I + X^T diag(D_l) X                (row blocks, FP32, summed in FP64)
-//   update    W_l -= H_l^-1 G_l                        (batched FP64 Cholesky, one CTA per label)
+//   partials  r = C (sigma(yz) - 1) y, D = C sigma (1 - sigma); X^T r and
+//             X^T diag(D) X of a block of 128 rows and one label, FP32
+//   sums      G = W + sum of the X^T r blocks (FP64), H = I + sum of the
+//             X^T D X blocks (error-free float pairs)
+//   update    W_l -= H_l^-1 G_l to FP64 accuracy: FP32 Cholesky, FP64 residuals
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -47,95 +48,182 @@ __global__ void gather_rows_kernel(const float *__restrict__ X, int64_t n, int64
     }
 }
 
-// In place: Z -> R = C (sigma(yz) - 1) y; D = C sigma(yz) (1 - sigma(yz)).
-__global__ void logistic_weights_kernel(float *__restrict__ Z, const float *__restrict__ Ys, int64_t count, float C,
-                                        float *__restrict__ D) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x) {
-        const float y = Ys[e];
-        const float sg = 1.0f / (1.0f + expf(-y * Z[e]));
-        Z[e] = C * (sg - 1.0f) * y;
-        D[e] = C * sg * (1.0f - sg);
+// Number of TS x TS tiles on and above the diagonal of a da x da matrix, and
+// the tile (ti, tj), ti <= tj, at position p in row order.
+__host__ __device__ inline int upper_tiles(int da, int ts) {
+    const int nt = (da + ts - 1) / ts;
+    return nt * (nt + 1) / 2;
+}
+__device__ __forceinline__ void upper_tile(int p, int nt, int *ti, int *tj) {
+    int i = 0;
+    while (p >= nt - i) {
+        p -= nt - i;
+        ++i;
     }
+    *ti = i;
+    *tj = i + p;
 }
 
-// partial[b][a][l] = sum over rows of block b of Xa[i][a] R[i][l].
-__global__ void grad_partial_kernel(const float *__restrict__ Xa, const float *__restrict__ R, int64_t m, int da, int L,
-                                    double *__restrict__ partial) {
-    const int64_t r0 = (int64_t)blockIdx.x * kEvalRows;
-    const int64_t r1 = imin64(m, r0 + kEvalRows);
-    double *out = partial + (int64_t)blockIdx.x * da * L;
-    for (int e = threadIdx.x; e < da * L; e += blockDim.x) {
-        const int a = e / L, l = e - a * L;
-        float acc = 0.f;
-        for (int64_t i = r0; i < r1; ++i) acc = fmaf(Xa[i * da + a], R[i * L + l], acc);
-        out[e] = acc;
-    }
-}
+// One block of kEvalRows rows and one label: gpart[b][l][a] = sum_r x_a R,
+// hpart[b][l][e][p] = sum_r (x_a D) x_c for entry e = (a % TS) TS + c % TS of
+// the upper tile p (entry-major, so that a warp's stores are contiguous), rows
+// in ascending order. Bound by the FP32 FMAs (rows x labels x da (da + 1) / 2):
+// a thread owns a TS x TS tile in registers, so a row costs it TS / 2 16-byte
+// shared-memory loads for TS^2 FMAs; rows are staged 32 at a time so that
+// several CTAs share an SM. TS = 8 for d >= 64, where the tiles fill the warps
+// (d = 128: 153 tiles on 160 threads); below, 4 x 4 tiles keep more threads
+// busy (d = 32: 45 tiles on 64 threads, with 8 x 8 15 on 32).
+// Staged rows with TS = 8 hold the first four columns of every tile, then the
+// last four, so that neighbouring tiles' 16-byte loads hit neighbouring banks.
+constexpr int kEvalStage = 32;
 
-// hpart[b][l][a][c] (a <= c) = sum over rows of block b of D[i][l] Xa[i][a] Xa[i][c];
-// CTA (row block, label): the block's rows and their D-weighted copies staged in
-// shared memory, one thread per entry (a, c) of the upper triangle.
-__global__ void __launch_bounds__(256) hess_partial_kernel(const float *__restrict__ Xa, const float *__restrict__ D,
-                                                           int64_t m, int da, int L, double *__restrict__ hpart) {
-    extern __shared__ float xs[];   // kEvalRows x dp rows, then the weighted rows
-    const int dp = (da + 7) & ~7;
+template <int TS>
+__global__ void __launch_bounds__(256) hess_partial_kernel(const float *__restrict__ Xa, const float *__restrict__ Z,
+                                                           const float *__restrict__ Ys, int64_t m, int da, int L,
+                                                           float C, int ntiles, float *__restrict__ hpart,
+                                                           float *__restrict__ gpart) {
+    extern __shared__ __align__(16) float xs[];   // kEvalStage rows, then their D-weighted copies
+    __shared__ float s_r[kEvalRows], s_d[kEvalRows];
+    const int nt = (da + TS - 1) / TS, pitch = nt * TS;
+    float *wx = xs + kEvalStage * pitch;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const int l = blockIdx.y;
     const int64_t r0 = (int64_t)blockIdx.x * kEvalRows;
     const int rows = (int)imin64(kEvalRows, m - r0);
-    float *wx = xs + kEvalRows * dp;
-    for (int e = threadIdx.x; e < rows * da; e += blockDim.x) {
-        const int r = e / da, a = e - r * da;
-        const float x = Xa[(r0 + r) * da + a];
-        xs[r * dp + a] = x;
-        wx[r * dp + a] = x * D[(r0 + r) * L + l];
+    for (int r = tid; r < rows; r += blockDim.x) {
+        const float y = Ys[(r0 + r) * L + l];
+        const float sg = 1.0f / (1.0f + expf(-y * Z[(r0 + r) * L + l]));
+        s_r[r] = C * (sg - 1.0f) * y;
+        s_d[r] = C * sg * (1.0f - sg);
     }
-    __syncthreads();
-    double *out = hpart + ((int64_t)blockIdx.x * L + l) * dp * dp;
-    for (int t = threadIdx.x; t < da * da; t += blockDim.x) {
-        const int a = t / da, c = t - a * da;
-        if (a > c) continue;
-        float acc = 0.f;
-        for (int r = 0; r < rows; ++r) acc = fmaf(wx[r * dp + a], xs[r * dp + c], acc);
-        out[a * dp + c] = acc;
-    }
-}
-
-// G = W + sum_b partial[b];  H_l = I + sum_b hpart[b][l] (mirrored), fixed order.
-__global__ void newton_reduce_kernel(const double *__restrict__ partial, const double *__restrict__ hpart, int nblk,
-                                     int da, int L, const double *__restrict__ W, double *__restrict__ G,
-                                     double *__restrict__ H) {
-    const int dp = (da + 7) & ~7;
-    const int64_t total_h = (int64_t)L * da * da;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total_h + da * L;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        if (e < total_h) {
-            const int l = (int)(e / ((int64_t)da * da));
-            const int rem = (int)(e - (int64_t)l * da * da);
-            const int a = rem / da, c = rem - a * da;
-            const int lo = min(a, c), hi = max(a, c);
-            double s = a == c ? 1.0 : 0.0;
-            for (int b = 0; b < nblk; ++b) s += hpart[((int64_t)b * L + l) * dp * dp + lo * dp + hi];
-            H[e] = s;
-        } else {
-            const int64_t f = e - total_h;
-            double s = W[f];
-            for (int b = 0; b < nblk; ++b) s += partial[(int64_t)b * da * L + f];
-            G[f] = s;
+    int ti = 0, tj = 0;
+    const bool active = tid < ntiles;
+    if (active) upper_tile(tid, nt, &ti, &tj);
+    auto at = [&](int c) { return TS == 8 ? (c & 4 ? nt * 4 : 0) + (c >> 3) * 4 + (c & 3) : c; };
+    float2 acc[TS][TS / 2];
+#pragma unroll
+    for (int u = 0; u < TS; ++u)
+#pragma unroll
+        for (int v = 0; v < TS / 2; ++v) acc[u][v] = make_float2(0.f, 0.f);
+    float g = 0.f;
+    const int ga = tid < da ? at(tid) : 0;
+    for (int s0 = 0; s0 < rows; s0 += kEvalStage) {
+        const int ns = min(kEvalStage, rows - s0);
+        __syncthreads();   // weights ready; the last stage's sums done
+        for (int r = warp; r < ns; r += nw) {
+            const float dr = s_d[s0 + r];
+            const float *src = Xa + (r0 + s0 + r) * da;
+            for (int c = lane; c < pitch; c += 32) {
+                const float x = c < da ? src[c] : 0.f;
+                const int e = r * pitch + at(c);
+                xs[e] = x;
+                wx[e] = x * dr;
+            }
         }
+        __syncthreads();
+        if (active) {
+#pragma unroll 2
+            for (int r = 0; r < ns; ++r) {
+                float a[TS], b[TS];
+#pragma unroll
+                for (int h = 0; h < TS / 4; ++h) {
+                    const float4 p = *reinterpret_cast<const float4 *>(wx + r * pitch + h * nt * 4 + ti * 4);
+                    const float4 q = *reinterpret_cast<const float4 *>(xs + r * pitch + h * nt * 4 + tj * 4);
+                    a[4 * h] = p.x, a[4 * h + 1] = p.y, a[4 * h + 2] = p.z, a[4 * h + 3] = p.w;
+                    b[4 * h] = q.x, b[4 * h + 1] = q.y, b[4 * h + 2] = q.z, b[4 * h + 3] = q.w;
+                }
+#pragma unroll
+                for (int u = 0; u < TS; ++u)
+#pragma unroll
+                    for (int v = 0; v < TS / 2; ++v)
+                        f2_add_prod(acc[u][v], make_float2(a[u], a[u]), make_float2(b[2 * v], b[2 * v + 1]));
+            }
+        }
+        if (tid < da)
+            for (int r = 0; r < ns; ++r) g = fmaf(xs[r * pitch + ga], s_r[s0 + r], g);
+    }
+    if (tid < da) gpart[((int64_t)blockIdx.x * L + l) * da + tid] = g;
+    if (!active) return;
+    float *out = hpart + ((int64_t)blockIdx.x * L + l) * ntiles * (TS * TS) + tid;
+#pragma unroll
+    for (int u = 0; u < TS; ++u)
+#pragma unroll
+        for (int v = 0; v < TS / 2; ++v) {
+            out[(int64_t)(u * TS + 2 * v) * ntiles] = acc[u][v].x;
+            out[(int64_t)(u * TS + 2 * v + 1) * ntiles] = acc[u][v].y;
+        }
+}
+
+// H_l = I + sum_b hpart[b][l] (both triangles, FP64) and G = W + sum_b gpart[b]
+// (FP64). The Hessian's sums over the row blocks are error-free float pairs
+// (two-sum; the pair holds about 46 bits): FP64 additions and conversions run
+// at 1/64 of the FP32 rate on this GPU and would bound this pass.
+template <int TS>
+__global__ void __launch_bounds__(256) newton_reduce_kernel(const float *__restrict__ gpart,
+                                                            const float *__restrict__ hpart, int nblk, int da, int L,
+                                                            int ntiles, const double *__restrict__ W,
+                                                            double *__restrict__ G, double *__restrict__ H) {
+    const int l = blockIdx.y;
+    const int64_t stride = (int64_t)L * ntiles * (TS * TS);
+    const int total = ntiles * TS * TS;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < total) {
+        const int q = e / ntiles, nt = (da + TS - 1) / TS;
+        int ti, tj;
+        upper_tile(e - q * ntiles, nt, &ti, &tj);
+        const int a = ti * TS + q / TS, c = tj * TS + q % TS;
+        if (a <= c && c < da) {
+            const float *src = hpart + (int64_t)l * total + e;
+            float hi = 0.f, lo = 0.f;
+#pragma unroll 8
+            for (int b = 0; b < nblk; ++b) {
+                const float p = src[b * stride];
+                const float s = __fadd_rn(hi, p), bb = __fsub_rn(s, hi);
+                lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb)));
+                hi = s;
+            }
+            const double s = (a == c ? 1.0 : 0.0) + (double)lo + (double)hi;
+            double *Hl = H + (int64_t)l * da * da;
+            Hl[a * da + c] = s;
+            Hl[c * da + a] = s;
+        }
+    } else if (e - total < da) {
+        const int a = e - total;
+        double s = W[a * L + l];
+        for (int b = 0; b < nblk; ++b) s += gpart[((int64_t)b * L + l) * da + a];
+        G[a * L + l] = s;
     }
 }
 
-// Per label (one CTA each): Cholesky of H_l (FP64, shared memory), solve
-// H_l delta = G[:, l], W[:, l] -= delta.
-__global__ void __launch_bounds__(512) newton_solve_kernel(const double *__restrict__ H, const double *__restrict__ G,
-                                                           int da, int L, double *__restrict__ W,
-                                                           int *__restrict__ status) {
-    extern __shared__ double A[];   // da x da, then the right-hand side
+// Per label (one CTA each): W[:, l] -= H_l^-1 G[:, l].
+//
+// H is factored in FP32 (blocked Cholesky in shared memory, 32-wide panels)
+// and the solution refined with FP64 residuals G - H x until the next
+// correction would be below an FP64 ulp of x, so x is as accurate as an FP64
+// factorisation's: FP64 FMAs run at 2 a cycle and SM here, which puts the FP64
+// factorisation alone at 170 us for d = 128 (129^3 / 3 FMAs), against 4 us for
+// a residual. Refinement converges when the condition number is below about
+// 1e6 (H = I + X^T D X: 1 + C |X|^2 / 4 at most); where it does not, or the
+// FP32 factorisation breaks down, the label takes the FP64 factorisation
+// (newton_solve_fp64).
+constexpr int kSolveThreads = 512;
+constexpr int kNB = 32;
+
+__host__ __device__ inline int solve_pad(int da) { return (da + kNB - 1) / kNB * kNB; }
+__host__ __device__ inline int solve_smem(int da) {
+    const int dp = solve_pad(da);
+    const int fp32 = (dp * (dp + 4) + (dp / kNB) * kNB * (kNB + 1) + 2 * dp) * 4 + (2 * da + 4 * da) * 8;
+    const int fp64 = (da * da + da) * 8;
+    return fp32 > fp64 ? fp32 : fp64;
+}
+
+// The FP64 factorisation of one label's Hessian (shared memory A: da x da,
+// then the right-hand side) and its solve; status bit 1: not positive definite.
+__device__ void newton_solve_fp64(const double *__restrict__ Hl, const double *__restrict__ G, int da, int L, int l,
+                                  double *A, double *__restrict__ W, int *__restrict__ status) {
     double *rhs = A + da * da;
-    const int l = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     __shared__ double s_inv;
-    const double *Hl = H + (int64_t)l * da * da;
     for (int e = tid; e < da * da; e += blockDim.x) A[e] = Hl[e];
     for (int a = tid; a < da; a += blockDim.x) rhs[a] = G[a * L + l];
     __syncthreads();
@@ -180,6 +268,234 @@ __global__ void __launch_bounds__(512) newton_solve_kernel(const double *__restr
     for (int a = tid; a < da; a += blockDim.x) W[a * L + l] -= rhs[a];
 }
 
+// FP32 upper Cholesky of the dp x dp matrix A (row stride ld, upper triangle;
+// dp a multiple of 32) by the CTA, and the inverses of its 32 x 32 diagonal
+// blocks (Dinv, row stride 33). *bad is set where a pivot is not positive and
+// finite. Ends with a barrier.
+__device__ __forceinline__ void chol32(float *A, int ld, int dp, float *Dinv, int *bad) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    for (int p0 = 0; p0 < dp; p0 += kNB) {
+        if (warp == 0) {   // diagonal block: lane j holds column j
+            float a[kNB];
+#pragma unroll
+            for (int i = 0; i < kNB; ++i) a[i] = i <= lane ? A[(p0 + i) * ld + p0 + lane] : 0.f;
+            bool ok = true;
+#pragma unroll
+            for (int k = 0; k < kNB; ++k) {
+                const float piv = __shfl_sync(0xffffffffu, a[k], k);
+                ok = ok && piv > 0.f && piv < 3.0e38f;
+                a[k] *= rsqrtf(piv);
+#pragma unroll
+                for (int i = k + 1; i < kNB; ++i)
+                    a[i] = fmaf(-__shfl_sync(0xffffffffu, a[k], i), a[k], a[i]);
+            }
+            if (!ok && lane == 0) *bad = 1;
+#pragma unroll
+            for (int i = 0; i < kNB; ++i)
+                if (i <= lane) A[(p0 + i) * ld + p0 + lane] = a[i];
+        }
+        __syncthreads();
+        const int j = p0 + kNB + tid;   // the panel's row block, a thread per column
+        if (j < dp) {
+            float x[kNB];
+#pragma unroll
+            for (int i = 0; i < kNB; ++i) x[i] = A[(p0 + i) * ld + j];
+#pragma unroll
+            for (int t = 0; t < kNB; ++t) {
+                const float *rt = A + (p0 + t) * ld + p0;
+                x[t] /= rt[t];
+#pragma unroll
+                for (int i = t + 1; i < kNB; ++i) x[i] = fmaf(-rt[i], x[t], x[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < kNB; ++i) A[(p0 + i) * ld + j] = x[i];
+        }
+        __syncthreads();
+        const int base = p0 + kNB, nt = (dp - base) / 4, pairs = nt * (nt + 1) / 2;
+        for (int q = tid; q < pairs; q += blockDim.x) {   // trailing 4 x 4 tiles
+            // tile row from the pairs before it: rows i hold nt - i pairs
+            int ti = (int)(((2 * nt + 1) - sqrtf((float)((2 * nt + 1) * (2 * nt + 1) - 8 * q))) * 0.5f);
+            while (ti > 0 && ti * nt - ti * (ti - 1) / 2 > q) --ti;
+            while ((ti + 1) * nt - (ti + 1) * ti / 2 <= q) ++ti;
+            const int tj = ti + q - (ti * nt - ti * (ti - 1) / 2);
+            float *ai = A + base + 4 * ti, *aj = A + base + 4 * tj;
+            float c[4][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float4 v = *reinterpret_cast<const float4 *>(aj + (base + 4 * ti + u) * ld);
+                c[u][0] = v.x, c[u][1] = v.y, c[u][2] = v.z, c[u][3] = v.w;
+            }
+#pragma unroll 8
+            for (int k = 0; k < kNB; ++k) {
+                const float4 x = *reinterpret_cast<const float4 *>(ai + (p0 + k) * ld);
+                const float4 y = *reinterpret_cast<const float4 *>(aj + (p0 + k) * ld);
+                const float xu[4] = {x.x, x.y, x.z, x.w}, yv[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) c[u][v] = fmaf(-xu[u], yv[v], c[u][v]);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                *reinterpret_cast<float4 *>(aj + (base + 4 * ti + u) * ld) =
+                    make_float4(c[u][0], c[u][1], c[u][2], c[u][3]);
+        }
+        __syncthreads();
+    }
+    // inverses of the diagonal blocks, a warp each, lane j its column j
+    for (int b = warp; b < dp / kNB; b += nw) {
+        const float *R = A + (b * kNB) * ld + b * kNB;
+        float *D = Dinv + b * kNB * (kNB + 1);
+        float x[kNB];
+#pragma unroll
+        for (int i = kNB - 1; i >= 0; --i) {
+            float s = i == lane ? 1.f : 0.f;
+#pragma unroll
+            for (int t = i + 1; t < kNB; ++t) s = fmaf(-R[i * ld + t], x[t], s);
+            x[i] = i <= lane ? s / R[i * ld + i] : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < kNB; ++i) D[i * (kNB + 1) + lane] = x[i];
+    }
+    __syncthreads();
+}
+
+// v <- R^-1 R^-T v (FP32, dp entries in shared memory). Ends with a barrier.
+__device__ __forceinline__ void solve32(const float *A, int ld, int dp, const float *Dinv, float *v) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = dp / kNB;
+    for (int p = 0; p < nb; ++p) {   // R^T y = v
+        const float *D = Dinv + p * kNB * (kNB + 1);
+        if (warp == 0) {
+            float s = 0.f;
+#pragma unroll
+            for (int i = 0; i < kNB; ++i) s = fmaf(D[i * (kNB + 1) + lane], v[p * kNB + i], s);
+            __syncwarp();
+            v[p * kNB + lane] = s;
+        }
+        __syncthreads();
+        const int j = (p + 1) * kNB + tid;
+        if (j < dp) {
+            float s = v[j];
+#pragma unroll
+            for (int i = 0; i < kNB; ++i) s = fmaf(-A[(p * kNB + i) * ld + j], v[p * kNB + i], s);
+            v[j] = s;
+        }
+        __syncthreads();
+    }
+    for (int p = nb - 1; p >= 0; --p) {   // R x = y
+        const float *D = Dinv + p * kNB * (kNB + 1);
+        if (warp == 0) {
+            float s = 0.f;
+#pragma unroll
+            for (int t = 0; t < kNB; ++t) s = fmaf(D[lane * (kNB + 1) + t], v[p * kNB + t], s);
+            __syncwarp();
+            v[p * kNB + lane] = s;
+        }
+        __syncthreads();
+        if (tid < p * kNB) {
+            float s = v[tid];
+#pragma unroll
+            for (int t = 0; t < kNB; t += 4) {
+                const float4 r = *reinterpret_cast<const float4 *>(A + tid * ld + p * kNB + t);
+                s = fmaf(-r.x, v[p * kNB + t], s);
+                s = fmaf(-r.y, v[p * kNB + t + 1], s);
+                s = fmaf(-r.z, v[p * kNB + t + 2], s);
+                s = fmaf(-r.w, v[p * kNB + t + 3], s);
+            }
+            v[tid] = s;
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kSolveThreads) newton_solve_kernel(const double *__restrict__ H,
+                                                                     const double *__restrict__ G, int da, int L,
+                                                                     double *__restrict__ W,
+                                                                     int *__restrict__ status) {
+    extern __shared__ __align__(16) double sm[];
+    const int l = blockIdx.x, tid = threadIdx.x;
+    const int dp = solve_pad(da), ld = dp + 4;
+    double *x = sm, *r = x + da, *part = r + da;   // part: up to 4 da
+    float *A = reinterpret_cast<float *>(part + 4 * da), *Dinv = A + dp * ld;
+    float *v = Dinv + (dp / kNB) * kNB * (kNB + 1);
+    __shared__ int s_bad, s_rexp;
+    __shared__ unsigned s_dmax, s_xmax;
+    const double *Hl = H + (int64_t)l * da * da;
+    if (tid == 0) {
+        s_bad = 0;
+        s_rexp = 0;
+    }
+    for (int e = tid; e < dp * dp; e += blockDim.x) {
+        const int i = e / dp, j = e - i * dp;
+        A[i * ld + j] = i < da && j < da ? (float)Hl[i * da + j] : i == j ? 1.f : 0.f;
+    }
+    for (int a = tid; a < da; a += blockDim.x) {
+        x[a] = 0.0;
+        r[a] = G[a * L + l];
+    }
+    __syncthreads();
+    chol32(A, ld, dp, Dinv, &s_bad);
+    // groups of da threads share a residual: group q sums columns q, q + ng, ..
+    const int ng = min(4, (int)blockDim.x / da), grp = tid / da, ra = tid - grp * da;
+    bool done = false;
+    float before = 3.0e38f;
+    for (int it = 0; it < 12 && !done && !s_bad; ++it) {
+        if (it > 0) {
+            if (grp < ng) {
+                double s = 0.0;
+                for (int j = grp; j < da; j += ng) s = fma(Hl[(int64_t)j * da + ra], x[j], s);
+                part[grp * da + ra] = s;
+            }
+            __syncthreads();
+            for (int a = tid; a < da; a += blockDim.x) {
+                double s = part[a];
+                for (int q = 1; q < ng; ++q) s += part[q * da + a];
+                r[a] = G[a * L + l] - s;
+            }
+        }
+        // the residual scaled by a power of two into FP32's range
+        if (tid == 0) s_dmax = s_xmax = 0u;
+        for (int a = tid; a < da; a += blockDim.x) atomicMax(&s_rexp, (__double2hiint(r[a]) >> 20) & 0x7ff);
+        __syncthreads();
+        const int re = s_rexp;
+        if (re == 0 || re == 0x7ff) {   // zero (or below FP64's normal range): nothing left to correct
+            if (re != 0 && tid == 0) s_bad = 1;
+            done = re == 0;
+            __syncthreads();
+            break;
+        }
+        const double up = __hiloint2double((2046 - re) << 20, 0), down = __hiloint2double(re << 20, 0);   // 2^-+(re - 1023)
+        for (int a = tid; a < dp; a += blockDim.x) v[a] = a < da ? (float)(r[a] * up) : 0.f;
+        __syncthreads();
+        solve32(A, ld, dp, Dinv, v);
+        for (int a = tid; a < da; a += blockDim.x) {
+            const double dx = (double)v[a] * down, xn = x[a] + dx;
+            x[a] = xn;
+            atomicMax(&s_dmax, __float_as_uint(fabsf((float)dx)));
+            atomicMax(&s_xmax, __float_as_uint(fabsf((float)xn)));
+        }
+        if (tid == 0) s_rexp = 0;
+        __syncthreads();
+        // the error left is about dmax^2 / before; stop when that is below an
+        // ulp of x, give up when the corrections shrink by less than 4
+        const float dmax = __uint_as_float(s_dmax), xmax = __uint_as_float(s_xmax);
+        if (!(dmax < 3.0e38f)) {
+            if (tid == 0) s_bad = 1;
+        } else if (it > 0) {
+            done = dmax <= 1.0e-16f * xmax || dmax * (dmax / before) <= 1.0e-16f * xmax;
+            if (!done && !(dmax <= 0.25f * before) && tid == 0) s_bad = 1;
+        }
+        before = dmax;
+        __syncthreads();
+    }
+    if (done && !s_bad) {
+        for (int a = tid; a < da; a += blockDim.x) W[a * L + l] -= x[a];
+        return;
+    }
+    __syncthreads();
+    newton_solve_fp64(Hl, G, da, L, l, sm, W, status);
+}
+
 // Top-k prediction and per-label TP / FP / FN counts.
 __global__ void topk_f1_kernel(const float *__restrict__ S, const float *__restrict__ Ys, int64_t m, int L,
                                unsigned long long *__restrict__ counts) {
@@ -210,16 +526,17 @@ int macro_f1(Workspace &ws, const float *X, int64_t n, int d, int64_t ldx, const
         return fail(LNE_ERR_INVALID, "bad Macro-F1 arguments");
     const int da = d + 1;
     if (da > 160) return fail(LNE_ERR_UNSUPPORTED, "Macro-F1 supports d <= 159");
-    const int dp = (da + 7) & ~7;
     const int64_t nblk = ceil_div(n_train, kEvalRows);
-    float *Xa = nullptr, *Ys = nullptr, *Z = nullptr, *Dw = nullptr, *Xt = nullptr, *Yt = nullptr, *St = nullptr;
-    double *W = nullptr, *G = nullptr, *H = nullptr, *gp = nullptr, *hp = nullptr;
+    const int ts = da > 64 ? 8 : 4;
+    const int ntiles = upper_tiles(da, ts);
+    float *Xa = nullptr, *Ys = nullptr, *Z = nullptr, *Xt = nullptr, *Yt = nullptr, *St = nullptr;
+    float *gp = nullptr, *hp = nullptr;
+    double *W = nullptr, *G = nullptr, *H = nullptr;
     unsigned long long *cnt = nullptr;
     int *status = nullptr;
     LNE_TRY(ws.get("eval.Xa", (size_t)(n_train * da), &Xa));
     LNE_TRY(ws.get("eval.Ys", (size_t)(n_train * L), &Ys));
     LNE_TRY(ws.get("eval.Z", (size_t)(n_train * L), &Z));
-    LNE_TRY(ws.get("eval.D", (size_t)(n_train * L), &Dw));
     LNE_TRY(ws.get("eval.Xt", (size_t)(n_test * da), &Xt));
     LNE_TRY(ws.get("eval.Yt", (size_t)(n_test * L), &Yt));
     LNE_TRY(ws.get("eval.St", (size_t)(n_test * L), &St));
@@ -227,7 +544,7 @@ int macro_f1(Workspace &ws, const float *X, int64_t n, int d, int64_t ldx, const
     LNE_TRY(ws.get("eval.G", (size_t)da * L, &G));
     LNE_TRY(ws.get("eval.H", (size_t)L * da * da, &H));
     LNE_TRY(ws.get("eval.gp", (size_t)(nblk * da * L), &gp));
-    LNE_TRY(ws.get("eval.hp", (size_t)(nblk * L * dp * dp), &hp));
+    LNE_TRY(ws.get("eval.hp", (size_t)nblk * L * ntiles * ts * ts, &hp));
     LNE_TRY(ws.get("eval.cnt", (size_t)3 * L, &cnt));
     LNE_TRY(ws.get("eval.status", 1, &status));
     LNE_CUDA_TRY(cudaMemsetAsync(W, 0, sizeof(double) * da * L, st));
@@ -242,24 +559,34 @@ int macro_f1(Workspace &ws, const float *X, int64_t n, int d, int64_t ldx, const
                                                                status);
         LNE_LAUNCH_CHECK();
     }
-    const int hsmem = 2 * kEvalRows * dp * 4;
-    if (hsmem > 48 * 1024) LNE_TRY(allow_dynamic_smem(hess_partial_kernel));
-    const int ssmem = (da * da + da) * 8;
+    const int threads = (std::max(ntiles, da) + 31) / 32 * 32;   // at most 224 (da = 160: 210 tiles)
+    const int hsmem = 2 * kEvalStage * ((da + ts - 1) / ts * ts) * 4;
+    const dim3 hgrid((unsigned)nblk, (unsigned)L);
+    const dim3 rgrid((unsigned)ceil_div((int64_t)ntiles * ts * ts + da, 256), (unsigned)L);
     LNE_TRY(allow_dynamic_smem(newton_solve_kernel));
     for (int it = 0; it < iters; ++it) {
         LNE_TRY(right_multiply(Xa, n_train, da, da, W, L, L, nullptr, Z, L, st));
         {
-            LNE_TRACE("logreg_newton", st);
-            logistic_weights_kernel<<<egrid(n_train * L), 256, 0, st>>>(Z, Ys, n_train * L, (float)C, Dw);
+            LNE_TRACE("newton_partials", st);
+            if (ts == 8)
+                hess_partial_kernel<8><<<hgrid, threads, hsmem, st>>>(Xa, Z, Ys, n_train, da, L, (float)C, ntiles, hp,
+                                                                      gp);
+            else
+                hess_partial_kernel<4><<<hgrid, threads, hsmem, st>>>(Xa, Z, Ys, n_train, da, L, (float)C, ntiles, hp,
+                                                                      gp);
             LNE_LAUNCH_CHECK();
-            grad_partial_kernel<<<(unsigned)nblk, 256, 0, st>>>(Xa, Z, n_train, da, L, gp);
+        }
+        {
+            LNE_TRACE("newton_sums", st);
+            if (ts == 8)
+                newton_reduce_kernel<8><<<rgrid, 256, 0, st>>>(gp, hp, (int)nblk, da, L, ntiles, W, G, H);
+            else
+                newton_reduce_kernel<4><<<rgrid, 256, 0, st>>>(gp, hp, (int)nblk, da, L, ntiles, W, G, H);
             LNE_LAUNCH_CHECK();
-            hess_partial_kernel<<<dim3((unsigned)nblk, (unsigned)L), 256, hsmem, st>>>(Xa, Dw, n_train, da, L, hp);
-            LNE_LAUNCH_CHECK();
-            newton_reduce_kernel<<<egrid((int64_t)L * da * da + da * L), 256, 0, st>>>(gp, hp, (int)nblk, da, L, W,
-                                                                                        G, H);
-            LNE_LAUNCH_CHECK();
-            newton_solve_kernel<<<L, 512, ssmem, st>>>(H, G, da, L, W, status);
+        }
+        {
+            LNE_TRACE("newton_solve", st);
+            newton_solve_kernel<<<L, kSolveThreads, solve_smem(da), st>>>(H, G, da, L, W, status);
             LNE_LAUNCH_CHECK();
         }
     }

@@ -132,12 +132,6 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// acc += a b on two packed floats, each one rounding (sm_100 and later).
-__device__ __forceinline__ void fma2(float2 &acc, float2 a, float2 b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;"
-        : "+l"(reinterpret_cast<uint64_t &>(acc))
-        : "l"(reinterpret_cast<const uint64_t &>(a)), "l"(reinterpret_cast<const uint64_t &>(b)));
-}
 __device__ __forceinline__ float2 bf2(uint32_t w) {   // a bfloat16 is the upper half of the FP32 with its value
     return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
 }
@@ -174,10 +168,10 @@ __device__ __forceinline__ void layer_chain(const uint32_t *w, int pitch, const 
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
             const float4 a = *reinterpret_cast<const float4 *>(in + i * ld + k);
-            fma2(acc[i], make_float2(a.x, a.x), w0);
-            fma2(acc[i], make_float2(a.y, a.y), w1);
-            fma2(acc[i], make_float2(a.z, a.z), w2);
-            fma2(acc[i], make_float2(a.w, a.w), w3);
+            f2_add_prod(acc[i], make_float2(a.x, a.x), w0);
+            f2_add_prod(acc[i], make_float2(a.y, a.y), w1);
+            f2_add_prod(acc[i], make_float2(a.z, a.z), w2);
+            f2_add_prod(acc[i], make_float2(a.w, a.w), w3);
         }
     }
 }
@@ -235,7 +229,7 @@ __device__ __forceinline__ void row_group(const RowArgs &A, char *sm, const RowB
         for (int k = 28; k < kIn; ++k) {
             const float2 wk = bf2(w[k * (kHid / 2)]);
 #pragma unroll
-            for (int i = 0; i < RPT; ++i) fma2(acc[i], make_float2(in[i * 32 + k], in[i * 32 + k]), wk);
+            for (int i = 0; i < RPT; ++i) f2_add_prod(acc[i], make_float2(in[i * 32 + k], in[i * 32 + k]), wk);
         }
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
@@ -430,8 +424,8 @@ __device__ __forceinline__ void weight_tile(const GradArgs &A, int tile, float *
                 const float *pk = ps + kk * kWPitch, *dj = ds + jq;
                 auto add = [&](float pr, int r) {
                     const float4 x = *reinterpret_cast<const float4 *>(dj + r * 32);
-                    fma2(acc0, make_float2(pr, pr), make_float2(x.x, x.y));
-                    fma2(acc1, make_float2(pr, pr), make_float2(x.z, x.w));
+                    f2_add_prod(acc0, make_float2(pr, pr), make_float2(x.x, x.y));
+                    f2_add_prod(acc1, make_float2(pr, pr), make_float2(x.z, x.w));
                 };
                 int r = 0;
 #pragma unroll 4
