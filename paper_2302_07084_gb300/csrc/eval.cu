@@ -22,23 +22,24 @@ namespace {
 
 constexpr int kEvalRows = 128;   // rows per FP32 partial sum (and per CTA)
 
-// Xa[i] = (X[idx[i]], 1), Ys[i][l] = +1 / -1. A row index outside [0, n) is
-// not read: its row becomes zeros (label -1) and status bit 2 is set, which
-// the host turns into LNE_ERR_INVALID.
+// Xa[i] = (X[idx[i]], 1, 0, ..) with rows of `pitch` floats, Ys[i][l] = +1 / -1.
+// A row index outside [0, n) is not read: its row becomes zeros (label -1) and
+// status bit 2 is set, which the host turns into LNE_ERR_INVALID.
 __global__ void gather_rows_kernel(const float *__restrict__ X, int64_t n, int64_t ldx, int d,
                                    const uint8_t *__restrict__ lab, int L, const int32_t *__restrict__ idx, int64_t m,
-                                   float *__restrict__ Xa, float *__restrict__ Ys, int *__restrict__ status) {
-    const int da = d + 1;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m * da; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = e / da;
-        const int j = (int)(e - i * da);
+                                   int pitch, float *__restrict__ Xa, float *__restrict__ Ys,
+                                   int *__restrict__ status) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m * pitch;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = e / pitch;
+        const int j = (int)(e - i * pitch);
         const int64_t r = idx[i];
         if (r < 0 || r >= n) {
             if (j == 0) atomicOr(status, 2);
             Xa[e] = 0.0f;
             continue;
         }
-        Xa[e] = j < d ? X[r * ldx + j] : 1.0f;
+        Xa[e] = j < d ? X[r * ldx + j] : j == d ? 1.0f : 0.0f;
     }
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m * L; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = e / L;
@@ -69,10 +70,14 @@ __device__ __forceinline__ void upper_tile(int p, int nt, int *ti, int *tj) {
 // the upper tile p (entry-major, so that a warp's stores are contiguous), rows
 // in ascending order. Bound by the FP32 FMAs (rows x labels x da (da + 1) / 2):
 // a thread owns a TS x TS tile in registers, so a row costs it TS / 2 16-byte
-// shared-memory loads for TS^2 FMAs; rows are staged 32 at a time so that
-// several CTAs share an SM. TS = 8 for d >= 64, where the tiles fill the warps
-// (d = 128: 153 tiles on 160 threads); below, 4 x 4 tiles keep more threads
-// busy (d = 32: 45 tiles on 64 threads, with 8 x 8 15 on 32).
+// shared-memory loads and TS multiplications by D for TS^2 FMAs; rows are
+// staged 32 at a time by asynchronous copies into two buffers, so the next
+// ones arrive during the sums. TS = 8 for d >= 64, where the tiles fill the
+// warps (d = 128: 153 tiles on 160 threads); below, 4 x 4 tiles keep more
+// threads busy (d = 32: 45 tiles on 64 threads, with 8 x 8 15 on 32).
+// Measured (5,156 rows, d = 128, 39 labels): 126 us a Newton step; the FP32 pipe
+// is about half busy, at 15 warps an SM (128 registers) the rest is latency and
+// the last wave. A thread per entry with two loads per FMA took 1.5 ms.
 // Staged rows with TS = 8 hold the first four columns of every tile, then the
 // last four, so that neighbouring tiles' 16-byte loads hit neighbouring banks.
 constexpr int kEvalStage = 32;
@@ -82,65 +87,70 @@ __global__ void __launch_bounds__(256) hess_partial_kernel(const float *__restri
                                                            const float *__restrict__ Ys, int64_t m, int da, int L,
                                                            float C, int ntiles, float *__restrict__ hpart,
                                                            float *__restrict__ gpart) {
-    extern __shared__ __align__(16) float xs[];   // kEvalStage rows, then their D-weighted copies
-    __shared__ float s_r[kEvalRows], s_d[kEvalRows];
-    const int nt = (da + TS - 1) / TS, pitch = nt * TS;
-    float *wx = xs + kEvalStage * pitch;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    extern __shared__ __align__(16) float xs[];   // two buffers of kEvalStage rows
+    __shared__ float2 s_w[kEvalRows];             // (D, R) of the rows
+    const int nt = (da + TS - 1) / TS, pitch = nt * TS, quads = pitch / 4;
+    const int tid = threadIdx.x;
     const int l = blockIdx.y;
     const int64_t r0 = (int64_t)blockIdx.x * kEvalRows;
     const int rows = (int)imin64(kEvalRows, m - r0);
+    auto stage = [&](int s0, float *to) {
+        const float *src = Xa + (r0 + s0) * pitch;
+        const int total = min(kEvalStage, rows - s0) * quads;
+        for (int e = tid; e < total; e += blockDim.x) {
+            const int r = e / quads, q = e - r * quads;
+            const int at = TS == 8 ? (q & 1) * nt + (q >> 1) : q;
+            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(to + r * pitch + 4 * at);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src + 4 * e) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    stage(0, xs);
     for (int r = tid; r < rows; r += blockDim.x) {
         const float y = Ys[(r0 + r) * L + l];
         const float sg = 1.0f / (1.0f + expf(-y * Z[(r0 + r) * L + l]));
-        s_r[r] = C * (sg - 1.0f) * y;
-        s_d[r] = C * sg * (1.0f - sg);
+        s_w[r] = make_float2(C * sg * (1.0f - sg), C * (sg - 1.0f) * y);
     }
     int ti = 0, tj = 0;
-    const bool active = tid < ntiles;
+    const bool active = tid < ntiles;   // threads without a tile sum tile (0, 0) along and store nothing
     if (active) upper_tile(tid, nt, &ti, &tj);
-    auto at = [&](int c) { return TS == 8 ? (c & 4 ? nt * 4 : 0) + (c >> 3) * 4 + (c & 3) : c; };
     float2 acc[TS][TS / 2];
 #pragma unroll
     for (int u = 0; u < TS; ++u)
 #pragma unroll
         for (int v = 0; v < TS / 2; ++v) acc[u][v] = make_float2(0.f, 0.f);
     float g = 0.f;
-    const int ga = tid < da ? at(tid) : 0;
-    for (int s0 = 0; s0 < rows; s0 += kEvalStage) {
+    const int gc = min(tid, pitch - 1);   // column tid of a staged row: the gradient's
+    const int ga = TS == 8 ? (gc & 4 ? nt * 4 : 0) + (gc >> 3) * 4 + (gc & 3) : gc;
+    for (int s0 = 0, buf = 0; s0 < rows; s0 += kEvalStage, buf ^= 1) {
         const int ns = min(kEvalStage, rows - s0);
-        __syncthreads();   // weights ready; the last stage's sums done
-        for (int r = warp; r < ns; r += nw) {
-            const float dr = s_d[s0 + r];
-            const float *src = Xa + (r0 + s0 + r) * da;
-            for (int c = lane; c < pitch; c += 32) {
-                const float x = c < da ? src[c] : 0.f;
-                const int e = r * pitch + at(c);
-                xs[e] = x;
-                wx[e] = x * dr;
-            }
+        const float *x = xs + buf * (kEvalStage * pitch);
+        if (s0 + kEvalStage < rows) {
+            stage(s0 + kEvalStage, xs + (buf ^ 1) * (kEvalStage * pitch));
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
-        if (active) {
 #pragma unroll 2
-            for (int r = 0; r < ns; ++r) {
-                float a[TS], b[TS];
+        for (int r = 0; r < ns; ++r) {
+            float a[TS], b[TS];
+            const float2 w = s_w[s0 + r];
 #pragma unroll
-                for (int h = 0; h < TS / 4; ++h) {
-                    const float4 p = *reinterpret_cast<const float4 *>(wx + r * pitch + h * nt * 4 + ti * 4);
-                    const float4 q = *reinterpret_cast<const float4 *>(xs + r * pitch + h * nt * 4 + tj * 4);
-                    a[4 * h] = p.x, a[4 * h + 1] = p.y, a[4 * h + 2] = p.z, a[4 * h + 3] = p.w;
-                    b[4 * h] = q.x, b[4 * h + 1] = q.y, b[4 * h + 2] = q.z, b[4 * h + 3] = q.w;
-                }
-#pragma unroll
-                for (int u = 0; u < TS; ++u)
-#pragma unroll
-                    for (int v = 0; v < TS / 2; ++v)
-                        f2_add_prod(acc[u][v], make_float2(a[u], a[u]), make_float2(b[2 * v], b[2 * v + 1]));
+            for (int h = 0; h < TS / 4; ++h) {
+                const float4 p = *reinterpret_cast<const float4 *>(x + r * pitch + h * nt * 4 + ti * 4);
+                const float4 q = *reinterpret_cast<const float4 *>(x + r * pitch + h * nt * 4 + tj * 4);
+                a[4 * h] = p.x * w.x, a[4 * h + 1] = p.y * w.x, a[4 * h + 2] = p.z * w.x, a[4 * h + 3] = p.w * w.x;
+                b[4 * h] = q.x, b[4 * h + 1] = q.y, b[4 * h + 2] = q.z, b[4 * h + 3] = q.w;
             }
+            g = fmaf(x[r * pitch + ga], w.y, g);
+#pragma unroll
+            for (int u = 0; u < TS; ++u)
+#pragma unroll
+                for (int v = 0; v < TS / 2; ++v)
+                    f2_add_prod(acc[u][v], make_float2(a[u], a[u]), make_float2(b[2 * v], b[2 * v + 1]));
         }
-        if (tid < da)
-            for (int r = 0; r < ns; ++r) g = fmaf(xs[r * pitch + ga], s_r[s0 + r], g);
+        __syncthreads();   // this buffer is refilled next
     }
     if (tid < da) gpart[((int64_t)blockIdx.x * L + l) * da + tid] = g;
     if (!active) return;
@@ -154,15 +164,23 @@ __global__ void __launch_bounds__(256) hess_partial_kernel(const float *__restri
         }
 }
 
-// H_l = I + sum_b hpart[b][l] (both triangles, FP64) and G = W + sum_b gpart[b]
-// (FP64). The Hessian's sums over the row blocks are error-free float pairs
+// (hi, lo) += p: hi takes the rounded sum, lo its exact rounding error.
+__device__ __forceinline__ void pair_add(float &hi, float &lo, float p) {
+    const float s = __fadd_rn(hi, p), b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(p, b)));
+    hi = s;
+}
+
+// H_l = I + sum_b hpart[b][l] (both triangles; FP64 in H, as a float pair in
+// Hp) and G = W + sum_b gpart[b] (FP64). The Hessian's sums over the row blocks are error-free float pairs
 // (two-sum; the pair holds about 46 bits): FP64 additions and conversions run
 // at 1/64 of the FP32 rate on this GPU and would bound this pass.
 template <int TS>
 __global__ void __launch_bounds__(256) newton_reduce_kernel(const float *__restrict__ gpart,
                                                             const float *__restrict__ hpart, int nblk, int da, int L,
                                                             int ntiles, const double *__restrict__ W,
-                                                            double *__restrict__ G, double *__restrict__ H) {
+                                                            double *__restrict__ G, double *__restrict__ H,
+                                                            float2 *__restrict__ Hp) {
     const int l = blockIdx.y;
     const int64_t stride = (int64_t)L * ntiles * (TS * TS);
     const int total = ntiles * TS * TS;
@@ -174,18 +192,14 @@ __global__ void __launch_bounds__(256) newton_reduce_kernel(const float *__restr
         const int a = ti * TS + q / TS, c = tj * TS + q % TS;
         if (a <= c && c < da) {
             const float *src = hpart + (int64_t)l * total + e;
-            float hi = 0.f, lo = 0.f;
-#pragma unroll 8
-            for (int b = 0; b < nblk; ++b) {
-                const float p = src[b * stride];
-                const float s = __fadd_rn(hi, p), bb = __fsub_rn(s, hi);
-                lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb)));
-                hi = s;
-            }
-            const double s = (a == c ? 1.0 : 0.0) + (double)lo + (double)hi;
-            double *Hl = H + (int64_t)l * da * da;
-            Hl[a * da + c] = s;
-            Hl[c * da + a] = s;
+            float hi = a == c ? 1.f : 0.f, lo = 0.f;
+#pragma unroll 16
+            for (int b = 0; b < nblk; ++b) pair_add(hi, lo, src[b * stride]);
+            const float s = __fadd_rn(hi, lo);
+            lo = __fsub_rn(lo, __fsub_rn(s, hi));   // |lo| <= |hi|: exact
+            const int64_t at = (int64_t)l * da * da;
+            H[at + a * da + c] = H[at + c * da + a] = (double)s + (double)lo;
+            Hp[at + a * da + c] = Hp[at + c * da + a] = make_float2(s, lo);
         }
     } else if (e - total < da) {
         const int a = e - total;
@@ -198,11 +212,13 @@ __global__ void __launch_bounds__(256) newton_reduce_kernel(const float *__restr
 // Per label (one CTA each): W[:, l] -= H_l^-1 G[:, l].
 //
 // H is factored in FP32 (blocked Cholesky in shared memory, 32-wide panels)
-// and the solution refined with FP64 residuals G - H x until the next
-// correction would be below an FP64 ulp of x, so x is as accurate as an FP64
+// and the solution refined with residuals G - H x, first in float-pair
+// arithmetic (about 46 bits, 1 us), then in FP64 until the next correction
+// would be below an FP64 ulp of x, so x is as accurate as an FP64
 // factorisation's: FP64 FMAs run at 2 a cycle and SM here, which puts the FP64
-// factorisation alone at 170 us for d = 128 (129^3 / 3 FMAs), against 4 us for
-// a residual. Refinement converges when the condition number is below about
+// factorisation alone at 170 us for d = 128 (129^3 / 3 FMAs), against 5 us for
+// an FP64 residual. Measured at d = 128: 64 us a step (the FP64 factorisation
+// with one-thread triangular solves: 0.5 ms). Refinement converges when the condition number is below about
 // 1e6 (H = I + X^T D X: 1 + C |X|^2 / 4 at most); where it does not, or the
 // FP32 factorisation breaks down, the label takes the FP64 factorisation
 // (newton_solve_fp64).
@@ -212,7 +228,7 @@ constexpr int kNB = 32;
 __host__ __device__ inline int solve_pad(int da) { return (da + kNB - 1) / kNB * kNB; }
 __host__ __device__ inline int solve_smem(int da) {
     const int dp = solve_pad(da);
-    const int fp32 = (dp * (dp + 4) + (dp / kNB) * kNB * (kNB + 1) + 2 * dp) * 4 + (2 * da + 4 * da) * 8;
+    const int fp32 = (dp * (dp + 4) + (dp / kNB) * kNB * (kNB + 1) + dp) * 4 + (7 * da + (da & 1)) * 8;
     const int fp64 = (da * da + da) * 8;
     return fp32 > fp64 ? fp32 : fp64;
 }
@@ -271,8 +287,8 @@ __device__ void newton_solve_fp64(const double *__restrict__ Hl, const double *_
 // FP32 upper Cholesky of the dp x dp matrix A (row stride ld, upper triangle;
 // dp a multiple of 32) by the CTA, and the inverses of its 32 x 32 diagonal
 // blocks (Dinv, row stride 33). *bad is set where a pivot is not positive and
-// finite. Ends with a barrier.
-__device__ __forceinline__ void chol32(float *A, int ld, int dp, float *Dinv, int *bad) {
+// finite; rdiag: dp floats, the diagonal's reciprocals. Ends with a barrier.
+__device__ __forceinline__ void chol32(float *A, int ld, int dp, float *Dinv, float *rdiag, int *bad) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     for (int p0 = 0; p0 < dp; p0 += kNB) {
         if (warp == 0) {   // diagonal block: lane j holds column j
@@ -284,7 +300,9 @@ __device__ __forceinline__ void chol32(float *A, int ld, int dp, float *Dinv, in
             for (int k = 0; k < kNB; ++k) {
                 const float piv = __shfl_sync(0xffffffffu, a[k], k);
                 ok = ok && piv > 0.f && piv < 3.0e38f;
-                a[k] *= rsqrtf(piv);
+                const float inv = rsqrtf(piv);
+                if (lane == k) rdiag[p0 + k] = inv;
+                a[k] *= inv;
 #pragma unroll
                 for (int i = k + 1; i < kNB; ++i)
                     a[i] = fmaf(-__shfl_sync(0xffffffffu, a[k], i), a[k], a[i]);
@@ -303,7 +321,7 @@ __device__ __forceinline__ void chol32(float *A, int ld, int dp, float *Dinv, in
 #pragma unroll
             for (int t = 0; t < kNB; ++t) {
                 const float *rt = A + (p0 + t) * ld + p0;
-                x[t] /= rt[t];
+                x[t] *= rdiag[p0 + t];
 #pragma unroll
                 for (int i = t + 1; i < kNB; ++i) x[i] = fmaf(-rt[i], x[t], x[i]);
             }
@@ -352,7 +370,7 @@ __device__ __forceinline__ void chol32(float *A, int ld, int dp, float *Dinv, in
             float s = i == lane ? 1.f : 0.f;
 #pragma unroll
             for (int t = i + 1; t < kNB; ++t) s = fmaf(-R[i * ld + t], x[t], s);
-            x[i] = i <= lane ? s / R[i * ld + i] : 0.f;
+            x[i] = i <= lane ? s * rdiag[b * kNB + i] : 0.f;
         }
 #pragma unroll
         for (int i = 0; i < kNB; ++i) D[i * (kNB + 1) + lane] = x[i];
@@ -409,6 +427,7 @@ __device__ __forceinline__ void solve32(const float *A, int ld, int dp, const fl
 }
 
 __global__ void __launch_bounds__(kSolveThreads) newton_solve_kernel(const double *__restrict__ H,
+                                                                     const float2 *__restrict__ Hp,
                                                                      const double *__restrict__ G, int da, int L,
                                                                      double *__restrict__ W,
                                                                      int *__restrict__ status) {
@@ -416,46 +435,63 @@ __global__ void __launch_bounds__(kSolveThreads) newton_solve_kernel(const doubl
     const int l = blockIdx.x, tid = threadIdx.x;
     const int dp = solve_pad(da), ld = dp + 4;
     double *x = sm, *r = x + da, *part = r + da;   // part: up to 4 da
-    float *A = reinterpret_cast<float *>(part + 4 * da), *Dinv = A + dp * ld;
+    float2 *xp = reinterpret_cast<float2 *>(part + 4 * da);   // x as float pairs
+    float *A = reinterpret_cast<float *>(xp + da + (da & 1)), *Dinv = A + dp * ld;
     float *v = Dinv + (dp / kNB) * kNB * (kNB + 1);
     __shared__ int s_bad, s_rexp;
     __shared__ unsigned s_dmax, s_xmax;
     const double *Hl = H + (int64_t)l * da * da;
+    const float2 *Hpl = Hp + (int64_t)l * da * da;
     if (tid == 0) {
         s_bad = 0;
         s_rexp = 0;
     }
     for (int e = tid; e < dp * dp; e += blockDim.x) {
         const int i = e / dp, j = e - i * dp;
-        A[i * ld + j] = i < da && j < da ? (float)Hl[i * da + j] : i == j ? 1.f : 0.f;
+        A[i * ld + j] = i < da && j < da ? Hpl[i * da + j].x : i == j ? 1.f : 0.f;
     }
     for (int a = tid; a < da; a += blockDim.x) {
         x[a] = 0.0;
         r[a] = G[a * L + l];
     }
     __syncthreads();
-    chol32(A, ld, dp, Dinv, &s_bad);
+    chol32(A, ld, dp, Dinv, v, &s_bad);   // v: scratch until the first solve
     // groups of da threads share a residual: group q sums columns q, q + ng, ..
     const int ng = min(4, (int)blockDim.x / da), grp = tid / da, ra = tid - grp * da;
-    bool done = false;
-    float before = 3.0e38f;
-    for (int it = 0; it < 12 && !done && !s_bad; ++it) {
+    bool done = false, fp64 = false;
+    float before = 3.0e38f, rate = 0.f;   // rate: the largest factor between corrections seen
+    for (int it = 0; it < 16 && !done && !s_bad; ++it) {
         if (it > 0) {
-            if (grp < ng) {
+            if (grp < ng && fp64) {
                 double s = 0.0;
-                for (int j = grp; j < da; j += ng) s = fma(Hl[(int64_t)j * da + ra], x[j], s);
+#pragma unroll 16
+                for (int j = grp; j < da; j += ng) s = fma(Hl[j * da + ra], x[j], s);
                 part[grp * da + ra] = s;
+            } else if (grp < ng) {
+                float hi = 0.f, lo = 0.f;
+#pragma unroll 16
+                for (int j = grp; j < da; j += ng) {
+                    const float2 h = Hpl[j * da + ra], xj = xp[j];
+                    const float p = __fmul_rn(h.x, xj.x);
+                    lo = __fadd_rn(lo, fmaf(h.x, xj.y, fmaf(h.y, xj.x, fmaf(h.x, xj.x, -p))));
+                    pair_add(hi, lo, p);
+                }
+                part[grp * da + ra] = (double)hi + (double)lo;
             }
             __syncthreads();
-            for (int a = tid; a < da; a += blockDim.x) {
-                double s = part[a];
-                for (int q = 1; q < ng; ++q) s += part[q * da + a];
-                r[a] = G[a * L + l] - s;
+            if (tid < da) {
+                double s = part[tid];
+                for (int q = 1; q < ng; ++q) s += part[q * da + tid];
+                r[tid] = G[tid * L + l] - s;
             }
         }
         // the residual scaled by a power of two into FP32's range
         if (tid == 0) s_dmax = s_xmax = 0u;
-        for (int a = tid; a < da; a += blockDim.x) atomicMax(&s_rexp, (__double2hiint(r[a]) >> 20) & 0x7ff);
+        if (tid < dp) {   // dp is a multiple of 32: whole warps
+            const unsigned e = tid < da ? (__double2hiint(r[tid]) >> 20) & 0x7ff : 0u;
+            const unsigned m = __reduce_max_sync(0xffffffffu, e);
+            if ((tid & 31) == 0) atomicMax(&s_rexp, (int)m);
+        }
         __syncthreads();
         const int re = s_rexp;
         if (re == 0 || re == 0x7ff) {   // zero (or below FP64's normal range): nothing left to correct
@@ -465,25 +501,43 @@ __global__ void __launch_bounds__(kSolveThreads) newton_solve_kernel(const doubl
             break;
         }
         const double up = __hiloint2double((2046 - re) << 20, 0), down = __hiloint2double(re << 20, 0);   // 2^-+(re - 1023)
-        for (int a = tid; a < dp; a += blockDim.x) v[a] = a < da ? (float)(r[a] * up) : 0.f;
+        if (tid < dp) v[tid] = tid < da ? (float)(r[tid] * up) : 0.f;
         __syncthreads();
         solve32(A, ld, dp, Dinv, v);
-        for (int a = tid; a < da; a += blockDim.x) {
-            const double dx = (double)v[a] * down, xn = x[a] + dx;
-            x[a] = xn;
-            atomicMax(&s_dmax, __float_as_uint(fabsf((float)dx)));
-            atomicMax(&s_xmax, __float_as_uint(fabsf((float)xn)));
+        if (tid < dp) {
+            unsigned db = 0u, xb = 0u;
+            if (tid < da) {
+                const double dx = (double)v[tid] * down, xn = x[tid] + dx;
+                x[tid] = xn;
+                const float xh = (float)xn;
+                xp[tid] = make_float2(xh, (float)(xn - (double)xh));
+                db = __float_as_uint(fabsf((float)dx));
+                xb = __float_as_uint(fabsf(xh));
+            }
+            db = __reduce_max_sync(0xffffffffu, db);
+            xb = __reduce_max_sync(0xffffffffu, xb);
+            if ((tid & 31) == 0) {
+                atomicMax(&s_dmax, db);
+                atomicMax(&s_xmax, xb);
+            }
         }
         if (tid == 0) s_rexp = 0;
         __syncthreads();
-        // the error left is about dmax^2 / before; stop when that is below an
-        // ulp of x, give up when the corrections shrink by less than 4
+        // the error left is about rate dmax: switch to FP64 residuals where
+        // the pairs' own error comes near, stop when it is below an ulp of x,
+        // give up when the corrections shrink by less than 4
         const float dmax = __uint_as_float(s_dmax), xmax = __uint_as_float(s_xmax);
         if (!(dmax < 3.0e38f)) {
             if (tid == 0) s_bad = 1;
         } else if (it > 0) {
-            done = dmax <= 1.0e-16f * xmax || dmax * (dmax / before) <= 1.0e-16f * xmax;
-            if (!done && !(dmax <= 0.25f * before) && tid == 0) s_bad = 1;
+            if (!fp64 && before > 0.f) rate = fmaxf(rate, fminf(dmax / before, 1.f));
+            const float left = rate * dmax;
+            if (!fp64) {
+                fp64 = left <= 1.0e-9f * xmax;
+                if (!fp64 && !(dmax <= 0.25f * before) && tid == 0) s_bad = 1;
+            } else {
+                done = dmax <= 1.0e-16f * xmax || left <= 1.0e-16f * xmax;
+            }
         }
         before = dmax;
         __syncthreads();
@@ -529,20 +583,23 @@ int macro_f1(Workspace &ws, const float *X, int64_t n, int d, int64_t ldx, const
     const int64_t nblk = ceil_div(n_train, kEvalRows);
     const int ts = da > 64 ? 8 : 4;
     const int ntiles = upper_tiles(da, ts);
+    const int pitch = (da + ts - 1) / ts * ts;
     float *Xa = nullptr, *Ys = nullptr, *Z = nullptr, *Xt = nullptr, *Yt = nullptr, *St = nullptr;
     float *gp = nullptr, *hp = nullptr;
     double *W = nullptr, *G = nullptr, *H = nullptr;
+    float2 *Hp = nullptr;   // H as float pairs
     unsigned long long *cnt = nullptr;
     int *status = nullptr;
-    LNE_TRY(ws.get("eval.Xa", (size_t)(n_train * da), &Xa));
+    LNE_TRY(ws.get("eval.Xa", (size_t)(n_train * pitch), &Xa));
     LNE_TRY(ws.get("eval.Ys", (size_t)(n_train * L), &Ys));
     LNE_TRY(ws.get("eval.Z", (size_t)(n_train * L), &Z));
-    LNE_TRY(ws.get("eval.Xt", (size_t)(n_test * da), &Xt));
+    LNE_TRY(ws.get("eval.Xt", (size_t)(n_test * pitch), &Xt));
     LNE_TRY(ws.get("eval.Yt", (size_t)(n_test * L), &Yt));
     LNE_TRY(ws.get("eval.St", (size_t)(n_test * L), &St));
     LNE_TRY(ws.get("eval.W", (size_t)da * L, &W));
     LNE_TRY(ws.get("eval.G", (size_t)da * L, &G));
     LNE_TRY(ws.get("eval.H", (size_t)L * da * da, &H));
+    LNE_TRY(ws.get("eval.Hp", (size_t)L * da * da, &Hp));
     LNE_TRY(ws.get("eval.gp", (size_t)(nblk * da * L), &gp));
     LNE_TRY(ws.get("eval.hp", (size_t)nblk * L * ntiles * ts * ts, &hp));
     LNE_TRY(ws.get("eval.cnt", (size_t)3 * L, &cnt));
@@ -552,20 +609,20 @@ int macro_f1(Workspace &ws, const float *X, int64_t n, int d, int64_t ldx, const
     LNE_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), st));
     {
         LNE_TRACE("eval_gather", st);
-        gather_rows_kernel<<<egrid(n_train * da), 256, 0, st>>>(X, n, ldx, d, labels, L, train_idx, n_train, Xa, Ys,
-                                                                status);
+        gather_rows_kernel<<<egrid(n_train * pitch), 256, 0, st>>>(X, n, ldx, d, labels, L, train_idx, n_train, pitch,
+                                                                   Xa, Ys, status);
         LNE_LAUNCH_CHECK();
-        gather_rows_kernel<<<egrid(n_test * da), 256, 0, st>>>(X, n, ldx, d, labels, L, test_idx, n_test, Xt, Yt,
-                                                               status);
+        gather_rows_kernel<<<egrid(n_test * pitch), 256, 0, st>>>(X, n, ldx, d, labels, L, test_idx, n_test, pitch, Xt,
+                                                                  Yt, status);
         LNE_LAUNCH_CHECK();
     }
     const int threads = (std::max(ntiles, da) + 31) / 32 * 32;   // at most 224 (da = 160: 210 tiles)
-    const int hsmem = 2 * kEvalStage * ((da + ts - 1) / ts * ts) * 4;
+    const int hsmem = 2 * kEvalStage * pitch * 4;
     const dim3 hgrid((unsigned)nblk, (unsigned)L);
     const dim3 rgrid((unsigned)ceil_div((int64_t)ntiles * ts * ts + da, 256), (unsigned)L);
     LNE_TRY(allow_dynamic_smem(newton_solve_kernel));
     for (int it = 0; it < iters; ++it) {
-        LNE_TRY(right_multiply(Xa, n_train, da, da, W, L, L, nullptr, Z, L, st));
+        LNE_TRY(right_multiply(Xa, n_train, da, pitch, W, L, L, nullptr, Z, L, st));
         {
             LNE_TRACE("newton_partials", st);
             if (ts == 8)
@@ -579,18 +636,18 @@ int macro_f1(Workspace &ws, const float *X, int64_t n, int d, int64_t ldx, const
         {
             LNE_TRACE("newton_sums", st);
             if (ts == 8)
-                newton_reduce_kernel<8><<<rgrid, 256, 0, st>>>(gp, hp, (int)nblk, da, L, ntiles, W, G, H);
+                newton_reduce_kernel<8><<<rgrid, 256, 0, st>>>(gp, hp, (int)nblk, da, L, ntiles, W, G, H, Hp);
             else
-                newton_reduce_kernel<4><<<rgrid, 256, 0, st>>>(gp, hp, (int)nblk, da, L, ntiles, W, G, H);
+                newton_reduce_kernel<4><<<rgrid, 256, 0, st>>>(gp, hp, (int)nblk, da, L, ntiles, W, G, H, Hp);
             LNE_LAUNCH_CHECK();
         }
         {
             LNE_TRACE("newton_solve", st);
-            newton_solve_kernel<<<L, kSolveThreads, solve_smem(da), st>>>(H, G, da, L, W, status);
+            newton_solve_kernel<<<L, kSolveThreads, solve_smem(da), st>>>(H, Hp, G, da, L, W, status);
             LNE_LAUNCH_CHECK();
         }
     }
-    LNE_TRY(right_multiply(Xt, n_test, da, da, W, L, L, nullptr, St, L, st));
+    LNE_TRY(right_multiply(Xt, n_test, da, pitch, W, L, L, nullptr, St, L, st));
     {
         LNE_TRACE("topk_f1", st);
         topk_f1_kernel<<<egrid(n_test), 256, 0, st>>>(St, Yt, n_test, L, cnt);
