@@ -2,7 +2,7 @@
 //
 //   sketch         Omega = randn(n, c) from Philox4x32-10 words (Box-Muller).
 //   gram           G = Y^T Y to FP64 accuracy: per-CTA partial Grams over row
-//                  blocks in error-free float-pair arithmetic, summed in FP64
+//                  blocks in exact FP32 steps (float pairs), summed in FP64
 //                  in a fixed order so the result is reproducible.
 //   chol           G = R^T R (upper Cholesky) in FP64, one CTA.
 //   trsm_rows      Q = Y R^-1 by forward substitution per row (FP32): each
@@ -62,28 +62,91 @@ __global__ void sketch_kernel(int64_t n, int c, uint32_t k0, uint32_t k1, float 
 
 // ---------------------------------------------------------------------------
 // Gram with FP64 accuracy from FP32 arithmetic: thread (ti, tj, half), ti <= tj,
-// owns 4 rows of an 8x8 tile of the upper half. Every product a*b is split exactly into
-// p + e (p = fl(a b), e = fma(a, b, -p)); p enters a float pair (hi, lo) by
-// an error-free two-sum, e and the two-sum's error go to lo. The pair carries
-// ~46 significant bits over a CTA's rows; CTAs are summed in FP64. FP64
-// arithmetic runs at a small fraction of the FP32 rate on this GPU, so this
-// is several times faster than FP64 FMAs. The _rn intrinsics keep the
-// compiler from contracting the error-free transformations.
+// owns 4 rows of an 8x8 tile of the upper half. FP64 arithmetic runs at 1/64 of
+// the FP32 rate on this GPU; four FP32 operations a product take its place:
+//
+//   Over a chunk of 64 rows entry (a, b) is accumulated in h, which starts at
+//   C = 3 u_a u_b, u the power of two above the column's norm over the chunk.
+//   |sum| <= u_a u_b keeps h inside [2, 4] u_a u_b, so every h <- h + a b is
+//   rounded to the same grid and h_old - h is exact; the rounding error
+//   a b + (h_old - h), one fma, goes to lo. (A general two-sum, which needs no
+//   such bound, takes ten operations.)
+//   After the chunk h - C (exact) and lo enter the entry's float pair by an
+//   error-free addition; CTAs are summed in FP64.
+//
+// h's grid is 2^-22 u_a u_b and lo keeps 24 bits below it, so the sum is good to
+// about 2^-44 of the column norms' product. Bound by the FP32 pipe (4 n c^2 / 2
+// operations a product, issued as packed pairs). Measured (n = 1e6, c = 144):
+// 4.5 ms with two-sums, 1.65 ms here, 78% of the FP32 pipe's rate; n = 10,312:
+// 64 -> 37 us.
+// The _rn intrinsics keep the compiler from contracting what has to be exact.
 // ---------------------------------------------------------------------------
-constexpr int kGramRows = 32;   // rows staged per step
+constexpr int kGramRows = 64;   // rows of a chunk (two buffers of them are staged)
 
 constexpr int kGramThreads = 384;
 
+__device__ __forceinline__ float2 f2_add(float2 a, float2 b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;"
+        : "=l"(d)
+        : "l"(reinterpret_cast<const uint64_t &>(a)), "l"(reinterpret_cast<const uint64_t &>(b)));
+    return reinterpret_cast<const float2 &>(d);
+}
+__device__ __forceinline__ float2 f2_sub(float2 a, float2 b) {
+    uint64_t d;
+    asm("sub.rn.f32x2 %0, %1, %2;"
+        : "=l"(d)
+        : "l"(reinterpret_cast<const uint64_t &>(a)), "l"(reinterpret_cast<const uint64_t &>(b)));
+    return reinterpret_cast<const float2 &>(d);
+}
+
+// C of an entry: 3 u_a u_b, or 0 where that is not finite (h then is a plain
+// running sum and lo collects what it rounds off).
+__device__ __forceinline__ float gram_shift(float ua, float ub) {
+    const float c = 3.0f * (ua * ub);
+    return c < 3.0e38f ? c : 0.f;
+}
+
+// VEC: rows are read by 16-byte copies (c, ld multiples of 4, Y 16-byte aligned).
+template <bool VEC>
 __global__ void __launch_bounds__(kGramThreads) gram_partial_kernel(const float *__restrict__ Y, int64_t n, int c,
                                                                     int64_t ld, int64_t rows_per_cta,
                                                                     double *__restrict__ partial) {
-    extern __shared__ float ys[];   // kGramRows x cp
+    // two chunks of kGramRows x cp, u of every column, then the threads' entry
+    // pairs (hi and lo of 4 x 8 entries, touched once a chunk)
+    extern __shared__ __align__(16) float ys[];
     const int cp = (c + 7) & ~7;
     const int nt = cp / 8;
     const int nitems = nt * (nt + 1);   // (tile, half): rows 0-3 or 4-7 of an 8x8 tile
     const int tid = threadIdx.x;
+    float *us = ys + 2 * kGramRows * cp;
+    float2 *acc = reinterpret_cast<float2 *>(us + cp) + tid;   // entry pair q: hi at q, lo at 16 + q (x kGramThreads)
     const int64_t r0 = (int64_t)blockIdx.x * rows_per_cta;
     const int64_t r1 = imin64(n, r0 + rows_per_cta);
+    for (int e = tid; e < 2 * kGramRows * (cp - c); e += kGramThreads) {   // padding columns
+        const int r = e / (cp - c);
+        ys[r * cp + c + (e - r * (cp - c))] = 0.f;
+    }
+    auto stage = [&](int64_t base, float *to) {
+        const int rows = (int)imin64(kGramRows, r1 - base);
+        if (VEC) {
+            const int q = c / 4;
+            for (int e = tid; e < rows * q; e += kGramThreads) {
+                const int r = e / q, k = e - r * q;
+                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(to + r * cp + 4 * k);
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(Y + (base + r) * ld + 4 * k)
+                             : "memory");
+            }
+        } else {
+            for (int e = tid; e < rows * c; e += kGramThreads) {
+                const int r = e / c, k = e - r * c;
+                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(to + r * cp + k);
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(Y + (base + r) * ld + k)
+                             : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
     // items are processed in groups of kGramThreads (uniform trip count for the barriers)
     for (int g0 = 0; g0 < nitems; g0 += kGramThreads) {
         const int item = g0 + tid;
@@ -99,51 +162,94 @@ __global__ void __launch_bounds__(kGramThreads) gram_partial_kernel(const float 
             tj = ti + rem;
         }
         const int xa = ti * 8 + half * 4;
-        float hi[4][8], lo[4][8];
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 8; ++b) hi[a][b] = lo[a][b] = 0.f;
-        for (int64_t base = r0; base < r1; base += kGramRows) {
+        for (int q = 0; q < 32; ++q) acc[q * kGramThreads] = make_float2(0.f, 0.f);
+        __syncthreads();   // the last group's chunks are done
+        if (r0 < r1) stage(r0, ys);
+        int buf = 0;
+        for (int64_t base = r0; base < r1; base += kGramRows, buf ^= 1) {
             const int rows = (int)imin64(kGramRows, r1 - base);
-#pragma unroll 4
-            for (int e = tid; e < kGramRows * cp; e += kGramThreads) {
-                int rr = e / cp, cc = e - rr * cp;
-                ys[e] = (rr < rows && cc < c) ? Y[(base + rr) * ld + cc] : 0.f;
+            const float *yb = ys + buf * (kGramRows * cp);
+            if (base + kGramRows < r1) {
+                stage(base + kGramRows, ys + (buf ^ 1) * (kGramRows * cp));
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            __syncthreads();
+            if (tid < cp) {   // u: a power of two above the norm of column tid
+                float s = 0.f;
+#pragma unroll 8
+                for (int r = 0; r < rows; ++r) s = fmaf(yb[r * cp + tid], yb[r * cp + tid], s);
+                // s (1 + 2^-10) in [2^E, 2^(E+1)): its root is below 2^(floor(E / 2) + 1)
+                const int E = (int)((__float_as_uint(s * 1.0009765625f) >> 23) & 0xFF) - 127;
+                us[tid] = s > 0.f ? __uint_as_float((uint32_t)((E >> 1) + 1 + 127) << 23) : 0.f;
             }
             __syncthreads();
             if (active) {
-                for (int rr = 0; rr < rows; ++rr) {
-                    const float *yr = ys + rr * cp;
-                    float av[4], bv[8];
+                float2 h[4][4], l[4][4];
+                float2 ub[4];
 #pragma unroll
-                    for (int t = 0; t < 4; ++t) av[t] = yr[xa + t];
+                for (int y = 0; y < 4; ++y) ub[y] = *reinterpret_cast<const float2 *>(us + tj * 8 + 2 * y);
 #pragma unroll
-                    for (int t = 0; t < 8; ++t) bv[t] = yr[tj * 8 + t];
+                for (int x = 0; x < 4; ++x) {
+                    const float ua = us[xa + x];
 #pragma unroll
-                    for (int x = 0; x < 4; ++x)
+                    for (int y = 0; y < 4; ++y) {
+                        h[x][y] = make_float2(gram_shift(ua, ub[y].x), gram_shift(ua, ub[y].y));
+                        l[x][y] = make_float2(0.f, 0.f);
+                    }
+                }
+#pragma unroll 2
+                for (int r = 0; r < rows; ++r) {
+                    const float *yr = yb + r * cp;
+                    const float4 a4 = *reinterpret_cast<const float4 *>(yr + xa);
+                    const float4 b0 = *reinterpret_cast<const float4 *>(yr + tj * 8);
+                    const float4 b1 = *reinterpret_cast<const float4 *>(yr + tj * 8 + 4);
+                    const float av[4] = {a4.x, a4.y, a4.z, a4.w};
+                    const float2 bv[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y),
+                                          make_float2(b1.z, b1.w)};
 #pragma unroll
-                        for (int y = 0; y < 8; ++y) {
-                            const float p = __fmul_rn(av[x], bv[y]);
-                            const float e = fmaf(av[x], bv[y], -p);
-                            const float h = hi[x][y];
-                            const float s = __fadd_rn(h, p);
-                            const float bb = __fsub_rn(s, h);
-                            const float err = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-                            hi[x][y] = s;
-                            lo[x][y] = __fadd_rn(lo[x][y], __fadd_rn(err, e));
+                    for (int x = 0; x < 4; ++x) {
+                        const float2 a2 = make_float2(av[x], av[x]);
+#pragma unroll
+                        for (int y = 0; y < 4; ++y) {
+                            float2 hn = h[x][y];
+                            f2_add_prod(hn, a2, bv[y]);
+                            float2 e = f2_sub(h[x][y], hn);   // exact: both on the chunk's grid
+                            f2_add_prod(e, a2, bv[y]);        // what the addition rounded off
+                            l[x][y] = f2_add(l[x][y], e);
+                            h[x][y] = hn;
                         }
+                    }
+                }
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const float ua = us[xa + x];
+#pragma unroll
+                    for (int y = 0; y < 4; ++y) {
+                        const float2 sh = make_float2(gram_shift(ua, ub[y].x), gram_shift(ua, ub[y].y));
+                        const float2 v = f2_sub(h[x][y], sh);   // exact
+                        float2 *at = acc + (x * 4 + y) * kGramThreads;
+                        const float2 o = at[0], s = f2_add(o, v), bb = f2_sub(s, o);
+                        const float2 err = f2_add(f2_sub(o, f2_sub(s, bb)), f2_sub(v, bb));
+                        at[0] = s;
+                        at[16 * kGramThreads] = f2_add(at[16 * kGramThreads], f2_add(err, l[x][y]));
+                    }
                 }
             }
-            __syncthreads();
+            __syncthreads();   // this buffer and u are rewritten next
         }
         if (active) {
             double *P = partial + (int64_t)blockIdx.x * cp * cp;
 #pragma unroll
             for (int x = 0; x < 4; ++x)
 #pragma unroll
-                for (int y = 0; y < 8; ++y)
-                    P[(xa + x) * cp + tj * 8 + y] = (double)hi[x][y] + (double)lo[x][y];
+                for (int y = 0; y < 4; ++y) {
+                    const float2 hi = acc[(x * 4 + y) * kGramThreads], lo = acc[(16 + x * 4 + y) * kGramThreads];
+                    P[(xa + x) * cp + tj * 8 + 2 * y] = (double)hi.x + (double)lo.x;
+                    P[(xa + x) * cp + tj * 8 + 2 * y + 1] = (double)hi.y + (double)lo.y;
+                }
         }
     }
 }
@@ -404,53 +510,160 @@ __global__ void __launch_bounds__(256, 1) chol_coop_kernel(double *__restrict__ 
     }
 }
 
-// Q = Y R^-1 for upper-triangular R (FP64, rounded to FP32): one warp per row
-// solves q R = y by forward substitution; lane l keeps the running sums of
-// columns l, l + 32, ...
-constexpr int kTrsmThreads = 512;   // 16 rows in flight per CTA (measured: 256 -> 512 threads, 15% faster)
+// Q = Y R^-1 for upper-triangular R (FP64, rounded to FP32): forward
+// substitution per row, q_l = (y_l - q_0 R_0l - .. - q_(l-1) R_(l-1)l) / R_ll with
+// the terms subtracted in that order. A warp owns 32 RPT rows, a lane the rows
+// lane and lane + 32, and takes their columns in blocks of 16: the terms of all
+// columns before the block are a small matrix product (the rows' earlier q from
+// shared memory, stored negated and by column; R's 16 entries of a row
+// broadcast), then the block's own triangle is solved in registers. Blocks of Y
+// and Q pass through a warp's staging rows, so that four lanes read or write a
+// row's 64 bytes together; the next block's loads are in flight meanwhile.
+// Per earlier column and RPT = 2: 6 shared-memory wavefronts for 32 FMAs a
+// thread, so the FP32 pipe bounds it (n c^2 / 2 FMAs). Measured (n = 1e6,
+// c = 144): 3.5 -> 0.73 ms; with a warp a row, a shuffle and c / 32 predicated
+// FMAs per column, most issue slots went to neither. One warp a scheduler (R and
+// the q of 256 rows fill shared memory), so latencies show: about half the
+// FP32 rate.
+constexpr int kTrsmB = 16;
+constexpr int kTrsmPitch = kTrsmB + 4;   // floats a staging row: 8 lanes' 16-byte accesses hit all banks once
 
-template <int NT>
-__global__ void __launch_bounds__(kTrsmThreads) trsm_rows_kernel(const float *__restrict__ Y, int64_t n, int c, int64_t ldy,
+// floats of R's column blocks before block b: block b holds the rows 0 .. 16 b + 15
+__host__ __device__ inline int trsm_block_at(int b) { return 128 * b * (b + 1); }
+inline int trsm_smem(int c, int tile_rows) {
+    const int nb = (c + kTrsmB - 1) / kTrsmB;
+    return (trsm_block_at(nb) + nb * kTrsmB + tile_rows * kTrsmPitch + (nb - 1) * kTrsmB * tile_rows) * 4;
+}
+
+// VEC: 16-byte accesses to Y and Q (c, ldy, ldq multiples of 4, both aligned).
+template <int RPT, bool VEC>
+__global__ void __launch_bounds__(128) trsm_rows_kernel(const float *__restrict__ Y, int64_t n, int c, int64_t ldy,
                                                         const double *__restrict__ R, float *__restrict__ Q,
                                                         int64_t ldq) {
-    extern __shared__ float Rs[];   // c x c, row-major, plus the reciprocal diagonal
-    float *rdiag = Rs + c * c;
-    // staged 8 loads at a time per thread: independent loads in flight instead
-    // of one L2 round trip per element
+    // R by column blocks, reciprocal diagonal, staging rows, -q by column
+    extern __shared__ __align__(16) float Rs[];
+    constexpr int WR = 32 * RPT, ITS = WR / 8;   // rows of a warp; its 16-byte accesses a lane and block
+    const int nb = (c + kTrsmB - 1) / kTrsmB, tile = blockDim.x * RPT, tid = threadIdx.x, lane = tid & 31;
+    const int wrow = (tid >> 5) * WR;            // the warp's first row in the tile
+    float *rdiag = Rs + trsm_block_at(nb), *stg = rdiag + nb * kTrsmB + wrow * kTrsmPitch;
+    float *qs = rdiag + nb * kTrsmB + tile * kTrsmPitch + wrow;
+    for (int b = 0; b < nb; ++b) {
+        float *to = Rs + trsm_block_at(b);
+        // staged 8 loads at a time per thread: independent loads in flight
 #pragma unroll 8
-    for (int e = threadIdx.x; e < c * c; e += blockDim.x) Rs[e] = (float)__ldg(R + e);
-    for (int j = threadIdx.x; j < c; j += blockDim.x) rdiag[j] = (float)(1.0 / R[j * c + j]);
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
-        float y[NT], q[NT];
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {
-            const int cc = lane + 32 * t;
-            y[t] = cc < c ? Y[i * ldy + cc] : 0.f;
-            q[t] = 0.f;
+        for (int e = tid; e < (b + 1) * (kTrsmB * kTrsmB); e += blockDim.x) {
+            const int j = e / kTrsmB, l = b * kTrsmB + e % kTrsmB;
+            to[e] = j < c && l < c ? (float)__ldg(R + j * c + l) : 0.f;
         }
-        // column j: q_j = y_j * rdiag_j; then y_l -= q_j R[j][l] for l > j
+    }
+    for (int j = tid; j < nb * kTrsmB; j += blockDim.x) rdiag[j] = j < c ? (float)(1.0 / R[j * c + j]) : 0.f;
+    __syncthreads();
+    const int sr = lane >> 2, sc = 4 * (lane & 3);   // access it of a block: row 8 it + sr, columns sc .. sc + 3
+    // columns l0 + sc .. of the warp's rows from row w0 on (zeros past the rows or the matrix)
+    auto load = [&](int64_t w0, int l0, float4 (&v)[ITS]) {
 #pragma unroll
-        for (int t = 0; t < NT; ++t) {
-            for (int jj = 0; jj < 32; ++jj) {
-                const int j = 32 * t + jj;
-                if (j >= c) break;
-                const float qj = __shfl_sync(0xffffffffu, y[t], jj) * rdiag[j];
-                if (lane == jj) q[t] = qj;
-                const float *rj = Rs + j * c;
-#pragma unroll
-                for (int u = 0; u < NT; ++u) {
-                    const int l = lane + 32 * u;
-                    if (u >= t && l > j && l < c) y[u] = fmaf(-qj, rj[l], y[u]);
-                }
+        for (int it = 0; it < ITS; ++it) {
+            const int64_t i = w0 + 8 * it + sr;
+            const float *src = Y + i * ldy + l0 + sc;
+            const int left = i < n ? c - (l0 + sc) : 0;
+            if (VEC) {
+                v[it] = left > 0 ? *reinterpret_cast<const float4 *>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+            } else {
+                v[it].x = left > 0 ? src[0] : 0.f;
+                v[it].y = left > 1 ? src[1] : 0.f;
+                v[it].z = left > 2 ? src[2] : 0.f;
+                v[it].w = left > 3 ? src[3] : 0.f;
             }
         }
+    };
+    for (int64_t t0 = (int64_t)blockIdx.x * tile; t0 < n; t0 += (int64_t)gridDim.x * tile) {
+        const int64_t w0 = t0 + wrow;
+        if (w0 >= n) continue;   // whole warps
+        float4 nxt[ITS];
+        load(w0, 0, nxt);
+        for (int b = 0; b < nb; ++b) {
 #pragma unroll
-        for (int t = 0; t < NT; ++t) {
-            const int cc = lane + 32 * t;
-            if (cc < c) Q[i * ldq + cc] = q[t];
+            for (int it = 0; it < ITS; ++it)
+                *reinterpret_cast<float4 *>(stg + (8 * it + sr) * kTrsmPitch + sc) = nxt[it];
+            __syncwarp();
+            if (b + 1 < nb) load(w0, (b + 1) * kTrsmB, nxt);   // arrives during this block's work
+            float2 y[RPT][kTrsmB / 2];
+#pragma unroll
+            for (int p = 0; p < RPT; ++p)
+#pragma unroll
+                for (int q = 0; q < kTrsmB / 4; ++q) {
+                    const float4 x =
+                        *reinterpret_cast<const float4 *>(stg + (lane + 32 * p) * kTrsmPitch + 4 * q);
+                    y[p][2 * q] = make_float2(x.x, x.y);
+                    y[p][2 * q + 1] = make_float2(x.z, x.w);
+                }
+            const float *Rb = Rs + trsm_block_at(b);
+#pragma unroll 4
+            for (int j = 0; j < b * kTrsmB; ++j) {
+                float nq[RPT];
+#pragma unroll
+                for (int p = 0; p < RPT; ++p) nq[p] = qs[j * tile + lane + 32 * p];
+#pragma unroll
+                for (int q = 0; q < kTrsmB / 4; ++q) {
+                    const float4 r = *reinterpret_cast<const float4 *>(Rb + j * kTrsmB + 4 * q);
+#pragma unroll
+                    for (int p = 0; p < RPT; ++p) {
+                        f2_add_prod(y[p][2 * q], make_float2(nq[p], nq[p]), make_float2(r.x, r.y));
+                        f2_add_prod(y[p][2 * q + 1], make_float2(nq[p], nq[p]), make_float2(r.z, r.w));
+                    }
+                }
+            }
+            // the block's own triangle
+            const float *Rd = Rb + b * (kTrsmB * kTrsmB);
+            float v[RPT][kTrsmB];
+#pragma unroll
+            for (int p = 0; p < RPT; ++p)
+#pragma unroll
+                for (int q = 0; q < kTrsmB / 2; ++q) v[p][2 * q] = y[p][q].x, v[p][2 * q + 1] = y[p][q].y;
+#pragma unroll
+            for (int l = 0; l < kTrsmB; ++l) {
+                const float rd = rdiag[b * kTrsmB + l];
+#pragma unroll
+                for (int p = 0; p < RPT; ++p) v[p][l] *= rd;
+#pragma unroll
+                for (int q = (l + 1) / 4; q < kTrsmB / 4; ++q) {
+                    const float4 r4 = *reinterpret_cast<const float4 *>(Rd + l * kTrsmB + 4 * q);
+                    const float r[4] = {r4.x, r4.y, r4.z, r4.w};
+#pragma unroll
+                    for (int m = 4 * q; m < 4 * q + 4; ++m)
+#pragma unroll
+                        for (int p = 0; p < RPT; ++p)
+                            if (m > l) v[p][m] = fmaf(-v[p][l], r[m - 4 * q], v[p][m]);
+                }
+            }
+#pragma unroll
+            for (int p = 0; p < RPT; ++p) {
+                if (b + 1 < nb) {   // read back by this lane only
+#pragma unroll
+                    for (int l = 0; l < kTrsmB; ++l) qs[(b * kTrsmB + l) * tile + lane + 32 * p] = -v[p][l];
+                }
+#pragma unroll
+                for (int q = 0; q < kTrsmB; q += 4)   // rows of the staging that only this lane has read
+                    *reinterpret_cast<float4 *>(stg + (lane + 32 * p) * kTrsmPitch + q) =
+                        make_float4(v[p][q], v[p][q + 1], v[p][q + 2], v[p][q + 3]);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int it = 0; it < ITS; ++it) {
+                const int64_t i = w0 + 8 * it + sr;
+                const int l0 = b * kTrsmB + sc, left = i < n ? c - l0 : 0;
+                const float4 x = *reinterpret_cast<const float4 *>(stg + (8 * it + sr) * kTrsmPitch + sc);
+                float *dst = Q + i * ldq + l0;
+                if (VEC) {
+                    if (left > 0) *reinterpret_cast<float4 *>(dst) = x;
+                } else {
+                    if (left > 0) dst[0] = x.x;
+                    if (left > 1) dst[1] = x.y;
+                    if (left > 2) dst[2] = x.z;
+                    if (left > 3) dst[3] = x.w;
+                }
+            }
+            __syncwarp();   // the staging rows are rewritten next
         }
     }
 }
@@ -1571,27 +1784,21 @@ int right_multiply(const float *Y, int64_t n, int c, int64_t ldy, const double *
 // G = Y^T Y (FP64, [c][c]).
 static int gram(Workspace &ws, const float *Y, int64_t n, int c, int64_t ld, double *G, cudaStream_t st) {
     const int cp = (c + 7) & ~7;
-    const int nt = cp / 8;
-    const int ntiles = nt * (nt + 1) / 2;
-    (void)ntiles;
     const int threads = kGramThreads;
+    const bool vec = c % 4 == 0 && ld % 4 == 0 && reinterpret_cast<uintptr_t>(Y) % 16 == 0;
+    const int smem = (2 * kGramRows * cp + cp + 64 * kGramThreads) * 4;   // cp <= 240: 217 KB
+    LNE_TRY(vec ? allow_dynamic_smem(gram_partial_kernel<true>) : allow_dynamic_smem(gram_partial_kernel<false>));
     // whole waves of resident CTAs (one per SM at this kernel's register use)
-    int per_sm = 1;
-    LNE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gram_partial_kernel, threads,
-                                                             kGramRows * cp * 4));
-    const int64_t slots = num_sms() * (int64_t)std::max(1, per_sm);
-    int64_t nblk = std::min<int64_t>(2 * slots, std::max<int64_t>(1, ceil_div(n, 64)));
-    if (nblk > slots) nblk = (nblk / slots) * slots;
+    const int64_t slots = num_sms();
+    int64_t nblk = std::min<int64_t>(slots, std::max<int64_t>(1, ceil_div(n, 32)));
     const int64_t rows_per = ceil_div(std::max<int64_t>(n, 1), nblk);
     nblk = ceil_div(std::max<int64_t>(n, 1), rows_per);
     double *partial = nullptr;
     LNE_TRY(ws.get("gram.partial", (size_t)nblk * cp * cp, &partial));
-    const int smem = kGramRows * cp * 4;
-    if (smem > 48 * 1024)
-        LNE_TRY(allow_dynamic_smem(gram_partial_kernel));
     {
         LNE_TRACE("gram_partial", st);
-        gram_partial_kernel<<<(unsigned)nblk, threads, smem, st>>>(Y, n, c, ld, rows_per, partial);
+        if (vec) gram_partial_kernel<true><<<(unsigned)nblk, threads, smem, st>>>(Y, n, c, ld, rows_per, partial);
+        else gram_partial_kernel<false><<<(unsigned)nblk, threads, smem, st>>>(Y, n, c, ld, rows_per, partial);
         LNE_LAUNCH_CHECK();
     }
     {
@@ -1659,35 +1866,30 @@ int status_check(Workspace &ws, cudaStream_t st) {
     return fail(LNE_ERR_NUMERIC, "Cholesky breakdown in CholeskyQR (Gram not positive definite)");
 }
 
+// Rows a tile: 256 (two a thread) where the earlier columns of that many fit in
+// shared memory beside R (c <= 144) and there are enough rows to give every SM
+// such a tile; else 128, else 64 (c up to 240).
 static int trsm_rows(const float *Y, int64_t n, int c, int64_t ldy, const double *R, float *Q, int64_t ldq,
                      cudaStream_t st) {
-    const int nt = (c + 31) / 32;
-    const int smem = (c * c + c) * 4;
-    // every CTA stages R in shared memory: one wave of resident CTAs, each
-    // walking many rows, loads it the fewest times
-    const int per_sm = std::max(1, std::min(8, (227 * 1024) / std::max(smem, 1)));
-    const int blocks = (int)std::min<int64_t>(ceil_div(n, 8), num_sms() * per_sm);
+    constexpr int kMost = 226 * 1024;
+    const bool vec = c % 4 == 0 && ldy % 4 == 0 && ldq % 4 == 0 && reinterpret_cast<uintptr_t>(Y) % 16 == 0 &&
+                     reinterpret_cast<uintptr_t>(Q) % 16 == 0;
     LNE_TRACE("trsm_rows", st);
-#define LNE_TRSM_CASE(K)                                                                               \
-    case K:                                                                                            \
-        if (smem > 48 * 1024) LNE_TRY(allow_dynamic_smem(trsm_rows_kernel<K>));                        \
-        trsm_rows_kernel<K><<<blocks, kTrsmThreads, smem, st>>>(Y, n, c, ldy, R, Q, ldq);                      \
-        break;
-    switch (nt) {
-        LNE_TRSM_CASE(1)
-        LNE_TRSM_CASE(2)
-        LNE_TRSM_CASE(3)
-        LNE_TRSM_CASE(4)
-        LNE_TRSM_CASE(5)
-        LNE_TRSM_CASE(6)
-        LNE_TRSM_CASE(7)
-        LNE_TRSM_CASE(8)
-        default:
-            return fail(LNE_ERR_UNSUPPORTED, "CholeskyQR supports at most 256 columns");
-    }
-#undef LNE_TRSM_CASE
-    LNE_LAUNCH_CHECK();
-    return 0;
+    auto launch = [&](auto kernel, int threads, int rpt) -> int {
+        const int tile = threads * rpt, smem = trsm_smem(c, tile);
+        LNE_TRY(allow_dynamic_smem(kernel));
+        const int per_sm = std::max(1, std::min(8, kMost / smem));
+        const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(n, tile), (int64_t)num_sms() * per_sm);
+        kernel<<<blocks, threads, smem, st>>>(Y, n, c, ldy, R, Q, ldq);
+        LNE_LAUNCH_CHECK();
+        return 0;
+    };
+    if (trsm_smem(c, 256) <= kMost && n >= (int64_t)num_sms() * 256)
+        return vec ? launch(trsm_rows_kernel<2, true>, 128, 2) : launch(trsm_rows_kernel<2, false>, 128, 2);
+    int threads = 128;
+    while (threads > 32 && (trsm_smem(c, threads) > kMost || n < (int64_t)num_sms() * threads)) threads /= 2;
+    if (trsm_smem(c, threads) > kMost) return fail(LNE_ERR_UNSUPPORTED, "CholeskyQR column count too large");
+    return vec ? launch(trsm_rows_kernel<1, true>, threads, 1) : launch(trsm_rows_kernel<1, false>, threads, 1);
 }
 
 int cholqr1(Workspace &ws, const float *Y, int64_t n, int c, int64_t ld, float *Q, int64_t ldq, cudaStream_t st) {
