@@ -880,33 +880,49 @@ __global__ void jacobi32_kernel(const double *__restrict__ R, int c, double *__r
     if (tid == 0 && sweeps_out) *sweeps_out = sweep;
 }
 
-// Register-resident variant of the same Jacobi (c <= 144). Each 8-thread
-// group holds its pair of columns of A in registers (E elements per column
-// and thread, as float2 chunks: element 16 q + 2 sub + {0, 1}), so a round
-// reads nothing from shared memory; columns move between groups through a
-// shared exchange buffer only when the pairing changes. The rotations W are
-// not accumulated here: every round's (cos, sin) and column labels are
-// recorded, and jacobi_replay_kernel applies them to the identity afterwards,
-// one row of W per warp on many SMs (the rows of W evolve independently).
+// Register-resident variant of the same Jacobi (c <= 144). The columns go in
+// blocks of two; each 8-thread group holds a pair of blocks in registers (E
+// elements per column and thread, as float2 chunks: element 16 q + 2 sub +
+// {0, 1}) and makes the four rotations between them, two at a time, before the
+// blocks move on through a shared exchange buffer. The rotations W are not
+// accumulated here: every rotation's (cos, sin) and column labels are recorded,
+// and jacobi_replay_kernel applies them to the identity afterwards, one row of W
+// per warp on many SMs (the rows of W evolve independently).
 //
-// The pairing order is chosen so that most rounds move one column of each
-// pair instead of both: a sweep over m = 2G columns takes the columns in slot
+// The order of the block pairs is chosen so that most rounds move one block of
+// each pair instead of both: a sweep over m = 2G blocks takes the blocks in slot
 // 0 as a set X and those in slot 1 as Y, and pairs X[i] with Y[(i + r) mod G]
 // for r = 0..G-1 (only Y moves, one group along); then X and Y are each split
 // in halves and the same is done inside X and inside Y in parallel, and so on
 // while the set size is even. Sets of odd size s then finish with s rounds of
-// the circle method (one column of each set idle per round). Every pair meets
-// exactly once per sweep; the layout a sweep ends with is the next sweep's
-// starting point, and a label per column records which column of R^T it
-// started as.
+// the circle method (one block of each set idle per round). Every pair of blocks
+// meets exactly once per sweep, the two columns of a block at its start; the
+// layout a sweep ends with is the next sweep's starting point, and a label per
+// column records which column of R^T it started as.
+//
+// One CTA, so a round is a chain: dot products, shuffles, the angle, the
+// update, the exchange. What shortens it: a rotation scales its columns lazily
+// (a0 <- a0 - t (d1 / d0) a1, a1 <- a1 + t (d0 / d1) a0, d <- cos d: one FMA an
+// entry) and keeps the squared norms up (only the dot product is formed: a
+// third of the sums and shuffles; both are refreshed at every level of a sweep,
+// two rounds' worth of work), and blocks of two halve the bytes that cross
+// shared memory per rotation, whose wavefronts (650 cycles a round of 72
+// columns of 144 entries, written and read) were the longest link with one
+// column a move. Straight-line code makes both rotations' chains overlap, with
+// one-instruction approximations where only the angle's quality depends on them.
+// Measured (start and replay of a random factor): c = 32 127 -> 90 us, c = 48
+// 211 -> 143, c = 128 990 -> 671, c = 144 1343 -> 1032 (0.25 us a round up to
+// c = 64, 0.68 at 144; the replay is 29 to 139 us of it).
 constexpr int kJacRegMaxC = 144;
 constexpr int kJacMaxSweeps = 20;
 
-template <int E>
-__host__ __device__ constexpr int jreg_stride() { return ((8 * E + 31) / 32) * 32 + 16; }
-
-// rounds per sweep of the order above for m (even) columns
-__host__ __device__ inline int jreg_rounds(int m) { return jorder_rounds(m); }
+// blocks of two columns, padded to an even number
+__host__ __device__ constexpr int jreg_blocks(int c) { return ((c + 1) / 2 + 1) / 2 * 2; }
+// floats of an exchange entry (two columns and their labels, norms and scales);
+// = 16 mod 32, so that neighbouring groups' float2 accesses hit distinct banks
+__host__ __device__ constexpr int jreg_stride(int E) { return 16 * E + 16; }
+// rounds of disjoint rotations per sweep for m blocks, m rotations each
+__host__ __device__ inline int jreg_rounds(int m) { return 2 * jorder_rounds(m) + 1; }
 
 // Paired FP32 arithmetic (fma.rn.f32x2 / mul.rn.f32x2, sm_100 and later):
 // one instruction for two lanes of a float2, each rounded as the scalar op.
@@ -926,8 +942,36 @@ __device__ __forceinline__ float2 f2_mul(float2 a, float2 b) {
     return *reinterpret_cast<const float2 *>(&d);
 }
 
+// Approximate square root, reciprocal and reciprocal square root (2 ulp or so),
+// denormals taken as zero: one instruction each.
+__device__ __forceinline__ float fast_sqrt(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float fast_rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float fast_rsqrt(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// One column of a group's pair of blocks: the calling thread's entries of it,
+// the column being scale * v, its squared norm, and the column of R^T it
+// started as.
 template <int E>
-__global__ void __launch_bounds__(32 * E, 1) jacobi_reg_kernel(const double *__restrict__ R, int c,
+struct JacCol {
+    float2 v[E / 2];
+    float nrm, scl;
+    int lab;
+};
+
+template <int E>
+__global__ void __launch_bounds__(16 * E, 1) jacobi_reg_kernel(const double *__restrict__ R, int c,
                                                                double *__restrict__ Vout,
                                                                float2 *__restrict__ rot,
                                                                uint32_t *__restrict__ rlab, int max_sweeps,
@@ -935,106 +979,176 @@ __global__ void __launch_bounds__(32 * E, 1) jacobi_reg_kernel(const double *__r
     constexpr int CP = 8 * E;            // padded column length
     constexpr int NQ = E / 2;            // float2 chunks per column and thread
     static_assert(E % 2 == 0, "columns are held as float2 chunks");
-    constexpr int ST = jreg_stride<E>(); // floats per exchange entry (= 16 mod 32: conflict-free float2)
-    extern __shared__ float xb[];        // 2 G entries: column [CP], label at CP
+    constexpr int ST = jreg_stride(E);   // floats per exchange entry: two columns, then their labels, norms, scales
+    extern __shared__ __align__(16) float xb[];   // 2 G entries
     __shared__ float red[32];
-    __shared__ int s_done;
-    const int m = c + (c & 1), G = m / 2, RD = jreg_rounds(m);
+    const int m = jreg_blocks(c), G = m / 2, SUB = jreg_rounds(m);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = tid >> 3, sub = tid & 7;
     const bool real = g < G;             // groups past G only fill the last warp
-    // element 2 q + t of a column is component t of chunk q (rows 16 q + 2 sub + t)
-    float2 a0[NQ], a1[NQ];
-    int lab0 = g, lab1 = g + G;
+    JacCol<E> A[2], B[2];                // the blocks in slots 0 and 1
+    float big = 0.f;
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const int i = 16 * q + 2 * sub;
-        const bool r0 = real && lab0 < c, r1 = real && lab1 < c;   // column lab of R^T
-        a0[q].x = r0 && i < c ? (float)R[(size_t)lab0 * c + i] : 0.f;
-        a0[q].y = r0 && i + 1 < c ? (float)R[(size_t)lab0 * c + i + 1] : 0.f;
-        a1[q].x = r1 && i < c ? (float)R[(size_t)lab1 * c + i] : 0.f;
-        a1[q].y = r1 && i + 1 < c ? (float)R[(size_t)lab1 * c + i + 1] : 0.f;
+    for (int k = 0; k < 4; ++k) {
+        JacCol<E> &x = k < 2 ? A[k & 1] : B[k & 1];
+        x.lab = 2 * (k < 2 ? g : g + G) + (k & 1);
+        x.nrm = 0.f;
+        const bool live = real && x.lab < c;   // column lab of R^T
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const int i = 16 * q + 2 * sub;
+            x.v[q].x = live && i < c ? (float)R[(size_t)x.lab * c + i] : 0.f;
+            x.v[q].y = live && i + 1 < c ? (float)R[(size_t)x.lab * c + i + 1] : 0.f;
+            big = fmaxf(big, fmaxf(fabsf(x.v[q].x), fabsf(x.v[q].y)));
+        }
     }
+    // scaled by a power of two so that the largest entry is in [1, 2): squares of
+    // squared norms stay in FP32's range, and nothing that is kept depends on it
+    big = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(big)));
+    if (lane == 0) red[warp] = big;
+    __syncthreads();
+    for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) big = fmaxf(big, red[w]);
+    const uint32_t bexp = __float_as_uint(big) >> 23;
+    const float unit = bexp >= 1 && bexp <= 253 ? __uint_as_float((254u - bexp) << 23) : 1.f;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) A[k].scl = B[k].scl = unit;   // multiplied in by the first renormalisation
     // stop at cosines of 0.4 c ulp (at least 8 ulp): the FP64 refinement's first-order
     // step needs the start's rotations this close where singular values are dense
     const float tol = fmaxf(0.4f * (float)c, 8.f) * 5.9604645e-8f;
     const int tz = jorder_levels(m);
     const int s_odd = m >> tz;           // set size the halving ends at
-    float local_max = 0.f;
-    int rec = 0;                         // record index of this round's group 0
+    const float tol2 = tol * tol;
+    bool rotated = false;                // a pair above the tolerance in this sweep
+    size_t rec = 0;                      // this round's first record
 
-    auto put = [&](int entry, const float2 (&a)[NQ], int lab) {
+    auto put = [&](int entry, const JacCol<E> (&x)[2]) {
         float *eb = xb + (size_t)entry * ST;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) *reinterpret_cast<float2 *>(eb + 16 * q + 2 * sub) = a[q];
-        if (sub == 0) reinterpret_cast<int *>(eb)[CP] = lab;
+        for (int k = 0; k < 2; ++k) {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) *reinterpret_cast<float2 *>(eb + k * CP + 16 * q + 2 * sub) = x[k].v[q];
+            if (sub == k)
+                *reinterpret_cast<float4 *>(eb + 2 * CP + 4 * k) =
+                    make_float4(__int_as_float(x[k].lab), x[k].nrm, x[k].scl, 0.f);
+        }
     };
-    auto take = [&](int entry, float2 (&a)[NQ], int &lab) {
+    auto take = [&](int entry, JacCol<E> (&x)[2]) {
         const float *eb = xb + (size_t)entry * ST;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) a[q] = *reinterpret_cast<const float2 *>(eb + 16 * q + 2 * sub);
-        lab = reinterpret_cast<const int *>(eb)[CP];
+        for (int k = 0; k < 2; ++k) {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) x[k].v[q] = *reinterpret_cast<const float2 *>(eb + k * CP + 16 * q + 2 * sub);
+            const float4 t = *reinterpret_cast<const float4 *>(eb + 2 * CP + 4 * k);
+            x[k].lab = __float_as_int(t.x);
+            x[k].nrm = t.y;
+            x[k].scl = t.z;
+        }
     };
-    // both columns of every group move (sources as group * 2 + slot)
+    // both blocks of every group move (sources as group * 2 + slot)
     auto move_both = [&](int src0, int src1) {
         __syncthreads();
         if (real) {
-            put(2 * g, a0, lab0);
-            put(2 * g + 1, a1, lab1);
+            put(2 * g, A);
+            put(2 * g + 1, B);
         }
         __syncthreads();
         if (real) {
-            take(src0, a0, lab0);
-            take(src1, a1, lab1);
+            take(src0, A);
+            take(src1, B);
         }
         __syncthreads();
     };
-    // one rotation of the group's pair (every lane takes part in the shuffles),
-    // recorded as (cos, sin) = (1, 0) when the pair is left as it is
-    auto rotate = [&](bool active) {
-        float2 al2 = make_float2(0.f, 0.f), be2 = al2, ga2 = al2;
+    // scales multiplied in, squared norms from the entries
+    auto renorm = [&](JacCol<E> &x) {
+        float2 n2 = make_float2(0.f, 0.f);
+        const float2 d = make_float2(x.scl, x.scl);
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
-            al2 = f2_fma(a0[q], a0[q], al2);
-            be2 = f2_fma(a1[q], a1[q], be2);
-            ga2 = f2_fma(a0[q], a1[q], ga2);
+            x.v[q] = f2_mul(d, x.v[q]);
+            n2 = f2_fma(x.v[q], x.v[q], n2);
         }
-        float al = al2.x + al2.y, be = be2.x + be2.y, ga = ga2.x + ga2.y;
+        float n = n2.x + n2.y;
+#pragma unroll
+        for (int off = 1; off < 8; off <<= 1) n += __shfl_xor_sync(0xffffffffu, n, off);
+        x.nrm = n;
+        x.scl = 1.f;
+    };
+    auto renorm_all = [&]() {
+        renorm(A[0]);
+        renorm(A[1]);
+        renorm(B[0]);
+        renorm(B[1]);
+    };
+    // one round: the rotations of the pairs (x0, y0) and (x1, y1), recorded as
+    // (cos, sin) = (1, 0) where a pair is left as it is. Straight-line code for
+    // both pairs at once, so that their chains overlap; t = tan of the angle
+    // = 2 g / (d + sign(d) sqrt(d^2 + 4 g^2)) for the dot product g and the squared
+    // norms' difference d. It only steers the convergence (approximate sqrt and
+    // division); (cos, sin) is a unit vector.
+    auto rotate = [&](JacCol<E> &x0, JacCol<E> &y0, JacCol<E> &x1, JacCol<E> &y1, bool active) {
+        JacCol<E> *const xs[2] = {&x0, &x1}, *const ys[2] = {&y0, &y1};
+        float ga[2], t[2], cs[2], r[2], ri[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            float2 a = make_float2(0.f, 0.f), b = a;
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                if (q & 1) b = f2_fma(xs[k]->v[q], ys[k]->v[q], b);
+                else a = f2_fma(xs[k]->v[q], ys[k]->v[q], a);
+            }
+            ga[k] = (a.x + a.y) + (b.x + b.y);
+            r[k] = ys[k]->scl * fast_rcp(xs[k]->scl);
+            ri[k] = xs[k]->scl * fast_rcp(ys[k]->scl);
+        }
 #pragma unroll
         for (int off = 1; off < 8; off <<= 1) {
-            al += __shfl_xor_sync(0xffffffffu, al, off);
-            be += __shfl_xor_sync(0xffffffffu, be, off);
-            ga += __shfl_xor_sync(0xffffffffu, ga, off);
+            ga[0] += __shfl_xor_sync(0xffffffffu, ga[0], off);
+            ga[1] += __shfl_xor_sync(0xffffffffu, ga[1], off);
         }
-        float cs = 1.f, sn = 0.f;
-        if (active && ga != 0.f && al > 0.f && be > 0.f) {
-            const float rel = fabsf(ga) * rsqrtf(al * be);
-            local_max = fmaxf(local_max, rel);
-            if (rel > tol) {
-                const float zeta = (be - al) / (2.f * ga);
-                const float t = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
-                cs = rsqrtf(1.f + t * t);
-                sn = cs * t;
-                const float2 c2 = make_float2(cs, cs), s2 = make_float2(sn, sn), ms2 = make_float2(-sn, -sn);
 #pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    const float2 x = a0[q], y = a1[q];
-                    a0[q] = f2_fma(c2, x, f2_mul(ms2, y));   // cs x - sn y
-                    a1[q] = f2_fma(c2, y, f2_mul(s2, x));    // sn x + cs y
-                }
+        for (int k = 0; k < 2; ++k) {
+            JacCol<E> &x = *xs[k], &y = *ys[k];
+            const float g1 = ga[k] * (x.scl * y.scl), g2 = g1 + g1, d = y.nrm - x.nrm;
+            const float tk = (d < 0.f ? -g2 : g2) * fast_rcp(fabsf(d) + fast_sqrt(fmaf(d, d, g2 * g2)));
+            const bool go = active && g1 * g1 > tol2 * (x.nrm * y.nrm) && x.nrm > 0.f && y.nrm > 0.f;
+            rotated = rotated || go;
+            t[k] = go ? tk : 0.f;
+            cs[k] = go ? fast_rsqrt(fmaf(tk, tk, 1.f)) : 1.f;
+            ga[k] = g1;
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            JacCol<E> &x = *xs[k], &y = *ys[k];
+            const float2 k0 = make_float2(-t[k] * r[k], -t[k] * r[k]), k1 = make_float2(t[k] * ri[k], t[k] * ri[k]);
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const float2 u = x.v[q];
+                x.v[q] = f2_fma(k0, y.v[q], u);
+                y.v[q] = f2_fma(k1, u, y.v[q]);
+            }
+            x.scl *= cs[k];
+            y.scl *= cs[k];
+            x.nrm = fmaxf(fmaf(-t[k], ga[k], x.nrm), 0.f);
+            y.nrm = fmaxf(fmaf(t[k], ga[k], y.nrm), 0.f);
+            if (real && sub == 4 * k) {
+                rot[rec + 2 * g + k] = make_float2(cs[k], cs[k] * t[k]);
+                rlab[rec + 2 * g + k] = (uint32_t)x.lab | ((uint32_t)y.lab << 16);
             }
         }
-        if (real && sub == 0) {
-            rot[(size_t)rec + g] = make_float2(cs, sn);
-            rlab[(size_t)rec + g] = (uint32_t)lab0 | ((uint32_t)lab1 << 16);
-        }
-        rec += G;
+        rec += m;
+    };
+    // the four rotations between a group's two blocks
+    auto cross = [&](bool active) {
+        rotate(A[0], B[0], A[1], B[1], active);
+        rotate(A[0], B[1], A[1], B[0], active);
     };
 
     int sweep = 0, par = 0;
     for (; sweep < max_sweeps; ++sweep) {
-        local_max = 0.f;
-        rec = sweep * RD * G;
+        rotated = false;
+        rec = (size_t)sweep * SUB * m;
+        renorm_all();
+        rotate(A[0], A[1], B[0], B[1], true);   // inside the blocks
         for (int lev = 0; lev < tz; ++lev) {
             const int h = m >> (lev + 1);   // ring length: pairs per set and rounds of this level
             if (lev > 0) {
@@ -1042,71 +1156,54 @@ __global__ void __launch_bounds__(32 * E, 1) jacobi_reg_kernel(const double *__r
                 int src0, src1;
                 jorder_split_sources(g, h, src0, src1);
                 move_both(src0, src1);   // every thread reaches the same barriers
+                renorm_all();
             }
-            const int ks = jorder_ring_source(g, h);   // slot-1 column comes from the next group
+            const int ks = jorder_ring_source(g, h);   // slot-1 block comes from the next group
             for (int r = 0; r < h; ++r) {
                 if (r > 0) {
                     // double-buffered halves: one barrier per round
-                    if (real) put(par * G + g, a1, lab1);
+                    if (real) put(par * G + g, B);
                     __syncthreads();
-                    if (real) take(par * G + ks, a1, lab1);
+                    if (real) take(par * G + ks, B);
                     par ^= 1;
                 }
-                rotate(true);
+                cross(true);
             }
         }
         if (s_odd > 1) {
             // circle method inside each set of odd size s: positions 1..k paired
             // with s-1..k+1 in k groups per set, position 0 idle (the two sets
-            // that share a parent put their idle columns in one group)
+            // that share a parent put their idle blocks in one group)
             const int s = s_odd;
             int e0, e1, r0, r1;
             bool idle;
             jorder_tail_sources(g, s, e0, e1, r0, r1, idle);
             for (int r = 0; r < s; ++r) {
                 move_both(r == 0 ? e0 : r0, r == 0 ? e1 : r1);
-                rotate(!idle);
+                if (r == 0) renorm_all();
+                cross(!idle);
             }
         }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) local_max = fmaxf(local_max, __shfl_xor_sync(0xffffffffu, local_max, off));
-        if (lane == 0) red[warp] = local_max;
-        __syncthreads();
-        if (tid == 0) {
-            float mx = 0.f;
-            for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) mx = fmaxf(mx, red[w]);
-            s_done = mx <= tol;
-        }
-        __syncthreads();
-        if (s_done) {
+        if (!__syncthreads_or(rotated)) {
             ++sweep;
             break;
         }
     }
     // right singular vectors of R: normalised columns of R^T W, by label
-    float2 n02 = make_float2(0.f, 0.f), n12 = n02;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        n02 = f2_fma(a0[q], a0[q], n02);
-        n12 = f2_fma(a1[q], a1[q], n12);
-    }
-    float n0 = n02.x + n02.y, n1 = n12.x + n12.y;
-#pragma unroll
-    for (int off = 1; off < 8; off <<= 1) {
-        n0 += __shfl_xor_sync(0xffffffffu, n0, off);
-        n1 += __shfl_xor_sync(0xffffffffu, n1, off);
-    }
-    const float q0 = n0 > 0.f ? rsqrtf(n0) : 0.f, q1 = n1 > 0.f ? rsqrtf(n1) : 0.f;
+    renorm_all();
     if (real) {
 #pragma unroll
-        for (int q = 0; q < NQ; ++q)
+        for (int k = 0; k < 4; ++k) {
+            const JacCol<E> &x = k < 2 ? A[k & 1] : B[k & 1];
+            const float inv = x.nrm > 0.f ? rsqrtf(x.nrm) : 0.f;
+            if (x.lab >= c) continue;
 #pragma unroll
-            for (int t = 0; t < 2; ++t) {
-                const int i = 16 * q + 2 * sub + t;
-                const float x0 = t ? a0[q].y : a0[q].x, x1 = t ? a1[q].y : a1[q].x;
-                if (i < c && lab0 < c) Vout[(size_t)i * c + lab0] = (double)(x0 * q0);
-                if (i < c && lab1 < c) Vout[(size_t)i * c + lab1] = (double)(x1 * q1);
+            for (int q = 0; q < NQ; ++q) {
+                const int i = 16 * q + 2 * sub;
+                if (i < c) Vout[(size_t)i * c + x.lab] = (double)(x.v[q].x * inv);
+                if (i + 1 < c) Vout[(size_t)(i + 1) * c + x.lab] = (double)(x.v[q].y * inv);
             }
+        }
     }
     if (tid == 0 && sweeps_out) *sweeps_out = sweep;
 }
@@ -1168,29 +1265,36 @@ __global__ void __launch_bounds__(kRpWarps * 32) jacobi_replay_kernel(const floa
         if (ch + 1 < nch) fetch(ch + 1);
         if (live) {
             const int nr = min(kRpChunk, total - ch * kRpChunk);
-            for (int r = 0; r < nr; ++r) {
-                // the round's pairs are disjoint: all reads first, then all writes
-                float2 cn[kRpPer];
-                int p[kRpPer], q[kRpPer];
-                float u[kRpPer], v[kRpPer];
+            // the round's pairs are disjoint: all reads first, then all writes;
+            // the next round's records are read before this round's rows
+            float2 cn[kRpPer];
+            uint32_t pq[kRpPer];
+            auto records = [&](int r) {
 #pragma unroll
                 for (int k = 0; k < kRpPer; ++k) {
                     const int g = lane + 32 * k;
                     cn[k] = g < G ? srot[b][r * G + g] : make_float2(1.f, 0.f);
-                    const uint32_t pq = g < G ? slab[b][r * G + g] : 0u;
-                    p[k] = (int)(pq & 0xFFFFu);
-                    q[k] = (int)(pq >> 16);
+                    pq[k] = g < G ? slab[b][r * G + g] : 0u;
                 }
+            };
+            records(0);
+            for (int r = 0; r < nr; ++r) {
+                float u[kRpPer], v[kRpPer];
+                float2 c0[kRpPer];
+                uint32_t l0[kRpPer];
 #pragma unroll
                 for (int k = 0; k < kRpPer; ++k) {
-                    u[k] = cn[k].y != 0.f ? row[p[k]] : 0.f;
-                    v[k] = cn[k].y != 0.f ? row[q[k]] : 0.f;
+                    c0[k] = cn[k];
+                    l0[k] = pq[k];
+                    u[k] = c0[k].y != 0.f ? row[l0[k] & 0xFFFFu] : 0.f;
+                    v[k] = c0[k].y != 0.f ? row[l0[k] >> 16] : 0.f;
                 }
+                if (r + 1 < nr) records(r + 1);
 #pragma unroll
                 for (int k = 0; k < kRpPer; ++k)
-                    if (cn[k].y != 0.f) {
-                        row[p[k]] = cn[k].x * u[k] - cn[k].y * v[k];
-                        row[q[k]] = cn[k].y * u[k] + cn[k].x * v[k];
+                    if (c0[k].y != 0.f) {
+                        row[l0[k] & 0xFFFFu] = c0[k].x * u[k] - c0[k].y * v[k];
+                        row[l0[k] >> 16] = c0[k].y * u[k] + c0[k].x * v[k];
                     }
                 __syncwarp();
             }
@@ -1204,21 +1308,21 @@ __global__ void __launch_bounds__(kRpWarps * 32) jacobi_replay_kernel(const floa
 
 // records a Jacobi run on c <= kJacRegMaxC columns may write
 inline size_t jreg_records(int c) {
-    const int m = c + (c & 1);
-    return (size_t)kJacMaxSweeps * jreg_rounds(m) * (m / 2);
+    const int m = jreg_blocks(c);
+    return (size_t)kJacMaxSweeps * jreg_rounds(m) * m;
 }
 
 template <int E>
 int launch_jacobi_reg_e(const double *R, int c, double *U, double *V, float2 *rot, uint32_t *rlab, int *sweeps,
                         cudaStream_t st) {
-    const int m = c + (c & 1);
+    const int m = jreg_blocks(c);
     const int threads = ((m / 2) * 8 + 31) / 32 * 32;
-    const int smem = m * jreg_stride<E>() * (int)sizeof(float);
+    const int smem = m * jreg_stride(E) * (int)sizeof(float);
     if (smem > 48 * 1024) LNE_TRY(allow_dynamic_smem(jacobi_reg_kernel<E>));
     jacobi_reg_kernel<E><<<1, threads, smem, st>>>(R, c, V, rot, rlab, kJacMaxSweeps, sweeps);
     LNE_LAUNCH_CHECK();
-    jacobi_replay_kernel<<<(unsigned)ceil_div(c, kRpWarps), kRpWarps * 32, 0, st>>>(rot, rlab, m / 2,
-                                                                                  jreg_rounds(m), sweeps, c, U);
+    jacobi_replay_kernel<<<(unsigned)ceil_div(c, kRpWarps), kRpWarps * 32, 0, st>>>(rot, rlab, m, jreg_rounds(m),
+                                                                                  sweeps, c, U);
     LNE_LAUNCH_CHECK();
     return 0;
 }
@@ -2068,7 +2172,7 @@ namespace {
 
 constexpr int kNoAllocMaxC = 160;
 constexpr size_t kNoAllocMat = (size_t)kNoAllocMaxC * kNoAllocMaxC;
-constexpr size_t kNoAllocRec = (size_t)kJacMaxSweeps * kJacRegMaxC * (kJacRegMaxC / 2);   // >= jreg_records(c)
+constexpr size_t kNoAllocRec = (size_t)kJacMaxSweeps * (kJacRegMaxC + 2) * (kJacRegMaxC / 2);   // >= jreg_records(c)
 constexpr size_t kNoAllocDoubles = 10 * kNoAllocMat + kNoAllocMaxC + 128 + kNoAllocRec + kNoAllocRec / 2;
 static_assert(4 * kOaParts + 8 <= 128, "partial sums and sweep count fit the reserve");
 static __device__ __align__(256) double g_svd_scratch[kNoAllocDoubles];
