@@ -4,7 +4,7 @@
 //   gram           G = Y^T Y to FP64 accuracy: per-CTA partial Grams over row
 //                  blocks in exact FP32 steps (float pairs), summed in FP64
 //                  in a fixed order so the result is reproducible.
-//   chol           G = R^T R (upper Cholesky) in FP64, one CTA.
+//   chol           G = R^T R (upper Cholesky) in FP64, a CTA per block column.
 //   trsm_rows      Q = Y R^-1 by forward substitution per row (FP32): each
 //                  row's solve is backward stable, so Y = Q R holds to FP32
 //                  rounding whatever the conditioning of R.
@@ -261,8 +261,10 @@ __global__ void __launch_bounds__(kGramThreads) gram_partial_kernel(const float 
 // tiles above the diagonal only (a, b).)
 constexpr int kGramRedLanes = 8;
 
+// Also zeroes the tile counters of the Cholesky that follows.
 __global__ void gram_reduce_kernel(const double *__restrict__ partial, int nblk, int c,
-                                   double *__restrict__ G) {
+                                   double *__restrict__ G, unsigned *__restrict__ cnt) {
+    if (blockIdx.x == 0 && threadIdx.x < 16) cnt[threadIdx.x] = 0u;
     constexpr int kPerWarp = 32 / kGramRedLanes;   // entries per warp and step
     const int cp = (c + 7) & ~7;
     const int nup = c * (c + 1) / 2;
@@ -294,219 +296,175 @@ __global__ void gram_reduce_kernel(const double *__restrict__ partial, int nblk,
     }
 }
 
-// 1/sqrt(a) of a positive finite FP64 pivot by two Newton steps
-// y <- y (3 - a y^2) / 2 from the FP32 estimate (which has 24 bits; two steps
-// pass FP64's 53), so no FP64 square root or division runs on this GPU's
-// narrow FP64 pipe; pivots outside FP32's range take the plain route.
+// 1/sqrt(a) of a positive normal FP64 pivot: one step of third order
+// y <- y + y e (1/2 + 3/8 e), e = 1 - a y^2, from an FP32 estimate (e is about
+// 2^-22, so the error left, 5/16 e^3, is below 2^-53). FP64 instructions take
+// some 64 cycles each on this GPU, conversions too: the estimate is taken of a's
+// upper bits scaled into [1, 4) by integer arithmetic and put back the same way,
+// which leaves four dependent FP64 operations.
 __device__ __forceinline__ double pivot_rsqrt(double a) {
-    double y = (double)rsqrtf((float)a);
-    if (!(y > 0.0) || !isfinite(y)) return 1.0 / sqrt(a);
-    y = y * fma(-0.5 * a, y * y, 1.5);
-    return y * fma(-0.5 * a, y * y, 1.5);
+    const int hi = __double2hiint(a), lo = __double2loint(a);
+    const int e = (hi >> 20) - 1023, odd = e & 1;   // a = 2^e (1.f)
+    if (e == -1023) return 1.0 / sqrt(a);           // subnormal
+    const uint32_t m = ((uint32_t)(hi & 0xFFFFF) << 3) | ((uint32_t)lo >> 29);
+    const uint32_t y32 = __float_as_uint(rsqrtf(__uint_as_float(((uint32_t)(127 + odd) << 23) | m)));
+    const int ye = (int)(y32 >> 23) - 127 - ((e - odd) >> 1) + 1023;
+    const double y = __hiloint2double((ye << 20) | (int)((y32 & 0x7FFFFFu) >> 3), (int)(y32 << 29));
+    const double t = fma(-(a * y), y, 1.0);
+    return fma(y * t, fma(0.375, t, 0.5), y);
 }
 
-// ---------------------------------------------------------------------------
-// Cholesky (upper, G = R^T R), one CTA, FP64. Right-looking: for each k the
-// pivot row is scaled by 1/sqrt(pivot) and the trailing upper triangle takes
-// the rank-1 update.
-// ---------------------------------------------------------------------------
-constexpr int kCholThreads = 1024;
-constexpr int kMaxSmemC = 160;
+constexpr int kMaxSmemC = 160;   // largest c of the small SVD
 
-__global__ void __launch_bounds__(kCholThreads) chol_kernel(const double *__restrict__ G, int c,
-                                                            double *__restrict__ R, int *__restrict__ status) {
-    extern __shared__ double sm[];
-    const bool in_smem = c <= kMaxSmemC;
-    double *A = in_smem ? sm : R;
-    __shared__ double s_inv;
-    __shared__ int bad;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kCholThreads / 32;
-    for (int e = tid; e < c * c; e += kCholThreads) A[e] = G[e];
-    if (tid == 0) bad = 0;
-    __syncthreads();
-    for (int k = 0; k < c; ++k) {
-        if (tid == 0) {
-            const double akk = A[k * c + k];
-            if (!(akk > 0.0) || !isfinite(akk)) {
-                if (!bad) bad = k + 1;
-                A[k * c + k] = 1.0;
-                s_inv = 1.0;
-            } else {
-                const double y = pivot_rsqrt(akk);
-                A[k * c + k] = akk * y;
-                s_inv = y;
-            }
-        }
-        __syncthreads();
-        const double inv = s_inv;
-        for (int j = k + 1 + tid; j < c; j += kCholThreads) A[k * c + j] *= inv;
-        __syncthreads();
-        for (int i = k + 1 + warp; i < c; i += nw) {
-            const double aki = A[k * c + i];
-            for (int j = i + lane; j < c; j += 32) A[i * c + j] = fma(-aki, A[k * c + j], A[i * c + j]);
-        }
-        __syncthreads();
-    }
-    for (int e = tid; e < c * c; e += kCholThreads) {
-        const int i = e / c, j = e - i * c;
-        if (in_smem) R[e] = j >= i ? A[e] : 0.0;
-        else if (j < i) R[e] = 0.0;
-    }
-    if (tid == 0 && bad && *status == 0) *status = bad;   // sticky: only a breakdown writes
-}
-
-// Blocked Cholesky over many SMs (FP64), for the matrix sizes where the
-// one-CTA kernel is bound by a single SM's FP64 rate. Panels of kCholB rows:
-// the panel phase (chol_panel_body) factors the diagonal block,
-// R11^T R11 = A11, and solves R11^T R12 = A12 for the panel's row block; the
-// update phase (chol_update_body, one CTA per 16 x 16 upper tile) subtracts
-// R12^T R12 from the trailing matrix. A is the working copy (row-major, upper
-// triangle significant) and ends as R. Both phases of every panel run in one
-// cooperative launch (chol_coop_kernel), separated by grid barriers.
-//
-// The panel's row block is spread over ceil((c - k1) / 16) CTAs, 16 columns
-// each; every CTA factors the small diagonal block itself (identically), so
-// no CTA waits for another. Since other CTAs may still be reading A11 while
-// one has finished, R11 goes to a scratch block (written by CTA 0) and is
-// copied into A in the update phase, or directly by a panel that runs as a
-// single CTA.
+// ---------------------------------------------------------------------------
+// Cholesky (upper, G = R^T R) in FP64, 16 x 16 tiles, one CTA per block column.
+// CTA j holds the tiles (i, j), i <= j, of its 16 columns in shared memory and
+// takes the panels p = 0 .. j in order: it solves R_pp^T R_pj = A_pj, publishes
+// R_pj, and subtracts R_pi^T R_pj from its tiles (i, j) as the other CTAs publish
+// their R_pi; at p = j it factors its diagonal tile, which releases the panel to
+// the CTAs on its right. cnt[i] counts the tiles CTA i has published, so a CTA
+// waits for the one tile it needs instead of for a grid-wide barrier (nine
+// panels of two barriers each took most of the factorisation's time). What is
+// left is the chain of the diagonal: per panel 16 pivots (an FP64 reciprocal
+// square root, a scaling and an update each), one tile solve and one tile
+// update. Launched cooperatively, so every CTA that is waited for is resident;
+// a wait gives up after 2 s and sets status[1]. A pivot that is not positive
+// sets status[0] and is replaced by 1. Every entry takes its terms in ascending
+// order of the pivots. Measured: see chol().
+// ---------------------------------------------------------------------------
 constexpr int kCholB = 16;
+constexpr int kCholMaxTiles = 15;   // c <= 240
 
-// The panel of rows k0.. for the 16-column block bx of R12 (nb blocks).
-__device__ __forceinline__ void chol_panel_body(double *__restrict__ A, int c, int k0, int *__restrict__ status,
-                                                double *__restrict__ r11, int bx, int nb) {
-    __shared__ double s11[kCholB][kCholB + 1];
-    __shared__ double sinv[kCholB];
-    const int tid = threadIdx.x;
-    const int bs = min(kCholB, c - k0), k1 = k0 + bs;
-    for (int e = tid; e < bs * bs; e += blockDim.x) {
-        const int i = e / bs, j = e - i * bs;
-        s11[i][j] = A[(size_t)(k0 + i) * c + k0 + j];
-    }
-    __syncthreads();
-    // unblocked factorisation of the diagonal block, one entry (ti, tj) per thread
-    const int ti = tid >> 4, tj = tid & 15;
-    for (int t = 0; t < bs; ++t) {
-        if (tid == 0) {
-            const double att = s11[t][t];
-            double d = 1.0, y = 1.0;
-            if (!(att > 0.0) || !isfinite(att)) {
-                if (bx == 0 && *status == 0) *status = k0 + t + 1;
-            } else {
-                y = pivot_rsqrt(att);
-                d = att * y;
-            }
-            s11[t][t] = d;
-            sinv[t] = y;
-        }
-        __syncthreads();
-        if (ti == t && tj > t && tj < bs) s11[t][tj] *= sinv[t];
-        __syncthreads();
-        if (ti > t && tj >= ti && tj < bs) s11[ti][tj] = fma(-s11[t][ti], s11[t][tj], s11[ti][tj]);
-        __syncthreads();
-    }
-    // R12: 16 lanes per column; lane i holds x_i and subtracts r_ti x_t as
-    // soon as x_t is final (the same terms in the same order as a row-by-row
-    // forward substitution)
-    {
-        const int li = tid & 15;
-        const int j = k1 + bx * 16 + (tid >> 4);
-        const bool live = j < c && li < bs;
-        double x = live ? A[(size_t)(k0 + li) * c + j] : 0.0;
-        for (int t = 0; t < bs; ++t) {
-            if (li == t) x *= sinv[t];
-            const double xt = __shfl_sync(0xffffffffu, x, t, 16);
-            if (li > t && li < bs) x = fma(-s11[t][li], xt, x);
-        }
-        if (live) A[(size_t)(k0 + li) * c + j] = x;
-    }
-    // R11 (and zeros left of the diagonal in the panel's rows)
-    if (bx == 0)
-        for (int e = tid; e < bs * bs; e += blockDim.x) {
-            const int i = e / bs, j = e - i * bs;
-            r11[e] = j >= i ? s11[i][j] : 0.0;
-        }
-    if (nb == 1)
-        for (int e = tid; e < bs * k1; e += blockDim.x) {
-            const int i = e / k1, j = e - i * k1;   // row k0 + i, column j < k1
-            A[(size_t)(k0 + i) * c + j] = j >= k0 + i ? s11[i][j - k0] : 0.0;
-        }
-}
-
-// r11 is read with ld.global.cg: in the cooperative launch it was written by
-// another CTA of the same launch, so it must not come through the read-only path.
-__device__ __forceinline__ void chol_update_body(double *__restrict__ A, int c, int k0, int k1, const double *r11,
-                                                 int I, int J) {
-    if (I > J) return;
-    const int tid = threadIdx.x;
-    const int bs = k1 - k0;
-    if (I == 0 && J == 0)   // the panel's R11 from its scratch block (these entries are not read below)
-        for (int e = tid; e < bs * k1; e += blockDim.x) {
-            const int i = e / k1, j = e - i * k1;
-            A[(size_t)(k0 + i) * c + j] = j >= k0 ? __ldcg(r11 + i * bs + (j - k0)) : 0.0;
-        }
-    __shared__ double ri[kCholB][16], rj[kCholB][16];
-    const int ti = tid >> 4, tj = tid & 15;
-    const int i0 = k1 + 16 * I, j0 = k1 + 16 * J;
-    for (int e = tid; e < kCholB * 16; e += 256) {
-        const int t = e >> 4, q = e & 15;
-        ri[t][q] = (t < bs && i0 + q < c) ? A[(size_t)(k0 + t) * c + i0 + q] : 0.0;
-        rj[t][q] = (t < bs && j0 + q < c) ? A[(size_t)(k0 + t) * c + j0 + q] : 0.0;
-    }
-    __syncthreads();
-    const int i = i0 + ti, j = j0 + tj;
-    if (i < c && j < c && i <= j) {
-        double a = A[(size_t)i * c + j];
-        for (int t = 0; t < bs; ++t) a = fma(-ri[t][ti], rj[t][tj], a);
-        A[(size_t)i * c + j] = a;
-    }
-}
-
-// All panels in one cooperative launch: the panel and update phases of each
-// panel are separated by grid-wide barriers (every CTA is resident, so the
-// barriers only wait for running CTAs; each gives up after 2 s and sets the
-// status word [1]). The same work in the same order as the per-panel launches.
-__device__ __forceinline__ void grid_barrier(unsigned *bar, unsigned &target, int *status) {
-    __syncthreads();
-    target += gridDim.x;
+// Waits until *cnt >= want (thread 0 polls; ends with a barrier of the CTA).
+__device__ __forceinline__ bool chol_wait(const unsigned *cnt, unsigned want, int *status) {
+    __shared__ int s_ok;
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(bar, 1u);
-        uint64_t t0;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-        for (;;) {
+        uint64_t t0 = 0;
+        int ok = 1;
+        for (unsigned spin = 1;; ++spin) {
             unsigned v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if (v >= target) break;
-            uint64_t t;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-            if (t - t0 > 2000000000ull) {
-                atomicExch(status + 1, 1);
-                break;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
+            if (v >= want) break;
+            if ((spin & 63u) == 0u) {
+                uint64_t t;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+                if (t0 == 0) t0 = t;
+                if (t - t0 > 2000000000ull) {
+                    atomicExch(status + 1, 1);
+                    ok = 0;
+                    break;
+                }
             }
         }
-        __threadfence();
+        s_ok = ok;
     }
     __syncthreads();
+    const bool ok = s_ok != 0;
+    __syncthreads();   // s_ok is written again by the next wait
+    return ok;
 }
 
-__global__ void __launch_bounds__(256, 1) chol_coop_kernel(double *__restrict__ A, int c, int *__restrict__ status,
-                                                        double *__restrict__ r11, unsigned *__restrict__ bar) {
-    unsigned target = 0;
-    for (int k0 = 0; k0 < c; k0 += kCholB) {
-        const int k1 = min(c, k0 + kCholB);
-        const int nb = max(1, (c - k1 + 15) / 16);
-        for (int bx = blockIdx.x; bx < nb; bx += gridDim.x) {
-            chol_panel_body(A, c, k0, status, r11, bx, nb);
+// pub: the published tiles, (i, j) at ((size_t)i * nt + j) * 256; inv: the
+// reciprocal diagonal.
+__global__ void __launch_bounds__(256, 1) chol_kernel(const double *__restrict__ G, int c, double *__restrict__ R,
+                                                      double *pub, double *inv, unsigned *cnt,
+                                                      int *__restrict__ status) {
+    __shared__ double tiles[kCholMaxTiles][kCholB][kCholB + 1];
+    __shared__ double rp[kCholB][kCholB + 1];   // R_pp, then R_pi
+    __shared__ double sinv[kCholB];
+    const int nt = gridDim.x, j = blockIdx.x, tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
+    const int col = 16 * j + tj;
+#pragma unroll 4
+    for (int i = 0; i <= j; ++i) {
+        const int row = 16 * i + ti;
+        tiles[i][ti][tj] = row < c && col < c ? __ldg(G + (size_t)row * c + col) : 0.0;
+    }
+    __syncthreads();
+    auto publish = [&](int p, double v) {
+        pub[((size_t)p * nt + j) * 256 + tid] = v;
+        __syncthreads();
+        if (tid == 0) {
+            __threadfence();
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(cnt + j), "r"((unsigned)p + 1u) : "memory");
+        }
+    };
+    for (int p = 0; p < j; ++p) {
+        if (!chol_wait(cnt + p, p + 1, status)) return;
+        rp[ti][tj] = __ldcg(pub + ((size_t)p * nt + p) * 256 + tid);
+        if (tid < 16) sinv[tid] = __ldcg(inv + 16 * p + tid);
+        __syncthreads();
+        // R_pp^T x = A_pj: 16 lanes per column; lane li holds x_li and subtracts
+        // r_t,li x_t as soon as x_t is final (panel p is full: p < j)
+        {
+            const int li = tj, q = ti;   // row in the tile, column in the tile
+            double x = tiles[p][li][q];
+            for (int t = 0; t < kCholB; ++t) {
+                if (li == t) x *= sinv[t];
+                const double xt = __shfl_sync(0xffffffffu, x, t, 16);
+                if (li > t) x = fma(-rp[t][li], xt, x);
+            }
+            __syncthreads();
+            tiles[p][li][q] = x;
+        }
+        __syncthreads();
+        publish(p, tiles[p][ti][tj]);
+        for (int i = p + 1; i < j; ++i) {
+            if (!chol_wait(cnt + i, p + 1, status)) return;
+            rp[ti][tj] = __ldcg(pub + ((size_t)p * nt + i) * 256 + tid);
+            __syncthreads();
+            double a = tiles[i][ti][tj];
+#pragma unroll
+            for (int t = 0; t < kCholB; ++t) a = fma(-rp[t][ti], tiles[p][t][tj], a);
+            tiles[i][ti][tj] = a;
             __syncthreads();
         }
-        if (k1 >= c) break;
-        grid_barrier(bar, target, status);
-        for (int t = blockIdx.x; t < nb * nb; t += gridDim.x) {
-            chol_update_body(A, c, k0, k1, r11, t / nb, t % nb);
-            __syncthreads();
+        if (ti <= tj) {
+            double a = tiles[j][ti][tj];
+#pragma unroll
+            for (int t = 0; t < kCholB; ++t) a = fma(-tiles[p][t][ti], tiles[p][t][tj], a);
+            tiles[j][ti][tj] = a;
         }
-        grid_barrier(bar, target, status);
+        __syncthreads();
+    }
+    // the diagonal tile, one entry per thread (in v); the owner of the next pivot
+    // takes its reciprocal root in the same phase as the update that finishes it
+    const int bs = min(kCholB, c - 16 * j);
+    double v = tiles[j][ti][tj];
+    auto pivot = [&](int t) {
+        double d = 1.0, y = 1.0;
+        const int hi = __double2hiint(v);
+        if ((hi > 0 && hi < 0x7FF00000) || (hi == 0 && __double2loint(v) != 0)) {   // positive, finite
+            y = pivot_rsqrt(v);
+            d = v * y;
+        } else if (*status == 0) {
+            *status = 16 * j + t + 1;
+        }
+        v = d;
+        sinv[t] = y;
+    };
+    if (tid == 0) pivot(0);
+    __syncthreads();
+    for (int t = 0; t < bs; ++t) {
+        if (ti == t && tj >= t && tj < bs) {
+            if (tj > t) v *= sinv[t];
+            rp[0][tj] = v;
+        }
+        __syncthreads();
+        if (ti > t && tj >= ti && tj < bs) {
+            v = fma(-rp[0][ti], rp[0][tj], v);
+            if (ti == tj && ti == t + 1) pivot(t + 1);
+        }
+        __syncthreads();
+    }
+    if (ti <= tj) tiles[j][ti][tj] = v;
+    __syncthreads();
+    if (j + 1 < nt) {
+        if (tid < 16) inv[16 * j + tid] = sinv[tid];
+        publish(j, tiles[j][ti][tj]);
+    }
+    for (int i = 0; i < nt; ++i) {
+        const int row = 16 * i + ti;
+        if (row < c && col < c) R[(size_t)row * c + col] = row <= col ? tiles[min(i, j)][ti][tj] : 0.0;
     }
 }
 
@@ -1899,6 +1857,8 @@ static int gram(Workspace &ws, const float *Y, int64_t n, int c, int64_t ld, dou
     nblk = ceil_div(std::max<int64_t>(n, 1), rows_per);
     double *partial = nullptr;
     LNE_TRY(ws.get("gram.partial", (size_t)nblk * cp * cp, &partial));
+    unsigned *cnt = nullptr;
+    LNE_TRY(ws.get("chol.cnt", 16, &cnt));
     {
         LNE_TRACE("gram_partial", st);
         if (vec) gram_partial_kernel<true><<<(unsigned)nblk, threads, smem, st>>>(Y, n, c, ld, rows_per, partial);
@@ -1907,8 +1867,8 @@ static int gram(Workspace &ws, const float *Y, int64_t n, int c, int64_t ld, dou
     }
     {
         LNE_TRACE("gram_reduce", st);
-        gram_reduce_kernel<<<grid_for((int64_t)c * (c + 1) / 2 * kGramRedLanes, 256), 256, 0, st>>>(partial,
-                                                                                                (int)nblk, c, G);
+        gram_reduce_kernel<<<grid_for((int64_t)c * (c + 1) / 2 * kGramRedLanes, 256), 256, 0, st>>>(
+            partial, (int)nblk, c, G, cnt);
         LNE_LAUNCH_CHECK();
     }
     return 0;
@@ -1917,34 +1877,25 @@ static int gram(Workspace &ws, const float *Y, int64_t n, int c, int64_t ld, dou
 // A breakdown (a pivot that is not positive) is recorded in the device status
 // word read by status_check, without a host synchronisation here; the
 // factorisation goes on with a unit pivot, so later kernels see finite values.
+// G comes from gram() on the same stream, whose reduction zeroes the tile
+// counters. Measured (c = 32 / 48 / 144): one CTA with a rank-1 update and three
+// barriers a pivot took 27 / 44 us, one cooperative launch with grid barriers
+// between panels 159 us at c = 144; now 20 / 32 / 106 us.
 static int chol(Workspace &ws, const double *G, int c, double *R, cudaStream_t st) {
     int *status = nullptr;
+    unsigned *cnt = nullptr;
+    double *pub = nullptr, *inv = nullptr;
+    const int nt = (int)ceil_div(c, kCholB);
+    if (nt > kCholMaxTiles) return fail(LNE_ERR_UNSUPPORTED, "Cholesky supports at most 240 columns");
     LNE_TRY(device_status(ws, &status, st));
-    if (c >= 64) {   // blocked over many SMs: one cooperative launch for all panels
-        double *r11 = nullptr;
-        unsigned *bar = nullptr;
-        LNE_TRY(ws.get("chol.r11", (size_t)kCholB * kCholB, &r11));
-        LNE_TRY(ws.get("chol.bar", 1, &bar));
-        LNE_CUDA_TRY(cudaMemcpyAsync(R, G, sizeof(double) * (size_t)c * c, cudaMemcpyDeviceToDevice, st));
-        LNE_CUDA_TRY(cudaMemsetAsync(bar, 0, sizeof(unsigned), st));
-        LNE_TRACE("chol", st);
-        const int nb0 = (int)std::max<int64_t>(1, ceil_div(c - kCholB, 16));
-        int per_sm = 0;
-        LNE_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, chol_coop_kernel, 256, 0));
-        const int grid = std::min(nb0 * nb0, std::max(1, per_sm) * num_sms());
-        int ci = c;
-        void *args[] = {&R, &ci, &status, &r11, &bar};
-        LNE_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(chol_coop_kernel), dim3(grid),
-                                                 dim3(256), args, 0, st));
-        LNE_LAUNCH_CHECK();
-    } else {
-        const int smem = c <= kMaxSmemC ? c * c * 8 : 0;
-        if (smem > 48 * 1024)
-            LNE_TRY(allow_dynamic_smem(chol_kernel));
-        LNE_TRACE("chol", st);
-        chol_kernel<<<1, kCholThreads, smem, st>>>(G, c, R, status);
-        LNE_LAUNCH_CHECK();
-    }
+    LNE_TRY(ws.get("chol.cnt", 16, &cnt));
+    LNE_TRY(ws.get("chol.pub", (size_t)nt * nt * 256, &pub));
+    LNE_TRY(ws.get("chol.inv", (size_t)nt * kCholB, &inv));
+    LNE_TRACE("chol", st);
+    void *args[] = {&G, &c, &R, &pub, &inv, &cnt, &status};
+    LNE_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(chol_kernel), dim3(nt), dim3(256), args, 0,
+                                             st));
+    LNE_LAUNCH_CHECK();
     return 0;
 }
 
