@@ -53,6 +53,40 @@ __device__ __forceinline__ void f2_add_prod(float2 &acc, float2 a, float2 b) {
         : "+l"(reinterpret_cast<uint64_t &>(acc))
         : "l"(reinterpret_cast<const uint64_t &>(a)), "l"(reinterpret_cast<const uint64_t &>(b)));
 }
+
+// A barrier over the grid of a cooperative launch (all CTAs resident). Gives
+// up after 2 s: status[1] is set and every CTA returns false, after which the
+// kernel ends.
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &target, int *status) {
+    __shared__ int ok_s;
+    __syncthreads();
+    target += gridDim.x;
+    if (threadIdx.x == 0) {
+        int ok = 1;
+        unsigned v;
+        __threadfence();
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        uint64_t t0 = 0;
+        for (unsigned spin = 1;; ++spin) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if ((int)(v - target) >= 0) break;   // the count may wrap
+            if ((spin & 63u) == 0u) {
+                uint64_t t;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+                if (t0 == 0) t0 = t;
+                if (t - t0 > 2000000000ull) {
+                    atomicExch(status + 1, 1);
+                    ok = 0;
+                    break;
+                }
+            }
+        }
+        __threadfence();
+        ok_s = ok;
+    }
+    __syncthreads();
+    return ok_s != 0;
+}
 #endif
 
 // Error state shared by host code of the library.

@@ -315,6 +315,8 @@ __device__ __forceinline__ double pivot_rsqrt(double a) {
 }
 
 constexpr int kMaxSmemC = 160;   // largest c of the small SVD
+constexpr int kOaSteps = 4;      // refinement steps at most
+constexpr int kOaSync = 8;       // words: grid barrier, then each step's largest correction (FP32 bits); two spare
 
 // ---------------------------------------------------------------------------
 // Cholesky (upper, G = R^T R) in FP64, 16 x 16 tiles, one CTA per block column.
@@ -724,7 +726,9 @@ __host__ __device__ __forceinline__ int jac_ld(int c) { return ((c + 23) / 32) *
 // rotations, so R = W Sigma Z^T -- left singular vectors U = W, right ones
 // V = normalised columns of R^T W.
 __global__ void jacobi32_kernel(const double *__restrict__ R, int c, double *__restrict__ Uout,
-                                double *__restrict__ Vout, int max_sweeps, int *__restrict__ sweeps_out) {
+                                double *__restrict__ Vout, int max_sweeps, int *__restrict__ sweeps_out,
+                                unsigned *__restrict__ sync) {
+    if (threadIdx.x < kOaSync) sync[threadIdx.x] = 0u;   // for the refinement that follows
     extern __shared__ float js[];
     const int ldc = jac_ld(c);
     float *A = js;              // column j at A + j * ldc
@@ -1181,7 +1185,9 @@ static_assert(kRpMaxG <= 32 * kRpPer, "records of a round fit the lanes");
 __global__ void __launch_bounds__(kRpWarps * 32) jacobi_replay_kernel(const float2 *__restrict__ rot,
                                                                       const uint32_t *__restrict__ rlab, int G,
                                                                       int RD, const int *__restrict__ sweeps,
-                                                                      int c, double *__restrict__ Uout) {
+                                                                      int c, double *__restrict__ Uout,
+                                                                      unsigned *__restrict__ sync) {
+    if (blockIdx.x == 0 && threadIdx.x < kOaSync) sync[threadIdx.x] = 0u;   // for the refinement that follows
     __shared__ float rows[kRpWarps][kJacRegMaxC + 1];
     __shared__ float2 srot[2][kRpChunk * kRpMaxG];
     __shared__ uint32_t slab[2][kRpChunk * kRpMaxG];
@@ -1272,7 +1278,7 @@ inline size_t jreg_records(int c) {
 
 template <int E>
 int launch_jacobi_reg_e(const double *R, int c, double *U, double *V, float2 *rot, uint32_t *rlab, int *sweeps,
-                        cudaStream_t st) {
+                        unsigned *sync, cudaStream_t st) {
     const int m = jreg_blocks(c);
     const int threads = ((m / 2) * 8 + 31) / 32 * 32;
     const int smem = m * jreg_stride(E) * (int)sizeof(float);
@@ -1280,7 +1286,7 @@ int launch_jacobi_reg_e(const double *R, int c, double *U, double *V, float2 *ro
     jacobi_reg_kernel<E><<<1, threads, smem, st>>>(R, c, V, rot, rlab, kJacMaxSweeps, sweeps);
     LNE_LAUNCH_CHECK();
     jacobi_replay_kernel<<<(unsigned)ceil_div(c, kRpWarps), kRpWarps * 32, 0, st>>>(rot, rlab, m, jreg_rounds(m),
-                                                                                  sweeps, c, U);
+                                                                                  sweeps, c, U, sync);
     LNE_LAUNCH_CHECK();
     return 0;
 }
@@ -1289,83 +1295,26 @@ int launch_jacobi_reg_e(const double *R, int c, double *U, double *V, float2 *ro
 // replay; rot / rlab hold jreg_records(c) records) up to c = 144, the
 // shared-memory one above.
 int launch_jacobi(const double *R, int c, double *U, double *V, float2 *rot, uint32_t *rlab, int *sweeps,
-                  cudaStream_t st) {
+                  unsigned *sync, cudaStream_t st) {
     switch ((c + 15) / 16) {
-    case 1: return launch_jacobi_reg_e<2>(R, c, U, V, rot, rlab, sweeps, st);
-    case 2: return launch_jacobi_reg_e<4>(R, c, U, V, rot, rlab, sweeps, st);
-    case 3: return launch_jacobi_reg_e<6>(R, c, U, V, rot, rlab, sweeps, st);
-    case 4: return launch_jacobi_reg_e<8>(R, c, U, V, rot, rlab, sweeps, st);
-    case 5: return launch_jacobi_reg_e<10>(R, c, U, V, rot, rlab, sweeps, st);
-    case 6: return launch_jacobi_reg_e<12>(R, c, U, V, rot, rlab, sweeps, st);
-    case 7: return launch_jacobi_reg_e<14>(R, c, U, V, rot, rlab, sweeps, st);
-    case 8: return launch_jacobi_reg_e<16>(R, c, U, V, rot, rlab, sweeps, st);
-    case 9: return launch_jacobi_reg_e<18>(R, c, U, V, rot, rlab, sweeps, st);
+    case 1: return launch_jacobi_reg_e<2>(R, c, U, V, rot, rlab, sweeps, sync, st);
+    case 2: return launch_jacobi_reg_e<4>(R, c, U, V, rot, rlab, sweeps, sync, st);
+    case 3: return launch_jacobi_reg_e<6>(R, c, U, V, rot, rlab, sweeps, sync, st);
+    case 4: return launch_jacobi_reg_e<8>(R, c, U, V, rot, rlab, sweeps, sync, st);
+    case 5: return launch_jacobi_reg_e<10>(R, c, U, V, rot, rlab, sweeps, sync, st);
+    case 6: return launch_jacobi_reg_e<12>(R, c, U, V, rot, rlab, sweeps, sync, st);
+    case 7: return launch_jacobi_reg_e<14>(R, c, U, V, rot, rlab, sweeps, sync, st);
+    case 8: return launch_jacobi_reg_e<16>(R, c, U, V, rot, rlab, sweeps, sync, st);
+    case 9: return launch_jacobi_reg_e<18>(R, c, U, V, rot, rlab, sweeps, sync, st);
     default: break;
     }
     const int m = c + (c & 1);
     const int threads = std::max(32, std::min(1024, (m / 2 * kJacTPP + 31) / 32 * 32));
     const int smem = 2 * c * jac_ld(c) * 4;
     if (smem > 48 * 1024) LNE_TRY(allow_dynamic_smem(jacobi32_kernel));
-    jacobi32_kernel<<<1, threads, smem, st>>>(R, c, U, V, kJacMaxSweeps, sweeps);
+    jacobi32_kernel<<<1, threads, smem, st>>>(R, c, U, V, kJacMaxSweeps, sweeps, sync);
     LNE_LAUNCH_CHECK();
     return 0;
-}
-
-// C = op(A) op(B) (+ C0 if given), all c x c row-major FP64; 16 x 16 tile per CTA.
-// 8 x 8 output tiles (64 threads, one output each; 324 CTAs for c = 144). The
-// CTA's 8 rows of op(A) and 8 columns of op(B) over the whole k range are
-// loaded into shared memory at once (one round of load latency instead of one
-// per k step), then each thread runs its dot product.
-constexpr int kDgTile = 8;
-constexpr int kDgMaxC = 160;
-
-// Two products with the same transposes may share a launch: blockIdx.z = 1
-// takes the second operand set (A2, B2, C02, C2).
-__global__ void __launch_bounds__(kDgTile * kDgTile) dgemm_small_kernel(const double *__restrict__ A, int ta,
-                                                                        const double *__restrict__ B, int tb,
-                                                                        const double *__restrict__ C0,
-                                                                        double *__restrict__ C, int c,
-                                                                        const double *__restrict__ A2,
-                                                                        const double *__restrict__ B2,
-                                                                        const double *__restrict__ C02,
-                                                                        double *__restrict__ C2) {
-    if (blockIdx.z == 1) {
-        A = A2;
-        B = B2;
-        C0 = C02;
-        C = C2;
-    }
-    __shared__ double As[kDgTile][kDgMaxC + 1], Bs[kDgMaxC][kDgTile + 1];
-    const int tid = threadIdx.x, tx = tid % kDgTile, ty = tid / kDgTile;
-    const int r0 = blockIdx.y * kDgTile, c0 = blockIdx.x * kDgTile;
-#pragma unroll 6
-    for (int e = tid; e < kDgTile * c; e += kDgTile * kDgTile) {
-        // op(A)[r0 + i][k]: for ta the k index runs along A's rows
-        const int i = ta ? e % kDgTile : e / c, k = ta ? e / kDgTile : e % c;
-        const int r = r0 + i;
-        As[i][k] = r < c ? (ta ? A[k * c + r] : A[r * c + k]) : 0.0;
-        // op(B)[k][c0 + j]
-        const int j = tb ? e / c : e % kDgTile, kb = tb ? e % c : e / kDgTile;
-        const int cc = c0 + j;
-        Bs[kb][j] = cc < c ? (tb ? B[cc * c + kb] : B[kb * c + cc]) : 0.0;
-    }
-    __syncthreads();
-    const int row = r0 + ty, col = c0 + tx;
-    double acc = 0.0;
-    for (int k = 0; k < c; ++k) acc = fma(As[ty][k], Bs[k][tx], acc);
-    if (row < c && col < c) C[row * c + col] = C0 ? C0[row * c + col] + acc : acc;
-}
-
-__device__ double block_sum(double v, double *red) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) t += red[w];
-    return t;
 }
 
 // One step of Ogita-Aishima refinement of an SVD A = U Sigma V^T (Ogita and
@@ -1380,98 +1329,194 @@ __device__ double block_sum(double v, double *red) {
 // taken as (p_ij / 2, q_ij / 2) when |s_i - s_j| <= delta (near-equal values),
 // delta = 2 (||offdiag T|| + max|s| (||P|| + ||Q||)). A itself is never squared,
 // so the accuracy does not depend on the condition number of A.
-// Also turns the Gram products into P := I - U^T U, Q := I - V^T V in place.
-// kOaParts CTAs each reduce a fixed slice of the c x c entries (FP64 is slow
-// on this GPU, so the three sums are spread over several SMs) and write
-// their partial sums; svd_oa_fg_kernel adds the partials in a fixed order,
-// so delta is the same on every run.
-constexpr int kOaParts = 16;
+//
+// Up to kOaSteps steps in one cooperative launch: quadratic convergence, but the
+// FP32 start may be loose in directions FP32 cannot resolve. A step is four
+// phases between grid barriers: P, Q (upper tiles, mirrored) and W = A V; T =
+// U^T W with sigma and the norms' partial sums; F and G; U + U F and V + V G. The
+// step whose corrections are all below 2^-43 is the last (the next one would be
+// below rounding, and T, which the cluster step reads, is U's to 2^-42); usually
+// the third. Bound by FP64 at large c (per step 6 c^3 multiply-adds at 2 a cycle
+// and SM: 29 us at c = 144) and by barriers and load latency at small c; as four
+// products and two element passes of their own launches a step took 38 us at
+// c = 32 and 84 us at 144.
+// A 64-thread group takes an 8 x 8 tile: its 8 rows of op(A) and 8 columns of B
+// over the whole k range go to shared memory at once (one round of load
+// latency), then each thread runs its dot product.
+constexpr int kOaTile = 8;
+constexpr int kOaGroups = 2;                    // 64-thread groups of a CTA
+constexpr int kOaThreads = 64 * kOaGroups;
 
-__global__ void svd_oa_norms_kernel(double *__restrict__ P, double *__restrict__ Q, const double *__restrict__ T,
-                                    int c, double *__restrict__ sig, double *__restrict__ part) {
-    __shared__ double red[32];
-    double o2 = 0.0, p2 = 0.0, q2 = 0.0, smax = 0.0;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < c * c; e += gridDim.x * blockDim.x) {
-        const int i = e / c, j = e - i * c;
-        const double d = i == j ? 1.0 : 0.0;
-        const double p = d - P[e], q = d - Q[e], t = T[e];
-        P[e] = p;
-        Q[e] = q;
-        if (i == j) {
-            const double sv = t / (1.0 - 0.5 * (p + q));
-            sig[i] = sv;
-            smax = fmax(smax, fabs(sv));
-        } else {
-            o2 = fma(t, t, o2);
-        }
-        p2 = fma(p, p, p2);
-        q2 = fma(q, q, q2);
+struct OaArgs {
+    const double *R;
+    double *U, *U2, *V, *V2, *W, *T, *P, *Q, *F, *G, *out, *sig;
+    double *part;       // 4 per CTA
+    unsigned *sync;     // kOaSync words, zeroed
+    int *status;        // [1] is set where a barrier gave up
+    int c;
+};
+
+struct OaSmem {
+    double a[kOaTile][kMaxSmemC + 1], b[kMaxSmemC][kOaTile + 1];
+};
+
+// Entry (r0 + ty, c0 + tx) of op(A) B, k ascending; the group's threads load the
+// operands together (read through L2: other CTAs of the launch wrote them).
+__device__ __forceinline__ double oa_tile(OaSmem &sm, const double *A, bool ta, const double *B, int c, int r0, int c0,
+                                          int gt, int grp) {
+    __syncwarp();
+    asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");   // the group's last tile is done
+#pragma unroll 6
+    for (int e = gt; e < kOaTile * c; e += 64) {
+        const int i = ta ? e % kOaTile : e / c, k = ta ? e / kOaTile : e % c;
+        const int r = r0 + i;
+        sm.a[i][k] = r < c ? __ldcg(ta ? A + k * c + r : A + r * c + k) : 0.0;
+        const int j = e % kOaTile, kb = e / kOaTile, cc = c0 + j;
+        sm.b[kb][j] = cc < c ? __ldcg(B + kb * c + cc) : 0.0;
     }
-    o2 = block_sum(o2, red);
-    p2 = block_sum(p2, red);
-    q2 = block_sum(q2, red);
-    {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, off));
-        __syncthreads();
-        if (lane == 0) red[warp] = smax;
-        __syncthreads();
-        double m = 0.0;
-        for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) m = fmax(m, red[w]);
-        smax = m;
-    }
-    if (threadIdx.x == 0) {
-        double *o = part + 4 * blockIdx.x;
-        o[0] = o2;
-        o[1] = p2;
-        o[2] = q2;
-        o[3] = smax;
-    }
+    __syncwarp();
+    asm volatile("bar.sync %0, 64;" ::"r"(grp + 1) : "memory");
+    const int tx = gt % kOaTile, ty = gt / kOaTile;
+    double acc = 0.0;
+    for (int k = 0; k < c; ++k) acc = fma(sm.a[ty][k], sm.b[k][tx], acc);
+    return acc;
 }
 
-// F, G of the update, one element per thread (the divisions spread over the GPU).
-__global__ void svd_oa_fg_kernel(const double *__restrict__ P, const double *__restrict__ Q,
-                                 const double *__restrict__ T, int c, const double *__restrict__ sig,
-                                 const double *__restrict__ part, double *__restrict__ F, double *__restrict__ Gm) {
+__global__ void __launch_bounds__(kOaThreads) svd_refine_kernel(OaArgs A) {
+    __shared__ OaSmem sm[kOaGroups];
+    __shared__ double red[4][kOaThreads / 32];
     __shared__ double s_delta;
-    if (threadIdx.x == 0) {
-        double o2 = 0.0, p2 = 0.0, q2 = 0.0, smax = 0.0;
-        for (int b = 0; b < kOaParts; ++b) {
-            o2 += part[4 * b];
-            p2 += part[4 * b + 1];
-            q2 += part[4 * b + 2];
-            smax = fmax(smax, part[4 * b + 3]);
-        }
-        s_delta = 2.0 * (sqrt(o2) + smax * (sqrt(p2) + sqrt(q2)));
-    }
-    __syncthreads();
-    const double delta = s_delta;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= c * c) return;
-    const int i = e / c, j = e - i * c;
-    const double pij = P[e], qij = Q[e];
-    double f = 0.5 * pij, g = 0.5 * qij;
-    if (i != j) {
-        const double si = sig[i], sj = sig[j];
-        if (fabs(sj - si) > delta) {
-            const double r1 = T[e] + pij * sj;
-            const double r2 = T[j * c + i] + qij * sj;
-            const double inv = 1.0 / ((sj - si) * (sj + si));
-            const double ff = (sj * r1 + si * r2) * inv;
-            const double gg = (si * r1 + sj * r2) * inv;
-            // outside the first-order regime this step only restores orthogonality:
-            // the correction must be small against the pair's relative gap, or its
-            // second-order error (|f|^2 (s_i + s_j) / |s_i - s_j|) would exceed it
-            const double mf = fmax(fabs(ff), fabs(gg));
-            if (mf <= 0.25 && mf * (fabs(si) + fabs(sj)) <= 0.25 * fabs(sj - si)) {
-                f = ff;
-                g = gg;
+    const int c = A.c, nt = (c + kOaTile - 1) / kOaTile, nup = nt * (nt + 1) / 2;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, grp = tid >> 6, gt = tid & 63;
+    const int g0 = blockIdx.x * kOaGroups + grp, ng = gridDim.x * kOaGroups;
+    const int tx = gt % kOaTile, ty = gt / kOaTile;
+    unsigned target = 0;
+    double *U = A.U, *U2 = A.U2, *V = A.V, *V2 = A.V2;
+    for (int it = 0; it < kOaSteps; ++it) {
+        // P = I - U^T U, Q = I - V^T V, W = R V
+        for (int q = g0; q < 2 * nup + nt * nt; q += ng) {
+            const int which = q < nup ? 0 : q < 2 * nup ? 1 : 2;
+            int ti, tj;
+            if (which == 2) {
+                ti = (q - 2 * nup) / nt;
+                tj = (q - 2 * nup) % nt;
+            } else {
+                int rem = q - which * nup;
+                for (ti = 0; rem >= nt - ti; ++ti) rem -= nt - ti;
+                tj = ti + rem;
+            }
+            const double *X = which == 0 ? U : V;
+            const double acc = which == 2 ? oa_tile(sm[grp], A.R, false, V, c, 8 * ti, 8 * tj, gt, grp)
+                                          : oa_tile(sm[grp], X, true, X, c, 8 * ti, 8 * tj, gt, grp);
+            const int row = 8 * ti + ty, col = 8 * tj + tx;
+            if (row >= c || col >= c) continue;
+            if (which == 2) {
+                A.W[row * c + col] = acc;
+            } else {
+                double *to = which == 0 ? A.P : A.Q;
+                const double v = (row == col ? 1.0 : 0.0) - acc;
+                to[row * c + col] = v;
+                to[col * c + row] = v;
             }
         }
+        if (!grid_barrier(A.sync, target, A.status)) return;
+        // T = U^T W; sigma; partial sums of |offdiag T|^2, |P|^2, |Q|^2 and max |sigma|
+        double o2 = 0.0, p2 = 0.0, q2 = 0.0, smax = 0.0;
+        for (int q = g0; q < nt * nt; q += ng) {
+            const int row = 8 * (q / nt) + ty, col = 8 * (q % nt) + tx;
+            const double t = oa_tile(sm[grp], U, true, A.W, c, 8 * (q / nt), 8 * (q % nt), gt, grp);
+            if (row >= c || col >= c) continue;
+            const double p = __ldcg(A.P + row * c + col), qq = __ldcg(A.Q + row * c + col);
+            A.T[row * c + col] = t;
+            if (row == col) {
+                const double sv = t / (1.0 - 0.5 * (p + qq));
+                A.sig[row] = sv;
+                smax = fmax(smax, fabs(sv));
+            } else {
+                o2 = fma(t, t, o2);
+            }
+            p2 = fma(p, p, p2);
+            q2 = fma(qq, qq, q2);
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            o2 += __shfl_xor_sync(0xffffffffu, o2, off);
+            p2 += __shfl_xor_sync(0xffffffffu, p2, off);
+            q2 += __shfl_xor_sync(0xffffffffu, q2, off);
+            smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, off));
+        }
+        if (lane == 0) red[0][warp] = o2, red[1][warp] = p2, red[2][warp] = q2, red[3][warp] = smax;
+        __syncthreads();
+        if (tid < 4) {
+            double v = red[tid][0];
+            for (int w = 1; w < kOaThreads / 32; ++w) v = tid < 3 ? v + red[tid][w] : fmax(v, red[tid][w]);
+            A.part[4 * blockIdx.x + tid] = v;
+        }
+        if (!grid_barrier(A.sync, target, A.status)) return;
+        // F and G, an element per thread
+        if (warp == 0) {
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int b = lane; b < (int)gridDim.x; b += 32) {
+                for (int k = 0; k < 3; ++k) s[k] += __ldcg(A.part + 4 * b + k);
+                s[3] = fmax(s[3], __ldcg(A.part + 4 * b + 3));
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                for (int k = 0; k < 3; ++k) s[k] += __shfl_xor_sync(0xffffffffu, s[k], off);
+                s[3] = fmax(s[3], __shfl_xor_sync(0xffffffffu, s[3], off));
+            }
+            if (lane == 0) s_delta = 2.0 * (sqrt(s[0]) + s[3] * (sqrt(s[1]) + sqrt(s[2])));
+        }
+        __syncthreads();
+        const double delta = s_delta;
+        float big = 0.f;
+        for (int e = blockIdx.x * kOaThreads + tid; e < c * c; e += gridDim.x * kOaThreads) {
+            const int i = e / c, j = e - i * c;
+            const double pij = __ldcg(A.P + e), qij = __ldcg(A.Q + e);
+            double f = 0.5 * pij, g = 0.5 * qij;
+            if (i != j) {
+                const double si = __ldcg(A.sig + i), sj = __ldcg(A.sig + j);
+                if (fabs(sj - si) > delta) {
+                    const double r1 = __ldcg(A.T + e) + pij * sj;
+                    const double r2 = __ldcg(A.T + j * c + i) + qij * sj;
+                    const double inv = 1.0 / ((sj - si) * (sj + si));
+                    const double ff = (sj * r1 + si * r2) * inv;
+                    const double gg = (si * r1 + sj * r2) * inv;
+                    // outside the first-order regime this step only restores orthogonality:
+                    // the correction must be small against the pair's relative gap, or its
+                    // second-order error (|f|^2 (s_i + s_j) / |s_i - s_j|) would exceed it
+                    const double mf = fmax(fabs(ff), fabs(gg));
+                    if (mf <= 0.25 && mf * (fabs(si) + fabs(sj)) <= 0.25 * fabs(sj - si)) {
+                        f = ff;
+                        g = gg;
+                    }
+                }
+            }
+            A.F[e] = f;
+            A.G[e] = g;
+            big = fmaxf(big, fmaxf(fabsf((float)f), fabsf((float)g)));
+        }
+        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(big));
+        if (lane == 0 && m) atomicMax(A.sync + 1 + it, m);
+        if (!grid_barrier(A.sync, target, A.status)) return;
+        const bool last = it + 1 == kOaSteps || __uint_as_float(__ldcg(A.sync + 1 + it)) <= 0x1p-43f;
+        // U + U F (the last step's goes to `out`), V + V G
+        double *to = last ? A.out : U2;
+        for (int q = g0; q < (last ? 1 : 2) * nt * nt; q += ng) {
+            const bool v = q >= nt * nt;
+            const int k = v ? q - nt * nt : q, row = 8 * (k / nt) + ty, col = 8 * (k % nt) + tx;
+            const double acc = oa_tile(sm[grp], v ? V : U, false, v ? A.G : A.F, c, 8 * (k / nt), 8 * (k % nt), gt, grp);
+            if (row < c && col < c) (v ? V2 : to)[row * c + col] = __ldcg((v ? V : U) + row * c + col) + acc;
+        }
+        if (last) return;
+        if (!grid_barrier(A.sync, target, A.status)) return;
+        double *x = U;
+        U = U2;
+        U2 = x;
+        x = V;
+        V = V2;
+        V2 = x;
     }
-    F[e] = f;
-    Gm[e] = g;
 }
 
 // The pairs the first-order step leaves (near-equal singular values, or a
@@ -1736,8 +1781,16 @@ __global__ void __launch_bounds__(kClusterThreads) svd_cluster_kernel(const doub
 // so the loads of the whole matrix are in flight together. Magnitudes are
 // compared and signs flipped on the bit patterns (non-negative doubles order
 // as their bits; integer operations instead of the slow FP64 pipe).
+// A refinement whose barrier gave up (status[1]) leaves NaN.
 __global__ void svd_finish_kernel(const double *__restrict__ U, const double *__restrict__ sg, int c,
-                                  double *__restrict__ UR, double *__restrict__ sigma) {
+                                  double *__restrict__ UR, double *__restrict__ sigma,
+                                  const int *__restrict__ status) {
+    if (status[1] != 0) {
+        const double nan = __longlong_as_double(0x7FF8000000000000ll);
+        for (int e = threadIdx.x; e < c * c; e += blockDim.x) UR[e] = nan;
+        for (int j = threadIdx.x; j < c; j += blockDim.x) sigma[j] = nan;
+        return;
+    }
     __shared__ long long s_abs[256];
     __shared__ int s_rank[256];
     __shared__ unsigned long long s_flip[256];
@@ -1985,59 +2038,41 @@ int cholqr2(Workspace &ws, float *Y, int64_t n, int c, int64_t ld, double *Rout,
     return 0;
 }
 
-// C = op(A) op(B) (+ C0), and when A2 is given also C2 = op(A2) op(B2) (+ C02)
-// in the same launch.
-static int dgemm_small(const double *A, bool ta, const double *B, bool tb, const double *C0, double *C, int c,
-                       cudaStream_t st, const double *A2 = nullptr, const double *B2 = nullptr,
-                       const double *C02 = nullptr, double *C2 = nullptr) {
-    if (c > kDgMaxC) return fail(LNE_ERR_UNSUPPORTED, "small FP64 products support c <= 160");
-    dim3 grid((unsigned)ceil_div(c, kDgTile), (unsigned)ceil_div(c, kDgTile), A2 ? 2u : 1u);
-    LNE_TRACE("dgemm_small", st);
-    dgemm_small_kernel<<<grid, kDgTile * kDgTile, 0, st>>>(A, ta ? 1 : 0, B, tb ? 1 : 0, C0, C, c, A2, B2, C02,
-                                                            C2);
-    LNE_LAUNCH_CHECK();
-    return 0;
-}
-
-// FP64 scratch of the refinement: ten c x c matrices, sigma (c) and the
-// norm partials (4 kOaParts).
+// FP64 scratch of the refinement: ten c x c matrices, sigma (c), the norm
+// partials (4 per CTA), the barrier and the status words.
 struct SvdScratch {
     double *U, *U2, *V, *V2, *W, *T, *P, *Q, *F, *Gm, *sg, *dl;
+    unsigned *sync;
+    int *status;
 };
+constexpr int kOaMaxCtas = 192;   // norm partials held
 
 // Refines the FP32 start (sc.U, sc.V) into the SVD of R in FP64 and writes
 // U_R and sigma (sorted descending).
 static int svd_refine_finish(const double *R, int c, SvdScratch sc, double *U_R, double *sigma, cudaStream_t st) {
     const size_t cc = (size_t)c * c;
-    double *U = sc.U, *U2 = sc.U2, *V = sc.V, *V2 = sc.V2;
-    // FP64 refinement of the SVD of R itself (quadratic convergence; the FP32
-    // start may be loose in directions FP32 cannot resolve, hence four steps)
-    for (int it = 0; it < 4; ++it) {
-        // P = U^T U and Q = V^T V (I - P, I - Q below)
-        LNE_TRY(dgemm_small(U, true, U, false, nullptr, sc.P, c, st, V, V, nullptr, sc.Q));
-        LNE_TRY(dgemm_small(R, false, V, false, nullptr, sc.W, c, st));   // W = R V
-        LNE_TRY(dgemm_small(U, true, sc.W, false, nullptr, sc.T, c, st)); // T = U^T R V
-        {
-            LNE_TRACE("svd_oa_update", st);
-            svd_oa_norms_kernel<<<kOaParts, 256, 0, st>>>(sc.P, sc.Q, sc.T, c, sc.sg, sc.dl);
-            LNE_LAUNCH_CHECK();
-            svd_oa_fg_kernel<<<(unsigned)ceil_div((int64_t)cc, 256), 256, 0, st>>>(sc.P, sc.Q, sc.T, c, sc.sg,
-                                                                                  sc.dl, sc.F, sc.Gm);
-            LNE_LAUNCH_CHECK();
-        }
-        LNE_TRY(dgemm_small(U, false, sc.F, false, U, U2, c, st, V, sc.Gm, V, V2));   // U2 = U + U F, V2 = V + V G
-        std::swap(U, U2);
-        std::swap(V, V2);
+    const int nt = (int)ceil_div(c, kOaTile);
+    {
+        LNE_TRACE("svd_refine", st);
+        // out: W's buffer, which the last step no longer reads
+        OaArgs A{R, sc.U, sc.U2, sc.V, sc.V2, sc.W, sc.T, sc.P, sc.Q, sc.F, sc.Gm, sc.W, sc.sg, sc.dl, sc.sync,
+                 sc.status, c};
+        const int ctas = (int)std::min<int64_t>(ceil_div(nt * (nt + 1) + nt * nt, kOaGroups),
+                                                std::min(num_sms(), kOaMaxCtas));
+        void *args[] = {&A};
+        LNE_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(svd_refine_kernel), dim3(ctas),
+                                                 dim3(kOaThreads), args, 0, st));
+        LNE_LAUNCH_CHECK();
     }
     {
         LNE_TRACE("svd_cluster", st);
         LNE_TRY(allow_dynamic_smem(svd_cluster_kernel));
-        svd_cluster_kernel<<<1, kClusterThreads, sizeof(double) * cc, st>>>(sc.T, c, U, sc.sg);
+        svd_cluster_kernel<<<1, kClusterThreads, sizeof(double) * cc, st>>>(sc.T, c, sc.W, sc.sg);
         LNE_LAUNCH_CHECK();
     }
     {
         LNE_TRACE("svd_finish", st);
-        svd_finish_kernel<<<1, 256, 0, st>>>(U, sc.sg, c, U_R, sigma);
+        svd_finish_kernel<<<1, 256, 0, st>>>(sc.W, sc.sg, c, U_R, sigma, sc.status);
         LNE_LAUNCH_CHECK();
     }
     return 0;
@@ -2061,7 +2096,11 @@ int small_svd(Workspace &ws, const double *R, int c, double *U_R, double *sigma,
     LNE_TRY(ws.get("svd.G", cc, &Gm));
     LNE_TRY(ws.get("svd.sg", (size_t)c, &sg));
     double *dl = nullptr;
-    LNE_TRY(ws.get("svd.delta", 4 * kOaParts, &dl));
+    unsigned *sync = nullptr;
+    int *status = nullptr;
+    LNE_TRY(ws.get("svd.delta", 4 * kOaMaxCtas, &dl));
+    LNE_TRY(ws.get("svd.sync", kOaSync, &sync));
+    LNE_TRY(device_status(ws, &status, st));
     LNE_TRY(ws.get("svd.sweeps", 1, &sweeps));
     float2 *jrot = nullptr;
     uint32_t *jlab = nullptr;
@@ -2072,9 +2111,9 @@ int small_svd(Workspace &ws, const double *R, int c, double *U_R, double *sigma,
     // starting point: FP32 one-sided Jacobi on R (U, V in FP64 storage)
     {
         LNE_TRACE("jacobi32", st);
-        LNE_TRY(launch_jacobi(R, c, U, V, jrot, jlab, sweeps, st));
+        LNE_TRY(launch_jacobi(R, c, U, V, jrot, jlab, sweeps, sync, st));
     }
-    SvdScratch sc{U, U2, V, V2, W, T, P, Q, F, Gm, sg, dl};
+    SvdScratch sc{U, U2, V, V2, W, T, P, Q, F, Gm, sg, dl, sync, status};
     return svd_refine_finish(R, c, sc, U_R, sigma, st);
 }
 
@@ -2124,8 +2163,9 @@ namespace {
 constexpr int kNoAllocMaxC = 160;
 constexpr size_t kNoAllocMat = (size_t)kNoAllocMaxC * kNoAllocMaxC;
 constexpr size_t kNoAllocRec = (size_t)kJacMaxSweeps * (kJacRegMaxC + 2) * (kJacRegMaxC / 2);   // >= jreg_records(c)
-constexpr size_t kNoAllocDoubles = 10 * kNoAllocMat + kNoAllocMaxC + 128 + kNoAllocRec + kNoAllocRec / 2;
-static_assert(4 * kOaParts + 8 <= 128, "partial sums and sweep count fit the reserve");
+constexpr size_t kNoAllocSmall = 4 * kOaMaxCtas + 16;   // norm partials; sweep count and sync words
+constexpr size_t kNoAllocDoubles = 10 * kNoAllocMat + kNoAllocMaxC + kNoAllocSmall + kNoAllocRec + kNoAllocRec / 2;
+static_assert((kOaSync + 2) * sizeof(unsigned) <= 16 * sizeof(double) && kOaSteps + 3 <= kOaSync, "the words fit the reserve");
 static __device__ __align__(256) double g_svd_scratch[kNoAllocDoubles];
 
 constexpr int kNoAllocMaxDevices = 64;
@@ -2164,11 +2204,13 @@ extern "C" int lne_svd_small_noalloc(const double *R_dev, int32_t c, double *U_d
            *T = base + 5 * cc, *P = base + 6 * cc, *Q = base + 7 * cc, *F = base + 8 * cc, *Gm = base + 9 * cc;
     double *sg = base + 10 * kNoAllocMat;
     double *dl = sg + kNoAllocMaxC;
-    int *sweeps = reinterpret_cast<int *>(dl + 4 * kOaParts);
-    float2 *jrot = reinterpret_cast<float2 *>(base + 10 * kNoAllocMat + kNoAllocMaxC + 128);
+    int *sweeps = reinterpret_cast<int *>(dl + 4 * kOaMaxCtas), *status = nullptr;
+    unsigned *sync = reinterpret_cast<unsigned *>(sweeps + 2);
+    status = reinterpret_cast<int *>(sync + kOaSync - 2);   // two words that each call zeroes with the others
+    float2 *jrot = reinterpret_cast<float2 *>(base + 10 * kNoAllocMat + kNoAllocMaxC + kNoAllocSmall);
     uint32_t *jlab = reinterpret_cast<uint32_t *>(jrot + kNoAllocRec);
-    LNE_TRY(launch_jacobi(R_dev, c, U, V, jrot, jlab, sweeps, st));
-    SvdScratch sc{U, U2, V, V2, W, T, P, Q, F, Gm, sg, dl};
+    LNE_TRY(launch_jacobi(R_dev, c, U, V, jrot, jlab, sweeps, sync, st));
+    SvdScratch sc{U, U2, V, V2, W, T, P, Q, F, Gm, sg, dl, sync, status};
     LNE_TRY(svd_refine_finish(R_dev, c, sc, U_dev, sigma_dev, st));
     return LNE_OK;
 }

@@ -518,40 +518,6 @@ __device__ __forceinline__ float adam_step(const AdamArgs &A, float c1, float c2
     return wi - A.lr * (mi / c1) / (sqrtf(vi / c2) + A.eps);
 }
 
-// A barrier over the grid of a cooperative launch (all CTAs resident). Gives
-// up after 2 s: status[1] is set and every CTA returns false, after which the
-// kernel ends.
-__device__ __forceinline__ bool grid_wait(unsigned *bar, unsigned &target, int *status) {
-    __shared__ int ok_s;
-    __syncthreads();
-    target += gridDim.x;
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        unsigned v;
-        __threadfence();
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-        uint64_t t0 = 0;
-        for (unsigned spin = 1;; ++spin) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if ((int)(v - target) >= 0) break;   // the count may wrap
-            if ((spin & 63u) == 0u) {
-                uint64_t t;
-                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-                if (t0 == 0) t0 = t;
-                if (t - t0 > 2000000000ull) {
-                    atomicExch(status + 1, 1);
-                    ok = 0;
-                    break;
-                }
-            }
-        }
-        __threadfence();
-        ok_s = ok;
-    }
-    __syncthreads();
-    return ok_s != 0;
-}
-
 // Whole passes over the training rows in one cooperative launch: `epochs`
 // orders of `rows` indices, mini-batches of `batch` rows, one Adam step each.
 // A step is the row pass, a grid barrier, the weight pass with Adam applied to
@@ -602,7 +568,7 @@ __global__ void __launch_bounds__(kThreads, 1) sur_train_kernel(TrainArgs T) {
             }
         }
         const float2 cc = __ldg(T.corr + s);
-        if (!grid_wait(T.bar, target, T.status)) return;
+        if (!grid_barrier(T.bar, target, T.status)) return;
         const GradArgs G{A.Xs, A.H1, A.H2, A.dy, A.dZ1, A.dZ2, A.B};
         if (s + 1 < steps) {
             A = batch_of(s + 1);
@@ -645,7 +611,7 @@ __global__ void __launch_bounds__(kThreads, 1) sur_train_kernel(TrainArgs T) {
                 });
             __syncthreads();
         }
-        if (s + 1 < steps && !grid_wait(T.bar, target, T.status)) return;
+        if (s + 1 < steps && !grid_barrier(T.bar, target, T.status)) return;
     }
 }
 
