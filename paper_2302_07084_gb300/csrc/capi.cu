@@ -288,46 +288,63 @@ lne::CsrView csr_view(const lne_csr *M) {
     return v;
 }
 
-// The CSR structure of a graph: bit 1 of *bad for an indptr entry below its
-// predecessor, bit 2 for a column index outside [0, n). Reads indptr[0..n]
-// and indices[0..nnz) only. With indptr[0] = 0 and indptr[n] = nnz (checked
-// on the host), a non-decreasing indptr keeps every row inside [0, nnz).
+// What the host needs of a graph's CSR arrays: the ends of indptr, whether the
+// structure is sound (bit 1 of bad: an indptr entry below its predecessor, bit
+// 2: a column index outside [0, n)), and the longest row.
+struct CsrInfo {
+    int64_t first, last;
+    unsigned long long max_row;
+    int bad;
+};
+
+// Reads indptr[0..n] and indices[0..nnz) only; *info is zero before. With
+// indptr[0] = 0 and indptr[n] = nnz (checked on the host), a non-decreasing
+// indptr keeps every row inside [0, nnz).
 __global__ void csr_structure_kernel(const int64_t *__restrict__ indptr, int64_t n,
-                                     const int32_t *__restrict__ indices, int64_t nnz, int *__restrict__ bad) {
+                                     const int32_t *__restrict__ indices, int64_t nnz, CsrInfo *__restrict__ info) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int f = 0;
-    for (int64_t i = t0; i < n; i += stride)
-        if (indptr[i + 1] < indptr[i]) f |= 1;
+    int64_t longest = 0;
+    if (t0 == 0) {
+        info->first = indptr[0];
+        info->last = indptr[n];
+    }
+    for (int64_t i = t0; i < n; i += stride) {
+        const int64_t len = indptr[i + 1] - indptr[i];
+        if (len < 0) f |= 1;
+        longest = max(longest, len);
+    }
     for (int64_t e = t0; e < nnz; e += stride) {
         const int32_t v = indices[e];
         if (v < 0 || (int64_t)v >= n) f |= 2;
     }
-    if (f) atomicOr(bad, f);
+    if (f) atomicOr(&info->bad, f);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) longest = max(longest, __shfl_xor_sync(0xffffffffu, longest, off));
+    if ((threadIdx.x & 31) == 0 && longest > 0) atomicMax(&info->max_row, (unsigned long long)longest);
 }
 
 // Checks the graph on the device before any kernel walks it: indptr starts at
-// 0, ends at nnz and never decreases, and every index lies in [0, n).
-int check_graph_device(lne_ctx *ctx, const lne_graph *g, cudaStream_t st) {
-    int64_t ends[2] = {0, 0};
-    int bad = 0;
-    int *bad_dev = nullptr;
-    LNE_TRY(ctx->ws.get("graph.check", 1, &bad_dev));
-    LNE_CUDA_TRY(cudaMemsetAsync(bad_dev, 0, sizeof(int), st));
+// 0, ends at nnz and never decreases, and every index lies in [0, n). *max_deg
+// receives the longest row.
+int check_graph_device(lne_ctx *ctx, const lne_graph *g, int64_t *max_deg, cudaStream_t st) {
+    CsrInfo h, *dev = nullptr;
+    LNE_TRY(ctx->ws.get("graph.check", 1, &dev));
+    LNE_CUDA_TRY(cudaMemsetAsync(dev, 0, sizeof(CsrInfo), st));
     {
         const int64_t work = std::max<int64_t>(std::max<int64_t>(g->n, g->nnz), 1);
         const unsigned blocks = (unsigned)std::min<int64_t>(lne::ceil_div(work, (int64_t)256), lne::num_sms() * 8);
-        csr_structure_kernel<<<blocks, 256, 0, st>>>(g->indptr, g->n, g->indices, g->nnz, bad_dev);
+        csr_structure_kernel<<<blocks, 256, 0, st>>>(g->indptr, g->n, g->indices, g->nnz, dev);
         LNE_LAUNCH_CHECK();
     }
-    LNE_CUDA_TRY(cudaMemcpyAsync(&ends[0], g->indptr, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    LNE_CUDA_TRY(cudaMemcpyAsync(&ends[1], g->indptr + g->n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    LNE_CUDA_TRY(cudaMemcpyAsync(&bad, bad_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
+    LNE_CUDA_TRY(cudaMemcpyAsync(&h, dev, sizeof(CsrInfo), cudaMemcpyDeviceToHost, st));
     LNE_CUDA_TRY(cudaStreamSynchronize(st));
-    if (ends[0] != 0 || ends[1] != g->nnz)
+    if (h.first != 0 || h.last != g->nnz)
         return lne::fail(LNE_ERR_INVALID, "graph indptr must start at 0 and end at nnz");
-    if (bad & 1) return lne::fail(LNE_ERR_INVALID, "graph indptr decreases");
-    if (bad & 2) return lne::fail(LNE_ERR_INVALID, "a graph index is outside [0, n)");
+    if (h.bad & 1) return lne::fail(LNE_ERR_INVALID, "graph indptr decreases");
+    if (h.bad & 2) return lne::fail(LNE_ERR_INVALID, "a graph index is outside [0, n)");
+    *max_deg = (int64_t)h.max_row;
     return 0;
 }
 
@@ -485,8 +502,10 @@ int lne_sample_pairs(lne_ctx *ctx, const lne_graph *g, const lne_params *p, int6
     if (rc == 0 && (!count_out || (capacity > 0 && (!u1_dev || !v1_dev))))
         rc = lne::fail(LNE_ERR_INVALID, "NULL output");
     cudaStream_t st = as_stream(stream);
-    if (rc == 0) rc = check_graph_device(ctx, g, st);
+    int64_t max_deg = 0;
+    if (rc == 0) rc = check_graph_device(ctx, g, &max_deg, st);
     lne::GraphView gv = view(g);
+    gv.max_deg = max_deg;
     if (rc == 0) rc = lne::prepare_weighted(ctx->ws, &gv, st);
     lne::SamplerSpec sp;
     if (rc == 0) rc = lne::make_sampler_spec(gv, p->T, p->s, p->samples, p->b, p->seed, &sp);
@@ -506,8 +525,10 @@ int lne_sparsifier_counts(lne_ctx *ctx, const lne_graph *g, const lne_params *p,
     if (rc == 0) rc = check_params(p, true);
     if (rc == 0 && !out) rc = lne::fail(LNE_ERR_INVALID, "NULL output");
     cudaStream_t st = as_stream(stream);
-    if (rc == 0) rc = check_graph_device(ctx, g, st);
+    int64_t max_deg = 0;
+    if (rc == 0) rc = check_graph_device(ctx, g, &max_deg, st);
     lne::GraphView gv = view(g);
+    gv.max_deg = max_deg;
     if (rc == 0) rc = lne::prepare_weighted(ctx->ws, &gv, st);
     lne::SamplerSpec sp;
     if (rc == 0) rc = lne::make_sampler_spec(gv, p->T, p->s, p->samples, p->b, p->seed, &sp);
@@ -535,8 +556,10 @@ int lne_sparsifier_csr(lne_ctx *ctx, const lne_graph *g, const lne_params *p, ln
     if (rc == 0) rc = check_params(p, true);
     if (rc == 0 && !out) rc = lne::fail(LNE_ERR_INVALID, "NULL output");
     cudaStream_t st = as_stream(stream);
-    if (rc == 0) rc = check_graph_device(ctx, g, st);
+    int64_t max_deg = 0;
+    if (rc == 0) rc = check_graph_device(ctx, g, &max_deg, st);
     lne::GraphView gv = view(g);
+    gv.max_deg = max_deg;
     if (rc == 0) rc = lne::prepare_weighted(ctx->ws, &gv, st);
     lne::SamplerSpec sp;
     if (rc == 0) rc = lne::make_sampler_spec(gv, p->T, p->s, p->samples, p->b, p->seed, &sp);
@@ -711,8 +734,10 @@ int lne_embed(lne_ctx *ctx, const lne_graph *g, const lne_params *p, float *X_de
     if (rc == 0 && !X_dev) rc = lne::fail(LNE_ERR_INVALID, "NULL embedding buffer");
     if (rc == 0 && (p->k < 0 || p->q < 0 || p->d < 1)) rc = lne::fail(LNE_ERR_INVALID, "need d >= 1, q >= 0, k >= 0");
     cudaStream_t st = as_stream(stream);
-    if (rc == 0) rc = check_graph_device(ctx, g, st);
+    int64_t max_deg = 0;
+    if (rc == 0) rc = check_graph_device(ctx, g, &max_deg, st);
     lne::GraphView gv = view(g);
+    gv.max_deg = max_deg;
     if (rc == 0) rc = lne::prepare_weighted(ctx->ws, &gv, st);
     lne::SamplerSpec sp;
     if (rc == 0) rc = lne::make_sampler_spec(gv, p->T, p->s, p->samples, p->b, p->seed, &sp);
@@ -748,8 +773,10 @@ int lne_tune_batch(lne_ctx *ctx, const lne_graph *g, const lne_params *cands, in
     if (rc == 0 && (!labels_dev || L < 1 || !train_dev || n_train < 1 || !test_dev || n_test < 1 || iters < 0))
         rc = lne::fail(LNE_ERR_INVALID, "bad evaluation split or labels");
     cudaStream_t st = as_stream(stream);
-    if (rc == 0) rc = check_graph_device(ctx, g, st);
+    int64_t max_deg = 0;
+    if (rc == 0) rc = check_graph_device(ctx, g, &max_deg, st);
     lne::GraphView gv = view(g);
+    gv.max_deg = max_deg;
     if (rc == 0) rc = lne::prepare_weighted(ctx->ws, &gv, st);
     if (rc == 0 && !ctx->prop_graph) ctx->prop_graph = lne::new_prop_cache();
     if (rc == 0)
@@ -777,9 +804,11 @@ int lne_tune_tasks(lne_ctx *ctx, const lne_task *tasks, int32_t ntasks, const ln
         if (rc == 0 && (!k.labels_dev || k.L < 1 || !k.train_dev || k.n_train < 1 || !k.test_dev || k.n_test < 1))
             rc = lne::fail(LNE_ERR_INVALID, "bad evaluation split or labels");
         for (int j = 0; rc == 0 && j < ncand; ++j) rc = check_params(&cands[(size_t)t * ncand + j], true);
-        if (rc == 0) rc = check_graph_device(ctx, &k.graph, st);
+        int64_t max_deg = 0;
+        if (rc == 0) rc = check_graph_device(ctx, &k.graph, &max_deg, st);
         if (rc == 0) {
             tt[t].g = view(&k.graph);
+            tt[t].g.max_deg = max_deg;
             tt[t].labels = k.labels_dev;
             tt[t].L = k.L;
             tt[t].train = k.train_dev;

@@ -188,7 +188,16 @@ int propagate(Workspace &ws, const GraphView &g, int d, int k, double theta, dou
     };
     // Y = op(A) X with X given in FP32; BF16 mode gathers X's BF16 copy and
     // keeps a BF16 copy of the output too
+    uint32_t *row_cnt = nullptr;
+    int32_t *slice_row = nullptr;
+    if (d % 4 == 0 && k > 1) {   // the merge path's products
+        LNE_TRY(merge_chain(ws, "prop.chain", g, d, &row_cnt, &slice_row));
+        LNE_TRY(merge_chain_prepare(g, row_cnt, slice_row, st));
+    }
     auto gspmm = [&](const float *Xin, float *Yout, SpmmEpilogue ep) -> int {
+        ep.row_cnt = row_cnt;
+        ep.slice_row = slice_row;
+        ep.max_row = g.max_deg;
         if (!bf16) return graph_spmm(ws, g, Xin, d, d, Yout, d, ep, st);
         ep.Yb = half_of(Yout);
         if (ep.G) ep.Gb = Gh;
@@ -321,8 +330,9 @@ struct PropBatchGraph {
 
 static int prop_batch_chain(Workspace &ws, const GraphView &g, int C, int kmax, const float *X0, float *F, float *Z,
                             float *Tbuf[3], float *G, float *P, const float *om, const float *hom, const float *gam,
-                            SpmmTile tile, cudaStream_t st) {
+                            SpmmTile tile, uint32_t *row_cnt, int32_t *slice_row, cudaStream_t st) {
     const int64_t cnt = g.n * C;
+    LNE_TRY(merge_chain_prepare(g, row_cnt, slice_row, st));
     {
         LNE_TRACE("scale_cols", st);
         scale_cols_kernel<<<elem_grid(cnt), 256, 0, st>>>(X0, gam, g.n, C, F);
@@ -338,6 +348,9 @@ static int prop_batch_chain(Workspace &ws, const GraphView &g, int C, int kmax, 
         e1.threads = tile.threads;
         e1.col_block = tile.col_block;
         e1.carry_tag = "pb.carry";
+        e1.row_cnt = row_cnt;
+        e1.slice_row = slice_row;
+        e1.max_row = g.max_deg;
         LNE_TRY(graph_spmm(ws, g, X0, C, C, Z, C, e1, st));
         SpmmEpilogue e2;
         e2.alpha = -0.5f;
@@ -352,6 +365,9 @@ static int prop_batch_chain(Workspace &ws, const GraphView &g, int C, int kmax, 
         e2.threads = tile.threads;
         e2.col_block = tile.col_block;
         e2.carry_tag = "pb.carry";
+        e2.row_cnt = row_cnt;
+        e2.slice_row = slice_row;
+        e2.max_row = g.max_deg;
         LNE_TRY(graph_spmm(ws, g, Z, C, C, Tbuf[0], C, e2, st));
         const float *prev = X0;
         float *cur = Tbuf[0];
@@ -371,6 +387,9 @@ static int prop_batch_chain(Workspace &ws, const GraphView &g, int C, int kmax, 
             ez.threads = tile.threads;
         ez.col_block = tile.col_block;
             ez.carry_tag = "pb.carry";
+            ez.row_cnt = row_cnt;
+            ez.slice_row = slice_row;
+            ez.max_row = g.max_deg;
             LNE_TRY(graph_spmm(ws, g, cur, C, C, Z, C, ez, st));
             SpmmEpilogue e;
             e.alpha = -1.f;
@@ -387,6 +406,9 @@ static int prop_batch_chain(Workspace &ws, const GraphView &g, int C, int kmax, 
             e.threads = tile.threads;
         e.col_block = tile.col_block;
             e.carry_tag = "pb.carry";
+            e.row_cnt = row_cnt;
+            e.slice_row = slice_row;
+            e.max_row = g.max_deg;
             LNE_TRY(graph_spmm(ws, g, Z, C, C, nxt, C, e, st));
             prev = cur;
             cur = nxt;
@@ -404,6 +426,9 @@ static int prop_batch_chain(Workspace &ws, const GraphView &g, int C, int kmax, 
     ep.threads = tile.threads;
     ep.col_block = tile.col_block;
     ep.carry_tag = "pb.carry";
+    ep.row_cnt = row_cnt;
+    ep.slice_row = slice_row;
+    ep.max_row = g.max_deg;
     return graph_spmm(ws, g, G, C, C, P, C, ep, st);
 }
 
@@ -441,15 +466,20 @@ int propagate_batch(Workspace &ws, PropBatchGraph *cache, const GraphView &g, in
     float4 *carry = nullptr;
     int64_t *carry_row = nullptr;
     LNE_TRY(merge_carry(ws, "pb.carry", g.nnz, g.n, C, &carry, &carry_row));
+    uint32_t *row_cnt = nullptr;
+    int32_t *slice_row = nullptr;
+    LNE_TRY(merge_chain(ws, "pb.chain", g, tile.col_block > 0 ? tile.col_block : C, &row_cnt, &slice_row));
     const float *om = coef, *hom = coef + C, *gam = coef + 2 * C;
-    if (!cache) return prop_batch_chain(ws, g, C, kmax, X0, F, Z, Tb, G, P, om, hom, gam, tile, st);
+    if (!cache) return prop_batch_chain(ws, g, C, kmax, X0, F, Z, Tb, G, P, om, hom, gam, tile, row_cnt, slice_row, st);
     // graph key: everything the captured launches depend on
     std::vector<uintptr_t> key = {(uintptr_t)g.indptr, (uintptr_t)g.indices, (uintptr_t)g.n,  (uintptr_t)g.nnz,
                                   (uintptr_t)C,        (uintptr_t)kmax,      (uintptr_t)X0,   (uintptr_t)P,
                                   (uintptr_t)coef,     (uintptr_t)F,         (uintptr_t)Z,    (uintptr_t)G,
                                   (uintptr_t)Tb[0],    (uintptr_t)Tb[1],     (uintptr_t)Tb[2], (uintptr_t)tile.threads,
                                   (uintptr_t)tile.col_block,
-                                  (uintptr_t)carry,    (uintptr_t)carry_row, (uintptr_t)g.wf, (uintptr_t)g.dinv};
+                                  (uintptr_t)row_cnt,  (uintptr_t)slice_row,
+                                  (uintptr_t)carry,    (uintptr_t)carry_row, (uintptr_t)g.wf, (uintptr_t)g.dinv,
+                                  (uintptr_t)g.max_deg};
     if (cache->valid && cache->key == key) {
         LNE_TRACE("propagate_batch_graph", st);
         LNE_CUDA_TRY(cudaGraphLaunch(cache->exec, st));
@@ -463,7 +493,7 @@ int propagate_batch(Workspace &ws, PropBatchGraph *cache, const GraphView &g, in
     }
     if (cache->seen == 0) {   // first run: eager (allocates every buffer the chain needs)
         cache->seen = 1;
-        return prop_batch_chain(ws, g, C, kmax, X0, F, Z, Tb, G, P, om, hom, gam, tile, st);
+        return prop_batch_chain(ws, g, C, kmax, X0, F, Z, Tb, G, P, om, hom, gam, tile, row_cnt, slice_row, st);
     }
     // second run with the same key: capture, instantiate, launch
     if (cache->exec) {
@@ -478,7 +508,8 @@ int propagate_batch(Workspace &ws, PropBatchGraph *cache, const GraphView &g, in
     if (!cache->capture) LNE_CUDA_TRY(cudaStreamCreateWithFlags(&cache->capture, cudaStreamNonBlocking));
     const int64_t before = launches_now();
     LNE_CUDA_TRY(cudaStreamBeginCapture(cache->capture, cudaStreamCaptureModeThreadLocal));
-    int rc = prop_batch_chain(ws, g, C, kmax, X0, F, Z, Tb, G, P, om, hom, gam, tile, cache->capture);
+    int rc = prop_batch_chain(ws, g, C, kmax, X0, F, Z, Tb, G, P, om, hom, gam, tile, row_cnt, slice_row,
+                              cache->capture);
     cudaError_t e = cudaStreamEndCapture(cache->capture, &graph);
     set_tracer(tracer);
     cache->kernels = launches_now() - before;

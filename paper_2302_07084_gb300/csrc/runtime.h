@@ -46,6 +46,7 @@ struct GraphView {
     int64_t nnz = 0;
     const int64_t *indptr = nullptr;
     const int32_t *indices = nullptr;
+    int64_t max_deg = 0;              // longest row (0 = not known)
     // weighted graphs (w = NULL: unweighted); the rest is derived from w by
     // prepare_weighted
     const uint32_t *w = nullptr;      // [nnz] positive integer arc weights, symmetric
@@ -193,6 +194,11 @@ struct SpmmEpilogue {
     int threads = 0;                    // CTA size of the merge kernel (0 = default)
     int col_block = 0;                  // merge products of more columns run in blocks of this many (0 = one)
     const char *carry_tag = nullptr;    // workspace name of the merge carry buffers (NULL = shared)
+    // products of a chain with one matrix (merge_chain): per-row arrival counters
+    // (zero before and after each product) and every slice's first row
+    uint32_t *row_cnt = nullptr;
+    const int32_t *slice_row = nullptr;
+    int64_t max_row = 0;                // the longest row, if known: short rows take a lane group each
 };
 // Device status words of the context (workspace "dev.status", zeroed when
 // created): [0] the first Cholesky breakdown, [1] a tensor-core pipeline wait
@@ -213,6 +219,11 @@ int dense_tc_spmm(Workspace &ws, const float *Ahi, const float *Alo, int64_t ld,
                   int64_t ldx, int c, float *Y, int64_t ldy, cudaStream_t st);
 // Carry buffers of the merge SpMM for nnz nonzeros over n rows and c columns, under the
 // workspace names tag + ".c" / tag + ".r" (tag NULL = "spmm.carry").
+// Buffers of a chain of products of g's matrix with c columns
+// (SpmmEpilogue::row_cnt, slice_row; NULL where none are needed), and the work
+// before the chain's first product.
+int merge_chain(Workspace &ws, const char *tag, const GraphView &g, int c, uint32_t **row_cnt, int32_t **slice_row);
+int merge_chain_prepare(const GraphView &g, uint32_t *row_cnt, int32_t *slice_row, cudaStream_t st);
 int merge_carry(Workspace &ws, const char *tag, int64_t nnz, int64_t n, int c, float4 **carry,
                 int64_t **carry_row);
 int graph_spmm(Workspace &ws, const GraphView &g, const float *X, int64_t ldx, int c, float *Y, int64_t ldy,

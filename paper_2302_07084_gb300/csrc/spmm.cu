@@ -11,7 +11,12 @@
 // warp's slice is finished there; a row crossing slice boundaries leaves its
 // partial sums in a carry buffer, and a fix-up kernel adds them in slice order.
 // Every sum has a fixed order, so results are deterministic and independent of
-// the degree distribution's skew.
+// the degree distribution's skew. A chain of products with one matrix (the
+// propagation) prepares each slice's first row once and lets the last slice of
+// a row to arrive add the partial sums itself, in the same order (row_cnt), so
+// that a product is one launch without a search: on the BlogCatalog-shaped graph
+// at d = 128 50 -> 44 us a product (8 gathered rows in flight instead of 4 are
+// part of it).
 // Fallback (other column counts): one warp per row, lane l owns columns l,
 // l+32, ...; rows longer than 512 nonzeros get a whole CTA.
 #include "runtime.h"
@@ -164,7 +169,11 @@ __device__ __forceinline__ void gather4(const int32_t *__restrict__ indices, con
     const int col = lane < cnt ? (STREAM ? __ldcs(indices + p + lane) : __ldg(indices + p + lane)) : 0;
     float v = 0.f;
     if (WEIGHTED) v = lane < cnt ? (STREAM ? __ldcs(vals + p + lane) : __ldg(vals + p + lane)) : 0.f;
-#pragma unroll 4
+    // rows in flight per warp: 8 for the unweighted products of up to 128 columns,
+    // 4 elsewhere. Batches held in registers with a predicated tail (64 to 80
+    // registers) were slower where the GPU is full of warps: 44 -> 52 us for the
+    // propagation product above, 4.4 -> 5.5 ms for 6e7 nonzeros x 144 columns
+#pragma unroll(NV == 1 && !WEIGHTED ? 8 : 4)
     for (int k = 0; k < cnt; ++k) {
         const int ck = __shfl_sync(0xffffffffu, col, k);
         const float vk = WEIGHTED ? __shfl_sync(0xffffffffu, v, k) : 1.f;
@@ -293,7 +302,8 @@ __device__ __forceinline__ int64_t row_of(const int64_t *__restrict__ indptr, in
 // block's virtual row offsets V (prefix sums of the rows' segment lengths);
 // row r's segment starts at indptr0[r] + segb[r] of indices / vals, so
 // position p of the row maps to p + indptr0[r] + segb[r] - V[r].
-template <int NV, bool WEIGHTED, typename TX, int LG = 32, bool VB = false>
+// CHAIN: a product of a chain (ep.row_cnt and ep.slice_row are set).
+template <int NV, bool WEIGHTED, typename TX, int LG = 32, bool VB = false, bool CHAIN = false>
 __global__ void __launch_bounds__(256) spmm_merge_kernel(int64_t n, int64_t nnz, const int64_t *__restrict__ indptr,
                                                          const int32_t *__restrict__ indices,
                                                          const float *__restrict__ vals, const TX *__restrict__ X,
@@ -306,13 +316,18 @@ __global__ void __launch_bounds__(256) spmm_merge_kernel(int64_t n, int64_t nnz,
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (w >= nwarps) return;
     const int64_t p0 = w * W, p1 = imin64(p0 + W, nnz);
-    if (lane == 0) {   // slots left from an earlier product must not be read
+    if (!CHAIN && lane == 0) {   // slots left from an earlier product must not be read
         carry_row[w * 2] = -1;
         carry_row[w * 2 + 1] = -1;
     }
-    int64_t r = row_of(indptr, n, p0);
-    // skip empty rows sharing the start offset
-    while (r + 1 < n && __ldg(indptr + r + 1) <= p0) ++r;
+    int64_t r;
+    if (CHAIN) {
+        r = __ldg(ep.slice_row + w);
+    } else {
+        r = row_of(indptr, n, p0);
+        // skip empty rows sharing the start offset
+        while (r + 1 < n && __ldg(indptr + r + 1) <= p0) ++r;
+    }
     int64_t p = p0;
     while (p < p1) {
         const int64_t rs = VB ? __ldcs(indptr + r) : __ldg(indptr + r);
@@ -350,11 +365,64 @@ __global__ void __launch_bounds__(256) spmm_merge_kernel(int64_t n, int64_t nnz,
 #pragma unroll
             for (int t = 0; t < NV; ++t)
                 if (lane + 32 * t < c4) dst[lane + 32 * t] = acc.v[t];
-            if (lane == 0) carry_row[w * 2 + slot] = r;
+            if (!CHAIN) {
+                if (lane == 0) carry_row[w * 2 + slot] = r;
+            } else {
+                // the row's last slice to arrive adds all of them, in slice order
+                const int64_t w0 = rs / W, w1 = (re - 1) / W;
+                unsigned seen = 0;
+                __threadfence();
+                __syncwarp();
+                if (lane == 0) seen = atomicAdd(ep.row_cnt + r, 1u);
+                seen = __shfl_sync(0xffffffffu, seen, 0);
+                if (seen == (unsigned)(w1 - w0)) {
+                    __threadfence();
+                    if (lane == 0) ep.row_cnt[r] = 0u;   // for the next product
+#pragma unroll
+                    for (int t = 0; t < NV; ++t) acc.v[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int64_t s = w0; s <= w1; ++s) {
+                        const float4 *src = carry + (s * 2 + (rs < s * W ? 0 : 1)) * (int64_t)(NV * 32);
+#pragma unroll
+                        for (int t = 0; t < NV; ++t) {
+                            if (lane + 32 * t < c4) {
+                                const float4 x = __ldcg(src + lane + 32 * t);
+                                acc.v[t].x += x.x;
+                                acc.v[t].y += x.y;
+                                acc.v[t].z += x.z;
+                                acc.v[t].w += x.w;
+                            }
+                        }
+                    }
+                    epilogue4<NV, VB>(r, re - rs, acc, lane, c4, Y, ldy, ep);
+                }
+            }
         }
         p = e;
         ++r;
         while (p < p1 && r + 1 < n && __ldg(indptr + r + 1) <= p) ++r;   // empty rows
+    }
+    if (!CHAIN) return;
+    // the empty rows' epilogues: 32 rows a warp step
+    const int64_t step = nwarps * 32;
+    for (int64_t b = w * 32; b < n; b += step) {
+        const int64_t i = b + lane;
+        unsigned m = __ballot_sync(0xffffffffu, i < n && __ldg(indptr + i + 1) == __ldg(indptr + i));
+        for (; m; m &= m - 1u) {
+            Acc4<NV> acc;
+#pragma unroll
+            for (int t = 0; t < NV; ++t) acc.v[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+            epilogue4<NV, VB>(b + __ffs(m) - 1, 0, acc, lane, c4, Y, ldy, ep);
+        }
+    }
+}
+
+// The row that holds nonzero w W (the first slice's first row with a nonzero), for every slice w.
+__global__ void slice_rows_kernel(const int64_t *__restrict__ indptr, int64_t n, int64_t W, int64_t nwarps,
+                                  int32_t *__restrict__ rows) {
+    for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < nwarps; w += (int64_t)gridDim.x * blockDim.x) {
+        int64_t r = row_of(indptr, n, w * W);
+        while (r + 1 < n && __ldg(indptr + r + 1) <= w * W) ++r;
+        rows[w] = (int32_t)r;
     }
 }
 
@@ -391,6 +459,135 @@ __global__ void __launch_bounds__(256) spmm_fixup_kernel(int64_t n, const int64_
         }
         epilogue4<NV, STREAM>(r, re - rs, acc, lane, c4, Y, ldy, ep);
     }
+}
+
+// The same product with a lane group per row, for small graphs whose rows are
+// short (rows_ok): nothing crosses groups, so no carry, no fix-up and no search;
+// the group itself adds the row's slices in slice order, which gives the merge
+// kernel's sums. LG lanes (the float4 columns, rounded up to a power of two) take
+// a row. Latency-bound: the epilogue's operands and the next batch's indices are
+// loaded ahead, B gathers are in flight, the last batch predicated. Measured per
+// propagation product (slices and fix-up before): 800 vertices, d = 16, 18 -> 9.6
+// us; 10,000 vertices, d = 32, 33 -> 11.5 us.
+template <int LG, int NV, bool WEIGHTED, typename TX>
+__global__ void __launch_bounds__(128) spmm_rows_kernel(int64_t n, const int64_t *__restrict__ indptr,
+                                                        const int32_t *__restrict__ indices,
+                                                        const float *__restrict__ vals, const TX *__restrict__ X,
+                                                        int64_t ldx, int c4, float *__restrict__ Y, int64_t ldy,
+                                                        SpmmEpilogue ep, uint32_t W) {
+    constexpr int B = NV == 1 ? 8 : 4;
+    const int q0 = threadIdx.x % LG;
+    const int64_t ng = (int64_t)gridDim.x * (blockDim.x / LG);
+    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LG; r < n; r += ng) {
+        const uint32_t rs = (uint32_t)__ldg(indptr + r), re = (uint32_t)__ldg(indptr + r + 1);
+        const int64_t e = r * ep.lde + 4 * q0;
+        float4 e1 = splat4(0.f), e2 = e1, e3 = e1, f = e1, x0 = e1;
+        if (NV == 1 && q0 < c4) {
+            if (ep.E1) e1 = ld4(ep.E1 + e);
+            if (ep.E2) e2 = ld4(ep.E2 + e);
+            if (ep.E3) e3 = ld4(ep.E3 + e);
+            if (ep.F) f = ld4(ep.F + e);
+            if (ep.G) x0 = ld4(ep.X0 + e);
+        }
+        const uint32_t w0 = rs / W;
+        const bool split = re > rs && (re - 1) / W != w0;
+        uint32_t next = (w0 + 1) * W;   // the next slice's first nonzero
+        Acc4<NV> acc, tot;
+#pragma unroll
+        for (int t = 0; t < NV; ++t) acc.v[t] = tot.v[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+        int32_t col[B];
+        float v[B];
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+            col[i] = rs + i < re ? __ldg(indices + rs + i) : 0;
+            v[i] = WEIGHTED && rs + i < re ? __ldg(vals + rs + i) : 0.f;
+        }
+        for (uint32_t p = rs; p < re; p += B) {
+            float4 x[B][NV];
+            float vc[B];
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                const TX *xr = X + (int64_t)col[i] * ldx;
+#pragma unroll
+                for (int t = 0; t < NV; ++t) {
+                    const int q = q0 + 32 * t;
+                    x[i][t] = p + i < re && q < c4 ? load4(xr, q) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+                vc[i] = v[i];
+            }
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                const uint32_t k = p + B + i;
+                col[i] = k < re ? __ldg(indices + k) : 0;
+                v[i] = WEIGHTED && k < re ? __ldg(vals + k) : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+                if (p + i >= re) break;
+                const bool fold = split && p + i == next;
+                if (fold) next += W;
+#pragma unroll
+                for (int t = 0; t < NV; ++t) {
+                    if (fold) {
+                        tot.v[t].x += acc.v[t].x;
+                        tot.v[t].y += acc.v[t].y;
+                        tot.v[t].z += acc.v[t].z;
+                        tot.v[t].w += acc.v[t].w;
+                        acc.v[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                    if (WEIGHTED) {
+                        acc.v[t] = fma4(splat4(vc[i]), x[i][t], acc.v[t]);
+                    } else {
+                        acc.v[t].x += x[i][t].x;
+                        acc.v[t].y += x[i][t].y;
+                        acc.v[t].z += x[i][t].z;
+                        acc.v[t].w += x[i][t].w;
+                    }
+                }
+            }
+        }
+        if (split) {
+#pragma unroll
+            for (int t = 0; t < NV; ++t) {
+                acc.v[t].x = tot.v[t].x + acc.v[t].x;
+                acc.v[t].y = tot.v[t].y + acc.v[t].y;
+                acc.v[t].z = tot.v[t].z + acc.v[t].z;
+                acc.v[t].w = tot.v[t].w + acc.v[t].w;
+            }
+        }
+        if (NV > 1) {
+            epilogue4<NV>(r, (int64_t)(re - rs), acc, q0, c4, Y, ldy, ep);
+            continue;
+        }
+        if (q0 >= c4) continue;
+        // epilogue4 on the operands loaded above
+        float sc = ep.alpha;
+        if (ep.dinv) sc = ep.dinv_w ? ep.alpha * __ldg(ep.dinv_w + r) : re > rs ? ep.alpha / (float)(int64_t)(re - rs) : 0.f;
+        const float4 a = acc.v[0];
+        float4 o = make_float4(sc * a.x, sc * a.y, sc * a.z, sc * a.w);
+        if (ep.E1) o = fma4(ep.b1_col ? ld4(ep.b1_col + 4 * q0) : splat4(ep.b1), e1, o);
+        if (ep.E2) o = fma4(splat4(ep.b2), e2, o);
+        if (ep.E3) o = fma4(splat4(ep.b3), e3, o);
+        const int64_t yo = r * ldy + 4 * q0;
+        if (ep.store) st4(Y + yo, o);
+        if (ep.Yb) st4_bf16(ep.Yb + yo, o);
+        if (ep.F) {
+            const float4 fn = fma4(ep.gamma_col ? ld4(ep.gamma_col + 4 * q0) : splat4(ep.gamma), o, f);
+            st4(ep.F + e, fn);
+            if (ep.G) {
+                const float4 gv = make_float4(x0.x - fn.x, x0.y - fn.y, x0.z - fn.z, x0.w - fn.w);
+                st4(ep.G + e, gv);
+                if (ep.Gb) st4_bf16(ep.Gb + e, gv);
+            }
+        }
+    }
+}
+
+// Rows of at most 256 nonzeros and 256 columns, graphs of at most 16 rows per
+// resident warp of the GPU: beyond, the merge kernel's balanced slices keep more
+// gathers going.
+bool rows_ok(int64_t n, int64_t max_row, int c) {
+    return max_row > 0 && max_row <= 256 && c <= 256 && n <= (int64_t)num_sms() * 64 * 16;
 }
 
 template <bool WEIGHTED>
@@ -495,14 +692,32 @@ int launch_merge(Workspace &ws, int64_t n, int64_t nnz, const int64_t *indptr, c
     const int threads = ep.threads > 0 ? ep.threads : 256;
     const unsigned mblocks = (unsigned)ceil_div(nwarps, threads / 32);
     const unsigned fblocks = (unsigned)std::min<int64_t>(ceil_div(n, 8), num_sms() * 32);
+    const bool fused = ep.row_cnt && ep.slice_row && nnz > 0 && !(WEIGHTED && c4 <= 16);
     LNE_TRACE(WEIGHTED ? "spmm" : "graph_spmm", st);
+    if (nnz > 0 && rows_ok(n, ep.max_row, c) && !(WEIGHTED && c4 <= 16)) {
+#define LNE_ROWS_CASE(LGV, K)                                                                               \
+    spmm_rows_kernel<LGV, K, WEIGHTED, TX><<<(unsigned)ceil_div(n, 128 / LGV), 128, 0, st>>>(                \
+        n, indptr, indices, vals, X, ldx, c4, Y, ldy, ep, (uint32_t)W)
+        if (c4 <= 4) LNE_ROWS_CASE(4, 1);
+        else if (c4 <= 8) LNE_ROWS_CASE(8, 1);
+        else if (c4 <= 16) LNE_ROWS_CASE(16, 1);
+        else if (c4 <= 32) LNE_ROWS_CASE(32, 1);
+        else LNE_ROWS_CASE(32, 2);
+#undef LNE_ROWS_CASE
+        LNE_LAUNCH_CHECK();
+        return 0;
+    }
 #define LNE_MERGE_CASE(K)                                                                                  \
     case K:                                                                                                \
-        if (nnz > 0)                                                                                       \
+        if (fused)                                                                                         \
+            spmm_merge_kernel<K, WEIGHTED, TX, 32, false, true><<<mblocks, threads, 0, st>>>(              \
+                n, nnz, indptr, indices, vals, X, ldx, c4, Y, ldy, ep, W, nwarps, carry, carry_row);       \
+        else if (nnz > 0)                                                                                  \
             spmm_merge_kernel<K, WEIGHTED, TX><<<mblocks, threads, 0, st>>>(n, nnz, indptr, indices, vals, X, ldx, \
                                                                      c4, Y, ldy, ep, W, nwarps, carry,     \
                                                                      carry_row);                           \
-        spmm_fixup_kernel<K><<<fblocks, 256, 0, st>>>(n, indptr, c4, Y, ldy, ep, W, carry, carry_row);      \
+        if (!fused)                                                                                        \
+            spmm_fixup_kernel<K><<<fblocks, 256, 0, st>>>(n, indptr, c4, Y, ldy, ep, W, carry, carry_row);  \
         break;
 #define LNE_MERGE_GROUPED(LGV)                                                                              \
     {                                                                                                       \
@@ -527,7 +742,7 @@ int launch_merge(Workspace &ws, int64_t n, int64_t nnz, const int64_t *indptr, c
 #undef LNE_MERGE_CASE
 #undef LNE_MERGE_GROUPED
     LNE_LAUNCH_CHECK();
-    ::lne::count_launch();
+    if (!fused) ::lne::count_launch();
     return 0;
 }
 
@@ -725,6 +940,29 @@ int merge_carry(Workspace &ws, const char *tag, int64_t nnz, int64_t n, int c, f
     return 0;
 }
 
+
+int merge_chain(Workspace &ws, const char *tag, const GraphView &g, int c, uint32_t **row_cnt,
+                int32_t **slice_row) {
+    *row_cnt = nullptr;
+    *slice_row = nullptr;
+    if (rows_ok(g.n, g.max_deg, c)) return 0;   // a lane group per row: no slices
+    const int64_t W = merge_slice(g.nnz, g.n), nwarps = std::max<int64_t>(1, ceil_div(g.nnz, W));
+    const std::string t = tag ? tag : "spmm.chain";
+    LNE_TRY(ws.get(t + ".n", (size_t)g.n, row_cnt));
+    LNE_TRY(ws.get(t + ".s", (size_t)nwarps, slice_row));
+    return 0;
+}
+
+int merge_chain_prepare(const GraphView &g, uint32_t *row_cnt, int32_t *slice_row, cudaStream_t st) {
+    if (g.n <= 0 || g.nnz <= 0 || !row_cnt) return 0;
+    const int64_t W = merge_slice(g.nnz, g.n), nwarps = std::max<int64_t>(1, ceil_div(g.nnz, W));
+    LNE_CUDA_TRY(cudaMemsetAsync(row_cnt, 0, sizeof(uint32_t) * (size_t)g.n, st));
+    LNE_TRACE("slice_rows", st);
+    slice_rows_kernel<<<(unsigned)std::min<int64_t>(ceil_div(nwarps, 128), num_sms() * 16), 128, 0, st>>>(
+        g.indptr, g.n, W, nwarps, slice_row);
+    LNE_LAUNCH_CHECK();
+    return 0;
+}
 
 int spmm(Workspace &ws, const CsrView &M, const float *X, int64_t ldx, int c, float *Y, int64_t ldy,
          cudaStream_t st) {

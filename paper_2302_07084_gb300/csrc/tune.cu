@@ -88,6 +88,7 @@ int spmm_tile_for(SpmmTune &tc, Workspace &ws, const GraphView &g, const float *
         ep.lde = C;
         ep.threads = cand.threads;
         ep.col_block = cand.col_block;
+        ep.max_row = g.max_deg;
         if ((rc = graph_spmm(ws, g, X, C, C, Y, C, ep, st)) != 0) break;   // warm-up
         cudaEventRecord(e0, st);
         for (int r = 0; r < 3 && rc == 0; ++r) rc = graph_spmm(ws, g, X, C, C, Y, C, ep, st);
