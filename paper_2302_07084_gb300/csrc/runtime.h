@@ -364,11 +364,13 @@ int scan_exclusive_i64(const int64_t *in, int64_t *out, int64_t n, cudaStream_t 
 // (rows of n + 1 entries).
 int scan_exclusive_rows_i64(int64_t *data, int64_t rows, int64_t n, cudaStream_t st);
 
-// Sorting of 64-bit keys (sort.cu). Stable LSD radix sort over the low `bits`
-// bits with an optional 32-bit payload (vals may be NULL); the result lands in
-// keys_alt / vals_alt when *in_alt is true, else in keys / vals.
+// Sorting of 64-bit keys (sort.cu). Stable LSD radix sort over the bits
+// [lo, hi) (whole bytes from lo on are compared: bits from hi to the byte's end
+// have to order alike) with an optional 32-bit payload (vals may be NULL); the
+// result lands in keys_alt / vals_alt when *in_alt is true, else in keys / vals.
+// Synchronises (its bounded waits are checked).
 int radix_sort_u64(Workspace &ws, uint64_t *keys, uint64_t *keys_alt, uint32_t *vals, uint32_t *vals_alt,
-                   int64_t n, int bits, bool *in_alt, cudaStream_t st);
+                   int64_t n, int lo, int hi, bool *in_alt, cudaStream_t st);
 // Unique keys of a sorted array and their multiplicities.
 int run_length(Workspace &ws, const uint64_t *keys, int64_t n, uint64_t *ukeys, uint32_t *counts,
                int64_t *nunique, cudaStream_t st);

@@ -2226,9 +2226,9 @@ int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *
                                               reinterpret_cast<int32_t *>(arc0), nullptr, nullptr, 0)));
     }
     bool in_alt = false;
-    LNE_TRY(radix_sort_u64(ws, k0, k1, arc0, arc1, total, bits, &in_alt, st));
+    LNE_TRY(radix_sort_u64(ws, k0, k1, arc0, arc1, total, 0, bits, &in_alt, st));
     uint64_t *sorted = in_alt ? k1 : k0, *spare = in_alt ? k0 : k1;
-    ws.release("sort.offs");
+    ws.release("sort.words");
     if (ds) {
         // the dropped draws sort last: run lengths over the kept ones only
         int64_t kept = 0;
@@ -2251,7 +2251,7 @@ int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *
 }
 
 void sort_release(Workspace &ws) {
-    for (const char *n : {"sort.k0", "sort.k1", "sort.cnt", "sort.w", "sort.a0", "sort.a1", "sort.bound", "sort.offs",
+    for (const char *n : {"sort.k0", "sort.k1", "sort.cnt", "sort.w", "sort.a0", "sort.a1", "sort.bound", "sort.words",
                           "sort.mk", "sort.mv",
                           "path.dcol", "path.dval", "path.tk", "path.tm", "path.ko", "path.mo", "path.deg",
                           "path.dlen", "path.rowlen", "path.dstart", "path.first", "path.end"})
@@ -2326,10 +2326,11 @@ int assemble_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, uint6
                                                                    dval, mk, mv);
         LNE_LAUNCH_CHECK();
     }
-    // mirrored entries sorted by (row y, column x); the unique keys and the
+    // mirrored entries sorted by (row y, column x): they come in order of x, so a
+    // stable sort by y alone does it (half the passes); the unique keys and the
     // values are no longer needed and serve as the sort's spare buffers
     bool in_alt = false;
-    LNE_TRY(radix_sort_u64(ws, mk, uk, mv, val, nm, 2 * sp.B, &in_alt, st));
+    LNE_TRY(radix_sort_u64(ws, mk, uk, mv, val, nm, sp.B, 2 * sp.B, &in_alt, st));
     const uint64_t *smk = in_alt ? uk : mk;
     const uint32_t *smv = in_alt ? val : mv;
     const unsigned mgrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(nm, 256), num_sms() * 16));
@@ -2708,9 +2709,9 @@ int strat_keys(Workspace &ws, const GraphView &g, const SamplerSpec &sp, int64_t
                                               tile_arcs, tile_off, k0, nullptr, nullptr, nullptr, 0)));
     }
     bool in_alt = false;
-    LNE_TRY(radix_sort_u64(ws, k0, k1, nullptr, nullptr, total, 2 * su.B + 4, &in_alt, st));
+    LNE_TRY(radix_sort_u64(ws, k0, k1, nullptr, nullptr, total, 0, 2 * su.B + 4, &in_alt, st));
     uint64_t *sorted = in_alt ? k1 : k0, *other = in_alt ? k0 : k1;
-    ws.release("sort.offs");
+    ws.release("sort.words");
     LNE_TRY(ws.get("sort.cnt", (size_t)std::max<int64_t>(total, 1), cnt));
     LNE_TRY(run_length(ws, sorted, total, other, *cnt, U, st));
     *total_out = total;

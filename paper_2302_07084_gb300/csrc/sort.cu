@@ -2,15 +2,15 @@
 // space does not fit a dense count table (the hash aggregation of Sec. 5.2
 // done as sort + run-length instead: exact counts, deterministic order).
 //
-// radix_sort_u64: stable LSD radix sort, 8 bits per pass over the low `bits`
-// bits, optional 32-bit payload. One pass = three launches:
-//   hist     per tile of 8192 keys, a 256-bin histogram -> offs[d][t];
-//   scan     one CTA per digit turns its row into exclusive offsets (row total
-//            last);
-//   scatter  each tile ranks its keys stably (rounds of 256 in input order,
-//            warp __match_any_sync groups per digit, a per-digit prefix over
-//            warps), stages them grouped by digit in shared memory and writes
-//            each digit's run contiguously to its global offset.
+// radix_sort_u64: stable LSD radix sort, 8 bits per pass over bits [lo, hi),
+// optional 32-bit payload. One kernel counts the digits of every pass; then a
+// pass is one launch that reads and writes the keys once: a tile of 6144 keys
+// ranks its keys by digit (each warp alone on 512 consecutive keys, by
+// __match_any_sync groups and its own row of counters), stages them in shared
+// memory in digit order, learns how many keys of each digit precede the tile from
+// the tiles before it (decoupled lookback: a tile publishes its counts, then its
+// prefix), and writes each digit's run contiguously. Bound by HBM: 16 bytes a key
+// (24 with a payload) and pass.
 // run_length: unique keys of a sorted array and their multiplicities (tile
 // flag counts, one scan over tiles, block scans inside tiles, each thread
 // summing the run segments among its own items); run_length_weighted sums a
@@ -25,20 +25,6 @@ constexpr int kSortThreads = 256;
 constexpr int kSortItems = 32;
 constexpr int kSortTile = kSortThreads * kSortItems;   // 8192 keys per tile
 constexpr int kSortWarps = kSortThreads / 32;
-
-__global__ void __launch_bounds__(kSortThreads) radix_hist_kernel(const uint64_t *__restrict__ keys, int64_t n,
-                                                                  int shift, int64_t ntiles,
-                                                                  int64_t *__restrict__ offs) {
-    __shared__ uint32_t h[256];
-    const int tid = threadIdx.x;
-    h[tid] = 0;
-    __syncthreads();
-    const int64_t i0 = (int64_t)blockIdx.x * kSortTile;
-    const int nt = (int)imin64(kSortTile, n - i0);
-    for (int i = tid; i < nt; i += kSortThreads) atomicAdd(&h[(uint32_t)(keys[i0 + i] >> shift) & 255u], 1u);
-    __syncthreads();
-    offs[(int64_t)tid * (ntiles + 1) + blockIdx.x] = h[tid];
-}
 
 // Exclusive scan of the 256 values v (one per thread) over the block.
 __device__ __forceinline__ int64_t block_scan256(int64_t v, int64_t *s_warp) {
@@ -57,78 +43,183 @@ __device__ __forceinline__ int64_t block_scan256(int64_t v, int64_t *s_warp) {
     return before + x - v;
 }
 
-template <bool VALS>
-__global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(
-    const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin, int64_t n, int shift, int64_t ntiles,
-    const int64_t *__restrict__ offs, uint64_t *__restrict__ kout, uint32_t *__restrict__ vout) {
-    extern __shared__ uint64_t sk[];                                   // kSortTile staged keys
-    uint32_t *sv = reinterpret_cast<uint32_t *>(sk + kSortTile);      // kSortTile staged payloads
-    __shared__ int64_t s_gbase[256];
-    __shared__ uint32_t s_lbase[256], s_run[256];
-    __shared__ uint32_t s_wc[kSortWarps][256];
-    __shared__ int64_t s_warp[kSortWarps];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t t = blockIdx.x, i0 = t * kSortTile;
-    const int nt = (int)imin64(kSortTile, n - i0);
-    {
-        const int64_t *row = offs + (int64_t)tid * (ntiles + 1);
-        const int64_t tot = row[ntiles], mine = row[t], cnt = row[t + 1] - row[t];
-        const int64_t dbase = block_scan256(tot, s_warp);    // start of digit tid in the output
-        const int64_t lbase = block_scan256(cnt, s_warp);    // start of digit tid in this tile
-        s_gbase[tid] = dbase + mine;
-        s_lbase[tid] = (uint32_t)lbase;
-        s_run[tid] = 0;
+constexpr int kPassThreads = 384;   // two CTAs an SM at 80 registers: 512 threads (64) spilled keys
+constexpr int kPassWarps = kPassThreads / 32;
+constexpr int kPassItems = 16;
+constexpr int kPassTile = kPassThreads * kPassItems;   // 6144 keys per tile
+constexpr int kMaxPasses = 8;
+
+// hist[p][d] = keys whose digit of pass p is d (zeroed before).
+__global__ void __launch_bounds__(512) radix_count_kernel(const uint64_t *__restrict__ keys, int64_t n, int lo,
+                                                          int passes, unsigned long long *__restrict__ hist) {
+    __shared__ uint32_t h[kMaxPasses][256];
+    for (int e = threadIdx.x; e < passes * 256; e += blockDim.x) h[e >> 8][e & 255] = 0;
+    __syncthreads();
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += 4 * stride) {
+        uint64_t k[4];
 #pragma unroll
-        for (int w = 0; w < kSortWarps; ++w) s_wc[w][tid] = 0;
+        for (int u = 0; u < 4; ++u) k[u] = i + u * stride < n ? __ldcs(keys + i + u * stride) : 0ull;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (i + u * stride >= n) break;
+            for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(uint32_t)(k[u] >> (lo + 8 * p)) & 255u], 1u);
+        }
     }
-    // every key (and payload) of the tile is requested up front: 32 independent
-    // loads per thread in flight instead of one per round
-    uint64_t kr[kSortItems];
-    uint32_t vr[kSortItems];
+    __syncthreads();
+    for (int e = threadIdx.x; e < passes * 256; e += blockDim.x) {
+        const uint32_t c = h[e >> 8][e & 255];
+        if (c) atomicAdd(hist + e, (unsigned long long)c);
+    }
+}
+
+// hist[p][.] -> exclusive prefix sums over the digits, one CTA of 256 per pass.
+__global__ void __launch_bounds__(256) radix_base_kernel(unsigned long long *__restrict__ hist) {
+    __shared__ int64_t s_warp[8];
+    unsigned long long *row = hist + 256 * blockIdx.x;
+    const int64_t v = (int64_t)row[threadIdx.x];
+    row[threadIdx.x] = (unsigned long long)block_scan256(v, s_warp);
+}
+
+// A tile's published word for a digit: the upper 8 bits say of which pass and
+// what (2 pass + 1: the tile's own count, 2 pass + 2: the count up to and with
+// the tile), the rest is the value. A pass does not see the words of the passes
+// before it (smaller tags), so the array is zeroed once per sort.
+__device__ __forceinline__ uint64_t tile_word(int tag, uint64_t v) { return ((uint64_t)tag << 56) | v; }
+__device__ __forceinline__ uint64_t ld_relaxed(const uint64_t *p) {
+    uint64_t v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_relaxed(uint64_t *p, uint64_t v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// One pass. Tiles are taken in order from a counter, so the tiles a tile waits
+// for are running or done. A wait gives up after 2 s, sets status[1] and the CTA
+// ends without writing (as do those that find it set).
+template <bool VALS>
+__global__ void __launch_bounds__(kPassThreads, 2) radix_pass_kernel(
+    const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin, int64_t n, int shift, int pass,
+    const unsigned long long *__restrict__ base, uint64_t *__restrict__ words, unsigned *__restrict__ next_tile,
+    uint64_t *__restrict__ kout, uint32_t *__restrict__ vout, int *status) {
+    extern __shared__ uint64_t sk[];                                   // kPassTile staged keys
+    uint32_t *sv = reinterpret_cast<uint32_t *>(sk + kPassTile);      // kPassTile staged payloads
+    __shared__ uint16_t s_wc[kPassWarps][256];   // per warp and digit: count, then where its keys start
+    __shared__ uint32_t s_lbase[256];            // start of the digit in the tile
+    __shared__ int64_t s_delta[256];             // output position minus tile position of the digit's keys
+    __shared__ int64_t s_warp[8];
+    __shared__ uint32_t s_tile;
+    __shared__ int s_fail;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        s_tile = atomicAdd(next_tile, 1u);
+        s_fail = 0;
+    }
+    for (int e = tid; e < kPassWarps * 256; e += kPassThreads) s_wc[e >> 8][e & 255] = 0;
+    __syncthreads();
+    const int64_t tile = s_tile, i0 = tile * kPassTile;
+    const int nt = (int)imin64(kPassTile, n - i0);
+    // the warp's 512 consecutive keys, all requested up front
+    const int w0 = warp * (32 * kPassItems);
+    uint64_t k[kPassItems];
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-        const int li = r * kSortThreads + tid;
-        kr[r] = li < nt ? kin[i0 + li] : 0ull;
-        vr[r] = (VALS && li < nt) ? vin[i0 + li] : 0u;
+    for (int i = 0; i < kPassItems; ++i) {
+        const int li = w0 + 32 * i + lane;
+        k[i] = li < nt ? __ldcs(kin + i0 + li) : 0ull;
+    }
+    uint32_t rank[kPassItems / 2];   // among the warp's keys of the same digit, two to a register
+#pragma unroll
+    for (int i = 0; i < kPassItems; ++i) {
+        const bool valid = w0 + 32 * i + lane < nt;
+        const uint32_t d = valid ? (uint32_t)(k[i] >> shift) & 255u : 256u;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t before = s_wc[warp][d & 255u];
+        const uint32_t lr = (uint32_t)__popc(peers & ((1u << lane) - 1u));
+        if (i & 1) rank[i / 2] |= (before + lr) << 16;
+        else rank[i / 2] = before + lr;
+        __syncwarp();
+        if (valid && lr == 0) s_wc[warp][d] = (uint16_t)(before + (uint32_t)__popc(peers));
+        __syncwarp();
+    }
+    __syncthreads();
+    uint64_t *mine = words + tile * 256 + tid;   // tid < 256: digit tid
+    int64_t count = 0;
+    if (tid < 256) {   // warps' counts -> their starting ranks; the tile's count is published
+        uint32_t c = 0;
+#pragma unroll
+        for (int w = 0; w < kPassWarps; ++w) {
+            const uint32_t x = s_wc[w][tid];
+            s_wc[w][tid] = (uint16_t)c;
+            c += x;
+        }
+        count = c;
+        st_relaxed(mine, tile_word(2 * pass + (tile == 0 ? 2 : 1), (uint64_t)count));
+    }
+    {   // exclusive scan of the 256 counts
+        int64_t x = count;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31 && warp < 8) s_warp[warp] = x;
+        __syncthreads();
+        if (tid < 256) {
+            int64_t p = x - count;
+            for (int w = 0; w < warp; ++w) p += s_warp[w];
+            s_lbase[tid] = (uint32_t)p;
+        }
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-        const int li = r * kSortThreads + tid;   // rounds in input order: stable
-        const bool valid = li < nt;
-        const uint64_t k = kr[r];
-        const uint32_t v = vr[r];
-        const uint32_t d = valid ? (uint32_t)(k >> shift) & 255u : 256u;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const uint32_t lr = (uint32_t)__popc(peers & ((1u << lane) - 1u));
-        if (valid && lr == 0) s_wc[warp][d] = (uint32_t)__popc(peers);
-        __syncthreads();
-        {   // thread tid owns digit tid: warps' counts -> their starting ranks
-            uint32_t p = s_run[tid];
-#pragma unroll
-            for (int w = 0; w < kSortWarps; ++w) {
-                const uint32_t c = s_wc[w][tid];
-                s_wc[w][tid] = p;
-                p += c;
-            }
-            s_run[tid] = p;
+    for (int i = 0; i < kPassItems; ++i) {
+        const int li = w0 + 32 * i + lane;
+        if (li < nt) {
+            const uint32_t d = (uint32_t)(k[i] >> shift) & 255u;
+            const uint32_t pos = s_lbase[d] + s_wc[warp][d] + ((i & 1) ? rank[i / 2] >> 16 : rank[i / 2] & 0xffffu);
+            sk[pos] = k[i];
+            if (VALS) sv[pos] = __ldcs(vin + i0 + li);
         }
-        __syncthreads();
-        if (valid) {
-            const uint32_t pos = s_lbase[d] + s_wc[warp][d] + lr;
-            sk[pos] = k;
-            if (VALS) sv[pos] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int w = 0; w < kSortWarps; ++w) s_wc[w][tid] = 0;
-        __syncthreads();
     }
-    for (int li = tid; li < nt; li += kSortThreads) {
-        const uint64_t k = sk[li];
-        const uint32_t d = (uint32_t)(k >> shift) & 255u;
-        const int64_t g = s_gbase[d] + (li - (int)s_lbase[d]);
-        kout[g] = k;
+    if (tid < 256) {   // keys of digit tid in the tiles before: four words at a time
+        int64_t sum = 0;
+        bool done = tile == 0;
+        uint64_t t0 = 0;
+        for (int64_t q = tile - 1; !done;) {
+            uint64_t x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = q - u >= 0 ? ld_relaxed(words + (q - u) * 256 + tid) : 0ull;
+            bool moved = false;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int tag = (int)(x[u] >> 56);
+                if (done || tag < 2 * pass + 1) break;   // not published yet: read it again
+                sum += (int64_t)(x[u] & 0x00FFFFFFFFFFFFFFull);
+                done = tag == 2 * pass + 2;
+                --q;
+                moved = true;
+            }
+            if (!done && !moved) {
+                uint64_t t;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+                if (t0 == 0) t0 = t;
+                if (t - t0 > 2000000000ull || *reinterpret_cast<volatile int *>(status + 1) != 0) {
+                    atomicExch(status + 1, 1);
+                    s_fail = 1;
+                    break;
+                }
+            }
+        }
+        if (tile > 0 && done) st_relaxed(mine, tile_word(2 * pass + 2, (uint64_t)(sum + count)));
+        s_delta[tid] = (int64_t)base[tid] + sum - (int64_t)s_lbase[tid];
+    }
+    __syncthreads();
+    if (s_fail) return;
+    for (int li = tid; li < nt; li += kPassThreads) {
+        const uint64_t x = sk[li];
+        const int64_t g = s_delta[(uint32_t)(x >> shift) & 255u] + li;
+        kout[g] = x;
         if (VALS) vout[g] = sv[li];
     }
 }
@@ -232,35 +323,55 @@ int count_below(Workspace &ws, const uint64_t *keys, int64_t n, uint64_t key, in
     return 0;
 }
 
+// Measured over 2e8 keys of 38 bits (five passes) and 1.1e8 mirrored ones with a
+// payload (five passes before, three over the row bits now): 14.3 ms with a
+// histogram, a scan and a scatter launch a pass (the scatter with four CTA
+// barriers per 256 keys), 9.0 ms now with the one count of all digits (0.57 ms).
 int radix_sort_u64(Workspace &ws, uint64_t *keys, uint64_t *keys_alt, uint32_t *vals, uint32_t *vals_alt,
-                   int64_t n, int bits, bool *in_alt, cudaStream_t st) {
+                   int64_t n, int lo, int hi, bool *in_alt, cudaStream_t st) {
     *in_alt = false;
-    if (n <= 1) return 0;
-    const int64_t ntiles = ceil_div(n, (int64_t)kSortTile);
-    int64_t *offs = nullptr;
-    LNE_TRY(ws.get("sort.offs", (size_t)256 * (ntiles + 1), &offs));
-    const int smem = kSortTile * (8 + (vals ? 4 : 0));
-    LNE_TRY(allow_dynamic_smem(radix_scatter_kernel<true>));
-    LNE_TRY(allow_dynamic_smem(radix_scatter_kernel<false>));
+    if (n <= 1 || hi <= lo) return 0;
+    const int passes = (hi - lo + 7) / 8;
+    if (lo < 0 || hi > 64 || passes > kMaxPasses) return fail(LNE_ERR_INVALID, "radix sort bits out of range");
+    const int64_t ntiles = ceil_div(n, (int64_t)kPassTile);
+    uint64_t *words = nullptr;
+    unsigned long long *hist = nullptr;
+    unsigned *next = nullptr;
+    int *status = nullptr;
+    LNE_TRY(ws.get("sort.words", (size_t)256 * ntiles, &words));
+    LNE_TRY(ws.get("sort.hist", (size_t)256 * kMaxPasses, &hist));
+    LNE_TRY(ws.get("sort.next", kMaxPasses, &next));
+    LNE_TRY(device_status(ws, &status, st));
+    const int smem = kPassTile * (8 + (vals ? 4 : 0));
+    LNE_TRY(allow_dynamic_smem(radix_pass_kernel<true>));
+    LNE_TRY(allow_dynamic_smem(radix_pass_kernel<false>));
+    {
+        LNE_TRACE("radix_count", st);
+        LNE_CUDA_TRY(cudaMemsetAsync(words, 0, sizeof(uint64_t) * 256 * (size_t)ntiles, st));
+        LNE_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * 256 * kMaxPasses, st));
+        LNE_CUDA_TRY(cudaMemsetAsync(next, 0, sizeof(unsigned) * kMaxPasses, st));
+        radix_count_kernel<<<(unsigned)std::min<int64_t>(ceil_div(n, 2048), num_sms() * 4), 512, 0, st>>>(
+            keys, n, lo, passes, hist);
+        LNE_LAUNCH_CHECK();
+        radix_base_kernel<<<passes, 256, 0, st>>>(hist);
+        LNE_LAUNCH_CHECK();
+    }
     uint64_t *ka = keys, *kb = keys_alt;
     uint32_t *va = vals, *vb = vals_alt;
-    for (int shift = 0; shift < bits; shift += 8) {
+    for (int p = 0; p < passes; ++p) {
         LNE_TRACE("radix_pass", st);
-        radix_hist_kernel<<<(unsigned)ntiles, kSortThreads, 0, st>>>(ka, n, shift, ntiles, offs);
-        LNE_LAUNCH_CHECK();
-        LNE_TRY(scan_exclusive_rows_i64(offs, 256, ntiles, st));
         if (vals)
-            radix_scatter_kernel<true><<<(unsigned)ntiles, kSortThreads, smem, st>>>(ka, va, n, shift, ntiles, offs,
-                                                                                     kb, vb);
+            radix_pass_kernel<true><<<(unsigned)ntiles, kPassThreads, smem, st>>>(
+                ka, va, n, lo + 8 * p, p, hist + 256 * p, words, next + p, kb, vb, status);
         else
-            radix_scatter_kernel<false><<<(unsigned)ntiles, kSortThreads, smem, st>>>(ka, nullptr, n, shift, ntiles,
-                                                                                      offs, kb, nullptr);
+            radix_pass_kernel<false><<<(unsigned)ntiles, kPassThreads, smem, st>>>(
+                ka, nullptr, n, lo + 8 * p, p, hist + 256 * p, words, next + p, kb, nullptr, status);
         LNE_LAUNCH_CHECK();
         std::swap(ka, kb);
         std::swap(va, vb);
         *in_alt = !*in_alt;
     }
-    return 0;
+    return status_check(ws, st);   // an expired wait leaves keys unwritten: nothing may use them
 }
 
 namespace {
