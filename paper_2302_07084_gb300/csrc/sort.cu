@@ -11,20 +11,18 @@
 // the tiles before it (decoupled lookback: a tile publishes its counts, then its
 // prefix), and writes each digit's run contiguously. Bound by HBM: 16 bytes a key
 // (24 with a payload) and pass.
-// run_length: unique keys of a sorted array and their multiplicities (tile
-// flag counts, one scan over tiles, block scans inside tiles, each thread
-// summing the run segments among its own items); run_length_weighted sums a
-// per-arc 64-bit weight over each run instead (edge downsampling).
+// run_length: unique keys of a sorted array and their multiplicities (run starts
+// counted per chunk of 1024 keys, one scan over the chunks, then a warp per chunk
+// writes its runs); run_length_weighted sums a per-arc 64-bit weight over each run
+// instead (edge downsampling).
 #include "common.cuh"
 #include "runtime.h"
 
 namespace lne {
 namespace {
 
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 32;
-constexpr int kSortTile = kSortThreads * kSortItems;   // 8192 keys per tile
-constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kRleThreads = 256;
+constexpr int kRleChunk = 1024;   // keys a warp
 
 // Exclusive scan of the 256 values v (one per thread) over the block.
 __device__ __forceinline__ int64_t block_scan256(int64_t v, int64_t *s_warp) {
@@ -224,80 +222,113 @@ __global__ void __launch_bounds__(kPassThreads, 2) radix_pass_kernel(
     }
 }
 
-// Run starts of a sorted array: count per tile.
-__global__ void __launch_bounds__(kSortThreads) rle_count_kernel(const uint64_t *__restrict__ keys, int64_t n,
-                                                                 uint32_t *__restrict__ tile_cnt) {
-    __shared__ uint32_t s;
-    if (threadIdx.x == 0) s = 0;
-    __syncthreads();
-    const int64_t i0 = (int64_t)blockIdx.x * kSortTile;
-    const int nt = (int)imin64(kSortTile, n - i0);
+// Run starts of a sorted array, counted per chunk of kRleChunk keys (a warp each).
+__global__ void __launch_bounds__(kRleThreads) rle_count_kernel(const uint64_t *__restrict__ keys, int64_t n,
+                                                                uint32_t *__restrict__ chunk_cnt) {
+    const int lane = threadIdx.x & 31;
+    const int64_t chunk = ((int64_t)blockIdx.x * kRleThreads + threadIdx.x) >> 5;
+    const int64_t i0 = chunk * kRleChunk;
+    if (i0 >= n) return;
+    const int64_t iend = imin64(n, i0 + kRleChunk);
     uint32_t c = 0;
-    for (int i = threadIdx.x; i < nt; i += kSortThreads) {
-        const int64_t g = i0 + i;
-        c += (g == 0 || keys[g] != keys[g - 1]) ? 1u : 0u;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(&s, c);
-    __syncthreads();
-    if (threadIdx.x == 0) tile_cnt[blockIdx.x] = s;
+#pragma unroll 8
+    for (int64_t g = i0 + lane; g < iend; g += 32) c += (g == 0 || keys[g] != keys[g - 1]) ? 1u : 0u;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0) chunk_cnt[chunk] = c;
 }
 
-// Unique keys and their run lengths (thread-blocked items, block scan). Each
-// thread adds up the segments of runs among its own items: a run that starts
-// and ends among them is stored, a piece of a run that crosses a thread
-// boundary is added atomically (integer sums, so the result does not depend
-// on the order), which keeps a run of any length parallel. The outputs are
-// zeroed beforehand. WEIGHTED: instead of the length, the 64-bit sum of
-// w[arc] over the run's payloads.
+// Unique keys and their run lengths, a warp per chunk: 32 consecutive keys at a
+// time, the run starts among them by ballot, so reads and writes are coalesced
+// (a thread per 32 consecutive keys read 32 sectors a load and took 2.4 of
+// run_length's 2.9 ms at 2e8 keys). A run that starts and ends in the chunk is
+// stored; the pieces of one that crosses a chunk's edge are added atomically
+// (integer sums, so the result does not depend on the order), which keeps a run
+// of any length parallel. The outputs are zeroed beforehand. WEIGHTED: instead of
+// the length, the 64-bit sum of w[arc] over the run's payloads.
 template <bool WEIGHTED>
-__global__ void __launch_bounds__(kSortThreads) rle_write_kernel(const uint64_t *__restrict__ keys, int64_t n,
-                                                                 const int64_t *__restrict__ tile_off,
-                                                                 uint64_t *__restrict__ ukeys,
-                                                                 uint32_t *__restrict__ counts,
-                                                                 const uint32_t *__restrict__ arcs,
-                                                                 const uint64_t *__restrict__ w,
-                                                                 uint64_t *__restrict__ wsum) {
-    __shared__ int64_t s_warp[kSortWarps];
-    const int tid = threadIdx.x;
-    const int64_t i0 = (int64_t)blockIdx.x * kSortTile + (int64_t)tid * kSortItems;
-    uint32_t flags = 0;
-    int c = 0;
-    for (int j = 0; j < kSortItems; ++j) {
-        const int64_t g = i0 + j;
-        if (g < n && (g == 0 || keys[g] != keys[g - 1])) {
-            flags |= 1u << j;
-            ++c;
-        }
-    }
-    // index of the run holding the item before this thread's first one
-    int64_t run = tile_off[blockIdx.x] + block_scan256(c, s_warp) - 1;
-    if (i0 >= n) return;
-    const int64_t iend = i0 + kSortItems < n ? i0 + kSortItems : n;
-    auto flush = [&](uint64_t acc, bool complete) {
-        if (WEIGHTED) {
-            if (complete) wsum[run] = acc;
-            else atomicAdd(reinterpret_cast<unsigned long long *>(wsum) + run, (unsigned long long)acc);
-        } else {
-            if (complete) counts[run] = (uint32_t)acc;
-            else atomicAdd(counts + run, (uint32_t)acc);
-        }
+__global__ void __launch_bounds__(kRleThreads) rle_write_kernel(const uint64_t *__restrict__ keys, int64_t n,
+                                                                const int64_t *__restrict__ chunk_off,
+                                                                uint64_t *__restrict__ ukeys,
+                                                                uint32_t *__restrict__ counts,
+                                                                const uint32_t *__restrict__ arcs,
+                                                                const uint64_t *__restrict__ w,
+                                                                uint64_t *__restrict__ wsum) {
+    constexpr int kAhead = 8;   // loads in flight a lane
+    const int lane = threadIdx.x & 31;
+    const int64_t chunk = ((int64_t)blockIdx.x * kRleThreads + threadIdx.x) >> 5;
+    const int64_t i0 = chunk * kRleChunk;
+    if (i0 >= n) return;   // whole warps
+    const int64_t iend = imin64(n, i0 + kRleChunk);
+    auto store = [&](int64_t run, uint64_t v) {
+        if (WEIGHTED) wsum[run] = v;
+        else counts[run] = (uint32_t)v;
     };
-    uint64_t acc = 0;
-    bool started_here = false;
-    for (int64_t g = i0; g < iend; ++g) {
-        if (flags & (1u << (int)(g - i0))) {
-            if (g > i0) flush(acc, started_here);   // the segment ends here
-            ++run;
-            ukeys[run] = keys[g];
-            acc = 0;
-            started_here = true;
+    auto add = [&](int64_t run, uint64_t v) {
+        if (WEIGHTED) atomicAdd(reinterpret_cast<unsigned long long *>(wsum) + run, (unsigned long long)v);
+        else atomicAdd(counts + run, (uint32_t)v);
+    };
+    int64_t run = chunk_off[chunk] - 1;   // the run that is open
+    uint64_t acc = 0;                     // its sum so far in this chunk
+    bool here = false;                    // whether it started in this chunk
+    uint64_t before = i0 > 0 ? keys[i0 - 1] : 0ull;
+    for (int64_t g0 = i0; g0 < iend; g0 += 32 * kAhead) {
+        uint64_t k[kAhead];
+        uint64_t x[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int64_t g = g0 + 32 * u + lane;
+            k[u] = g < iend ? keys[g] : 0ull;
+            x[u] = WEIGHTED ? (g < iend ? __ldg(w + arcs[g]) : 0ull) : 0ull;
         }
-        acc += WEIGHTED ? __ldg(w + arcs[g]) : 1ull;
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int64_t g = g0 + 32 * u + lane;
+            const int nv = (int)imin64(32, iend - (g0 + 32 * u));   // keys of this step
+            if (nv <= 0) break;
+            uint64_t prev = __shfl_up_sync(0xffffffffu, k[u], 1);
+            if (lane == 0) prev = before;
+            before = __shfl_sync(0xffffffffu, k[u], nv - 1);
+            const bool head = lane < nv && (g == 0 || k[u] != prev);
+            const unsigned heads = __ballot_sync(0xffffffffu, head);
+            uint64_t upto = (uint64_t)lane + 1;   // sum over the lanes up to and with this one
+            if (WEIGHTED) {
+                upto = x[u];
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint64_t y = __shfl_up_sync(0xffffffffu, upto, o);
+                    if (lane >= o) upto += y;
+                }
+            }
+            const uint64_t all = WEIGHTED ? __shfl_sync(0xffffffffu, upto, 31) : (uint64_t)nv;
+            if (heads == 0) {
+                acc += all;
+                continue;
+            }
+            const int first = __ffs(heads) - 1, last = 31 - __clz(heads);
+            const unsigned above = lane < 31 ? heads & ~((2u << lane) - 1u) : 0u;   // starts after this lane
+            const int next = above ? __ffs(above) - 1 : 32;
+            uint64_t below = __shfl_up_sync(0xffffffffu, upto, 1);
+            if (lane == 0) below = 0;
+            const uint64_t at_next = __shfl_sync(0xffffffffu, upto, (next - 1) & 31);
+            acc += __shfl_sync(0xffffffffu, below, first);
+            if (lane == 0) {   // the open run ends here
+                if (here) store(run, acc);
+                else if (acc) add(run, acc);
+            }
+            if (head) {
+                const int64_t r = run + 1 + __popc(heads & ((1u << lane) - 1u));
+                ukeys[r] = k[u];
+                if (next < 32) store(r, at_next - below);
+            }
+            run += __popc(heads);
+            acc = all - __shfl_sync(0xffffffffu, below, last);
+            here = true;
+        }
     }
-    const bool ends = iend >= n || keys[iend] != keys[iend - 1];
-    flush(acc, started_here && ends);
+    if (lane == 0) {
+        if (here && (iend >= n || keys[iend] != before)) store(run, acc);
+        else if (acc) add(run, acc);
+    }
 }
 
 // Number of keys below `key` in a sorted array (one thread, binary search).
@@ -380,26 +411,25 @@ int run_length_impl(Workspace &ws, const uint64_t *keys, int64_t n, uint64_t *uk
                     const uint32_t *arcs, const uint64_t *w, uint64_t *wsum, int64_t *nunique, cudaStream_t st) {
     *nunique = 0;
     if (n <= 0) return 0;
-    const int64_t ntiles = ceil_div(n, (int64_t)kSortTile);
-    uint32_t *tc = nullptr;
-    int64_t *toff = nullptr;
-    LNE_TRY(ws.get("rle.tile_cnt", (size_t)ntiles, &tc));
-    LNE_TRY(ws.get("rle.tile_off", (size_t)ntiles + 1, &toff));
+    const int64_t nchunks = ceil_div(n, (int64_t)kRleChunk);
+    const unsigned grid = (unsigned)ceil_div(n, (int64_t)kRleChunk * (kRleThreads / 32));
+    uint32_t *cc = nullptr;
+    int64_t *coff = nullptr;
+    LNE_TRY(ws.get("rle.cnt", (size_t)nchunks, &cc));
+    LNE_TRY(ws.get("rle.off", (size_t)nchunks + 1, &coff));
     LNE_TRACE("run_length", st);
-    rle_count_kernel<<<(unsigned)ntiles, kSortThreads, 0, st>>>(keys, n, tc);
+    rle_count_kernel<<<grid, kRleThreads, 0, st>>>(keys, n, cc);
     LNE_LAUNCH_CHECK();
-    LNE_TRY(scan_exclusive_u32_to_i64(tc, toff, ntiles, st));
+    LNE_TRY(scan_exclusive_u32_to_i64(cc, coff, nchunks, st));
     int64_t u = 0;
-    LNE_CUDA_TRY(cudaMemcpyAsync(&u, toff + ntiles, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    LNE_CUDA_TRY(cudaMemcpyAsync(&u, coff + nchunks, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     LNE_CUDA_TRY(cudaStreamSynchronize(st));
     if (wsum) LNE_CUDA_TRY(cudaMemsetAsync(wsum, 0, sizeof(uint64_t) * (size_t)u, st));
     else LNE_CUDA_TRY(cudaMemsetAsync(counts, 0, sizeof(uint32_t) * (size_t)u, st));
     if (wsum)
-        rle_write_kernel<true><<<(unsigned)ntiles, kSortThreads, 0, st>>>(keys, n, toff, ukeys, nullptr, arcs, w,
-                                                                           wsum);
+        rle_write_kernel<true><<<grid, kRleThreads, 0, st>>>(keys, n, coff, ukeys, nullptr, arcs, w, wsum);
     else
-        rle_write_kernel<false><<<(unsigned)ntiles, kSortThreads, 0, st>>>(keys, n, toff, ukeys, counts, nullptr,
-                                                                            nullptr, nullptr);
+        rle_write_kernel<false><<<grid, kRleThreads, 0, st>>>(keys, n, coff, ukeys, counts, nullptr, nullptr, nullptr);
     LNE_LAUNCH_CHECK();
     LNE_CUDA_TRY(cudaStreamSynchronize(st));
     *nunique = u;
