@@ -4,9 +4,9 @@
 //
 // radix_sort_u64: stable LSD radix sort, 8 bits per pass over bits [lo, hi),
 // optional 32-bit payload. One kernel counts the digits of every pass; then a
-// pass is one launch that reads and writes the keys once: a tile of 6144 keys
+// pass is one launch that reads and writes the keys once: a tile of 4096 keys
 // ranks its keys by digit (each warp alone on 512 consecutive keys, by
-// __match_any_sync groups and its own row of counters), stages them in shared
+// groups of equal digits and its own row of counters), stages them in shared
 // memory in digit order, learns how many keys of each digit precede the tile from
 // the tiles before it (decoupled lookback: a tile publishes its counts, then its
 // prefix), and writes each digit's run contiguously. Bound by HBM: 16 bytes a key
@@ -41,10 +41,14 @@ __device__ __forceinline__ int64_t block_scan256(int64_t v, int64_t *s_warp) {
     return before + x - v;
 }
 
-constexpr int kPassThreads = 384;   // two CTAs an SM at 80 registers: 512 threads (64) spilled keys
+// 256 threads with 16 keys each. Measured over 2e8 keys (five passes and the
+// count): 5.4 ms without a payload at four CTAs an SM (three 5.7, 384 threads 5.8,
+// 12 or 24 keys a thread 6.2 and 5.7), 6.8 ms with one at three (four spill: 7.2).
+constexpr int kPassThreads = 256;
+static_assert(kPassThreads == 256, "a thread per digit");
 constexpr int kPassWarps = kPassThreads / 32;
 constexpr int kPassItems = 16;
-constexpr int kPassTile = kPassThreads * kPassItems;   // 6144 keys per tile
+constexpr int kPassTile = kPassThreads * kPassItems;   // 4096 keys per tile
 constexpr int kMaxPasses = 8;
 
 // hist[p][d] = keys whose digit of pass p is d (zeroed before).
@@ -93,18 +97,33 @@ __device__ __forceinline__ void st_relaxed(uint64_t *p, uint64_t v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// Which lanes of the warp hold the same digit: __match_any_sync for every fourth
+// group of keys, eight ballots for the others. Match alone keeps its pipe busy 63%
+// of the pass (7.3 ms for the five passes instead of 5.8, 384 threads), ballots
+// alone the issue slots (6.0).
+constexpr int kMatchEvery = 4;
+// The lanes whose digit d is this lane's.
+__device__ __forceinline__ unsigned same_digit(uint32_t d) {
+    unsigned peers = 0xffffffffu;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const unsigned one = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+        peers &= ~(one ^ (unsigned)((int)(d << (31 - b)) >> 31));
+    }
+    return peers;
+}
+
 // One pass. Tiles are taken in order from a counter, so the tiles a tile waits
 // for are running or done. A wait gives up after 2 s, sets status[1] and the CTA
 // ends without writing (as do those that find it set).
 template <bool VALS>
-__global__ void __launch_bounds__(kPassThreads, 2) radix_pass_kernel(
+__global__ void __launch_bounds__(kPassThreads, VALS ? 3 : 4) radix_pass_kernel(
     const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin, int64_t n, int shift, int pass,
     const unsigned long long *__restrict__ base, uint64_t *__restrict__ words, unsigned *__restrict__ next_tile,
     uint64_t *__restrict__ kout, uint32_t *__restrict__ vout, int *status) {
     extern __shared__ uint64_t sk[];                                   // kPassTile staged keys
     uint32_t *sv = reinterpret_cast<uint32_t *>(sk + kPassTile);      // kPassTile staged payloads
-    __shared__ uint16_t s_wc[kPassWarps][256];   // per warp and digit: count, then where its keys start
-    __shared__ uint32_t s_lbase[256];            // start of the digit in the tile
+    __shared__ uint16_t s_wc[kPassWarps][256];   // per warp and digit: count, then where its keys go in the tile
     __shared__ int64_t s_delta[256];             // output position minus tile position of the digit's keys
     __shared__ int64_t s_warp[8];
     __shared__ uint32_t s_tile;
@@ -124,26 +143,26 @@ __global__ void __launch_bounds__(kPassThreads, 2) radix_pass_kernel(
 #pragma unroll
     for (int i = 0; i < kPassItems; ++i) {
         const int li = w0 + 32 * i + lane;
-        k[i] = li < nt ? __ldcs(kin + i0 + li) : 0ull;
+        k[i] = li < nt ? __ldcs(kin + i0 + li) : ~0ull;   // past the end: the largest digit, ranked last
     }
     uint32_t rank[kPassItems / 2];   // among the warp's keys of the same digit, two to a register
 #pragma unroll
     for (int i = 0; i < kPassItems; ++i) {
-        const bool valid = w0 + 32 * i + lane < nt;
-        const uint32_t d = valid ? (uint32_t)(k[i] >> shift) & 255u : 256u;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const uint32_t before = s_wc[warp][d & 255u];
+        const uint32_t d = (uint32_t)(k[i] >> shift) & 255u;
+        const unsigned peers = i % kMatchEvery == 0 ? __match_any_sync(0xffffffffu, d) : same_digit(d);
+        const uint32_t before = s_wc[warp][d];
         const uint32_t lr = (uint32_t)__popc(peers & ((1u << lane) - 1u));
         if (i & 1) rank[i / 2] |= (before + lr) << 16;
         else rank[i / 2] = before + lr;
         __syncwarp();
-        if (valid && lr == 0) s_wc[warp][d] = (uint16_t)(before + (uint32_t)__popc(peers));
+        if (lr == 0) s_wc[warp][d] = (uint16_t)(before + (uint32_t)__popc(peers));
         __syncwarp();
     }
     __syncthreads();
-    uint64_t *mine = words + tile * 256 + tid;   // tid < 256: digit tid
+    uint64_t *mine = words + tile * 256 + tid;   // thread = digit from here on
     int64_t count = 0;
-    if (tid < 256) {   // warps' counts -> their starting ranks; the tile's count is published
+    uint32_t lbase = 0;   // start of the digit in the tile
+    {   // warps' counts -> their starting ranks; the tile's count is published
         uint32_t c = 0;
 #pragma unroll
         for (int w = 0; w < kPassWarps; ++w) {
@@ -151,36 +170,22 @@ __global__ void __launch_bounds__(kPassThreads, 2) radix_pass_kernel(
             s_wc[w][tid] = (uint16_t)c;
             c += x;
         }
-        count = c;
+        count = c - (tid == 255 ? (uint32_t)(kPassTile - nt) : 0u);
         st_relaxed(mine, tile_word(2 * pass + (tile == 0 ? 2 : 1), (uint64_t)count));
-    }
-    {   // exclusive scan of the 256 counts
-        int64_t x = count;
+        lbase = (uint32_t)block_scan256(count, s_warp);
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31 && warp < 8) s_warp[warp] = x;
-        __syncthreads();
-        if (tid < 256) {
-            int64_t p = x - count;
-            for (int w = 0; w < warp; ++w) p += s_warp[w];
-            s_lbase[tid] = (uint32_t)p;
-        }
+        for (int w = 0; w < kPassWarps; ++w) s_wc[w][tid] += (uint16_t)lbase;
     }
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < kPassItems; ++i) {
         const int li = w0 + 32 * i + lane;
-        if (li < nt) {
-            const uint32_t d = (uint32_t)(k[i] >> shift) & 255u;
-            const uint32_t pos = s_lbase[d] + s_wc[warp][d] + ((i & 1) ? rank[i / 2] >> 16 : rank[i / 2] & 0xffffu);
-            sk[pos] = k[i];
-            if (VALS) sv[pos] = __ldcs(vin + i0 + li);
-        }
+        const uint32_t d = (uint32_t)(k[i] >> shift) & 255u;
+        const uint32_t pos = s_wc[warp][d] + ((i & 1) ? rank[i / 2] >> 16 : rank[i / 2] & 0xffffu);
+        sk[pos] = k[i];
+        if (VALS && li < nt) sv[pos] = __ldcs(vin + i0 + li);
     }
-    if (tid < 256) {   // keys of digit tid in the tiles before: four words at a time
+    {   // keys of digit tid in the tiles before: four words at a time
         int64_t sum = 0;
         bool done = tile == 0;
         uint64_t t0 = 0;
@@ -210,7 +215,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) radix_pass_kernel(
             }
         }
         if (tile > 0 && done) st_relaxed(mine, tile_word(2 * pass + 2, (uint64_t)(sum + count)));
-        s_delta[tid] = (int64_t)base[tid] + sum - (int64_t)s_lbase[tid];
+        s_delta[tid] = (int64_t)base[tid] + sum - (int64_t)lbase;
     }
     __syncthreads();
     if (s_fail) return;
@@ -357,7 +362,7 @@ int count_below(Workspace &ws, const uint64_t *keys, int64_t n, uint64_t key, in
 // Measured over 2e8 keys of 38 bits (five passes) and 1.1e8 mirrored ones with a
 // payload (five passes before, three over the row bits now): 14.3 ms with a
 // histogram, a scan and a scatter launch a pass (the scatter with four CTA
-// barriers per 256 keys), 9.0 ms now with the one count of all digits (0.57 ms).
+// barriers per 256 keys), 7.5 ms now with the one count of all digits (0.58 ms).
 int radix_sort_u64(Workspace &ws, uint64_t *keys, uint64_t *keys_alt, uint32_t *vals, uint32_t *vals_alt,
                    int64_t n, int lo, int hi, bool *in_alt, cudaStream_t st) {
     *in_alt = false;
