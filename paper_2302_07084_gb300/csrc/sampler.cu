@@ -905,6 +905,231 @@ __global__ void __launch_bounds__(kTabThreads, kTabMinBlocks) walk_table_kernel(
     }
 }
 
+// ---------------------------------------------------------------------------
+// The key-emitting walk of unweighted graphs without downsampling or window
+// strata: the draws of walk_emit_kernel (the same Philox words), with each warp
+// alone on batches of 256 consecutive samples as in walk_table_kernel, ranked by
+// window length. The keys go to the sort, so a batch writes them in the order in
+// which it walks them (coalesced), not in sample order.
+//
+// REC: a step reads the 16-byte record of the arc that it takes, which holds the
+// next vertex's offset, degree and reciprocal. Otherwise it reads the 4-byte
+// neighbour, and the neighbour's vertex record unless the step is the last of
+// its side (then the id is all that is needed): two dependent loads, over a
+// quarter of the bytes (the rule stands at kKeyRecordArcs).
+//
+// Bound by gathers that miss L1 (one a step and one a vertex record, from L2).
+// Measured at 400k vertices, 16M arcs, 2e8 draws, T = 5: 3.7 ms. walk_emit_kernel
+// took 8.8: tiles of 4096 arcs left three CTAs of four warps an SM, and its CTA
+// barriers and DRAM-resident records kept those waiting.
+// ---------------------------------------------------------------------------
+constexpr int kKeyMaxTileArcs = 512;
+constexpr int kKeyTileSamples = 8192;
+
+struct KeyDraw {
+    uint32_t j;
+    int64_t arc;
+    int steps, sigma;
+    u32x4 nb;            // current Philox block
+    WalkCur cur, v;      // current vertex; the arc's target
+    int32_t uend;
+};
+
+__device__ __forceinline__ WalkCur walk_record(const WalkArgs &A, int32_t x, bool need) {
+    uint4 r = make_uint4(0u, 0u, 0u, 0u);
+    if (need) r = __ldg(A.vinfo + x);
+    return WalkCur{x, r.x, r.y, r.z};
+}
+
+__device__ __forceinline__ void key_begin(const WalkArgs &A, int64_t arc, uint32_t j, int r, int sigma, uint32_t w3,
+                                          int32_t u, int32_t v, KeyDraw &d) {
+    d.j = j;
+    d.arc = arc;
+    d.steps = r - 1;
+    d.sigma = sigma;
+    d.nb = u32x4{0u, 0u, 0u, w3};
+    const bool from_v = sigma == 0 && d.steps > 0;
+    d.v = walk_record(A, v, d.steps > sigma);
+    d.cur = walk_record(A, u, d.steps > 0 && sigma > 0);
+    d.uend = u;
+    if (from_v) d.cur = d.v;
+}
+
+// Step K (word 3 + K) of the draw, if it has one.
+template <int K, bool REC>
+__device__ __forceinline__ void key_step(const WalkArgs &A, KeyDraw &d) {
+    if (K >= d.steps) return;
+    constexpr int widx = 3 + K;
+    if ((widx & 3) == 0)
+        d.nb = philox_rk(u32x4{d.j, (uint32_t)(uint64_t)d.arc, (uint32_t)((uint64_t)d.arc >> 32), (uint32_t)(widx >> 2)},
+                         A.rk);
+    const uint32_t w = (widx & 3) == 0 ? d.nb.x : (widx & 3) == 1 ? d.nb.y : (widx & 3) == 2 ? d.nb.z : d.nb.w;
+    if (REC) {
+        walk_step<false>(A, d.cur, w);
+    } else {
+        uint32_t deg = d.cur.hidg >> 8;
+        if (deg != 0) {   // degree 0 only on graphs that break the contract: stay
+            const int64_t off = (int64_t)d.cur.off_lo | ((int64_t)(d.cur.hidg & 0xFF) << 32);
+            uint32_t jj;
+            if (deg == 0xFFFFFFu) {
+                deg = (uint32_t)(__ldg(A.indptr + d.cur.x + 1) - __ldg(A.indptr + d.cur.x));
+                jj = w % deg;
+            } else {
+                jj = barrett_mod(w, d.cur.m, deg);   // m of degree 1 makes it 0
+            }
+            const int32_t x = __ldg(A.indices + off + jj);
+            d.cur = walk_record(A, x, K + 1 != d.sigma && K + 1 != d.steps);
+        }
+    }
+    if (K + 1 == d.sigma && K + 1 < d.steps) {   // u side done: continue from v
+        d.uend = d.cur.x;
+        d.cur = d.v;
+    }
+}
+
+template <int K, bool REC>
+struct KeySteps {
+    __device__ __forceinline__ static void run(const WalkArgs &A, KeyDraw &a, KeyDraw &b, int kmax) {
+        if (K >= kmax) return;
+        key_step<K, REC>(A, a);
+        key_step<K, REC>(A, b);
+        KeySteps<K + 1, REC>::run(A, a, b, kmax);
+    }
+};
+template <bool REC>
+struct KeySteps<15, REC> {
+    __device__ __forceinline__ static void run(const WalkArgs &, KeyDraw &, KeyDraw &, int) {}
+};
+
+__device__ __forceinline__ uint64_t key_end(const KeyDraw &d, int B) {
+    const bool one_sided = d.sigma >= d.steps;   // every step on the u side (or none at all)
+    const int32_t pu = one_sided && d.steps > 0 ? d.cur.x : d.uend;
+    const int32_t pv = one_sided ? d.v.x : d.cur.x;
+    return ((uint64_t)(uint32_t)min(pu, pv) << B) | (uint64_t)(uint32_t)max(pu, pv);
+}
+
+template <bool REC>
+__global__ void __launch_bounds__(kTabThreads, 8) walk_keys_kernel(WalkArgs A, int tile_arcs,
+                                                                   const int64_t *__restrict__ tile_off,
+                                                                   uint64_t *__restrict__ keys) {
+    extern __shared__ uint32_t smem[];
+    __shared__ __align__(16) uint8_t s_rlut[4096];
+    __shared__ uint32_t s_rmod[17];
+    __shared__ uint32_t s_ent[kTabWarps][kTabBatch];    // arc in tile | r << 12 | sigma << 17 | rank << 21
+    __shared__ uint32_t s_w3[kTabWarps][kTabBatch];     // word 3 of each draw
+    __shared__ uint8_t s_sorted[kTabWarps][kTabBatch];  // batch index at each ranked position
+    __shared__ uint32_t s_hist[kTabWarps][32];          // draws per r so far in the batch
+    __shared__ int32_t s_first, s_last;                 // sources of the tile's first and last arc
+    uint32_t *s_off = smem;                             // tile_arcs + 1
+    int32_t *s_src = reinterpret_cast<int32_t *>(s_off + tile_arcs + 1);
+    int32_t *s_dst = s_src + tile_arcs;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t a0 = (int64_t)blockIdx.x * tile_arcs;
+    const int na = (int)imin64(tile_arcs, A.n_arcs - a0);
+    for (int b = tid; b < 4096 / 16; b += kTabThreads)
+        reinterpret_cast<uint4 *>(s_rlut)[b] = __ldg(reinterpret_cast<const uint4 *>(A.rlut) + b);
+    if (tid < 17) s_rmod[tid] = A.rmod[tid];
+    s_hist[warp][lane] = 0;
+    if (tid == 0) s_first = arc_source(A.indptr, A.n, a0);
+    if (tid == 32) s_last = arc_source(A.indptr, A.n, a0 + na - 1);
+    __syncthreads();
+    for (int i = tid; i < na; i += kTabThreads) {
+        s_off[i] = arc_count(A, a0 + i);
+        s_dst[i] = __ldg(A.indices + a0 + i);
+        int64_t lo = s_first, hi = (int64_t)s_last + 1;   // indptr[lo] <= a0 + i < indptr[hi]
+        while (hi - lo > 1) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (__ldg(A.indptr + mid) <= a0 + i) lo = mid; else hi = mid;
+        }
+        s_src[i] = (int32_t)lo;
+    }
+    __syncthreads();
+    const uint32_t total = block_exclusive_scan<kTabThreads>(s_off, na);
+    if (tid == 0) s_off[na] = total;
+    __syncthreads();
+    uint64_t *out = keys + tile_off[blockIdx.x];
+    const bool uniform = A.thr_frac == 0;
+    uint32_t *ent = s_ent[warp];
+    uint32_t *w3s = s_w3[warp];
+    uint8_t *sorted = s_sorted[warp];
+    uint32_t *hist = s_hist[warp];
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    const uint32_t nbatch = (total + kTabBatch - 1) / kTabBatch;
+    for (uint32_t bt = warp; bt < nbatch; bt += kTabWarps) {
+        const uint32_t bbase = bt * kTabBatch;
+        // heads and ranks by r (r = 0: past the tile's last sample)
+#pragma unroll 2
+        for (int t = 0; t < kTabBatch / 32; ++t) {
+            const uint32_t idx = (uint32_t)t * 32 + lane;
+            const uint32_t s = bbase + idx;
+            int r = 0, sg = 0, lo = 0;
+            uint32_t w3 = 0;
+            if (s < total) {
+                if (uniform) {
+                    lo = A.base == 1 ? (int)s : (int)fastdiv32(s, A.base_magic);
+                } else {
+                    int hi = na;   // s_off[lo] <= s < s_off[hi]
+                    while (hi - lo > 1) {
+                        const int mid = (lo + hi) >> 1;
+                        if (s_off[mid] <= s) lo = mid; else hi = mid;
+                    }
+                }
+                uint32_t coin;
+                draw_head(A, s_rlut, s_rmod, a0 + lo, s - s_off[lo], &r, &sg, &coin, &w3);
+            }
+            const unsigned grp = __match_any_sync(0xffffffffu, r);
+            const int leader = __ffs(grp) - 1;
+            uint32_t base = 0;
+            if (lane == leader) {
+                base = hist[r];
+                hist[r] = base + (uint32_t)__popc(grp);
+            }
+            base = __shfl_sync(0xffffffffu, base, leader);
+            const uint32_t rank = base + (uint32_t)__popc(grp & lt_mask);
+            ent[idx] = (uint32_t)lo | ((uint32_t)r << 12) | ((uint32_t)sg << 17) | (rank << 21);
+            w3s[idx] = w3;
+            __syncwarp();   // the next group leader reads what this one wrote
+        }
+        // exclusive scan of the 17 bins: lane r holds the first position of r
+        const uint32_t h = lane < 17 ? hist[lane] : 0u;
+        uint32_t incl = h;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const uint32_t start = incl - h;
+        hist[lane] = 0;
+#pragma unroll 1
+        for (int t = 0; t < kTabBatch / 32; ++t) {
+            const uint32_t idx = (uint32_t)t * 32 + lane;
+            const uint32_t e = ent[idx];
+            const uint32_t pos = __shfl_sync(0xffffffffu, start, (e >> 12) & 31) + (e >> 21);
+            sorted[pos] = (uint8_t)idx;
+        }
+        __syncwarp();
+        // walks in r order, two draws per lane, 32 ranks apart
+        const uint32_t first = __shfl_sync(0xffffffffu, start, 1);
+#pragma unroll 1
+        for (uint32_t q = first + (uint32_t)lane; q < (uint32_t)kTabBatch; q += 64) {
+            const bool has1 = q + 32 < (uint32_t)kTabBatch;
+            const uint32_t i0 = sorted[q], i1 = sorted[has1 ? q + 32 : q];
+            const uint32_t e0 = ent[i0], e1 = ent[i1];
+            const uint32_t lo0 = e0 & 0xFFFu, lo1 = e1 & 0xFFFu;
+            KeyDraw d0, d1;
+            key_begin(A, a0 + lo0, bbase + i0 - s_off[lo0], (int)((e0 >> 12) & 31), (int)((e0 >> 17) & 15), w3s[i0],
+                      s_src[lo0], s_dst[lo0], d0);
+            key_begin(A, a0 + lo1, bbase + i1 - s_off[lo1], (int)((e1 >> 12) & 31), (int)((e1 >> 17) & 15), w3s[i1],
+                      s_src[lo1], s_dst[lo1], d1);
+            if (!has1) d1.steps = 0;
+            KeySteps<0, REC>::run(A, d0, d1, max(d0.steps, d1.steps));
+            out[bbase + q - first] = key_end(d0, A.B);
+            if (has1) out[bbase + q + 32 - first] = key_end(d1, A.B);
+        }
+        __syncwarp();
+    }
+}
+
 // Exact 32-bit counts from the packed table and its wrap records, in place in
 // the 32-bit table (upper triangle only: nothing else was counted). Field i
 // of a word received its counter's c_i increments plus one carry per wrap of
@@ -1787,7 +2012,7 @@ WalkArgs make_walk_args(const GraphView &g, const SamplerSpec &sp) {
 }
 
 // Builds the per-vertex walk records into the workspace.
-int attach_vinfo(Workspace &ws, const GraphView &g, WalkArgs *A, cudaStream_t st) {
+int attach_vinfo(Workspace &ws, const GraphView &g, WalkArgs *A, cudaStream_t st, bool arc_records = true) {
     uint4 *vi = nullptr;
     LNE_TRY(ws.get("walk.vinfo", (size_t)std::max<int64_t>(g.n, 1), &vi));
     LNE_TRACE("build_vinfo", st);
@@ -1795,15 +2020,15 @@ int attach_vinfo(Workspace &ws, const GraphView &g, WalkArgs *A, cudaStream_t st
         g.indptr, g.n, vi);
     LNE_LAUNCH_CHECK();
     A->vinfo = vi;
-    uint4 *ar = nullptr;
-    LNE_TRY(ws.get("walk.arcrec", (size_t)std::max<int64_t>(g.nnz, 1), &ar));
-    {
+    if (arc_records) {
+        uint4 *ar = nullptr;
+        LNE_TRY(ws.get("walk.arcrec", (size_t)std::max<int64_t>(g.nnz, 1), &ar));
         LNE_TRACE("build_arcrec", st);
         build_arcrec_kernel<<<(unsigned)std::min<int64_t>(ceil_div(std::max<int64_t>(g.nnz, 1), 256), num_sms() * 16), 256, 0,
                               st>>>(g.indices, g.nnz, vi, ar);
         LNE_LAUNCH_CHECK();
+        A->arcrec = ar;
     }
-    A->arcrec = ar;
     uint8_t *lut = nullptr;
     LNE_TRY(ws.get("walk.rlut", 4096, &lut));
     build_rlut_kernel<<<16, 256, 0, st>>>(*A, lut);
@@ -1843,8 +2068,17 @@ int attach_downsample(Workspace &ws, const GraphView &g, const SamplerSpec &sp, 
     return 0;
 }
 
-// Tile size: aim for ~32k samples per CTA but at least ~8 CTAs per SM overall.
-int choose_tile_arcs(int64_t n_arcs, double rate) {
+// Most arcs for which walk_keys_kernel reads per-arc records: 64 MB of them, half
+// of L2. Measured (records / neighbour and vertex record, 8e7 to 1e8 draws): 2M
+// arcs 1.01 / 1.02 ms at T = 5 and 2.0 / 2.5 at T = 10, 8M arcs 2.1 / 1.7 and
+// 6.0 / 3.6, 16M arcs (2e8 draws, T = 5) 4.4 / 3.7.
+constexpr int64_t kKeyRecordArcs = (int64_t)4 << 20;
+
+// Tile size: aim for ~32k samples per CTA but at least ~8 CTAs per SM overall, and
+// at most max_arcs: 12 bytes of shared memory an arc, so 1024 leave room for
+// seven CTAs an SM. With 4096 (three CTAs) the downsampled walk of 16M arcs took
+// 7.3 ms instead of 5.0.
+int choose_tile_arcs(int64_t n_arcs, double rate, int max_arcs = 1024) {
     double per_arc = rate < 1.0 ? 1.0 : rate;
     double total = per_arc * (double)n_arcs;
     double want = total / ((double)num_sms() * 8.0);
@@ -1852,7 +2086,7 @@ int choose_tile_arcs(int64_t n_arcs, double rate) {
     if (want < 2048.0) want = 2048.0;
     int64_t t = (int64_t)(want / per_arc);
     if (t < 1) t = 1;
-    if (t > 4096) t = 4096;
+    if (t > max_arcs) t = max_arcs;
     return (int)t;
 }
 
@@ -1878,11 +2112,12 @@ template <typename KeyT, int MODE>
 int launch_walk_emit(const WalkArgs &A, unsigned grid, int smem, cudaStream_t st, int64_t a_begin, int64_t a_end,
                      int tile_arcs, const int64_t *tile_off, KeyT *keys, int32_t *u1, int32_t *v1,
                      uint32_t *bucket_cnt, int nb_smem) {
-    if (A.ds_thr || A.cum || A.w || A.strat) {
+    // the plain walks of MODE 2 and 3 are walk_table_kernel's and walk_keys_kernel's
+    if (MODE == 2 || MODE == 3 || A.ds_thr || A.cum || A.w || A.strat) {
         LNE_TRY(allow_dynamic_smem(walk_emit_kernel<KeyT, MODE, true>));
         walk_emit_kernel<KeyT, MODE, true><<<grid, kWalkThreads, smem, st>>>(A, a_begin, a_end, tile_arcs, tile_off,
                                                                             keys, u1, v1, bucket_cnt, nb_smem);
-    } else {
+    } else if constexpr (MODE != 2 && MODE != 3) {
         LNE_TRY(allow_dynamic_smem(walk_emit_kernel<KeyT, MODE, false>));
         walk_emit_kernel<KeyT, MODE, false><<<grid, kWalkThreads, smem, st>>>(A, a_begin, a_end, tile_arcs, tile_off,
                                                                              keys, u1, v1, bucket_cnt, nb_smem);
@@ -1893,9 +2128,9 @@ int launch_walk_emit(const WalkArgs &A, unsigned grid, int smem, cudaStream_t st
 
 int tile_offsets(Workspace &ws, const WalkArgs &A, int64_t a0, int64_t a1, int tile_arcs,
                  int64_t **tile_off, int64_t *total, cudaStream_t st) {
-    if (A.w) {   // a tile's sample count is a 32-bit sum: bound it by the heaviest arc
+    if (A.w) {   // a tile's sample count is a 32-bit sum: bound it by the heaviest arc (and tiles of 4096 arcs)
         const double max_rate = A.S * (double)A.wmax / A.vol;
-        if ((max_rate + 1.0) * (double)tile_arcs >= 2147483648.0)
+        if ((max_rate + 1.0) * (double)choose_tile_arcs(a1 - a0, (double)A.base + 0.5, 4096) >= 2147483648.0)
             return fail(LNE_ERR_UNSUPPORTED, "an arc's weight share of S is too large for the sample tiles");
     }
     const int64_t ntiles = ceil_div(a1 - a0, tile_arcs);
@@ -2189,14 +2424,18 @@ struct SortRaw {
 int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *R, cudaStream_t st) {
     if (2 * sp.B > 64) return fail(LNE_ERR_UNSUPPORTED, "pair keys need 2 ceil(log2 n) <= 64 bits");
     WalkArgs A = make_walk_args(g, sp);
-    LNE_TRY(attach_vinfo(ws, g, &A, st));
+    const bool lean = !(sp.ds_C > 0.0) && !A.w && !A.strat;   // walk_keys_kernel takes it
+    const bool arc_records = !lean || g.nnz <= kKeyRecordArcs;
+    LNE_TRY(attach_vinfo(ws, g, &A, st, arc_records));
     LNE_TRY(attach_downsample(ws, g, sp, &A, st));
     const bool ds = A.ds_thr != nullptr;
     const int bits = 2 * sp.B + ((ds && ((int64_t)1 << sp.B) == g.n) ? 1 : 0);
     if (bits > 64) return fail(LNE_ERR_UNSUPPORTED, "downsampled pair keys need 2 ceil(log2 n) + 1 <= 64 bits");
     if (ds && g.nnz > (int64_t)UINT32_MAX)
         return fail(LNE_ERR_UNSUPPORTED, "edge downsampling on the sort path needs fewer than 2^32 arcs");
-    const int tile_arcs = choose_tile_arcs(g.nnz, (double)sp.base + 0.5);
+    const double rate = (double)sp.base + 0.5;
+    const int tile_arcs = lean ? (int)std::min<double>(kKeyMaxTileArcs, std::max(1.0, kKeyTileSamples / rate))
+                               : choose_tile_arcs(g.nnz, rate);
     int64_t *tile_off = nullptr;
     int64_t total = 0;
     LNE_TRY(tile_offsets(ws, A, 0, g.nnz, tile_arcs, &tile_off, &total, st));
@@ -2213,8 +2452,16 @@ int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *
     const int smem = walk_smem_bytes(tile_arcs, 0);
     {
         LNE_TRACE("walk_keys", st);
-        LNE_TRY((launch_walk_emit<uint64_t, 3>(A, (unsigned)ntiles, smem, st, 0, g.nnz, tile_arcs, tile_off, k0,
-                                              reinterpret_cast<int32_t *>(arc0), nullptr, nullptr, 0)));
+        if (lean) {
+            if (arc_records)
+                walk_keys_kernel<true><<<(unsigned)ntiles, kTabThreads, smem, st>>>(A, tile_arcs, tile_off, k0);
+            else
+                walk_keys_kernel<false><<<(unsigned)ntiles, kTabThreads, smem, st>>>(A, tile_arcs, tile_off, k0);
+            LNE_LAUNCH_CHECK();
+        } else {
+            LNE_TRY((launch_walk_emit<uint64_t, 3>(A, (unsigned)ntiles, smem, st, 0, g.nnz, tile_arcs, tile_off, k0,
+                                                  reinterpret_cast<int32_t *>(arc0), nullptr, nullptr, 0)));
+        }
     }
     bool in_alt = false;
     LNE_TRY(radix_sort_u64(ws, k0, k1, arc0, arc1, total, 0, bits, &in_alt, st));

@@ -72,6 +72,19 @@ def test_counts_and_csr(ctx, g, T, rate):
     np.testing.assert_allclose(to_np(out["data"]), sp["data"], rtol=1e-6, atol=1e-7)
 
 
+@pytest.mark.parametrize("T,rate", [(1, 1.0), (5, 0.4), (16, 0.5)])
+def test_walk_without_arc_records(ctx, T, rate):
+    """Graphs of more than 2^22 arcs walk through neighbours and vertex records
+    instead of arc records: the oracle's pairs all the same."""
+    g = synth.ring((1 << 21) + 3)
+    p = make_params(T, np.full(T, 1.0 / T), rate * g.n_arcs, seed=5)
+    res = ctx.sparsifier_counts(lne.DeviceGraph.from_graph(g), p)
+    x, y, c = oracle_counts(g, p)
+    assert np.array_equal(to_np(res["x"]).astype(np.int64), x)
+    assert np.array_equal(to_np(res["y"]).astype(np.int64), y)
+    assert np.array_equal(to_np(res["count"]).astype(np.int64), c)
+
+
 @pytest.mark.parametrize("n,rate", [(513, 1.0), (3073, 4.0), (9001, 2.5)])
 @pytest.mark.parametrize("C", [0.7, 4.0])
 def test_downsampled_sums_equal_the_table(ctx, n, rate, C):
