@@ -72,7 +72,7 @@ struct WalkArgs {
     // (first j with word < cum[off + j], cum = floor(2^32 prefix_j / d_x))
     const uint32_t *w;
     const uint32_t *cum;
-    const uint32_t *guide;        // per arc b of x: the answer for the smallest word of bucket b
+    const uint4 *wstep;           // per arc b of x: bracket and thresholds of bucket b (build_wstep_kernel)
     double S, vol;
     uint32_t wmax;                // host copy of the largest weight (tile size bounds)
 };
@@ -174,42 +174,28 @@ __global__ void build_cum_kernel(const int64_t *__restrict__ indptr, const uint3
         const int64_t a0 = indptr[x], a1 = indptr[x + 1];
         const uint64_t d = __ldg(wdeg + x);
         uint64_t carry = 0;
-        for (int64_t base = a0; base < a1; base += 32) {
-            const int64_t a = base + lane;
-            uint64_t v = a < a1 ? (uint64_t)__ldg(w + a) : 0ull;
+        for (int64_t base = a0; base < a1; base += 128) {   // four chunks' loads and scans in flight
+            uint64_t own[4], pre[4];
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint64_t y = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += y;
+            for (int c = 0; c < 4; ++c) {
+                const int64_t a = base + 32 * c + lane;
+                own[c] = a < a1 ? (uint64_t)__ldg(w + a) : 0ull;
             }
-            const uint64_t prefix = carry + v;
-            // the last arc's threshold would be 2^32: it is never read
-            const uint64_t t = (prefix << 32) / d;
-            if (a < a1) cum[a] = t > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)t;
-            carry += __shfl_sync(0xffffffffu, v, 31);
-        }
-    }
-}
-
-// Guide of the weighted step: for bucket b of vertex x (words w with
-// floor(w deg / 2^32) = b) the answer for the bucket's smallest word
-// ceil(b 2^32 / deg); the inverse CDF is monotone in w, so a word of bucket b
-// takes an arc between guide[b] and guide[b + 1] (or the last arc).
-__global__ void build_guide_kernel(const int64_t *__restrict__ indptr, const uint32_t *__restrict__ cum, int64_t n,
-                                   uint32_t *__restrict__ guide) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t x = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); x < n; x += warps) {
-        const int64_t a0 = indptr[x];
-        const uint64_t deg = (uint64_t)(indptr[x + 1] - a0);
-        for (uint64_t b = lane; b < deg; b += 32) {
-            const uint64_t w0 = ((b << 32) + deg - 1) / deg;   // ceil(b 2^32 / deg) < 2^32
-            uint32_t lo = 0, hi = (uint32_t)deg - 1;           // first j with w0 < cum[j], else the last
-            while (lo < hi) {
-                const uint32_t mid = (lo + hi) >> 1;
-                if (w0 < (uint64_t)cum[a0 + mid]) hi = mid; else lo = mid + 1;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (base + 32 * c >= a1) break;
+                pre[c] = own[c];
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint64_t y = __shfl_up_sync(0xffffffffu, pre[c], o);
+                    if (lane >= o) pre[c] += y;
+                }
+                const int64_t a = base + 32 * c + lane;
+                // the last arc's threshold would be 2^32: it is never read
+                const uint64_t t = ((carry + pre[c]) << 32) / d;
+                if (a < a1) cum[a] = t > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)t;
+                carry += __shfl_sync(0xffffffffu, pre[c], 31);
             }
-            guide[a0 + (int64_t)b] = lo;
         }
     }
 }
@@ -222,6 +208,54 @@ __device__ __forceinline__ int32_t arc_source(const int64_t *__restrict__ indptr
         if (__ldg(indptr + mid) <= a) lo = mid; else hi = mid;
     }
     return (int32_t)lo;
+}
+
+// Record of the weighted step, 16 bytes: for bucket b of vertex x (words w with
+// floor(w deg / 2^32) = b) the answer lo for the bucket's smallest word
+// ceil(b 2^32 / deg), the answer hi for the next bucket's (the last arc for the
+// last bucket) and the thresholds of arcs lo and lo + 1. The inverse CDF is
+// monotone in w, so a word of bucket b takes an arc of lo..hi, and one load
+// settles it when hi <= lo + 2. A thread per arc (a hub's arcs by a single warp
+// held the build up): tiles of 1024 arcs, whose sources lie between those of the
+// tile's ends.
+constexpr int kStepTile = 1024;
+__global__ void __launch_bounds__(256) build_wstep_kernel(const int64_t *__restrict__ indptr,
+                                                          const uint32_t *__restrict__ cum, int64_t n, int64_t nnz,
+                                                          uint4 *__restrict__ wstep) {
+    __shared__ uint32_t s_lo[kStepTile + 1];
+    __shared__ int32_t s_x[kStepTile + 1];
+    __shared__ int32_t s_first, s_last;
+    const int64_t p0 = (int64_t)blockIdx.x * kStepTile;
+    const int np = (int)imin64(kStepTile + 1, nnz - p0);   // with the next tile's first arc
+    if (threadIdx.x == 0) s_first = arc_source(indptr, n, p0);
+    if (threadIdx.x == 32) s_last = arc_source(indptr, n, p0 + np - 1);
+    __syncthreads();
+    for (int i = threadIdx.x; i < np; i += 256) {
+        int64_t xl = s_first, xh = (int64_t)s_last + 1;   // indptr[xl] <= p0 + i < indptr[xh]
+        while (xh - xl > 1) {
+            const int64_t mid = (xl + xh) >> 1;
+            if (__ldg(indptr + mid) <= p0 + i) xl = mid; else xh = mid;
+        }
+        const int64_t a0 = __ldg(indptr + xl);
+        const uint64_t deg = (uint64_t)(__ldg(indptr + xl + 1) - a0), b = (uint64_t)(p0 + i - a0);
+        const uint64_t w0 = ((b << 32) + deg - 1) / deg;   // ceil(b 2^32 / deg) < 2^32
+        uint32_t lo = 0, hi = (uint32_t)deg - 1;           // first j with w0 < cum[j], else the last
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (w0 < (uint64_t)__ldg(cum + a0 + mid)) hi = mid; else lo = mid + 1;
+        }
+        s_lo[i] = lo;
+        s_x[i] = (int32_t)xl;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kStepTile && i < np; i += 256) {
+        if (p0 + i >= nnz) break;
+        const int32_t x = s_x[i];
+        const int64_t a0 = __ldg(indptr + x);
+        const uint32_t deg = (uint32_t)(__ldg(indptr + x + 1) - a0), lo = s_lo[i];
+        const uint32_t hi = i + 1 < np && s_x[i + 1] == x ? s_lo[i + 1] : deg - 1;
+        wstep[p0 + i] = make_uint4(lo, hi, __ldg(cum + a0 + lo), lo + 1 < deg ? __ldg(cum + a0 + lo + 1) : 0xFFFFFFFFu);
+    }
 }
 
 // Walk state: the current vertex and its walk record.
@@ -256,16 +290,21 @@ __device__ __forceinline__ void walk_step(const WalkArgs &A, WalkCur &c, uint32_
     if (deg == 0xFFFFFFu) deg = (uint32_t)(__ldg(A.indptr + c.x + 1) - __ldg(A.indptr + c.x));
     if (GEN && A.cum) {
         // weighted: inverse CDF over the vertex's thresholds (the last is
-        // 2^32). The word's bucket b = floor(w deg / 2^32) brackets the
-        // answer between the guides of buckets b and b + 1, usually one arc.
-        const uint32_t b = __umulhi(w, deg);
-        uint32_t lo = __ldg(A.guide + off + b);
-        uint32_t hi = b + 1 < deg ? __ldg(A.guide + off + b + 1) : deg - 1;
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (w < __ldg(A.cum + off + mid)) hi = mid; else lo = mid + 1;
+        // 2^32): the first arc of the word's bracket lo..hi whose threshold is
+        // above the word, else hi
+        const uint4 g = __ldg(A.wstep + off + __umulhi(w, deg));
+        if (g.x == g.y || w < g.z) {
+            j = g.x;
+        } else if (g.x + 1 == g.y || w < g.w) {
+            j = g.x + 1;
+        } else {
+            uint32_t lo = g.x + 2, hi = g.y;
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (w < __ldg(A.cum + off + mid)) hi = mid; else lo = mid + 1;
+            }
+            j = lo;
         }
-        j = lo;
     } else if ((c.hidg >> 8) == 0xFFFFFFu) {
         j = w % deg;
     } else {
@@ -916,7 +955,7 @@ __global__ void __launch_bounds__(kTabThreads, kTabMinBlocks) walk_table_kernel(
 // next vertex's offset, degree and reciprocal. Otherwise it reads the 4-byte
 // neighbour, and the neighbour's vertex record unless the step is the last of
 // its side (then the id is all that is needed): two dependent loads, over a
-// quarter of the bytes (the rule stands at kKeyRecordArcs).
+// quarter of the bytes (the rule stands at kRecordArcs).
 //
 // Bound by gathers that miss L1 (one a step and one a vertex record, from L2).
 // Measured at 400k vertices, 16M arcs, 2e8 draws, T = 5: 3.7 ms. walk_emit_kernel
@@ -1970,7 +2009,7 @@ __global__ void path_mirror_fill_kernel(const uint64_t *__restrict__ mk, const u
 }
 
 WalkArgs make_walk_args(const GraphView &g, const SamplerSpec &sp) {
-    WalkArgs A;
+    WalkArgs A = {};   // no records, weights or coins until they are attached
     A.indptr = g.indptr;
     A.indices = g.indices;
     A.n = g.n;
@@ -2000,7 +2039,7 @@ WalkArgs make_walk_args(const GraphView &g, const SamplerSpec &sp) {
     A.strat = sp.stratified;
     A.w = g.w;
     A.cum = nullptr;
-    A.guide = nullptr;
+    A.wstep = nullptr;
     A.S = sp.S;
     A.vol = g.vol;
     A.wmax = g.wmax;
@@ -2012,6 +2051,13 @@ WalkArgs make_walk_args(const GraphView &g, const SamplerSpec &sp) {
 }
 
 // Builds the per-vertex walk records into the workspace.
+// Most arcs for which walk_keys_kernel reads per-arc records: 64 MB of them, half
+// of L2. Measured (records / neighbour and vertex record, 8e7 to 1e8 draws): 2M
+// arcs 1.01 / 1.02 ms at T = 5 and 2.0 / 2.5 at T = 10, 8M arcs 2.1 / 1.7 and
+// 6.0 / 3.6, 16M arcs (2e8 draws, T = 5) 4.4 / 3.7. The weighted step, which has a
+// record of its own per arc, is better off with them at 16M arcs too (13.9 / 15.6).
+constexpr int64_t kRecordArcs = (int64_t)4 << 20;
+
 int attach_vinfo(Workspace &ws, const GraphView &g, WalkArgs *A, cudaStream_t st, bool arc_records = true) {
     uint4 *vi = nullptr;
     LNE_TRY(ws.get("walk.vinfo", (size_t)std::max<int64_t>(g.n, 1), &vi));
@@ -2041,13 +2087,13 @@ int attach_vinfo(Workspace &ws, const GraphView &g, WalkArgs *A, cudaStream_t st
         build_cum_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(g.n, 8), num_sms() * 16)), 256, 0,
                            st>>>(g.indptr, g.w, g.wdeg, g.n, cum);
         LNE_LAUNCH_CHECK();
-        uint32_t *guide = nullptr;
-        LNE_TRY(ws.get("walk.guide", (size_t)std::max<int64_t>(g.nnz, 1), &guide));
-        build_guide_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(g.n, 8), num_sms() * 16)), 256, 0,
-                             st>>>(g.indptr, cum, g.n, guide);
+        uint4 *wstep = nullptr;
+        LNE_TRY(ws.get("walk.wstep", (size_t)std::max<int64_t>(g.nnz, 1), &wstep));
+        build_wstep_kernel<<<(unsigned)std::max<int64_t>(1, ceil_div(g.nnz, (int64_t)kStepTile)), 256, 0, st>>>(
+            g.indptr, cum, g.n, g.nnz, wstep);
         LNE_LAUNCH_CHECK();
         A->cum = cum;
-        A->guide = guide;
+        A->wstep = wstep;
     }
     return 0;
 }
@@ -2068,21 +2114,17 @@ int attach_downsample(Workspace &ws, const GraphView &g, const SamplerSpec &sp, 
     return 0;
 }
 
-// Most arcs for which walk_keys_kernel reads per-arc records: 64 MB of them, half
-// of L2. Measured (records / neighbour and vertex record, 8e7 to 1e8 draws): 2M
-// arcs 1.01 / 1.02 ms at T = 5 and 2.0 / 2.5 at T = 10, 8M arcs 2.1 / 1.7 and
-// 6.0 / 3.6, 16M arcs (2e8 draws, T = 5) 4.4 / 3.7.
-constexpr int64_t kKeyRecordArcs = (int64_t)4 << 20;
-
-// Tile size: aim for ~32k samples per CTA but at least ~8 CTAs per SM overall, and
-// at most max_arcs: 12 bytes of shared memory an arc, so 1024 leave room for
-// seven CTAs an SM. With 4096 (three CTAs) the downsampled walk of 16M arcs took
-// 7.3 ms instead of 5.0.
-int choose_tile_arcs(int64_t n_arcs, double rate, int max_arcs = 1024) {
+// Tile size: at most max_samples samples per CTA, at least ~8 CTAs per SM overall
+// (but 2048 samples), and at most max_arcs, whose 12 bytes each of shared memory
+// leave the L1 cache less. Measured with 4096 samples and up to 512 arcs / 32768
+// and 4096: weighted walk of 16M arcs 7.9 / 17.7 ms (8192 samples 8.4, 16384 and
+// 1024 arcs 13.8), downsampled 4.1 / 7.3, weighted downsampled of 668k arcs, 100
+// draws each, 2.0 / 2.5 (there the last wave was nearly empty).
+int choose_tile_arcs(int64_t n_arcs, double rate, double max_samples = 4096.0, int max_arcs = 512) {
     double per_arc = rate < 1.0 ? 1.0 : rate;
     double total = per_arc * (double)n_arcs;
     double want = total / ((double)num_sms() * 8.0);
-    if (want > 32768.0) want = 32768.0;
+    if (want > max_samples) want = max_samples;
     if (want < 2048.0) want = 2048.0;
     int64_t t = (int64_t)(want / per_arc);
     if (t < 1) t = 1;
@@ -2130,7 +2172,7 @@ int tile_offsets(Workspace &ws, const WalkArgs &A, int64_t a0, int64_t a1, int t
                  int64_t **tile_off, int64_t *total, cudaStream_t st) {
     if (A.w) {   // a tile's sample count is a 32-bit sum: bound it by the heaviest arc (and tiles of 4096 arcs)
         const double max_rate = A.S * (double)A.wmax / A.vol;
-        if ((max_rate + 1.0) * (double)choose_tile_arcs(a1 - a0, (double)A.base + 0.5, 4096) >= 2147483648.0)
+        if ((max_rate + 1.0) * (double)choose_tile_arcs(a1 - a0, (double)A.base + 0.5, 32768.0, 4096) >= 2147483648.0)
             return fail(LNE_ERR_UNSUPPORTED, "an arc's weight share of S is too large for the sample tiles");
     }
     const int64_t ntiles = ceil_div(a1 - a0, tile_arcs);
@@ -2243,7 +2285,8 @@ int sample_and_reduce(Workspace &ws, const GraphView &g, const SamplerSpec &sp, 
         return fail(LNE_ERR_UNSUPPORTED, "graphs with more than 65536 vertices need 64-bit pair keys (not in this build)");
     WalkArgs A = make_walk_args(g, sp);
     LNE_TRY(attach_vinfo(ws, g, &A, st));
-    const int tile_arcs = choose_tile_arcs(g.nnz, (double)sp.base + 0.5);
+    // a tile flushes its whole bucket histogram: larger tiles than the other walks take
+    const int tile_arcs = choose_tile_arcs(g.nnz, (double)sp.base + 0.5, 32768.0, 4096);
     int64_t *tile_off = nullptr;
     int64_t total = 0;
     LNE_TRY(tile_offsets(ws, A, 0, g.nnz, tile_arcs, &tile_off, &total, st));
@@ -2425,8 +2468,7 @@ int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *
     if (2 * sp.B > 64) return fail(LNE_ERR_UNSUPPORTED, "pair keys need 2 ceil(log2 n) <= 64 bits");
     WalkArgs A = make_walk_args(g, sp);
     const bool lean = !(sp.ds_C > 0.0) && !A.w && !A.strat;   // walk_keys_kernel takes it
-    const bool arc_records = !lean || g.nnz <= kKeyRecordArcs;
-    LNE_TRY(attach_vinfo(ws, g, &A, st, arc_records));
+    LNE_TRY(attach_vinfo(ws, g, &A, st, !lean || g.nnz <= kRecordArcs));
     LNE_TRY(attach_downsample(ws, g, sp, &A, st));
     const bool ds = A.ds_thr != nullptr;
     const int bits = 2 * sp.B + ((ds && ((int64_t)1 << sp.B) == g.n) ? 1 : 0);
@@ -2453,7 +2495,7 @@ int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *
     {
         LNE_TRACE("walk_keys", st);
         if (lean) {
-            if (arc_records)
+            if (A.arcrec)
                 walk_keys_kernel<true><<<(unsigned)ntiles, kTabThreads, smem, st>>>(A, tile_arcs, tile_off, k0);
             else
                 walk_keys_kernel<false><<<(unsigned)ntiles, kTabThreads, smem, st>>>(A, tile_arcs, tile_off, k0);
@@ -2667,14 +2709,15 @@ int sample_table(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Table
     tb->nt = nt;
     LNE_CUDA_TRY(cudaMemsetAsync(tb->T, 0, sizeof(uint32_t) * (size_t)(ld * ld), st));
     WalkArgs A = make_walk_args(g, sp);
+    const bool plain = !(sp.ds_C > 0.0) && !A.w && !A.strat;   // walk_table_kernel takes it
     LNE_TRY(attach_vinfo(ws, g, &A, st));
     LNE_TRY(attach_downsample(ws, g, sp, &A, st));
     const int tile_arcs = choose_tile_arcs(g.nnz, (double)sp.base + 0.5);
     const int64_t ntiles = ceil_div(g.nnz, tile_arcs);
     const int smem = walk_smem_bytes(tile_arcs, 0);
-    if (!A.ds_thr && !A.w && !A.strat) {
+    if (plain) {
         // tiles of at most kTabMaxTileArcs arcs, whose walk records sit in shared memory
-        const int tab_arcs = std::min(tile_arcs, kTabMaxTileArcs);
+        const int tab_arcs = choose_tile_arcs(g.nnz, (double)sp.base + 0.5, 32768.0, kTabMaxTileArcs);
         const int64_t tab_tiles = ceil_div(g.nnz, tab_arcs);
         const int tab_smem = tab_arcs * 32 + (tab_arcs + 1) * 4;
         // packed narrow counters, decoded into the 32-bit table afterwards
