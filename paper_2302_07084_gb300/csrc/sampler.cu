@@ -279,6 +279,20 @@ __device__ __forceinline__ uint32_t barrett_mod(uint32_t w, uint32_t m, uint32_t
     return r >= d ? r - d : r;
 }
 
+// The arc that word w takes from a vertex of a weighted graph (inverse CDF over its
+// thresholds, the last of which is 2^32): the first of the word's bracket lo..hi
+// whose threshold is above the word, else hi. g: the bracket's record.
+__device__ __forceinline__ uint32_t weighted_arc(const WalkArgs &A, int64_t off, uint4 g, uint32_t w) {
+    if (g.x == g.y || w < g.z) return g.x;
+    if (g.x + 1 == g.y || w < g.w) return g.x + 1;
+    uint32_t lo = g.x + 2, hi = g.y;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (w < __ldg(A.cum + off + mid)) hi = mid; else lo = mid + 1;
+    }
+    return lo;
+}
+
 // One walk step: x <- nbr(x)[w mod deg(x)] (Sec. 5.2), reading the taken
 // arc's record. GEN: the variant that also handles weighted graphs.
 template <bool GEN>
@@ -289,22 +303,7 @@ __device__ __forceinline__ void walk_step(const WalkArgs &A, WalkCur &c, uint32_
     uint32_t j;
     if (deg == 0xFFFFFFu) deg = (uint32_t)(__ldg(A.indptr + c.x + 1) - __ldg(A.indptr + c.x));
     if (GEN && A.cum) {
-        // weighted: inverse CDF over the vertex's thresholds (the last is
-        // 2^32): the first arc of the word's bracket lo..hi whose threshold is
-        // above the word, else hi
-        const uint4 g = __ldg(A.wstep + off + __umulhi(w, deg));
-        if (g.x == g.y || w < g.z) {
-            j = g.x;
-        } else if (g.x + 1 == g.y || w < g.w) {
-            j = g.x + 1;
-        } else {
-            uint32_t lo = g.x + 2, hi = g.y;
-            while (lo < hi) {
-                const uint32_t mid = (lo + hi) >> 1;
-                if (w < __ldg(A.cum + off + mid)) hi = mid; else lo = mid + 1;
-            }
-            j = lo;
-        }
+        j = weighted_arc(A, off, __ldg(A.wstep + off + __umulhi(w, deg)), w);
     } else if ((c.hidg >> 8) == 0xFFFFFFu) {
         j = w % deg;
     } else {
@@ -464,13 +463,10 @@ __global__ void __launch_bounds__(kWalkThreads) tile_counts_kernel(WalkArgs A, i
 }
 
 // MODE 0: write ordered endpoint pairs (u1, v1). MODE 1: write canonical keys
-// and count key buckets. MODE 2: add the pair into the dense count table
-// table[x * ld + y] (x <= y); `keys` is the table, ld = nb_smem. MODE 3: write
-// the canonical key at the sample's position (no counting). GEN = false is the
-// variant for unweighted graphs without downsampling or window strata (the
-// checks for those compiled out); GEN = true handles everything.
+// and count key buckets. GEN = false is the variant for unweighted graphs without
+// downsampling (the checks for those compiled out); GEN = true handles everything.
 template <typename KeyT, int MODE, bool GEN>
-__global__ void __launch_bounds__(kWalkThreads, MODE == 2 ? 10 : 8) walk_emit_kernel(
+__global__ void __launch_bounds__(kWalkThreads, 8) walk_emit_kernel(
     WalkArgs A, int64_t a_begin, int64_t a_end, int tile_arcs, const int64_t *__restrict__ tile_off,
     KeyT *__restrict__ keys, int32_t *__restrict__ u1, int32_t *__restrict__ v1,
     uint32_t *__restrict__ bucket_cnt, int nb_smem) {
@@ -524,32 +520,17 @@ __global__ void __launch_bounds__(kWalkThreads, MODE == 2 ? 10 : 8) walk_emit_ke
         j = s - s_off[lo];
     };
     // a draw the downsampling coin drops leaves a marker at its position:
-    // (-1, -1) for raw draws, a key above every pair key for the sort
-    auto emit_dropped = [&](uint32_t s, int64_t arc) {
+    // (-1, -1) for raw draws
+    auto emit_dropped = [&](uint32_t s) {
         if (MODE == 0) {
             u1[out0 + s] = -1;
             v1[out0 + s] = -1;
-        } else if (MODE == 3) {
-            keys[out0 + s] = ~(KeyT)0;
-            if (u1) reinterpret_cast<uint32_t *>(u1)[out0 + s] = (uint32_t)arc;
         }
     };
-    auto emit = [&](uint32_t s, int64_t arc, int32_t pu, int32_t pv, uint32_t r) {
+    auto emit = [&](uint32_t s, int32_t pu, int32_t pv) {
         if (MODE == 0) {
             u1[out0 + s] = pu;
             v1[out0 + s] = pv;
-        } else if (MODE == 2) {
-            const uint32_t x = (uint32_t)min(pu, pv), y = (uint32_t)max(pu, pv);
-            const size_t at = (size_t)x * (uint32_t)nb_smem + y;
-            if (sizeof(KeyT) == 8)   // downsampled: weights, 2^-32 fixed point
-                atomicAdd(reinterpret_cast<unsigned long long *>(keys) + at, (unsigned long long)A.ds_w[arc]);
-            else
-                atomicAdd(reinterpret_cast<uint32_t *>(keys) + at, 1u);
-        } else if (MODE == 3) {
-            const uint32_t x = (uint32_t)min(pu, pv), y = (uint32_t)max(pu, pv);
-            const KeyT key = ((KeyT)x << A.B) | (KeyT)y;
-            keys[out0 + s] = (GEN && A.strat) ? (key << 4) | (KeyT)(r - 1u) : key;
-            if (u1) reinterpret_cast<uint32_t *>(u1)[out0 + s] = (uint32_t)arc;   // the draw's arc
         } else {
             const uint32_t x = (uint32_t)min(pu, pv), y = (uint32_t)max(pu, pv);
             const KeyT key = ((KeyT)x << A.B) | (KeyT)y;
@@ -582,7 +563,7 @@ __global__ void __launch_bounds__(kWalkThreads, MODE == 2 ? 10 : 8) walk_emit_ke
                 draw_head(A, s_rlut, s_rmod, a0 + lo, j, &r, &sg, &coin, &w3);
                 // edge downsampling (Algorithm 3): the draw walks only if its coin comes up heads
                 if (GEN && A.ds_thr && (uint64_t)coin >= __ldg(A.ds_thr + a0 + lo)) {
-                    emit_dropped(cb + idx, a0 + lo);
+                    emit_dropped(cb + idx);
                     r = 0;
                 }
             }
@@ -648,10 +629,10 @@ __global__ void __launch_bounds__(kWalkThreads, MODE == 2 ? 10 : 8) walk_emit_ke
             StepAll<0, GEN>::run(A, d0, d1, max(d0.steps, d1.steps));
             int32_t pu, pv;
             draw_end(d0, &pu, &pv);
-            emit(s0, a0 + lo0, pu, pv, (pk0 >> 11) & 31);
+            emit(s0, pu, pv);
             if (has1) {
                 draw_end(d1, &pu, &pv);
-                emit(s1, a0 + lo1, pu, pv, (pk1 >> 11) & 31);
+                emit(s1, pu, pv);
             }
         }
         __syncthreads();
@@ -667,8 +648,8 @@ __global__ void __launch_bounds__(kWalkThreads, MODE == 2 ? 10 : 8) walk_emit_ke
 
 // ---------------------------------------------------------------------------
 // The dense-table walk of unweighted graphs without downsampling or window
-// strata (the benchmark's case). Same draws as walk_emit_kernel<.., 2, false>
-// (Algorithms 1 and 3, the same Philox words), organised for fewer
+// strata (the benchmark's case). The draws of Algorithms 1 and 3 from the same
+// Philox words as every other walk here, organised for fewer
 // instructions and less DRAM traffic per draw:
 //
 // * each warp works alone on batches of kTabBatch consecutive samples of the
@@ -945,25 +926,29 @@ __global__ void __launch_bounds__(kTabThreads, kTabMinBlocks) walk_table_kernel(
 }
 
 // ---------------------------------------------------------------------------
-// The key-emitting walk of unweighted graphs without downsampling or window
-// strata: the draws of walk_emit_kernel (the same Philox words), with each warp
-// alone on batches of 256 consecutive samples as in walk_table_kernel, ranked by
-// window length. The keys go to the sort, so a batch writes them in the order in
-// which it walks them (coalesced), not in sample order.
+// The walks that feed the key sort, and the dense-table walks with edge
+// downsampling, weights or window strata (GEN): the draws of Algorithms 1 and 3
+// from the same Philox words, with each warp alone on batches of 256 consecutive
+// samples as in walk_table_kernel, ranked by window length. Keys go to the sort, so
+// a batch of plain keys is written in the order in which it walks (coalesced), not
+// in sample order.
 //
-// REC: a step reads the 16-byte record of the arc that it takes, which holds the
-// next vertex's offset, degree and reciprocal. Otherwise it reads the 4-byte
-// neighbour, and the neighbour's vertex record unless the step is the last of
-// its side (then the id is all that is needed): two dependent loads, over a
-// quarter of the bytes (the rule stands at kRecordArcs).
+// kKeysRec: a step reads the 16-byte record of the arc that it takes, which holds
+// the next vertex's offset, degree and reciprocal. kKeysNbr: it reads the 4-byte
+// neighbour, and the neighbour's vertex record unless the step is the last of its
+// side (then the id is all that is needed): two dependent loads, over a quarter of
+// the bytes (the rule stands at kRecordArcs). GEN steps are not unrolled (the
+// instruction cache missed) and load for both of a lane's draws before either is
+// settled.
 //
 // Bound by gathers that miss L1 (one a step and one a vertex record, from L2).
-// Measured at 400k vertices, 16M arcs, 2e8 draws, T = 5: 3.7 ms. walk_emit_kernel
-// took 8.8: tiles of 4096 arcs left three CTAs of four warps an SM, and its CTA
-// barriers and DRAM-resident records kept those waiting.
+// Measured at 400k vertices, 16M arcs, 2e8 draws, T = 5: 3.7 ms. A CTA per chunk of
+// 512 ranked samples took 8.8: tiles of 4096 arcs left three CTAs of four warps an
+// SM, and its CTA barriers and DRAM-resident records kept those waiting. GEN: 668k
+// arcs, weighted, downsampled, 67M draws: 1.75 ms (the CTA-wide kernel 1.96); 16M arcs
+// weighted 7.5 (7.9).
 // ---------------------------------------------------------------------------
-constexpr int kKeyMaxTileArcs = 512;
-constexpr int kKeyTileSamples = 8192;
+enum WalkOut { kKeysRec, kKeysNbr, kKeysGen, kCountsGen, kWeightsGen };
 
 struct KeyDraw {
     uint32_t j;
@@ -1040,17 +1025,75 @@ struct KeySteps<15, REC> {
     __device__ __forceinline__ static void run(const WalkArgs &, KeyDraw &, KeyDraw &, int) {}
 };
 
-__device__ __forceinline__ uint64_t key_end(const KeyDraw &d, int B) {
+// Step k of two draws on any graph, their loads in flight together.
+__device__ __forceinline__ void gen_step(const WalkArgs &A, KeyDraw &d0, KeyDraw &d1, int k) {
+    const int widx = 3 + k;
+    const bool on0 = k < d0.steps, on1 = k < d1.steps;
+    if ((widx & 3) == 0) {
+        if (on0)
+            d0.nb = philox_rk(u32x4{d0.j, (uint32_t)(uint64_t)d0.arc, (uint32_t)((uint64_t)d0.arc >> 32),
+                                    (uint32_t)(widx >> 2)}, A.rk);
+        if (on1)
+            d1.nb = philox_rk(u32x4{d1.j, (uint32_t)(uint64_t)d1.arc, (uint32_t)((uint64_t)d1.arc >> 32),
+                                    (uint32_t)(widx >> 2)}, A.rk);
+    }
+    auto word = [&](const u32x4 &b) { return (widx & 2) ? ((widx & 1) ? b.w : b.z) : ((widx & 1) ? b.y : b.x); };
+    auto degree = [&](const WalkCur &c) {
+        const uint32_t deg = c.hidg >> 8;
+        return deg == 0xFFFFFFu ? (uint32_t)(__ldg(A.indptr + c.x + 1) - __ldg(A.indptr + c.x)) : deg;
+    };
+    const uint32_t w0 = word(d0.nb), w1 = word(d1.nb);
+    const uint32_t deg0 = on0 ? degree(d0.cur) : 0u, deg1 = on1 ? degree(d1.cur) : 0u;
+    const int64_t off0 = (int64_t)d0.cur.off_lo | ((int64_t)(d0.cur.hidg & 0xFF) << 32);
+    const int64_t off1 = (int64_t)d1.cur.off_lo | ((int64_t)(d1.cur.hidg & 0xFF) << 32);
+    uint32_t j0 = 0, j1 = 0;
+    if (A.cum) {
+        uint4 g0 = make_uint4(0u, 0u, 0u, 0u), g1 = g0;
+        if (deg0) g0 = __ldg(A.wstep + off0 + __umulhi(w0, deg0));
+        if (deg1) g1 = __ldg(A.wstep + off1 + __umulhi(w1, deg1));
+        j0 = weighted_arc(A, off0, g0, w0);
+        j1 = weighted_arc(A, off1, g1, w1);
+    } else {
+        auto plain = [&](const WalkCur &c, uint32_t deg, uint32_t w) {
+            return (c.hidg >> 8) == 0xFFFFFFu ? w % deg : deg < 2 ? 0u : barrett_mod(w, c.m, deg);
+        };
+        j0 = plain(d0.cur, deg0, w0);
+        j1 = plain(d1.cur, deg1, w1);
+    }
+    uint4 r0 = make_uint4(0u, 0u, 0u, 0u), r1 = r0;
+    if (deg0) r0 = __ldg(A.arcrec + off0 + j0);
+    if (deg1) r1 = __ldg(A.arcrec + off1 + j1);
+    if (deg0) d0.cur = WalkCur{(int32_t)r0.x, r0.y, r0.z, r0.w};   // degree 0 only on graphs that break the contract
+    if (deg1) d1.cur = WalkCur{(int32_t)r1.x, r1.y, r1.z, r1.w};
+    if (k + 1 == d0.sigma && k + 1 < d0.steps) {   // u side done: continue from v
+        d0.uend = d0.cur.x;
+        d0.cur = d0.v;
+    }
+    if (k + 1 == d1.sigma && k + 1 < d1.steps) {
+        d1.uend = d1.cur.x;
+        d1.cur = d1.v;
+    }
+}
+
+// The draw's pair, x <= y.
+__device__ __forceinline__ void key_end(const KeyDraw &d, uint32_t *x, uint32_t *y) {
     const bool one_sided = d.sigma >= d.steps;   // every step on the u side (or none at all)
     const int32_t pu = one_sided && d.steps > 0 ? d.cur.x : d.uend;
     const int32_t pv = one_sided ? d.v.x : d.cur.x;
-    return ((uint64_t)(uint32_t)min(pu, pv) << B) | (uint64_t)(uint32_t)max(pu, pv);
+    *x = (uint32_t)min(pu, pv);
+    *y = (uint32_t)max(pu, pv);
 }
 
-template <bool REC>
-__global__ void __launch_bounds__(kTabThreads, 8) walk_keys_kernel(WalkArgs A, int tile_arcs,
-                                                                   const int64_t *__restrict__ tile_off,
-                                                                   uint64_t *__restrict__ keys) {
+// Keys: written from tile_off[tile] on; with downsampling each key's arc into arcs,
+// and a dropped draw's key is all ones. Counts (kCountsGen) and weights (kWeightsGen):
+// added at x ld + y of the 32-bit table cnt or the 64-bit table keys.
+template <WalkOut OUT>
+__global__ void __launch_bounds__(kTabThreads, 8) walk_batch_kernel(WalkArgs A, int tile_arcs,
+                                                                    const int64_t *__restrict__ tile_off,
+                                                                    uint64_t *__restrict__ keys,
+                                                                    uint32_t *__restrict__ arcs,
+                                                                    uint32_t *__restrict__ cnt, uint32_t ld) {
+    constexpr bool GEN = OUT >= kKeysGen, KEYS = OUT <= kKeysGen;
     extern __shared__ uint32_t smem[];
     __shared__ __align__(16) uint8_t s_rlut[4096];
     __shared__ uint32_t s_rmod[17];
@@ -1086,8 +1129,8 @@ __global__ void __launch_bounds__(kTabThreads, 8) walk_keys_kernel(WalkArgs A, i
     const uint32_t total = block_exclusive_scan<kTabThreads>(s_off, na);
     if (tid == 0) s_off[na] = total;
     __syncthreads();
-    uint64_t *out = keys + tile_off[blockIdx.x];
-    const bool uniform = A.thr_frac == 0;
+    const int64_t out0 = KEYS ? tile_off[blockIdx.x] : 0;
+    const bool uniform = A.thr_frac == 0 && !(GEN && A.w);
     uint32_t *ent = s_ent[warp];
     uint32_t *w3s = s_w3[warp];
     uint8_t *sorted = s_sorted[warp];
@@ -1115,6 +1158,14 @@ __global__ void __launch_bounds__(kTabThreads, 8) walk_keys_kernel(WalkArgs A, i
                 }
                 uint32_t coin;
                 draw_head(A, s_rlut, s_rmod, a0 + lo, s - s_off[lo], &r, &sg, &coin, &w3);
+                // edge downsampling (Algorithm 3): the draw walks only if its coin comes up heads
+                if (GEN && A.ds_thr && (uint64_t)coin >= __ldg(A.ds_thr + a0 + lo)) {
+                    r = 0;
+                    if (KEYS) {
+                        keys[out0 + s] = ~0ull;
+                        if (arcs) arcs[out0 + s] = (uint32_t)(a0 + lo);
+                    }
+                }
             }
             const unsigned grp = __match_any_sync(0xffffffffu, r);
             const int leader = __ffs(grp) - 1;
@@ -1161,9 +1212,33 @@ __global__ void __launch_bounds__(kTabThreads, 8) walk_keys_kernel(WalkArgs A, i
             key_begin(A, a0 + lo1, bbase + i1 - s_off[lo1], (int)((e1 >> 12) & 31), (int)((e1 >> 17) & 15), w3s[i1],
                       s_src[lo1], s_dst[lo1], d1);
             if (!has1) d1.steps = 0;
-            KeySteps<0, REC>::run(A, d0, d1, max(d0.steps, d1.steps));
-            out[bbase + q - first] = key_end(d0, A.B);
-            if (has1) out[bbase + q + 32 - first] = key_end(d1, A.B);
+            if constexpr (GEN) {
+                const int kmax = max(d0.steps, d1.steps);
+#pragma unroll 1
+                for (int k = 0; k < kmax; ++k) gen_step(A, d0, d1, k);
+            } else {
+                KeySteps<0, OUT == kKeysRec>::run(A, d0, d1, max(d0.steps, d1.steps));
+            }
+            // a plain key goes to its rank's place, a general one to its sample's
+            auto emit = [&](const KeyDraw &d, uint32_t q_at, uint32_t i, uint32_t e) {
+                uint32_t x, y;
+                key_end(d, &x, &y);
+                if (KEYS) {
+                    const uint64_t key = ((uint64_t)x << A.B) | y;
+                    const int64_t at = out0 + bbase + (GEN ? i : q_at - first);
+                    keys[at] = GEN && A.strat ? (key << 4) | (uint64_t)(((e >> 12) & 31) - 1u) : key;
+                    if (GEN && arcs) arcs[at] = (uint32_t)d.arc;
+                } else {
+                    const size_t at = (size_t)x * ld + y;
+                    if (OUT == kWeightsGen)   // downsampled: weights, 2^-32 fixed point
+                        atomicAdd(reinterpret_cast<unsigned long long *>(keys) + at,
+                                  (unsigned long long)__ldg(A.ds_w + d.arc));
+                    else
+                        atomicAdd(cnt + at, 1u);
+                }
+            };
+            emit(d0, q, i0, e0);
+            if (has1) emit(d1, q + 32, i1, e1);
         }
         __syncwarp();
     }
@@ -2051,7 +2126,7 @@ WalkArgs make_walk_args(const GraphView &g, const SamplerSpec &sp) {
 }
 
 // Builds the per-vertex walk records into the workspace.
-// Most arcs for which walk_keys_kernel reads per-arc records: 64 MB of them, half
+// Most arcs for which a plain key walk (walk_batch_kernel) reads per-arc records: 64 MB of them, half
 // of L2. Measured (records / neighbour and vertex record, 8e7 to 1e8 draws): 2M
 // arcs 1.01 / 1.02 ms at T = 5 and 2.0 / 2.5 at T = 10, 8M arcs 2.1 / 1.7 and
 // 6.0 / 3.6, 16M arcs (2e8 draws, T = 5) 4.4 / 3.7. The weighted step, which has a
@@ -2154,16 +2229,24 @@ template <typename KeyT, int MODE>
 int launch_walk_emit(const WalkArgs &A, unsigned grid, int smem, cudaStream_t st, int64_t a_begin, int64_t a_end,
                      int tile_arcs, const int64_t *tile_off, KeyT *keys, int32_t *u1, int32_t *v1,
                      uint32_t *bucket_cnt, int nb_smem) {
-    // the plain walks of MODE 2 and 3 are walk_table_kernel's and walk_keys_kernel's
-    if (MODE == 2 || MODE == 3 || A.ds_thr || A.cum || A.w || A.strat) {
+    if (A.ds_thr || A.cum || A.w) {
         LNE_TRY(allow_dynamic_smem(walk_emit_kernel<KeyT, MODE, true>));
         walk_emit_kernel<KeyT, MODE, true><<<grid, kWalkThreads, smem, st>>>(A, a_begin, a_end, tile_arcs, tile_off,
                                                                             keys, u1, v1, bucket_cnt, nb_smem);
-    } else if constexpr (MODE != 2 && MODE != 3) {
+    } else {
         LNE_TRY(allow_dynamic_smem(walk_emit_kernel<KeyT, MODE, false>));
         walk_emit_kernel<KeyT, MODE, false><<<grid, kWalkThreads, smem, st>>>(A, a_begin, a_end, tile_arcs, tile_off,
                                                                              keys, u1, v1, bucket_cnt, nb_smem);
     }
+    LNE_LAUNCH_CHECK();
+    return 0;
+}
+
+template <WalkOut OUT>
+int launch_walk_batch(const WalkArgs &A, int tile_arcs, const int64_t *tile_off, uint64_t *keys, uint32_t *arcs,
+                      uint32_t *cnt, uint32_t ld, cudaStream_t st) {
+    walk_batch_kernel<OUT><<<(unsigned)ceil_div(A.n_arcs, tile_arcs), kTabThreads, walk_smem_bytes(tile_arcs, 0), st>>>(
+        A, tile_arcs, tile_off, keys, arcs, cnt, ld);
     LNE_LAUNCH_CHECK();
     return 0;
 }
@@ -2467,7 +2550,7 @@ struct SortRaw {
 int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *R, cudaStream_t st) {
     if (2 * sp.B > 64) return fail(LNE_ERR_UNSUPPORTED, "pair keys need 2 ceil(log2 n) <= 64 bits");
     WalkArgs A = make_walk_args(g, sp);
-    const bool lean = !(sp.ds_C > 0.0) && !A.w && !A.strat;   // walk_keys_kernel takes it
+    const bool lean = !(sp.ds_C > 0.0) && !A.w && !A.strat;   // walk_batch_kernel<kKeysRec or kKeysNbr>
     LNE_TRY(attach_vinfo(ws, g, &A, st, !lean || g.nnz <= kRecordArcs));
     LNE_TRY(attach_downsample(ws, g, sp, &A, st));
     const bool ds = A.ds_thr != nullptr;
@@ -2476,8 +2559,7 @@ int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *
     if (ds && g.nnz > (int64_t)UINT32_MAX)
         return fail(LNE_ERR_UNSUPPORTED, "edge downsampling on the sort path needs fewer than 2^32 arcs");
     const double rate = (double)sp.base + 0.5;
-    const int tile_arcs = lean ? (int)std::min<double>(kKeyMaxTileArcs, std::max(1.0, kKeyTileSamples / rate))
-                               : choose_tile_arcs(g.nnz, rate);
+    const int tile_arcs = choose_tile_arcs(g.nnz, rate);
     int64_t *tile_off = nullptr;
     int64_t total = 0;
     LNE_TRY(tile_offsets(ws, A, 0, g.nnz, tile_arcs, &tile_off, &total, st));
@@ -2490,20 +2572,11 @@ int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *
         LNE_TRY(ws.get("sort.a0", (size_t)std::max<int64_t>(total, 1), &arc0));
         LNE_TRY(ws.get("sort.a1", (size_t)std::max<int64_t>(total, 1), &arc1));
     }
-    const int64_t ntiles = ceil_div(g.nnz, tile_arcs);
-    const int smem = walk_smem_bytes(tile_arcs, 0);
     {
         LNE_TRACE("walk_keys", st);
-        if (lean) {
-            if (A.arcrec)
-                walk_keys_kernel<true><<<(unsigned)ntiles, kTabThreads, smem, st>>>(A, tile_arcs, tile_off, k0);
-            else
-                walk_keys_kernel<false><<<(unsigned)ntiles, kTabThreads, smem, st>>>(A, tile_arcs, tile_off, k0);
-            LNE_LAUNCH_CHECK();
-        } else {
-            LNE_TRY((launch_walk_emit<uint64_t, 3>(A, (unsigned)ntiles, smem, st, 0, g.nnz, tile_arcs, tile_off, k0,
-                                                  reinterpret_cast<int32_t *>(arc0), nullptr, nullptr, 0)));
-        }
+        if (!lean) LNE_TRY(launch_walk_batch<kKeysGen>(A, tile_arcs, tile_off, k0, arc0, nullptr, 0, st));
+        else if (A.arcrec) LNE_TRY(launch_walk_batch<kKeysRec>(A, tile_arcs, tile_off, k0, nullptr, nullptr, 0, st));
+        else LNE_TRY(launch_walk_batch<kKeysNbr>(A, tile_arcs, tile_off, k0, nullptr, nullptr, 0, st));
     }
     bool in_alt = false;
     LNE_TRY(radix_sort_u64(ws, k0, k1, arc0, arc1, total, 0, bits, &in_alt, st));
@@ -2713,8 +2786,6 @@ int sample_table(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Table
     LNE_TRY(attach_vinfo(ws, g, &A, st));
     LNE_TRY(attach_downsample(ws, g, sp, &A, st));
     const int tile_arcs = choose_tile_arcs(g.nnz, (double)sp.base + 0.5);
-    const int64_t ntiles = ceil_div(g.nnz, tile_arcs);
-    const int smem = walk_smem_bytes(tile_arcs, 0);
     if (plain) {
         // tiles of at most kTabMaxTileArcs arcs, whose walk records sit in shared memory
         const int tab_arcs = choose_tile_arcs(g.nnz, (double)sp.base + 0.5, 32768.0, kTabMaxTileArcs);
@@ -2747,11 +2818,9 @@ int sample_table(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Table
     if (A.ds_thr) {   // downsampled: 64-bit weight sums
         LNE_TRY(ws.get("table.W", (size_t)(ld * ld), &tb->W));
         LNE_CUDA_TRY(cudaMemsetAsync(tb->W, 0, sizeof(uint64_t) * (size_t)(ld * ld), st));
-        LNE_TRY((launch_walk_emit<uint64_t, 2>(A, (unsigned)ntiles, smem, st, 0, g.nnz, tile_arcs, nullptr, tb->W,
-                                              nullptr, nullptr, nullptr, (int)ld)));
+        LNE_TRY(launch_walk_batch<kWeightsGen>(A, tile_arcs, nullptr, tb->W, nullptr, nullptr, (uint32_t)ld, st));
     } else {
-        LNE_TRY((launch_walk_emit<uint32_t, 2>(A, (unsigned)ntiles, smem, st, 0, g.nnz, tile_arcs, nullptr, tb->T,
-                                              nullptr, nullptr, nullptr, (int)ld)));
+        LNE_TRY(launch_walk_batch<kCountsGen>(A, tile_arcs, nullptr, nullptr, nullptr, tb->T, (uint32_t)ld, st));
     }
     return 0;
 }
@@ -2982,11 +3051,9 @@ int strat_keys(Workspace &ws, const GraphView &g, const SamplerSpec &sp, int64_t
     uint64_t *k0 = nullptr, *k1 = nullptr;
     LNE_TRY(ws.get("sort.k0", (size_t)std::max<int64_t>(total, 1), &k0));
     LNE_TRY(ws.get("sort.k1", (size_t)std::max<int64_t>(total, 1), &k1));
-    const int64_t ntiles = ceil_div(g.nnz, tile_arcs);
     {
         LNE_TRACE("walk_keys", st);
-        LNE_TRY((launch_walk_emit<uint64_t, 3>(A, (unsigned)ntiles, walk_smem_bytes(tile_arcs, 0), st, 0, g.nnz,
-                                              tile_arcs, tile_off, k0, nullptr, nullptr, nullptr, 0)));
+        LNE_TRY(launch_walk_batch<kKeysGen>(A, tile_arcs, tile_off, k0, nullptr, nullptr, 0, st));
     }
     bool in_alt = false;
     LNE_TRY(radix_sort_u64(ws, k0, k1, nullptr, nullptr, total, 0, 2 * su.B + 4, &in_alt, st));
