@@ -142,9 +142,22 @@ void trace_end(cudaStream_t st) {
     r.closed = true;
 }
 
+// Bytes of all workspaces' retired buffers.
+static std::atomic<int64_t> g_idle_bytes{0};
+
+void Workspace::free_buf(Buf &b) {
+    if (b.idle) g_idle_bytes -= (int64_t)b.bytes;
+    if (b.p) cudaFree(b.p);
+    b = Buf();
+}
+
 int Workspace::get(const std::string &name, size_t bytes, void **ptr) {
     if (bytes == 0) bytes = 1;
     Buf &b = bufs_[name];
+    if (b.idle) {
+        g_idle_bytes -= (int64_t)b.bytes;
+        b.idle = false;
+    }
     if (b.bytes < bytes) {
         if (b.p) {
             cudaError_t e = cudaFree(b.p);
@@ -156,6 +169,16 @@ int Workspace::get(const std::string &name, size_t bytes, void **ptr) {
         size_t want = bytes + std::min(bytes / 8, (size_t)1 << 28);
         want = (want + 255) & ~(size_t)255;
         cudaError_t e = cudaMalloc(&b.p, want);
+        if (e == cudaErrorMemoryAllocation) {   // once more without the retired buffers
+            cudaGetLastError();
+            bool freed = false;
+            for (auto &kv : bufs_) {
+                if (!kv.second.idle) continue;
+                free_buf(kv.second);
+                freed = true;
+            }
+            if (freed) e = cudaMalloc(&b.p, want);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             b.p = nullptr;
@@ -172,16 +195,32 @@ int Workspace::get(const std::string &name, size_t bytes, void **ptr) {
 }
 
 void Workspace::release() {
-    for (auto &kv : bufs_)
-        if (kv.second.p) cudaFree(kv.second.p);
+    for (auto &kv : bufs_) free_buf(kv.second);
     bufs_.clear();
 }
 
 void Workspace::release(const std::string &name) {
     auto it = bufs_.find(name);
     if (it == bufs_.end()) return;
-    if (it->second.p) cudaFree(it->second.p);
+    free_buf(it->second);
     bufs_.erase(it);
+}
+
+void Workspace::retire(const std::string &name) {
+    static const int64_t kKeep = [] {
+        int dev = 0;
+        cudaDeviceProp prop;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return (int64_t)0;
+        return (int64_t)(prop.totalGlobalMem / 8);
+    }();
+    auto it = bufs_.find(name);
+    if (it == bufs_.end() || it->second.idle) return;
+    if ((g_idle_bytes += (int64_t)it->second.bytes) > kKeep) {
+        g_idle_bytes -= (int64_t)it->second.bytes;
+        release(name);
+    } else {
+        it->second.idle = true;
+    }
 }
 
 int64_t Workspace::bytes() const {

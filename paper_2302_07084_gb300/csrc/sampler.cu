@@ -2534,7 +2534,7 @@ struct Table {
 
 // Samples of every arc as 64-bit keys, sorted, as unique keys with counts.
 // On return the unique keys are in *uk ("sort.k0" or "sort.k1"), counts in
-// "sort.cnt"; the other key buffer and the run starts are released. With edge
+// "sort.cnt"; the other key buffer is retired. With edge
 // downsampling each key carries its arc, a dropped draw's key is all ones
 // (sorted past every pair: the sort takes one more bit when n = 2^B, where the
 // all-ones pair of B-bit halves is a real vertex pair), and *w gets the summed
@@ -2581,15 +2581,15 @@ int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *
     bool in_alt = false;
     LNE_TRY(radix_sort_u64(ws, k0, k1, arc0, arc1, total, 0, bits, &in_alt, st));
     uint64_t *sorted = in_alt ? k1 : k0, *spare = in_alt ? k0 : k1;
-    ws.release("sort.words");
+    ws.retire("sort.words");
     if (ds) {
         // the dropped draws sort last: run lengths over the kept ones only
         int64_t kept = 0;
         LNE_TRY(count_below(ws, sorted, total, ~0ull, &kept, st));
         LNE_TRY(ws.get("sort.w", (size_t)std::max<int64_t>(kept, 1), &R->w));
         LNE_TRY(run_length_weighted(ws, sorted, in_alt ? arc1 : arc0, A.ds_w, kept, spare, R->w, &R->U, st));
-        ws.release("sort.a0");
-        ws.release("sort.a1");
+        ws.retire("sort.a0");
+        ws.retire("sort.a1");
         LNE_TRY(ws.get("sort.cnt", (size_t)std::max<int64_t>(R->U, 1), &R->cnt));
     } else {
         LNE_TRY(ws.get("sort.cnt", (size_t)std::max<int64_t>(total, 1), &R->cnt));
@@ -2599,7 +2599,7 @@ int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *
     R->uk = spare;
     R->uk_name = in_alt ? "sort.k0" : "sort.k1";
     R->spare_name = in_alt ? "sort.k1" : "sort.k0";
-    ws.release(R->spare_name);
+    ws.retire(R->spare_name);
     return 0;
 }
 
@@ -2608,7 +2608,7 @@ void sort_release(Workspace &ws) {
                           "sort.mk", "sort.mv",
                           "path.dcol", "path.dval", "path.tk", "path.tm", "path.ko", "path.mo", "path.deg",
                           "path.dend", "path.rowlen", "path.dstart", "path.first", "path.end"})
-        ws.release(n);
+        ws.retire(n);
 }
 
 int sort_counts(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CountsResult *out, cudaStream_t st) {
@@ -2639,7 +2639,7 @@ int sort_counts(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Counts
 // Symmetric CSR from U ascending unique pair keys uk and their Eq. 1 value
 // bits val (0 = dropped), with per-tile (kPathTile) kept / kept off-diagonal
 // counts tk / tm. uk and val (workspace buffers uk_name / val_name) serve as
-// spare buffers of the mirrored sort and are released.
+// spare buffers of the mirrored sort and are retired.
 int assemble_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, uint64_t *uk, uint32_t *val, int64_t U,
                  const uint32_t *tk, const uint32_t *tm, const char *uk_name, const char *val_name, CsrResult *out,
                  cudaStream_t st) {
@@ -2701,11 +2701,11 @@ int assemble_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, uint6
     LNE_CUDA_TRY(cudaStreamSynchronize(st));
     // the buffers not holding the sorted mirrored entries are free now
     if (in_alt) {
-        ws.release("sort.mk");
-        ws.release("sort.mv");
+        ws.retire("sort.mk");
+        ws.retire("sort.mv");
     } else {
-        ws.release(uk_name);
-        ws.release(val_name);
+        ws.retire(uk_name);
+        ws.retire(val_name);
     }
     LNE_TRY(ws.get("csr.indices", (size_t)std::max<int64_t>(nnz, 1), &out->indices));
     LNE_TRY(ws.get("csr.data", (size_t)std::max<int64_t>(nnz, 1), &out->data));
@@ -2722,18 +2722,18 @@ int assemble_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, uint6
     }
     LNE_CUDA_TRY(cudaStreamSynchronize(st));
     sort_release(ws);
-    ws.release(uk_name);
-    ws.release(val_name);
+    ws.retire(uk_name);
+    ws.retire(val_name);
     out->n = n;
     out->nnz = nnz;
     return 0;
 }
 
 int sort_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CsrResult *out, cudaStream_t st) {
-    // a previous sparsifier's arrays are rebuilt below: free them before the
+    // a previous sparsifier's arrays are rebuilt below: retire them before the
     // sort's peak (tens of GB for billions of samples)
-    ws.release("csr.indices");
-    ws.release("csr.data");
+    ws.retire("csr.indices");
+    ws.retire("csr.data");
     SortRaw R;
     LNE_TRY(sort_raw(ws, g, sp, &R, st));
     const int64_t U = R.U, n = g.n;
@@ -3058,7 +3058,7 @@ int strat_keys(Workspace &ws, const GraphView &g, const SamplerSpec &sp, int64_t
     bool in_alt = false;
     LNE_TRY(radix_sort_u64(ws, k0, k1, nullptr, nullptr, total, 0, 2 * su.B + 4, &in_alt, st));
     uint64_t *sorted = in_alt ? k1 : k0, *other = in_alt ? k0 : k1;
-    ws.release("sort.words");
+    ws.retire("sort.words");
     LNE_TRY(ws.get("sort.cnt", (size_t)std::max<int64_t>(total, 1), cnt));
     LNE_TRY(run_length(ws, sorted, total, other, *cnt, U, st));
     *total_out = total;
@@ -3153,7 +3153,7 @@ int stratified_sample(Workspace &ws, const GraphView &g, const SamplerSpec &sp, 
     LNE_TRY(scan_exclusive_u32_to_i64(seglen, seg, P, st));
     LNE_CUDA_TRY(cudaStreamSynchronize(st));
     for (const char *nm : {"sort.k0", "sort.k1", "sort.cnt", "strat.seglen", "rle.cnt", "rle.off"})
-        ws.release(nm);
+        ws.retire(nm);
     out->total = total;
     out->U = U;
     out->P = P;
@@ -3175,8 +3175,8 @@ int stratified_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, con
                    cudaStream_t st) {
     if (S.T != sp.T || S.B != sp.B || S.g_n != g.n || S.g_nnz != g.nnz)
         return fail(LNE_ERR_INVALID, "strata belong to another graph or window size");
-    ws.release("csr.indices");
-    ws.release("csr.data");
+    ws.retire("csr.indices");
+    ws.retire("csr.data");
     StratW w = {};
     for (int r = 0; r < sp.T; ++r) w.w[r] = strat_weight(sp, r);
     const int64_t P = S.P, n = g.n;
@@ -3207,7 +3207,7 @@ int stratified_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, con
 void stratified_release(Workspace &ws) {
     for (const char *nm : {"strat.r", "strat.cnt", "strat.pair", "strat.seglen", "strat.seg", "strat.cuk",
                            "strat.cval"})
-        ws.release(nm);
+        ws.retire(nm);
 }
 
 namespace {

@@ -100,3 +100,23 @@ def test_downsampled_sums_equal_the_table(ctx, n, rate, C):
     table.close()
     for k in ("indptr", "indices", "data"):
         assert np.array_equal(a[k], b[k]), k
+
+
+def test_kept_buffers_serve_every_size(ctx):
+    """Calls of changing sizes and kinds in one context equal those of fresh ones."""
+    gs = [synth.ring(3000), synth.chung_lu(2000, 12000, 2.1, seed=4, n_labels=5), synth.ring(50)]
+    ps = [make_params(5, np.full(5, 0.2), r * g.n_arcs, seed=2) for g, r in zip(gs, (9.0, 6.0, 300.0))]
+    def run(c, i, C):
+        ps[i].downsample_C = C
+        return {k: to_np(v).copy() for k, v in c.sparsifier_csr(lne.DeviceGraph.from_graph(gs[i]), ps[i]).items()
+                if torch.is_tensor(v)}
+    for i, C in [(0, 0.0), (2, 0.0), (1, 0.0), (1, 2.0), (0, 2.0), (0, 0.0), (2, 0.0)]:
+        fresh = lne.Context(0)
+        fresh.set_option(lne.OPT_AGGREGATION, lne.AGG_SORT)
+        a, b = run(ctx, i, C), run(fresh, i, C)
+        fresh.close()
+        for k in a:
+            assert np.array_equal(a[k], b[k]), (i, C, k)
+    before = ctx.workspace_bytes()
+    run(ctx, 1, 0.0)
+    assert ctx.workspace_bytes() == before   # nothing new for a size it has served
