@@ -204,13 +204,9 @@ __device__ __forceinline__ void gather4(const int32_t *__restrict__ indices, con
 // column group q. The groups' partial sums are combined by a fixed xor tree at
 // the end of each row segment, so the result is deterministic.
 template <int LG, bool WEIGHTED, typename TX>
-__device__ __forceinline__ void gather4_grouped(const int32_t *__restrict__ indices, const float *__restrict__ vals,
-                                                int64_t p, int cnt, const TX *__restrict__ X, int64_t ldx, int c4,
-                                                int lane, float4 &acc) {
+__device__ __forceinline__ void gather4_grouped(int col, float v, int cnt, const TX *__restrict__ X, int64_t ldx,
+                                                int c4, int lane, float4 &acc) {
     constexpr int G = 32 / LG;
-    const int col = lane < cnt ? __ldg(indices + p + lane) : 0;
-    float v = 0.f;
-    if (WEIGHTED) v = lane < cnt ? __ldg(vals + p + lane) : 0.f;
     const int g = lane / LG, q = lane % LG;
 #pragma unroll 4
     for (int k0 = 0; k0 < cnt; k0 += G) {
@@ -344,8 +340,17 @@ __global__ void __launch_bounds__(256) spmm_merge_kernel(int64_t n, int64_t nnz,
 #pragma unroll
         for (int t = 0; t < NV; ++t) acc.v[t] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (LG < 32) {
-            for (int64_t q = p; q < e; q += 32)
-                gather4_grouped<LG, WEIGHTED, TX>(ind, val, q, (int)imin64(32, e - q), X, ldx, c4, lane, acc.v[0]);
+            // the next 32 nonzeros are on their way while these rows of X are gathered
+            int col = p + lane < e ? __ldg(ind + p + lane) : 0;
+            float v = WEIGHTED && p + lane < e ? __ldg(val + p + lane) : 0.f;
+            for (int64_t q = p; q < e; q += 32) {
+                const bool more = q + 32 + lane < e;
+                const int col1 = more ? __ldg(ind + q + 32 + lane) : 0;
+                const float v1 = WEIGHTED && more ? __ldg(val + q + 32 + lane) : 0.f;
+                gather4_grouped<LG, WEIGHTED, TX>(col, v, (int)imin64(32, e - q), X, ldx, c4, lane, acc.v[0]);
+                col = col1;
+                v = v1;
+            }
 #pragma unroll
             for (int off = LG; off < 32; off <<= 1) {
                 acc.v[0].x += __shfl_xor_sync(0xffffffffu, acc.v[0].x, off);
@@ -728,8 +733,12 @@ int launch_merge(Workspace &ws, int64_t n, int64_t nnz, const int64_t *indptr, c
     }
     // weighted products with at most 16 float4 column groups: several nonzeros
     // per warp step (the graph products keep one, so batched propagation sums
-    // in the same order as a single candidate's)
-    if (WEIGHTED && c4 <= 8) LNE_MERGE_GROUPED(8)
+    // in the same order as a single candidate's). Up to 16 columns eight of them:
+    // 1.9e8 nonzeros, 16 columns 2.56 ms with four (half the lanes idle), 1.74 with
+    // eight, 1.61 with the next indices loaded ahead; 64 bytes of X a nonzero from
+    // L2 bound it
+    if (WEIGHTED && c4 <= 4) LNE_MERGE_GROUPED(4)
+    else if (WEIGHTED && c4 <= 8) LNE_MERGE_GROUPED(8)
     else if (WEIGHTED && c4 <= 16) LNE_MERGE_GROUPED(16)
     else switch (nv) {
         LNE_MERGE_CASE(1)
