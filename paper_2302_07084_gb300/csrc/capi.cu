@@ -784,7 +784,12 @@ int lne_embed(lne_ctx *ctx, const lne_graph *g, const lne_params *p, float *X_de
     sp.ds_C = p->downsample_C;
     sp.stratified = ctx->stratified;
     lne::CsrResult M;
-    if (rc == 0) rc = lne::sparsifier_csr(ctx->ws, gv, sp, &M, st);
+    lne::ProductWant want;
+    if (lne::table_products(p->precision, sketch_of(p))) {
+        want.dense_mode = ctx->dense_mode;
+        want.c = p->d + oversample_of(p);
+    }
+    if (rc == 0) rc = lne::sparsifier_csr(ctx->ws, gv, sp, &M, st, want);
     float *X0 = nullptr;
     if (rc == 0) rc = ctx->ws.get("embed.x0", (size_t)g->n * p->d, &X0);
     if (rc == 0) {

@@ -1479,17 +1479,42 @@ __device__ __forceinline__ float netmf_value_w(uint64_t wsum, int64_t dx, int64_
     return netmf_value_fixed(wsum, 2.3283064e-10f, 2.3283064365386963e-10, dx, dy, diag, k);   // 2^-32
 }
 
+// The value passes also count the entries of the symmetric matrix that they keep
+// (a pair off the diagonal twice): the host decides by the total whether the
+// products take the table or a CSR. Spread over kNnzSlots counters.
+constexpr int kNnzSlots = 64;
+__device__ __forceinline__ void add_kept(unsigned kept, unsigned long long *__restrict__ nnz) {
+    __shared__ unsigned s_kept;
+    if (threadIdx.x == 0) s_kept = 0;
+    __syncthreads();
+    kept = __reduce_add_sync(0xffffffffu, kept);
+    if ((threadIdx.x & 31) == 0 && kept) atomicAdd(&s_kept, kept);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_kept) atomicAdd(nnz + blockIdx.x % kNnzSlots, (unsigned long long)s_kept);
+}
+
 // Weighted table -> the float-bits value table (upper triangle).
-__global__ void table_values_w_kernel(const uint64_t *__restrict__ W, uint32_t *__restrict__ T, int64_t ld, int n,
-                                      const int64_t *__restrict__ indptr, NetmfConst kc) {
+__global__ void __launch_bounds__(256) table_values_w_kernel(const uint64_t *__restrict__ W, uint32_t *__restrict__ T,
+                                                             int64_t ld, int n, const int64_t *__restrict__ indptr,
+                                                             NetmfConst kc, unsigned long long *__restrict__ nnz) {
+    constexpr int kAhead = 4;   // loads in flight a thread
     const int x = blockIdx.x;
     const int64_t dx = eq1_degree(kc, indptr, x);
-    for (int y = x + threadIdx.x; y < n; y += blockDim.x) {
-        const uint64_t w = W[(size_t)x * ld + y];
-        if (w == 0) continue;
-        const int64_t dy = eq1_degree(kc, indptr, y);
-        T[(size_t)x * ld + y] = __float_as_uint(netmf_value_w(w, dx, dy, x == y, kc));
+    unsigned kept = 0;
+    for (int y0 = x + threadIdx.x; y0 < n; y0 += kAhead * 256) {
+        uint64_t w[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) w[u] = y0 + 256 * u < n ? __ldcs(W + (size_t)x * ld + y0 + 256 * u) : 0ull;
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            if (w[u] == 0) continue;
+            const int y = y0 + 256 * u;
+            const float v = netmf_value_w(w[u], dx, eq1_degree(kc, indptr, y), x == y, kc);
+            T[(size_t)x * ld + y] = __float_as_uint(v);
+            if (__float_as_uint(v) != 0u) kept += x == y ? 1u : 2u;
+        }
     }
+    add_kept(kept, nnz);
 }
 
 // Per arc u -> v: the coin threshold min(2^32, floor(p 2^32)) and the weight
@@ -1616,8 +1641,9 @@ constexpr int kTile = 64;
 
 // Counts -> Eq. 1 values in place (float bits; 0 = not kept). One CTA per row
 // x of the upper triangle (y >= x).
-__global__ void table_values_kernel(uint32_t *__restrict__ T, int64_t ld, int n,
-                                    const int64_t *__restrict__ indptr, NetmfConst kc) {
+__global__ void table_values_kernel(uint32_t *__restrict__ T, int64_t ld, int n, const int64_t *__restrict__ indptr,
+                                    NetmfConst kc, unsigned long long *__restrict__ nnz) {
+    unsigned kept = 0;
     const int x = blockIdx.x;
     const int64_t dx = eq1_degree(kc, indptr, x);
     uint32_t *row = T + (size_t)x * ld;
@@ -1625,8 +1651,11 @@ __global__ void table_values_kernel(uint32_t *__restrict__ T, int64_t ld, int n,
         const uint32_t c = row[y];
         if (c == 0) continue;
         const int64_t dy = eq1_degree(kc, indptr, y);
-        row[y] = __float_as_uint(netmf_value(c, dx, dy, x == y, kc));
+        const float v = netmf_value(c, dx, dy, x == y, kc);
+        row[y] = __float_as_uint(v);
+        if (__float_as_uint(v) != 0u) kept += x == y ? 1u : 2u;
     }
+    add_kept(kept, nnz);
 }
 
 // table_decode_kernel and table_values_kernel in one pass, for the CSR: the
@@ -1634,35 +1663,55 @@ __global__ void table_values_kernel(uint32_t *__restrict__ T, int64_t ld, int n,
 // records (see table_decode_kernel), then its Eq. 1 value written as float
 // bits in place of the wrap record (which is 0 where nothing was counted).
 template <int BITS>
-__global__ void table_decode_values_kernel(const uint32_t *__restrict__ tp, uint32_t *__restrict__ T, int64_t ld,
-                                           int n, const int64_t *__restrict__ indptr, NetmfConst kc) {
+__global__ void __launch_bounds__(256) table_decode_values_kernel(const uint32_t *__restrict__ tp,
+                                                                  uint32_t *__restrict__ T, int64_t ld, int n,
+                                                                  const int64_t *__restrict__ indptr, NetmfConst kc,
+                                                                  unsigned long long *__restrict__ nnz) {
     constexpr int P = TabPack<BITS>::P;
     constexpr uint32_t mask = TabPack<BITS>::mask;
+    static_assert(P == 4, "a word's counters are one 16-byte group of the table");
     const int x = blockIdx.x;
     const int64_t dx = eq1_degree(kc, indptr, x);
     const int64_t k0 = ((int64_t)x * ld + x) / P, k1 = ((int64_t)x * ld + ld) / P;
-    for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
-        const uint32_t w = tp[k];
-        uint32_t wr[P];
+    uint4 *T4 = reinterpret_cast<uint4 *>(T);
+    unsigned kept = 0;
+    constexpr int kAhead = 2;   // words in flight a thread
+    for (int64_t kb = k0 + threadIdx.x; kb < k1; kb += kAhead * 256) {
+        uint32_t w[kAhead];
+        uint4 r[kAhead];
 #pragma unroll
-        for (int i = 0; i < P; ++i) wr[i] = T[P * k + i];
-        uint32_t prev = 0;
+        for (int u = 0; u < kAhead; ++u) {
+            const bool in = kb + 256 * u < k1;
+            w[u] = in ? __ldcs(tp + kb + 256 * u) : 0u;
+            r[u] = in ? T4[kb + 256 * u] : make_uint4(0u, 0u, 0u, 0u);
+        }
 #pragma unroll
-        for (int i = 0; i < P; ++i) {
-            const uint32_t cnt = ((w >> (BITS * i)) & mask) + (wr[i] << BITS) - prev;
-            prev = wr[i];
-            const int64_t y = P * k + i - (int64_t)x * ld;
-            // left of the diagonal, padding, or nothing counted: value 0. The
-            // record is 0 there unless the field took the carries of a
-            // neighbour that wrapped 2^BITS times and wrapped itself (a
-            // neighbour past 2^16 counts): clear it
-            if (y < x || y >= n || cnt == 0) {
-                if (wr[i] != 0u) T[P * k + i] = 0u;
-                continue;
+        for (int u = 0; u < kAhead; ++u) {
+            const int64_t k = kb + 256 * u;
+            const uint32_t wr[P] = {r[u].x, r[u].y, r[u].z, r[u].w};
+            if ((w[u] | wr[0] | wr[1] | wr[2] | wr[3]) == 0u) continue;   // nothing counted, nothing to clear
+            uint32_t out[P];
+            uint32_t prev = 0;
+#pragma unroll
+            for (int i = 0; i < P; ++i) {
+                const uint32_t cnt = ((w[u] >> (BITS * i)) & mask) + (wr[i] << BITS) - prev;
+                prev = wr[i];
+                const int64_t y = P * k + i - (int64_t)x * ld;
+                // left of the diagonal, padding, or nothing counted: value 0. The
+                // record is 0 there unless the field took the carries of a
+                // neighbour that wrapped 2^BITS times and wrapped itself (a
+                // neighbour past 2^16 counts): cleared
+                out[i] = 0u;
+                if (y >= x && y < n && cnt != 0u) {
+                    const float v = netmf_value(cnt, dx, eq1_degree(kc, indptr, y), x == y, kc);
+                    out[i] = __float_as_uint(v);
+                    if (__float_as_uint(v) != 0u) kept += x == y ? 1u : 2u;
+                }
             }
-            T[P * k + i] = __float_as_uint(netmf_value(cnt, dx, eq1_degree(kc, indptr, y), x == y, kc));
+            T4[k] = make_uint4(out[0], out[1], out[2], out[3]);
         }
     }
+    add_kept(kept, nnz);
 }
 
 // table_decode_values_kernel for sparse tables: a warp decodes 32
@@ -1677,7 +1726,8 @@ template <int BITS>
 __global__ void __launch_bounds__(kDvThreads) table_decode_values_sparse_kernel(const uint32_t *__restrict__ tp,
                                                                         uint32_t *__restrict__ T, int64_t ld, int n,
                                                                         const int64_t *__restrict__ indptr,
-                                                                        NetmfConst kc) {
+                                                                        NetmfConst kc,
+                                                                        unsigned long long *__restrict__ nnz) {
     constexpr int P = TabPack<BITS>::P;
     constexpr uint32_t mask = TabPack<BITS>::mask;
     static_assert(P * 32 + 31 <= kDvQueue, "queue holds a chunk's counters and the leftovers");
@@ -1688,12 +1738,15 @@ __global__ void __launch_bounds__(kDvThreads) table_decode_values_sparse_kernel(
     const int64_t k0 = ((int64_t)x * ld + x) / P, k1 = ((int64_t)x * ld + ld) / P;
     uint32_t *qi = s_qi[warp], *qc = s_qc[warp];
     int qn = 0;   // queued entries (the same in every lane)
+    unsigned kept = 0;
     // values of queued entries [q0, q0 + cnt), cnt <= 32, one per lane
     auto values = [&](int q0, int cnt) {
         if (lane < cnt) {
             const uint32_t idx = qi[q0 + lane], c = qc[q0 + lane];
             const int64_t y = (int64_t)idx - (int64_t)x * ld;
-            T[idx] = __float_as_uint(netmf_value(c, dx, eq1_degree(kc, indptr, y), x == y, kc));
+            const float v = netmf_value(c, dx, eq1_degree(kc, indptr, y), x == y, kc);
+            T[idx] = __float_as_uint(v);
+            if (__float_as_uint(v) != 0u) kept += x == y ? 1u : 2u;
         }
     };
     const unsigned lt = (1u << lane) - 1u;
@@ -1732,6 +1785,7 @@ __global__ void __launch_bounds__(kDvThreads) table_decode_values_sparse_kernel(
         }
     }
     values(0, qn);
+    add_kept(kept, nnz);
 }
 
 // Distinct pairs per upper-triangle row (for the counts output).
@@ -2869,7 +2923,8 @@ int table_counts(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Count
     return 0;
 }
 
-int table_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CsrResult *out, cudaStream_t st) {
+int table_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CsrResult *out, cudaStream_t st,
+              const ProductWant &want) {
     Table tb;
     LNE_TRY(sample_table(ws, g, sp, &tb, st, false));
     const int n = (int)g.n;
@@ -2878,18 +2933,32 @@ int table_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CsrResul
     // 39k-vertex graph, 0.18 -> 0.21 ms at 41% on the benchmark's)
     const double samples = (double)g.nnz * ((double)sp.base + (double)sp.thr_frac / 4294967296.0);
     const bool sparse = 2.0 * samples < 0.15 * (double)n * (double)n;
+    unsigned long long *kept = nullptr;
+    LNE_TRY(ws.get("table.kept", kNnzSlots, &kept));
+    LNE_CUDA_TRY(cudaMemsetAsync(kept, 0, sizeof(unsigned long long) * kNnzSlots, st));
     {
         LNE_TRACE("table_values", st);
-        if (tb.W) table_values_w_kernel<<<(unsigned)n, 256, 0, st>>>(tb.W, tb.T, tb.ld, n, g.indptr, netmf_const(sp));
+        if (tb.W) table_values_w_kernel<<<(unsigned)n, 256, 0, st>>>(tb.W, tb.T, tb.ld, n, g.indptr, netmf_const(sp),
+                                                                        kept);
         else if (tb.packed && sparse)
             table_decode_values_sparse_kernel<kTabBits><<<(unsigned)n, kDvThreads, 0, st>>>(
-                tb.packed, tb.T, tb.ld, n, g.indptr, netmf_const(sp));
+                tb.packed, tb.T, tb.ld, n, g.indptr, netmf_const(sp), kept);
         else if (tb.packed)
             table_decode_values_kernel<kTabBits><<<(unsigned)n, 256, 0, st>>>(tb.packed, tb.T, tb.ld, n, g.indptr,
-                                                                             netmf_const(sp));
-        else table_values_kernel<<<(unsigned)n, 256, 0, st>>>(tb.T, tb.ld, n, g.indptr, netmf_const(sp));
+                                                                             netmf_const(sp), kept);
+        else table_values_kernel<<<(unsigned)n, 256, 0, st>>>(tb.T, tb.ld, n, g.indptr, netmf_const(sp), kept);
         LNE_LAUNCH_CHECK();
     }
+    unsigned long long slots[kNnzSlots];
+    LNE_CUDA_TRY(cudaMemcpyAsync(slots, kept, sizeof(slots), cudaMemcpyDeviceToHost, st));
+    LNE_CUDA_TRY(cudaStreamSynchronize(st));
+    int64_t nnz = 0;
+    for (unsigned long long s : slots) nnz += (int64_t)s;
+    out->n = g.n;
+    out->nnz = nnz;
+    out->dense = reinterpret_cast<const float *>(tb.T);
+    out->dense_ld = tb.ld;
+    if (want.c > 0 && product_view(*out, want.dense_mode, want.c).dense) return 0;
     uint32_t *rowtile = nullptr, *rowcnt = nullptr;
     LNE_TRY(ws.get("table.rowtile", (size_t)n * tb.nt, &rowtile));
     LNE_TRY(ws.get("table.rowcnt", (size_t)n, &rowcnt));
@@ -2906,9 +2975,6 @@ int table_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CsrResul
         LNE_LAUNCH_CHECK();
     }
     LNE_TRY(scan_exclusive_u32_to_i64(rowcnt, out->indptr, n, st));
-    int64_t nnz = 0;
-    LNE_CUDA_TRY(cudaMemcpyAsync(&nnz, out->indptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    LNE_CUDA_TRY(cudaStreamSynchronize(st));
     LNE_TRY(ws.get("csr.indices", (size_t)std::max<int64_t>(nnz, 1), &out->indices));
     LNE_TRY(ws.get("csr.data", (size_t)std::max<int64_t>(nnz, 1), &out->data));
     {
@@ -2916,10 +2982,6 @@ int table_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CsrResul
         tile_fill_kernel<<<grid, 256, 0, st>>>(tb.T, tb.ld, n, tb.nt, rowtile, out->indptr, out->indices, out->data);
         LNE_LAUNCH_CHECK();
     }
-    out->n = g.n;
-    out->nnz = nnz;
-    out->dense = reinterpret_cast<const float *>(tb.T);
-    out->dense_ld = tb.ld;
     return 0;
 }
 
@@ -3250,7 +3312,8 @@ int sparsifier_counts(Workspace &ws, const GraphView &g, const SamplerSpec &sp, 
     return 0;
 }
 
-int sparsifier_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CsrResult *out, cudaStream_t st) {
+int sparsifier_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CsrResult *out, cudaStream_t st,
+                   const ProductWant &want) {
     if (sp.stratified) {
         Strata S;
         LNE_TRY(stratified_sample(ws, g, sp, &S, st));
@@ -3260,7 +3323,7 @@ int sparsifier_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Csr
     }
     if (sp.ds_C > 0.0 && !use_table(g, sp) && sp.aggregation == LNE_AGG_BUCKET)
         return fail(LNE_ERR_UNSUPPORTED, "edge downsampling needs the table or the sort aggregation");
-    if (use_table(g, sp)) return table_csr(ws, g, sp, out, st);
+    if (use_table(g, sp)) return table_csr(ws, g, sp, out, st, want);
     if (sp.aggregation == LNE_AGG_BUCKET) return bucket_csr(ws, g, sp, out, st);
     return sort_csr(ws, g, sp, out, st);
 }

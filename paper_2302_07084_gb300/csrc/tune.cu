@@ -154,6 +154,9 @@ int tune_batch(Workspace &ws, PropBatchGraph *cache, SpmmTune &tc, int aggregati
         LNE_TRY(make_sampler_spec(g, p.T, p.s, p.samples, p.b, p.seed, &sp));
         sp.aggregation = aggregation;
         sp.ds_C = p.downsample_C;
+        SketchSpec sk;
+        sk.kind = p.sketch;
+        sk.zeta = p.sketch_zeta;
         CsrResult M;
         if (stratified) {
             if (!have_strata || strata.T != sp.T || strata.S != sp.S || strata.seed != sp.seed) {
@@ -162,11 +165,13 @@ int tune_batch(Workspace &ws, PropBatchGraph *cache, SpmmTune &tc, int aggregati
             }
             LNE_TRY(stratified_csr(ws, g, sp, strata, &M, st));
         } else {
-            LNE_TRY(sparsifier_csr(ws, g, sp, &M, st));
+            ProductWant want;
+            if (table_products(p.precision, sk)) {
+                want.dense_mode = dense_mode;
+                want.c = d + os_of(p);
+            }
+            LNE_TRY(sparsifier_csr(ws, g, sp, &M, st, want));
         }
-        SketchSpec sk;
-        sk.kind = p.sketch;
-        sk.zeta = p.sketch_zeta;
         LNE_TRY(rsvd(ws, product_view(M, dense_mode, d + os_of(p)), d, os_of(p), p.q, p.seed, p.precision, nullptr, nullptr,
                      X0s + (size_t)q * n * d, st, sk));
     }
