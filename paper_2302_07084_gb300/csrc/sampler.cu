@@ -1402,31 +1402,24 @@ struct NetmfConst {
 };
 
 // The degree of Eq. 1: weighted when the graph is, else the arc count.
-__device__ __forceinline__ int64_t eq1_degree(const NetmfConst &k, const int64_t *__restrict__ indptr, int64_t x) {
-    return k.wdeg ? (int64_t)__ldg(k.wdeg + x) : __ldg(indptr + x + 1) - __ldg(indptr + x);
+// (Below 2^32, so the offsets' low words give it.)
+__device__ __forceinline__ uint32_t eq1_degree(const NetmfConst &k, const int64_t *__restrict__ indptr, int64_t x) {
+    const uint32_t *lo = reinterpret_cast<const uint32_t *>(indptr);
+    return k.wdeg ? __ldg(k.wdeg + x) : __ldg(lo + 2 * x + 2) - __ldg(lo + 2 * x);
 }
 
 // Eq. 1 entry with the truncated log for count K of pair (x, y):
 // v = fl(fl(K alpha) / fl(d_x d_y)), kept iff v > 1, value log(v) as float32
 // (0 means dropped; log v > 0 for every kept entry).
-// Fast path: D = K alpha - q (q = d_x d_y) in FP32 with alpha split into a
-// float pair; fmaf makes the product exact, so D carries a relative error of
-// ~1e-7. Whenever |D| > 1e-5 q its sign is the FP64 decision and
-// log1p(D / q) is accurate to a few ulp. Otherwise (v within 1e-5 of 1, or
-// operands beyond 2^24) the exact FP64 rule decides: a correctly rounded
-// quotient exceeds 1 iff p >= 2q or (p > q and (p - q) 2^53 > q), with p - q
-// exact there (Sterbenz), so no division is needed.
-__device__ __forceinline__ float netmf_value(uint32_t cnt, int64_t dx, int64_t dy, bool diag,
-                                             const NetmfConst &k) {
-    const int64_t q64 = dx * dy;
-    if (cnt < (1u << 24) && q64 < (1ll << 24)) {
-        const float cf = (float)cnt, qf = (float)q64;
-        const float hi = diag ? k.diag_hi : k.off_hi, lo = diag ? k.diag_lo : k.off_lo;
-        const float dq = fmaf(cf, hi, -qf) + cf * lo;
-        if (fabsf(dq) > 1e-5f * qf) return dq > 0.f ? log1pf(__fdiv_rn(dq, qf)) : 0.f;
-    }
-    const double p = __dmul_rn((double)cnt, diag ? k.a_diag : k.a_off);
-    const double q = __ll2double_rn(q64);
+// Fast path: D = K alpha - q (q = d_x d_y) in FP32 with alpha and q split into
+// float pairs (q's low part is 0 below 2^24); fmaf makes the products exact, so D
+// carries a relative error of ~1e-7. Whenever |D| > 1e-5 q its sign is the FP64
+// decision, and log1p(D / q) is accurate to a few ulp where q is a float.
+// Otherwise (v within 1e-5 of 1, v > 1 and q beyond 2^24, or a count or degree of
+// 2^24 and more) the exact FP64 rule decides: a correctly rounded quotient exceeds
+// 1 iff p >= 2q or (p > q and (p - q) 2^53 > q), with p - q exact there
+// (Sterbenz), so no division is needed.
+__device__ __forceinline__ float netmf_value_exact(double p, double q) {
     if (!(p > q)) return 0.f;
     const double q2 = __dmul_rn(2.0, q);
     if (p < q2) {
@@ -1436,6 +1429,19 @@ __device__ __forceinline__ float netmf_value(uint32_t cnt, int64_t dx, int64_t d
     }
     if (p < 1e30) return logf(__fdiv_rn((float)p, (float)q));
     return (float)(log(p) - log(q));
+}
+
+__device__ __forceinline__ float netmf_value(uint32_t cnt, uint32_t dx, uint32_t dy, bool diag,
+                                             const NetmfConst &k) {
+    if ((cnt | dx | dy) < (1u << 24)) {
+        const float cf = (float)cnt, xf = (float)dx, yf = (float)dy, qf = __fmul_rn(xf, yf);
+        const float hi = diag ? k.diag_hi : k.off_hi, lo = diag ? k.diag_lo : k.off_lo;
+        const float dq = fmaf(cf, lo, fmaf(cf, hi, -qf) - fmaf(xf, yf, -qf));
+        if (dq < -1e-5f * qf) return 0.f;
+        if (dq > 1e-5f * qf && qf < 16777216.f) return log1pf(__fdiv_rn(dq, qf));
+    }
+    return netmf_value_exact(__dmul_rn((double)cnt, diag ? k.a_diag : k.a_off),
+                             __ll2double_rn((int64_t)dx * (int64_t)dy));
 }
 
 // Eq. 1 entry from a fixed-point count: K = wsum * unit (2^-32 for summed
@@ -1446,35 +1452,25 @@ __device__ __forceinline__ float netmf_value(uint32_t cnt, int64_t dx, int64_t d
 // carries an error of ~1e-7 |D| + 1e-14 q; when |D| > 1e-5 q its sign is the
 // FP64 decision. Otherwise the exact FP64 rule (no division) decides.
 // unit_f / unit_d: the power of two that one unit of wsum stands for.
-__device__ __forceinline__ float netmf_value_fixed(uint64_t wsum, float unit_f, double unit_d, int64_t dx,
-                                                   int64_t dy, bool diag, const NetmfConst &k) {
-    const int64_t q64 = dx * dy;
-    if (q64 < (1ll << 24)) {
+__device__ __forceinline__ float netmf_value_fixed(uint64_t wsum, float unit_f, double unit_d, uint32_t dx,
+                                                   uint32_t dy, bool diag, const NetmfConst &k) {
+    if ((dx | dy) < (1u << 24)) {
         const float kh = __ull2float_rn(wsum);
         // kh is an integer below 2^64 (unless wsum rounds up to 2^64): the
         // residual wsum - kh is exact in 64-bit arithmetic
         const float kl = kh < 1.8446744e19f ? (float)(int64_t)(wsum - __float2ull_rn(kh)) : 0.f;
         const float khs = kh * unit_f, kls = kl * unit_f;
-        const float qf = (float)q64;
+        const float xf = (float)dx, yf = (float)dy, qf = __fmul_rn(xf, yf);
         const float hi = diag ? k.diag_hi : k.off_hi, lo = diag ? k.diag_lo : k.off_lo;
-        const float dq = fmaf(khs, hi, -qf) + fmaf(khs, lo, kls * hi);
-        if (fabsf(dq) > 1e-5f * qf) return dq > 0.f ? log1pf(__fdiv_rn(dq, qf)) : 0.f;
+        const float dq = (fmaf(khs, hi, -qf) - fmaf(xf, yf, -qf)) + fmaf(khs, lo, kls * hi);
+        if (dq < -1e-5f * qf) return 0.f;
+        if (dq > 1e-5f * qf && qf < 16777216.f) return log1pf(__fdiv_rn(dq, qf));
     }
     const double K = __dmul_rn(__ull2double_rn(wsum), unit_d);
-    const double p = __dmul_rn(K, diag ? k.a_diag : k.a_off);
-    const double q = __ll2double_rn(q64);
-    if (!(p > q)) return 0.f;
-    const double q2 = __dmul_rn(2.0, q);
-    if (p < q2) {
-        const double dd = __dsub_rn(p, q);
-        if (!(__dmul_rn(dd, 9007199254740992.0) > q)) return 0.f;
-        return log1pf(__fdiv_rn((float)dd, (float)q));
-    }
-    if (p < 1e30) return logf(__fdiv_rn((float)p, (float)q));
-    return (float)(log(p) - log(q));
+    return netmf_value_exact(__dmul_rn(K, diag ? k.a_diag : k.a_off), __ll2double_rn((int64_t)dx * (int64_t)dy));
 }
 
-__device__ __forceinline__ float netmf_value_w(uint64_t wsum, int64_t dx, int64_t dy, bool diag,
+__device__ __forceinline__ float netmf_value_w(uint64_t wsum, uint32_t dx, uint32_t dy, bool diag,
                                                const NetmfConst &k) {
     return netmf_value_fixed(wsum, 2.3283064e-10f, 2.3283064365386963e-10, dx, dy, diag, k);   // 2^-32
 }
@@ -1493,27 +1489,61 @@ __device__ __forceinline__ void add_kept(unsigned kept, unsigned long long *__re
     if (threadIdx.x == 0 && s_kept) atomicAdd(nnz + blockIdx.x % kNnzSlots, (unsigned long long)s_kept);
 }
 
-// Weighted table -> the float-bits value table (upper triangle).
-__global__ void __launch_bounds__(256) table_values_w_kernel(const uint64_t *__restrict__ W, uint32_t *__restrict__ T,
-                                                             int64_t ld, int n, const int64_t *__restrict__ indptr,
-                                                             NetmfConst kc, unsigned long long *__restrict__ nnz) {
-    constexpr int kAhead = 4;   // loads in flight a thread
-    const int x = blockIdx.x;
-    const int64_t dx = eq1_degree(kc, indptr, x);
+// Weighted table -> the float-bits value table (upper triangle). A warp queues the
+// nonzero weights that it finds and takes their values 32 at a time, one per lane:
+// the arithmetic bounds the pass, and downsampled tables are mostly empty.
+// 10k vertices, 67M weighted downsampled draws: 123 us (a value per lane that found a
+// weight: 278, with 64-bit degree products 368).
+constexpr int kWvThreads = 256;
+constexpr int kWvAhead = 4;                      // loads in flight a lane
+constexpr int kWvQueue = 31 + 32 * kWvAhead;     // left over + new
+__global__ void __launch_bounds__(kWvThreads) table_values_w_kernel(const uint64_t *__restrict__ W,
+                                                                    uint32_t *__restrict__ T, int64_t ld, int n,
+                                                                    const int64_t *__restrict__ indptr, NetmfConst kc,
+                                                                    unsigned long long *__restrict__ nnz) {
+    __shared__ uint64_t s_qw[kWvThreads / 32][kWvQueue + 1];
+    __shared__ int s_qy[kWvThreads / 32][kWvQueue + 1];
+    const int x = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t dx = eq1_degree(kc, indptr, x);
+    const size_t row = (size_t)x * ld;
+    uint64_t *qw = s_qw[warp];
+    int *qy = s_qy[warp];
+    int qn = 0;   // queued entries (the same in every lane)
     unsigned kept = 0;
-    for (int y0 = x + threadIdx.x; y0 < n; y0 += kAhead * 256) {
-        uint64_t w[kAhead];
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u) w[u] = y0 + 256 * u < n ? __ldcs(W + (size_t)x * ld + y0 + 256 * u) : 0ull;
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u) {
-            if (w[u] == 0) continue;
-            const int y = y0 + 256 * u;
-            const float v = netmf_value_w(w[u], dx, eq1_degree(kc, indptr, y), x == y, kc);
-            T[(size_t)x * ld + y] = __float_as_uint(v);
+    auto values = [&](int q0, int cnt) {   // of queued entries [q0, q0 + cnt), cnt <= 32
+        if (lane < cnt) {
+            const int y = qy[q0 + lane];
+            const float v = netmf_value_w(qw[q0 + lane], dx, eq1_degree(kc, indptr, y), x == y, kc);
+            T[row + y] = __float_as_uint(v);
             if (__float_as_uint(v) != 0u) kept += x == y ? 1u : 2u;
         }
+    };
+    const unsigned lt = (1u << lane) - 1u;
+    for (int yb = x + 32 * kWvAhead * warp; yb < n; yb += kWvThreads * kWvAhead) {
+        uint64_t w[kWvAhead];
+#pragma unroll
+        for (int u = 0; u < kWvAhead; ++u) {
+            const int y = yb + 32 * u + lane;
+            w[u] = y < n ? __ldcs(W + row + y) : 0ull;
+        }
+#pragma unroll
+        for (int u = 0; u < kWvAhead; ++u) {
+            const unsigned bal = __ballot_sync(0xffffffffu, w[u] != 0ull);
+            if (w[u] != 0ull) {
+                const int pos = qn + __popc(bal & lt);
+                qw[pos] = w[u];
+                qy[pos] = yb + 32 * u + lane;
+            }
+            qn += __popc(bal);
+        }
+        __syncwarp();
+        while (qn >= 32) {   // the last 32 queued
+            values(qn - 32, 32);
+            qn -= 32;
+            __syncwarp();
+        }
     }
+    values(0, qn);
     add_kept(kept, nnz);
 }
 
@@ -1551,8 +1581,8 @@ __global__ void trunclog_kernel(const int32_t *__restrict__ x, const int32_t *__
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nnz;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t xi = x[i], yi = y[i];
-        const int64_t dx = eq1_degree(kc, indptr, xi);
-        const int64_t dy = eq1_degree(kc, indptr, yi);
+        const uint32_t dx = eq1_degree(kc, indptr, xi);
+        const uint32_t dy = eq1_degree(kc, indptr, yi);
         const float v = netmf_value(cnt[i], dx, dy, xi == yi, kc);
         const bool k = v > 0.f;
         if (k) {
@@ -1645,12 +1675,12 @@ __global__ void table_values_kernel(uint32_t *__restrict__ T, int64_t ld, int n,
                                     NetmfConst kc, unsigned long long *__restrict__ nnz) {
     unsigned kept = 0;
     const int x = blockIdx.x;
-    const int64_t dx = eq1_degree(kc, indptr, x);
+    const uint32_t dx = eq1_degree(kc, indptr, x);
     uint32_t *row = T + (size_t)x * ld;
     for (int y = x + threadIdx.x; y < n; y += blockDim.x) {
         const uint32_t c = row[y];
         if (c == 0) continue;
-        const int64_t dy = eq1_degree(kc, indptr, y);
+        const uint32_t dy = eq1_degree(kc, indptr, y);
         const float v = netmf_value(c, dx, dy, x == y, kc);
         row[y] = __float_as_uint(v);
         if (__float_as_uint(v) != 0u) kept += x == y ? 1u : 2u;
@@ -1671,7 +1701,7 @@ __global__ void __launch_bounds__(256) table_decode_values_kernel(const uint32_t
     constexpr uint32_t mask = TabPack<BITS>::mask;
     static_assert(P == 4, "a word's counters are one 16-byte group of the table");
     const int x = blockIdx.x;
-    const int64_t dx = eq1_degree(kc, indptr, x);
+    const uint32_t dx = eq1_degree(kc, indptr, x);
     const int64_t k0 = ((int64_t)x * ld + x) / P, k1 = ((int64_t)x * ld + ld) / P;
     uint4 *T4 = reinterpret_cast<uint4 *>(T);
     unsigned kept = 0;
@@ -1685,7 +1715,7 @@ __global__ void __launch_bounds__(256) table_decode_values_kernel(const uint32_t
             w[u] = in ? __ldcs(tp + kb + 256 * u) : 0u;
             r[u] = in ? T4[kb + 256 * u] : make_uint4(0u, 0u, 0u, 0u);
         }
-#pragma unroll
+#pragma unroll 1
         for (int u = 0; u < kAhead; ++u) {
             const int64_t k = kb + 256 * u;
             const uint32_t wr[P] = {r[u].x, r[u].y, r[u].z, r[u].w};
@@ -1717,8 +1747,8 @@ __global__ void __launch_bounds__(256) table_decode_values_kernel(const uint32_t
 // table_decode_values_kernel for sparse tables: a warp decodes 32
 // consecutive words at a time and queues the counted (index, count) pairs in
 // shared memory; the values are taken 32 at a time, one per lane, so a sparse
-// row does not run the value arithmetic with most lanes idle (each value is
-// independent: the order does not matter).
+// row does not run the value arithmetic, which bounds the pass, with most lanes
+// idle (each value is independent: the order does not matter).
 constexpr int kDvThreads = 256;
 constexpr int kDvQueue = 160;   // 31 left over + 4 x 32 new
 
@@ -1734,7 +1764,7 @@ __global__ void __launch_bounds__(kDvThreads) table_decode_values_sparse_kernel(
     __shared__ uint32_t s_qi[kDvThreads / 32][kDvQueue], s_qc[kDvThreads / 32][kDvQueue];
     const int x = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t dx = eq1_degree(kc, indptr, x);
+    const uint32_t dx = eq1_degree(kc, indptr, x);
     const int64_t k0 = ((int64_t)x * ld + x) / P, k1 = ((int64_t)x * ld + ld) / P;
     uint32_t *qi = s_qi[warp], *qc = s_qc[warp];
     int qn = 0;   // queued entries (the same in every lane)
@@ -1750,13 +1780,20 @@ __global__ void __launch_bounds__(kDvThreads) table_decode_values_sparse_kernel(
         }
     };
     const unsigned lt = (1u << lane) - 1u;
+    const uint4 *T4 = reinterpret_cast<const uint4 *>(T);
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    // the next words are on their way while these are decoded
+    uint32_t wn = k0 + 32 * warp + lane < k1 ? __ldcs(tp + k0 + 32 * warp + lane) : 0u;
+    uint4 rn = k0 + 32 * warp + lane < k1 ? T4[k0 + 32 * warp + lane] : zero;
+#pragma unroll 1
     for (int64_t kb = k0 + 32 * warp; kb < k1; kb += kDvThreads) {
         const int64_t k = kb + lane;
         const bool valid = k < k1;
-        const uint32_t w = valid ? tp[k] : 0u;
-        uint32_t wr[P];
-#pragma unroll
-        for (int i = 0; i < P; ++i) wr[i] = valid ? T[P * k + i] : 0u;
+        const uint32_t w = wn;
+        const uint32_t wr[P] = {rn.x, rn.y, rn.z, rn.w};
+        const bool more = k + kDvThreads < k1;
+        wn = more ? __ldcs(tp + k + kDvThreads) : 0u;
+        rn = more ? T4[k + kDvThreads] : zero;
         uint32_t prev = 0;
 #pragma unroll
         for (int i = 0; i < P; ++i) {
@@ -2928,11 +2965,12 @@ int table_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CsrResul
     Table tb;
     LNE_TRY(sample_table(ws, g, sp, &tb, st, false));
     const int n = (int)g.n;
-    // the samples bound the counted pairs: below ~15% of all pairs the value
-    // pass queues its counters (measured: 2.02 -> 1.09 ms at 3% on a
-    // 39k-vertex graph, 0.18 -> 0.21 ms at 41% on the benchmark's)
+    // the fewer samples a pair has, the fewer counters are not zero: below three a
+    // pair (half the pairs, both ways) the value pass queues its counters. Measured
+    // at n = 10312, queue / a value per lane: 7e6 samples 0.08 / 0.13 ms, 2.7e7 0.11 /
+    // 0.18, 1.1e8 0.15 / 0.18, 6.7e8 0.21 / 0.18; equal near 3.2e8
     const double samples = (double)g.nnz * ((double)sp.base + (double)sp.thr_frac / 4294967296.0);
-    const bool sparse = 2.0 * samples < 0.15 * (double)n * (double)n;
+    const bool sparse = 2.0 * samples < 6.0 * (double)n * (double)n;
     unsigned long long *kept = nullptr;
     LNE_TRY(ws.get("table.kept", kNnzSlots, &kept));
     LNE_CUDA_TRY(cudaMemsetAsync(kept, 0, sizeof(unsigned long long) * kNnzSlots, st));

@@ -120,3 +120,29 @@ def test_kept_buffers_serve_every_size(ctx):
     before = ctx.workspace_bytes()
     run(ctx, 1, 0.0)
     assert ctx.workspace_bytes() == before   # nothing new for a size it has served
+
+
+@pytest.mark.parametrize("rate", [0.3, 40.0, 900.0])
+@pytest.mark.parametrize("hub", [False, True])
+def test_table_values_sparse_and_dense(ctx, rate, hub):
+    """The table's value passes (queued below three samples a pair, a value per lane
+    above) against the oracle; hub: degree products beyond 2^24, where FP32 decides
+    only what is dropped. One FP32 log of a quotient with a relative error of 1e-7:
+    1e-6 as for every other value here."""
+    n = 4200 if hub else 300
+    if hub:      # two vertices joined to all the others: 4199^2 > 2^24
+        u = np.concatenate([np.zeros(n - 1, np.int64), np.ones(n - 2, np.int64)])
+        v = np.concatenate([np.arange(1, n), np.arange(2, n)])
+        g = synth.Graph(n, *synth.csr_from_edges(n, u, v), None, "hubs")
+    else:
+        g = synth.chung_lu(n, 2000, 2.2, seed=8, n_labels=2)
+    p = make_params(3, [0.2, 0.3, 0.5], rate * g.n_arcs, seed=4)
+    with_table = lne.Context(0)
+    with_table.set_option(lne.OPT_AGGREGATION, lne.AGG_TABLE)
+    out = {k: to_np(v).copy() for k, v in with_table.sparsifier_csr(lne.DeviceGraph.from_graph(g), p).items()
+           if torch.is_tensor(v)}
+    with_table.close()
+    sp = oracle.sparsifier(g.indptr, g.indices, p.T, p.s, p.samples, p.seed, p.b)
+    assert np.array_equal(out["indptr"], sp["indptr"])
+    assert np.array_equal(out["indices"].astype(np.int64), sp["indices"])
+    np.testing.assert_allclose(out["data"], sp["data"], rtol=1e-6, atol=1e-7)
