@@ -647,9 +647,16 @@ __global__ void upper_matmul_kernel(const double *__restrict__ A, const double *
 constexpr int kMMTile = 64;
 constexpr int kMMK = 32;
 
+// BATCH: independent products at fixed strides (a compile-time choice: the strides
+// alone cost a single product 10%).
+template <bool BATCH>
 __global__ void __launch_bounds__(256) right_multiply_kernel(
-    const float *__restrict__ Y, int64_t n, int c, int64_t ldy, const double *__restrict__ W,
-    int64_t ldw, int dout, const double *__restrict__ colscale, float *__restrict__ out, int64_t ldo) {
+    const float *__restrict__ Y0, int64_t n, int c, int64_t ldy, const double *__restrict__ W0,
+    int64_t ldw, int dout, const double *__restrict__ colscale, float *__restrict__ out0, int64_t ldo, int64_t sy,
+    int64_t sw, int64_t so) {
+    const float *__restrict__ Y = BATCH ? Y0 + blockIdx.z * sy : Y0;
+    const double *__restrict__ W = BATCH ? W0 + blockIdx.z * sw : W0;
+    float *__restrict__ out = BATCH ? out0 + blockIdx.z * so : out0;
     __shared__ float ys[kMMTile][kMMK + 1];
     __shared__ float ws[kMMK][kMMTile];
     const int tid = threadIdx.x;
@@ -1893,12 +1900,16 @@ int gaussian_sketch(int64_t n, int c, uint64_t seed, float *out, int64_t ld, cud
 }
 
 int right_multiply(const float *Y, int64_t n, int c, int64_t ldy, const double *W, int64_t ldw,
-                   int dout, const double *colscale, float *out, int64_t ldo, cudaStream_t st) {
+                   int dout, const double *colscale, float *out, int64_t ldo, cudaStream_t st, int batch, int64_t sy,
+                   int64_t sw, int64_t so) {
     if (n <= 0 || dout <= 0) return 0;
-    dim3 grid((unsigned)ceil_div(n, kMMTile), (unsigned)ceil_div(dout, kMMTile));
+    dim3 grid((unsigned)ceil_div(n, kMMTile), (unsigned)ceil_div(dout, kMMTile), (unsigned)batch);
     {
         LNE_TRACE("right_multiply", st);
-        right_multiply_kernel<<<grid, 256, 0, st>>>(Y, n, c, ldy, W, ldw, dout, colscale, out, ldo);
+        if (batch > 1)
+            right_multiply_kernel<true><<<grid, 256, 0, st>>>(Y, n, c, ldy, W, ldw, dout, colscale, out, ldo, sy, sw, so);
+        else
+            right_multiply_kernel<false><<<grid, 256, 0, st>>>(Y, n, c, ldy, W, ldw, dout, colscale, out, ldo, 0, 0, 0);
         LNE_LAUNCH_CHECK();
     }
     return 0;

@@ -21,6 +21,7 @@ namespace lne {
 namespace {
 
 constexpr int kEvalRows = 128;   // rows per FP32 partial sum (and per CTA)
+constexpr double kEvalBatchBytes = 256e6;   // buffers of a batch of more than one candidate
 
 // Xa[i] = (X[idx[i]], 1, 0, ..) with rows of `pitch` floats, Ys[i][l] = +1 / -1.
 // A row index outside [0, n) is not read: its row becomes zeros (label -1) and
@@ -82,16 +83,18 @@ __device__ __forceinline__ void upper_tile(int p, int nt, int *ti, int *tj) {
 // last four, so that neighbouring tiles' 16-byte loads hit neighbouring banks.
 constexpr int kEvalStage = 32;
 
-template <int TS>
+template <int TS, bool BATCH>
 __global__ void __launch_bounds__(256) hess_partial_kernel(const float *__restrict__ Xa, const float *__restrict__ Z,
                                                            const float *__restrict__ Ys, int64_t m, int da, int L,
+                                                           int Ly,
                                                            float C, int ntiles, float *__restrict__ hpart,
                                                            float *__restrict__ gpart) {
     extern __shared__ __align__(16) float xs[];   // two buffers of kEvalStage rows
     __shared__ float2 s_w[kEvalRows];             // (D, R) of the rows
     const int nt = (da + TS - 1) / TS, pitch = nt * TS, quads = pitch / 4;
     const int tid = threadIdx.x;
-    const int l = blockIdx.y;
+    const int l = blockIdx.y, cand = BATCH ? l / Ly : 0;   // the candidate's rows; its labels are every candidate's
+    if (BATCH) Xa += cand * m * pitch;
     const int64_t r0 = (int64_t)blockIdx.x * kEvalRows;
     const int rows = (int)imin64(kEvalRows, m - r0);
     auto stage = [&](int s0, float *to) {
@@ -107,7 +110,7 @@ __global__ void __launch_bounds__(256) hess_partial_kernel(const float *__restri
     };
     stage(0, xs);
     for (int r = tid; r < rows; r += blockDim.x) {
-        const float y = Ys[(r0 + r) * L + l];
+        const float y = Ys[(r0 + r) * Ly + (l - cand * Ly)];
         const float sg = 1.0f / (1.0f + expf(-y * Z[(r0 + r) * L + l]));
         s_w[r] = make_float2(C * sg * (1.0f - sg), C * (sg - 1.0f) * y);
     }
@@ -553,6 +556,8 @@ __global__ void __launch_bounds__(kSolveThreads) newton_solve_kernel(const doubl
 // Top-k prediction and per-label TP / FP / FN counts.
 __global__ void topk_f1_kernel(const float *__restrict__ S, const float *__restrict__ Ys, int64_t m, int L,
                                unsigned long long *__restrict__ counts) {
+    S += blockIdx.y * m * L;   // the candidate's
+    counts += 3 * L * blockIdx.y;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
         const float *si = S + i * L;
         const float *yi = Ys + i * L;
@@ -573,105 +578,153 @@ int egrid(int64_t work) { return (int)std::min<int64_t>(ceil_div(std::max<int64_
 
 }  // namespace
 
-int macro_f1(Workspace &ws, const float *X, int64_t n, int d, int64_t ldx, const uint8_t *labels, int L,
-             const int32_t *train_idx, int64_t n_train, const int32_t *test_idx, int64_t n_test, double C, int iters,
-             double *macro, double *micro, cudaStream_t st) {
+// Candidates are scored together: one launch a Newton step for all of them, as many
+// as fit the buffer bound. A small candidate's kernels (33 features, a few labels)
+// are all latency: 4 tasks of 8 candidates each took 26.3 ms one candidate at a
+// time, 22.2 together (both with everything else alike).
+int eval_batch_init(Workspace &ws, EvalBatch *b, int ncand, int64_t n, int d, const uint8_t *labels, int L,
+                    const int32_t *train_idx, int64_t n_train, const int32_t *test_idx, int64_t n_test, double C,
+                    int iters, cudaStream_t st) {
     if (d < 1 || L < 1 || n_train < 1 || n_test < 1 || iters < 0 || !(C > 0.0))
         return fail(LNE_ERR_INVALID, "bad Macro-F1 arguments");
     const int da = d + 1;
     if (da > 160) return fail(LNE_ERR_UNSUPPORTED, "Macro-F1 supports d <= 159");
-    const int64_t nblk = ceil_div(n_train, kEvalRows);
-    const int ts = da > 64 ? 8 : 4;
-    const int ntiles = upper_tiles(da, ts);
-    const int pitch = (da + ts - 1) / ts * ts;
-    float *Xa = nullptr, *Ys = nullptr, *Z = nullptr, *Xt = nullptr, *Yt = nullptr, *St = nullptr;
-    float *gp = nullptr, *hp = nullptr;
-    double *W = nullptr, *G = nullptr, *H = nullptr;
-    float2 *Hp = nullptr;   // H as float pairs
-    unsigned long long *cnt = nullptr;
-    int *status = nullptr;
-    LNE_TRY(ws.get("eval.Xa", (size_t)(n_train * pitch), &Xa));
-    LNE_TRY(ws.get("eval.Ys", (size_t)(n_train * L), &Ys));
-    LNE_TRY(ws.get("eval.Z", (size_t)(n_train * L), &Z));
-    LNE_TRY(ws.get("eval.Xt", (size_t)(n_test * pitch), &Xt));
-    LNE_TRY(ws.get("eval.Yt", (size_t)(n_test * L), &Yt));
-    LNE_TRY(ws.get("eval.St", (size_t)(n_test * L), &St));
-    LNE_TRY(ws.get("eval.W", (size_t)da * L, &W));
-    LNE_TRY(ws.get("eval.G", (size_t)da * L, &G));
-    LNE_TRY(ws.get("eval.H", (size_t)L * da * da, &H));
-    LNE_TRY(ws.get("eval.Hp", (size_t)L * da * da, &Hp));
-    LNE_TRY(ws.get("eval.gp", (size_t)(nblk * da * L), &gp));
-    LNE_TRY(ws.get("eval.hp", (size_t)nblk * L * ntiles * ts * ts, &hp));
-    LNE_TRY(ws.get("eval.cnt", (size_t)3 * L, &cnt));
-    LNE_TRY(ws.get("eval.status", 1, &status));
-    LNE_CUDA_TRY(cudaMemsetAsync(W, 0, sizeof(double) * da * L, st));
-    LNE_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * 3 * L, st));
-    LNE_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), st));
-    {
-        LNE_TRACE("eval_gather", st);
-        gather_rows_kernel<<<egrid(n_train * pitch), 256, 0, st>>>(X, n, ldx, d, labels, L, train_idx, n_train, pitch,
-                                                                   Xa, Ys, status);
-        LNE_LAUNCH_CHECK();
-        gather_rows_kernel<<<egrid(n_test * pitch), 256, 0, st>>>(X, n, ldx, d, labels, L, test_idx, n_test, pitch, Xt,
-                                                                  Yt, status);
-        LNE_LAUNCH_CHECK();
-    }
+    b->n = n;
+    b->n_train = n_train;
+    b->n_test = n_test;
+    b->d = d;
+    b->L = L;
+    b->iters = iters;
+    b->C = C;
+    b->labels = labels;
+    b->train_idx = train_idx;
+    b->test_idx = test_idx;
+    b->nblk = ceil_div(n_train, kEvalRows);
+    b->ts = da > 64 ? 8 : 4;
+    b->ntiles = upper_tiles(da, b->ts);
+    b->pitch = (da + b->ts - 1) / b->ts * b->ts;
+    const size_t hp = (size_t)b->nblk * L * b->ntiles * b->ts * b->ts;
+    const double bytes = 4.0 * ((double)(n_train + n_test) * (b->pitch + L) + (double)b->nblk * da * L + (double)hp) +
+                         16.0 * da * L * (da + 1);
+    b->cap = (int)std::max(1.0, std::min({(double)ncand, kEvalBatchBytes / bytes, 65535.0 / L}));
+    b->ids.clear();
+    const size_t cap = (size_t)b->cap;
+    LNE_TRY(ws.get("eval.Xa", cap * (size_t)(n_train * b->pitch), &b->Xa));
+    LNE_TRY(ws.get("eval.Ys", (size_t)(n_train * L), &b->Ys));
+    LNE_TRY(ws.get("eval.Z", cap * (size_t)(n_train * L), &b->Z));
+    LNE_TRY(ws.get("eval.Xt", cap * (size_t)(n_test * b->pitch), &b->Xt));
+    LNE_TRY(ws.get("eval.Yt", (size_t)(n_test * L), &b->Yt));
+    LNE_TRY(ws.get("eval.St", cap * (size_t)(n_test * L), &b->St));
+    LNE_TRY(ws.get("eval.W", cap * (size_t)da * L, &b->W));
+    LNE_TRY(ws.get("eval.G", cap * (size_t)da * L, &b->G));
+    LNE_TRY(ws.get("eval.H", cap * (size_t)L * da * da, &b->H));
+    LNE_TRY(ws.get("eval.Hp", cap * (size_t)L * da * da, &b->Hp));
+    LNE_TRY(ws.get("eval.gp", cap * (size_t)(b->nblk * da * L), &b->gp));
+    LNE_TRY(ws.get("eval.hp", cap * hp, &b->hp));
+    LNE_TRY(ws.get("eval.cnt", cap * (size_t)3 * L, &b->cnt));
+    LNE_TRY(ws.get("eval.status", 1, &b->status));
+    LNE_CUDA_TRY(cudaMemsetAsync(b->status, 0, sizeof(int), st));
+    return 0;
+}
+
+// Gathers candidate id's rows of X (free to be reused on the stream afterwards);
+// runs the batch first when it is full.
+int eval_batch_add(EvalBatch *b, int id, const float *X, int64_t ldx, double *macro, double *micro, cudaStream_t st) {
+    if ((int)b->ids.size() == b->cap) LNE_TRY(eval_batch_run(b, macro, micro, st));
+    const int64_t slot = (int64_t)b->ids.size();
+    b->ids.push_back(id);
+    LNE_TRACE("eval_gather", st);
+    gather_rows_kernel<<<egrid(b->n_train * b->pitch), 256, 0, st>>>(
+        X, b->n, ldx, b->d, b->labels, b->L, b->train_idx, b->n_train, b->pitch, b->Xa + slot * b->n_train * b->pitch,
+        b->Ys, b->status);
+    LNE_LAUNCH_CHECK();
+    gather_rows_kernel<<<egrid(b->n_test * b->pitch), 256, 0, st>>>(
+        X, b->n, ldx, b->d, b->labels, b->L, b->test_idx, b->n_test, b->pitch, b->Xt + slot * b->n_test * b->pitch,
+        b->Yt, b->status);
+    LNE_LAUNCH_CHECK();
+    return 0;
+}
+
+// Scores the gathered candidates: macro[id], micro[id]. Synchronises.
+int eval_batch_run(EvalBatch *b, double *macro, double *micro, cudaStream_t st) {
+    const int m = (int)b->ids.size(), L = b->L, da = b->d + 1, ntiles = b->ntiles, ts = b->ts, pitch = b->pitch;
+    if (m == 0) return 0;
+    LNE_CUDA_TRY(cudaMemsetAsync(b->W, 0, sizeof(double) * da * L * m, st));
+    LNE_CUDA_TRY(cudaMemsetAsync(b->cnt, 0, sizeof(unsigned long long) * 3 * L * m, st));
     const int threads = (std::max(ntiles, da) + 31) / 32 * 32;   // at most 224 (da = 160: 210 tiles)
     const int hsmem = 2 * kEvalStage * pitch * 4;
-    const dim3 hgrid((unsigned)nblk, (unsigned)L);
-    const dim3 rgrid((unsigned)ceil_div((int64_t)ntiles * ts * ts + da, 256), (unsigned)L);
+    // the labels of all candidates in a row: label l of candidate j is column j L + l
+    const int Lm = L * m;
+    const dim3 hgrid((unsigned)b->nblk, (unsigned)Lm);
+    const dim3 rgrid((unsigned)ceil_div((int64_t)ntiles * ts * ts + da, 256), (unsigned)Lm);
     LNE_TRY(allow_dynamic_smem(newton_solve_kernel));
-    for (int it = 0; it < iters; ++it) {
-        LNE_TRY(right_multiply(Xa, n_train, da, pitch, W, L, L, nullptr, Z, L, st));
+    for (int it = 0; it < b->iters; ++it) {
+        LNE_TRY(right_multiply(b->Xa, b->n_train, da, pitch, b->W, Lm, L, nullptr, b->Z, Lm, st, m,
+                               b->n_train * pitch, L, L));
         {
             LNE_TRACE("newton_partials", st);
-            if (ts == 8)
-                hess_partial_kernel<8><<<hgrid, threads, hsmem, st>>>(Xa, Z, Ys, n_train, da, L, (float)C, ntiles, hp,
-                                                                      gp);
-            else
-                hess_partial_kernel<4><<<hgrid, threads, hsmem, st>>>(Xa, Z, Ys, n_train, da, L, (float)C, ntiles, hp,
-                                                                      gp);
+            auto *hess = m > 1 ? (ts == 8 ? hess_partial_kernel<8, true> : hess_partial_kernel<4, true>)
+                               : (ts == 8 ? hess_partial_kernel<8, false> : hess_partial_kernel<4, false>);
+            hess<<<hgrid, threads, hsmem, st>>>(b->Xa, b->Z, b->Ys, b->n_train, da, Lm, L, (float)b->C, ntiles, b->hp,
+                                                b->gp);
             LNE_LAUNCH_CHECK();
         }
         {
             LNE_TRACE("newton_sums", st);
             if (ts == 8)
-                newton_reduce_kernel<8><<<rgrid, 256, 0, st>>>(gp, hp, (int)nblk, da, L, ntiles, W, G, H, Hp);
+                newton_reduce_kernel<8><<<rgrid, 256, 0, st>>>(b->gp, b->hp, (int)b->nblk, da, Lm, ntiles, b->W, b->G,
+                                                               b->H, b->Hp);
             else
-                newton_reduce_kernel<4><<<rgrid, 256, 0, st>>>(gp, hp, (int)nblk, da, L, ntiles, W, G, H, Hp);
+                newton_reduce_kernel<4><<<rgrid, 256, 0, st>>>(b->gp, b->hp, (int)b->nblk, da, Lm, ntiles, b->W, b->G,
+                                                               b->H, b->Hp);
             LNE_LAUNCH_CHECK();
         }
         {
             LNE_TRACE("newton_solve", st);
-            newton_solve_kernel<<<L, kSolveThreads, solve_smem(da), st>>>(H, Hp, G, da, L, W, status);
+            newton_solve_kernel<<<Lm, kSolveThreads, solve_smem(da), st>>>(b->H, b->Hp, b->G, da, Lm, b->W, b->status);
             LNE_LAUNCH_CHECK();
         }
     }
-    LNE_TRY(right_multiply(Xt, n_test, da, pitch, W, L, L, nullptr, St, L, st));
+    LNE_TRY(right_multiply(b->Xt, b->n_test, da, pitch, b->W, Lm, L, nullptr, b->St, L, st, m, b->n_test * pitch, L,
+                           b->n_test * L));
     {
         LNE_TRACE("topk_f1", st);
-        topk_f1_kernel<<<egrid(n_test), 256, 0, st>>>(St, Yt, n_test, L, cnt);
+        topk_f1_kernel<<<dim3((unsigned)egrid(b->n_test), (unsigned)m), 256, 0, st>>>(b->St, b->Yt, b->n_test, L,
+                                                                                     b->cnt);
         LNE_LAUNCH_CHECK();
     }
-    std::vector<unsigned long long> h(3 * L);
+    std::vector<unsigned long long> h((size_t)3 * L * m);
     int hs = 0;
-    LNE_CUDA_TRY(cudaMemcpyAsync(h.data(), cnt, sizeof(unsigned long long) * 3 * L, cudaMemcpyDeviceToHost, st));
-    LNE_CUDA_TRY(cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st));
+    LNE_CUDA_TRY(cudaMemcpyAsync(h.data(), b->cnt, sizeof(unsigned long long) * h.size(), cudaMemcpyDeviceToHost, st));
+    LNE_CUDA_TRY(cudaMemcpyAsync(&hs, b->status, sizeof(int), cudaMemcpyDeviceToHost, st));
     LNE_CUDA_TRY(cudaStreamSynchronize(st));
     if (hs & 2) return fail(LNE_ERR_INVALID, "a train or test row index is outside [0, n)");
     if (hs) return fail(LNE_ERR_NUMERIC, "a logistic-regression Hessian was not positive definite");
-    double f1sum = 0.0, tp = 0, fp = 0, fn = 0;
-    for (int l = 0; l < L; ++l) {
-        const double a = (double)h[3 * l], b = (double)h[3 * l + 1], c = (double)h[3 * l + 2];
-        const double den = 2 * a + b + c;
-        f1sum += den > 0 ? 2 * a / den : 0.0;
-        tp += a;
-        fp += b;
-        fn += c;
+    for (int j = 0; j < m; ++j) {
+        const unsigned long long *hj = h.data() + (size_t)3 * L * j;
+        double f1sum = 0.0, tp = 0, fp = 0, fn = 0;
+        for (int l = 0; l < L; ++l) {
+            const double t = (double)hj[3 * l], p = (double)hj[3 * l + 1], q = (double)hj[3 * l + 2];
+            const double den = 2 * t + p + q;
+            f1sum += den > 0 ? 2 * t / den : 0.0;
+            tp += t;
+            fp += p;
+            fn += q;
+        }
+        macro[b->ids[j]] = f1sum / L;
+        micro[b->ids[j]] = (2 * tp + fp + fn) > 0 ? 2 * tp / (2 * tp + fp + fn) : 0.0;
     }
-    *macro = f1sum / L;
-    *micro = (2 * tp + fp + fn) > 0 ? 2 * tp / (2 * tp + fp + fn) : 0.0;
+    b->ids.clear();
     return 0;
+}
+
+int macro_f1(Workspace &ws, const float *X, int64_t n, int d, int64_t ldx, const uint8_t *labels, int L,
+             const int32_t *train_idx, int64_t n_train, const int32_t *test_idx, int64_t n_test, double C, int iters,
+             double *macro, double *micro, cudaStream_t st) {
+    EvalBatch b;
+    LNE_TRY(eval_batch_init(ws, &b, 1, n, d, labels, L, train_idx, n_train, test_idx, n_test, C, iters, st));
+    LNE_TRY(eval_batch_add(&b, 0, X, ldx, macro, micro, st));
+    return eval_batch_run(&b, macro, micro, st);
 }
 
 }  // namespace lne

@@ -181,7 +181,8 @@ int small_svd(Workspace &ws, const double *R, int c, double *U_R, double *sigma,
 // out[n][dout] = Y[n][c] * W[c][dout] (W FP64 row-major with leading dim ldw),
 // optionally scaled per output column by colscale (FP64, length dout).
 int right_multiply(const float *Y, int64_t n, int c, int64_t ldy, const double *W, int64_t ldw,
-                   int dout, const double *colscale, float *out, int64_t ldo, cudaStream_t st);
+                   int dout, const double *colscale, float *out, int64_t ldo, cudaStream_t st, int batch = 1, int64_t sy = 0,
+                   int64_t sw = 0, int64_t so = 0);
 // Flip columns of U [n][d] so that each column's largest-magnitude entry is
 // positive; if X is not NULL also writes X = U diag(sqrt(sigma)).
 int sign_fix_embed(Workspace &ws, float *U, int64_t n, int d, int64_t ld, const double *sigma,
@@ -379,6 +380,27 @@ int surrogate_train(Surrogate &S, Workspace &ws, const float *X, const float *t,
 int macro_f1(Workspace &ws, const float *X, int64_t n, int d, int64_t ldx, const uint8_t *labels, int L,
              const int32_t *train_idx, int64_t n_train, const int32_t *test_idx, int64_t n_test, double C, int iters,
              double *macro, double *micro, cudaStream_t st);
+// Several embeddings scored together on one split: init, add each (its rows are
+// gathered at once, so X may be reused), run; a full batch runs when the next is added.
+struct EvalBatch {
+    int64_t n = 0, n_train = 0, n_test = 0, nblk = 0;
+    int d = 0, L = 0, iters = 0, ts = 0, ntiles = 0, pitch = 0, cap = 0;
+    double C = 0.0;
+    const uint8_t *labels = nullptr;
+    const int32_t *train_idx = nullptr, *test_idx = nullptr;
+    float *Xa = nullptr, *Ys = nullptr, *Z = nullptr, *Xt = nullptr, *Yt = nullptr, *St = nullptr, *gp = nullptr,
+          *hp = nullptr;
+    double *W = nullptr, *G = nullptr, *H = nullptr;
+    float2 *Hp = nullptr;   // H as float pairs
+    unsigned long long *cnt = nullptr;
+    int *status = nullptr;
+    std::vector<int> ids;   // candidates gathered so far
+};
+int eval_batch_init(Workspace &ws, EvalBatch *b, int ncand, int64_t n, int d, const uint8_t *labels, int L,
+                    const int32_t *train_idx, int64_t n_train, const int32_t *test_idx, int64_t n_test, double C,
+                    int iters, cudaStream_t st);
+int eval_batch_add(EvalBatch *b, int id, const float *X, int64_t ldx, double *macro, double *micro, cudaStream_t st);
+int eval_batch_run(EvalBatch *b, double *macro, double *micro, cudaStream_t st);
 
 // Exclusive scan helpers (scan.cu).
 int scan_exclusive_u32_to_i64(const uint32_t *in, int64_t *out, int64_t n, cudaStream_t st);

@@ -183,12 +183,13 @@ int tune_batch(Workspace &ws, PropBatchGraph *cache, SpmmTune &tc, int aggregati
     LNE_TRY(ws.get("tune.r", (size_t)d * d, &R));
     LNE_TRY(ws.get("tune.ur", (size_t)d * d, &UR));
     LNE_TRY(ws.get("tune.sig", (size_t)d, &sig));
+    EvalBatch eb;
+    LNE_TRY(eval_batch_init(ws, &eb, ncand, n, d, labels, L, train, n_train, test, n_test, Creg, iters, st));
     auto score = [&](int j, const float *Xj) -> int {
         if (X_out)
             LNE_CUDA_TRY(cudaMemcpyAsync(X_out + (size_t)j * n * d, Xj, sizeof(float) * n * d,
                                          cudaMemcpyDeviceToDevice, st));
-        return macro_f1(ws, Xj, n, d, d, labels, L, train, n_train, test, n_test, Creg, iters, &macro[j], &micro[j],
-                        st);
+        return eval_batch_add(&eb, j, Xj, d, macro, micro, st);
     };
     // k = 0: the embedding is X0 itself
     std::vector<int> prop;
@@ -230,7 +231,7 @@ int tune_batch(Workspace &ws, PropBatchGraph *cache, SpmmTune &tc, int aggregati
         }
         LNE_TRY(status_check(ws, st));
     }
-    return 0;
+    return eval_batch_run(&eb, macro, micro, st);
 }
 
 }  // namespace lne
