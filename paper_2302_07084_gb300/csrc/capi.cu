@@ -215,8 +215,11 @@ void Workspace::retire(const std::string &name) {
     }();
     auto it = bufs_.find(name);
     if (it == bufs_.end() || it->second.idle) return;
-    if ((g_idle_bytes += (int64_t)it->second.bytes) > kKeep) {
-        g_idle_bytes -= (int64_t)it->second.bytes;
+    const int64_t size = (int64_t)it->second.bytes;
+    if (size > kKeep / 8) {
+        release(name);
+    } else if ((g_idle_bytes += size) > kKeep) {
+        g_idle_bytes -= size;
         release(name);
     } else {
         it->second.idle = true;

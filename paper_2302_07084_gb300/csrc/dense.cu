@@ -1987,7 +1987,7 @@ int status_check(Workspace &ws, cudaStream_t st) {
     LNE_CUDA_TRY(cudaStreamSynchronize(st));
     if (h[0] == 0 && h[1] == 0 && h[2] == 0) return 0;
     LNE_CUDA_TRY(cudaMemsetAsync(status, 0, 4 * sizeof(int), st));
-    if (h[1] != 0) return fail(LNE_ERR_TIMEOUT, "a bounded device wait expired (tensor-core pipeline or Cholesky grid barrier)");
+    if (h[1] != 0) return fail(LNE_ERR_TIMEOUT, "a bounded device wait expired (tensor-core pipeline, Cholesky, small SVD or key sort)");
     if (h[2] != 0)
         return fail(LNE_ERR_UNSUPPORTED, "a row of the very sparse projection has more than 12 nonzeros (raise s)");
     return fail(LNE_ERR_NUMERIC, "Cholesky breakdown in CholeskyQR (Gram not positive definite)");

@@ -32,9 +32,9 @@ public:
     // Frees one named buffer (no-op if absent).
     void release(const std::string &name);
     // Done with a named buffer until the next get() of it (no-op if absent). Kept,
-    // contents undefined, while all workspaces together keep at most 1/8 of the
-    // device's memory this way, else freed; a workspace's kept ones are freed when
-    // one of its allocations fails. Freeing and allocating the sort path's buffers on
+    // contents undefined, if it takes at most 1/64 of the device's memory and all
+    // workspaces together then keep at most 1/8 of it this way, else freed; a
+    // workspace's kept ones are freed when one of its allocations fails. Freeing and allocating the sort path's buffers on
     // every call took 8 of 26 ms at 2e8 samples (7 GB); a run of tens of GB still
     // hands them back as it goes.
     void retire(const std::string &name);

@@ -19,12 +19,15 @@
 //                      exact decision), log(v) as float32.
 //   6. csr_fill/sort   symmetric CSR of the kept entries, rows sorted.
 //
-// For graphs whose pair space fits a dense table (n <= 65536) the counting is
-// direct instead: the walk adds each sample into an n x n table of counters
-// (upper triangle, fire-and-forget atomics), one pass turns counts into Eq. 1
-// values in place, and 64 x 64 tiles of the symmetric matrix (the lower half
-// read through a shared-memory transpose) give row counts and then the CSR in
-// column order -- no key buffers, no sort.
+// That is the bucket aggregation. For graphs whose pair space fits a dense table
+// (n <= 65536) the counting is direct instead: the walk (walk_table_kernel, or
+// walk_batch_kernel with downsampling, weights or strata) adds each sample into an
+// n x n table of counters (upper triangle), one pass turns counts into Eq. 1
+// values in place, and, where a CSR is wanted, 64 x 64 tiles of the symmetric
+// matrix (the lower half read through a shared-memory transpose) give row counts
+// and then the CSR in column order -- no key buffers, no sort. Otherwise
+// walk_batch_kernel writes the keys, sort.cu sorts them, and path_* kernels
+// assemble the CSR from the sorted pairs.
 //
 // Every integer result (counts, keep decisions, CSR structure) is independent of
 // scheduling, so it equals the CPU oracle bit for bit.
