@@ -1830,9 +1830,8 @@ __global__ void svd_finish_kernel(const double *__restrict__ U, const double *__
 // Per column: the largest |u| and, among equal magnitudes, the smallest row,
 // packed as (|u| bits << 32) | ~row so that one max orders both. Each thread
 // keeps a running maximum over a strided set of rows of one column, and a CTA
-// adds one atomic per column: they bound the kernel (all CTAs meet at the same d
-// words), so there is one CTA an SM. 10k x 32: 4 us, with an atomic per thread
-// and eight CTAs an SM 41.
+// adds one atomic per column (all CTAs meet at the same d words: with an atomic per
+// thread and a row a thread they bound the kernel, 41 us at 10k x 32, 4 us now).
 __global__ void __launch_bounds__(256) col_absmax_kernel(const float *__restrict__ U, int64_t n, int d, int64_t ld,
                                                          unsigned long long *__restrict__ best) {
     const int sub = blockDim.x / d;               // row subsets per CTA (d <= 256)
@@ -2149,7 +2148,9 @@ int sign_fix_embed(Workspace &ws, float *U, int64_t n, int d, int64_t ld, const 
     const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, sub), num_sms() * 8));
     {
         LNE_TRACE("col_absmax", st);
-        col_absmax_kernel<<<std::min<unsigned>(blocks, num_sms()), 256, 0, st>>>(U, n, d, ld, best);
+        // at least 16 rows a thread before the CTAs fill the GPU
+        const unsigned cblocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 16 * sub), num_sms() * 8));
+        col_absmax_kernel<<<cblocks, 256, 0, st>>>(U, n, d, ld, best);
         LNE_LAUNCH_CHECK();
     }
     {
