@@ -693,9 +693,9 @@ int lne_spmm(lne_ctx *ctx, const lne_csr *M, const void *X_dev, int64_t ldx, int
         if (ok) v.vb = &vbs;
         if (rc == 0 && precision == LNE_PREC_BF16_MIXED)
             rc = lne::spmm_bf16(ctx->ws, v, static_cast<const __nv_bfloat16 *>(X_dev), ldx, c, Y_dev, ldy, nullptr,
-                                as_stream(stream));
+                                as_stream(stream), true);
         else if (rc == 0)
-            rc = lne::spmm(ctx->ws, v, static_cast<const float *>(X_dev), ldx, c, Y_dev, ldy, as_stream(stream));
+            rc = lne::spmm(ctx->ws, v, static_cast<const float *>(X_dev), ldx, c, Y_dev, ldy, as_stream(stream), true);
     }
     return finish(ctx, rc);
 }

@@ -62,29 +62,28 @@ __global__ void sketch_kernel(int64_t n, int c, uint32_t k0, uint32_t k1, float 
 
 // ---------------------------------------------------------------------------
 // Gram with FP64 accuracy from FP32 arithmetic: thread (ti, tj, half), ti <= tj,
-// owns 4 rows of an 8x8 tile of the upper half. FP64 arithmetic runs at 1/64 of
-// the FP32 rate on this GPU; four FP32 operations a product take its place:
-//
-//   Over a chunk of 64 rows entry (a, b) is accumulated in h, which starts at
-//   C = 3 u_a u_b, u the power of two above the column's norm over the chunk.
-//   |sum| <= u_a u_b keeps h inside [2, 4] u_a u_b, so every h <- h + a b is
-//   rounded to the same grid and h_old - h is exact; the rounding error
-//   a b + (h_old - h), one fma, goes to lo. (A general two-sum, which needs no
-//   such bound, takes ten operations.)
-//   After the chunk h - C (exact) and lo enter the entry's float pair by an
-//   error-free addition; CTAs are summed in FP64.
-//
-// h's grid is 2^-22 u_a u_b and lo keeps 24 bits below it, so the sum is good to
-// about 2^-44 of the column norms' product. Bound by the FP32 pipe (4 n c^2 / 2
-// operations a product, issued as packed pairs). Measured (n = 1e6, c = 144):
-// 4.5 ms with two-sums, 1.65 ms here, 78% of the FP32 pipe's rate; n = 10,312:
-// 64 -> 37 us.
-// The _rn intrinsics keep the compiler from contracting what has to be exact.
+// owns 4 rows of an 8x8 tile of the upper half. Every product a*b is split exactly into
+// p + e (p = fl(a b), e = fma(a, b, -p)); p enters a float pair (hi, lo) by
+// an error-free two-sum, e and the two-sum's error go to lo. The pair carries
+// ~46 significant bits over a CTA's rows; CTAs are summed in FP64. FP64
+// arithmetic runs at a small fraction of the FP32 rate on this GPU, so this
+// is several times faster than FP64 FMAs. The _rn operations keep the
+// compiler from contracting the error-free transformations.
+// Bound by the FP32 pipe (ten operations a product, issued as packed pairs); chunks
+// of rows arrive by asynchronous copies during the sums of the chunk before. Measured
+// (n = 1e6, c = 144): 4.5 ms with scalar operations and a barrier between load and
+// sums, 3.7 now; n = 10,312: 64 -> 59 us. Sums on a fixed grid per chunk (a shift
+// above the running sum: four operations, 1.65 ms) were given up: their error is
+// relative to the columns' norms instead of to the sum, and the changed rounding
+// moved tuning scores (each a count of decisions, some of them near ties). Picking
+// the larger operand by compare and select (three operations fewer): 4.2 ms.
 // ---------------------------------------------------------------------------
 constexpr int kGramRows = 64;   // rows of a chunk (two buffers of them are staged)
 
 constexpr int kGramThreads = 384;
 
+// Paired FP32 arithmetic (f32x2, sm_100 and later): one instruction for two lanes
+// of a float2, each rounded as the scalar operation.
 __device__ __forceinline__ float2 f2_add(float2 a, float2 b) {
     uint64_t d;
     asm("add.rn.f32x2 %0, %1, %2;"
@@ -99,12 +98,20 @@ __device__ __forceinline__ float2 f2_sub(float2 a, float2 b) {
         : "l"(reinterpret_cast<const uint64_t &>(a)), "l"(reinterpret_cast<const uint64_t &>(b)));
     return reinterpret_cast<const float2 &>(d);
 }
-
-// C of an entry: 3 u_a u_b, or 0 where that is not finite (h then is a plain
-// running sum and lo collects what it rounds off).
-__device__ __forceinline__ float gram_shift(float ua, float ub) {
-    const float c = 3.0f * (ua * ub);
-    return c < 3.0e38f ? c : 0.f;
+__device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(d)
+        : "l"(reinterpret_cast<const uint64_t &>(a)), "l"(reinterpret_cast<const uint64_t &>(b)),
+          "l"(reinterpret_cast<const uint64_t &>(c)));
+    return reinterpret_cast<const float2 &>(d);
+}
+__device__ __forceinline__ float2 f2_mul(float2 a, float2 b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;"
+        : "=l"(d)
+        : "l"(reinterpret_cast<const uint64_t &>(a)), "l"(reinterpret_cast<const uint64_t &>(b)));
+    return reinterpret_cast<const float2 &>(d);
 }
 
 // VEC: rows are read by 16-byte copies (c, ld multiples of 4, Y 16-byte aligned).
@@ -112,15 +119,11 @@ template <bool VEC>
 __global__ void __launch_bounds__(kGramThreads) gram_partial_kernel(const float *__restrict__ Y, int64_t n, int c,
                                                                     int64_t ld, int64_t rows_per_cta,
                                                                     double *__restrict__ partial) {
-    // two chunks of kGramRows x cp, u of every column, then the threads' entry
-    // pairs (hi and lo of 4 x 8 entries, touched once a chunk)
-    extern __shared__ __align__(16) float ys[];
+    extern __shared__ __align__(16) float ys[];   // two chunks of kGramRows x cp
     const int cp = (c + 7) & ~7;
     const int nt = cp / 8;
     const int nitems = nt * (nt + 1);   // (tile, half): rows 0-3 or 4-7 of an 8x8 tile
     const int tid = threadIdx.x;
-    float *us = ys + 2 * kGramRows * cp;
-    float2 *acc = reinterpret_cast<float2 *>(us + cp) + tid;   // entry pair q: hi at q, lo at 16 + q (x kGramThreads)
     const int64_t r0 = (int64_t)blockIdx.x * rows_per_cta;
     const int64_t r1 = imin64(n, r0 + rows_per_cta);
     for (int e = tid; e < 2 * kGramRows * (cp - c); e += kGramThreads) {   // padding columns
@@ -162,8 +165,11 @@ __global__ void __launch_bounds__(kGramThreads) gram_partial_kernel(const float 
             tj = ti + rem;
         }
         const int xa = ti * 8 + half * 4;
+        float2 hi[4][4], lo[4][4];
 #pragma unroll
-        for (int q = 0; q < 32; ++q) acc[q * kGramThreads] = make_float2(0.f, 0.f);
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) hi[x][y] = lo[x][y] = make_float2(0.f, 0.f);
         __syncthreads();   // the last group's chunks are done
         if (r0 < r1) stage(r0, ys);
         int buf = 0;
@@ -177,30 +183,7 @@ __global__ void __launch_bounds__(kGramThreads) gram_partial_kernel(const float 
                 asm volatile("cp.async.wait_group 0;" ::: "memory");
             }
             __syncthreads();
-            if (tid < cp) {   // u: a power of two above the norm of column tid
-                float s = 0.f;
-#pragma unroll 8
-                for (int r = 0; r < rows; ++r) s = fmaf(yb[r * cp + tid], yb[r * cp + tid], s);
-                // s (1 + 2^-10) in [2^E, 2^(E+1)): its root is below 2^(floor(E / 2) + 1)
-                const int E = (int)((__float_as_uint(s * 1.0009765625f) >> 23) & 0xFF) - 127;
-                us[tid] = s > 0.f ? __uint_as_float((uint32_t)((E >> 1) + 1 + 127) << 23) : 0.f;
-            }
-            __syncthreads();
             if (active) {
-                float2 h[4][4], l[4][4];
-                float2 ub[4];
-#pragma unroll
-                for (int y = 0; y < 4; ++y) ub[y] = *reinterpret_cast<const float2 *>(us + tj * 8 + 2 * y);
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    const float ua = us[xa + x];
-#pragma unroll
-                    for (int y = 0; y < 4; ++y) {
-                        h[x][y] = make_float2(gram_shift(ua, ub[y].x), gram_shift(ua, ub[y].y));
-                        l[x][y] = make_float2(0.f, 0.f);
-                    }
-                }
-#pragma unroll 2
                 for (int r = 0; r < rows; ++r) {
                     const float *yr = yb + r * cp;
                     const float4 a4 = *reinterpret_cast<const float4 *>(yr + xa);
@@ -211,34 +194,21 @@ __global__ void __launch_bounds__(kGramThreads) gram_partial_kernel(const float 
                                           make_float2(b1.z, b1.w)};
 #pragma unroll
                     for (int x = 0; x < 4; ++x) {
-                        const float2 a2 = make_float2(av[x], av[x]);
+                        const float2 a2 = make_float2(av[x], av[x]), na2 = make_float2(-av[x], -av[x]);
 #pragma unroll
                         for (int y = 0; y < 4; ++y) {
-                            float2 hn = h[x][y];
-                            f2_add_prod(hn, a2, bv[y]);
-                            float2 e = f2_sub(h[x][y], hn);   // exact: both on the chunk's grid
-                            f2_add_prod(e, a2, bv[y]);        // what the addition rounded off
-                            l[x][y] = f2_add(l[x][y], e);
-                            h[x][y] = hn;
+                            const float2 p = f2_mul(a2, bv[y]);
+                            const float2 ne = f2_fma(na2, bv[y], p);   // p - a b
+                            const float2 h = hi[x][y], s = f2_add(h, p);
+                            const float2 bb = f2_sub(s, h);
+                            const float2 err = f2_add(f2_sub(h, f2_sub(s, bb)), f2_sub(p, bb));
+                            hi[x][y] = s;
+                            lo[x][y] = f2_add(lo[x][y], f2_sub(err, ne));
                         }
                     }
                 }
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    const float ua = us[xa + x];
-#pragma unroll
-                    for (int y = 0; y < 4; ++y) {
-                        const float2 sh = make_float2(gram_shift(ua, ub[y].x), gram_shift(ua, ub[y].y));
-                        const float2 v = f2_sub(h[x][y], sh);   // exact
-                        float2 *at = acc + (x * 4 + y) * kGramThreads;
-                        const float2 o = at[0], s = f2_add(o, v), bb = f2_sub(s, o);
-                        const float2 err = f2_add(f2_sub(o, f2_sub(s, bb)), f2_sub(v, bb));
-                        at[0] = s;
-                        at[16 * kGramThreads] = f2_add(at[16 * kGramThreads], f2_add(err, l[x][y]));
-                    }
-                }
             }
-            __syncthreads();   // this buffer and u are rewritten next
+            __syncthreads();   // this buffer is rewritten next
         }
         if (active) {
             double *P = partial + (int64_t)blockIdx.x * cp * cp;
@@ -246,9 +216,8 @@ __global__ void __launch_bounds__(kGramThreads) gram_partial_kernel(const float 
             for (int x = 0; x < 4; ++x)
 #pragma unroll
                 for (int y = 0; y < 4; ++y) {
-                    const float2 hi = acc[(x * 4 + y) * kGramThreads], lo = acc[(16 + x * 4 + y) * kGramThreads];
-                    P[(xa + x) * cp + tj * 8 + 2 * y] = (double)hi.x + (double)lo.x;
-                    P[(xa + x) * cp + tj * 8 + 2 * y + 1] = (double)hi.y + (double)lo.y;
+                    P[(xa + x) * cp + tj * 8 + 2 * y] = (double)hi[x][y].x + (double)lo[x][y].x;
+                    P[(xa + x) * cp + tj * 8 + 2 * y + 1] = (double)hi[x][y].y + (double)lo[x][y].y;
                 }
         }
     }
@@ -296,27 +265,33 @@ __global__ void gram_reduce_kernel(const double *__restrict__ partial, int nblk,
     }
 }
 
-// 1/sqrt(a) of a positive normal FP64 pivot: one step of third order
-// y <- y + y e (1/2 + 3/8 e), e = 1 - a y^2, from an FP32 estimate (e is about
-// 2^-22, so the error left, 5/16 e^3, is below 2^-53). FP64 instructions take
-// some 64 cycles each on this GPU, conversions too: the estimate is taken of a's
-// upper bits scaled into [1, 4) by integer arithmetic and put back the same way,
-// which leaves four dependent FP64 operations.
+// 1/sqrt(a) of a positive finite FP64 pivot by two Newton steps
+// y <- y (3 - a y^2) / 2 from the FP32 estimate (which has 24 bits; two steps
+// pass FP64's 53), so no FP64 square root or division runs on this GPU's
+// narrow FP64 pipe. FP64 instructions take some 64 cycles each, conversions too: the
+// FP32 rounding of the pivot and the estimate's FP64 form are taken on the bits
+// where both are normal floats; pivots outside FP32's range take the plain route.
 __device__ __forceinline__ double pivot_rsqrt(double a) {
-    const int hi = __double2hiint(a), lo = __double2loint(a);
-    const int e = (hi >> 20) - 1023, odd = e & 1;   // a = 2^e (1.f)
-    if (e == -1023) return 1.0 / sqrt(a);           // subnormal
-    const uint32_t m = ((uint32_t)(hi & 0xFFFFF) << 3) | ((uint32_t)lo >> 29);
-    const uint32_t y32 = __float_as_uint(rsqrtf(__uint_as_float(((uint32_t)(127 + odd) << 23) | m)));
-    const int ye = (int)(y32 >> 23) - 127 - ((e - odd) >> 1) + 1023;
-    const double y = __hiloint2double((ye << 20) | (int)((y32 & 0x7FFFFFu) >> 3), (int)(y32 << 29));
-    const double t = fma(-(a * y), y, 1.0);
-    return fma(y * t, fma(0.375, t, 0.5), y);
+    const uint64_t bits = (uint64_t)__double_as_longlong(a);
+    const int e = (int)(bits >> 52) - 1023;
+    double y;
+    if (e >= -126 && e < 127) {   // rounded to nearest even: at most 2^127
+        uint32_t f = (uint32_t)((bits >> 29) - ((uint64_t)896 << 23));
+        const uint32_t rest = (uint32_t)bits & 0x1FFFFFFFu;
+        f += rest > 0x10000000u || (rest == 0x10000000u && (f & 1u)) ? 1u : 0u;
+        const uint32_t r = __float_as_uint(rsqrtf(__uint_as_float(f)));
+        y = __longlong_as_double((long long)(((uint64_t)r + ((uint64_t)896 << 23)) << 29));
+    } else {
+        y = (double)rsqrtf((float)a);
+        if (!(y > 0.0) || !isfinite(y)) return 1.0 / sqrt(a);
+    }
+    y = y * fma(-0.5 * a, y * y, 1.5);
+    return y * fma(-0.5 * a, y * y, 1.5);
 }
 
 constexpr int kMaxSmemC = 160;   // largest c of the small SVD
-constexpr int kOaSteps = 4;      // refinement steps at most
-constexpr int kOaSync = 8;       // words: grid barrier, then each step's largest correction (FP32 bits); two spare
+constexpr int kOaSteps = 4;      // refinement steps
+constexpr int kOaSync = 8;       // words: grid barrier; two are lne_svd_small_noalloc's status, the others spare
 
 // ---------------------------------------------------------------------------
 // Cholesky (upper, G = R^T R) in FP64, 16 x 16 tiles, one CTA per block column.
@@ -849,98 +824,40 @@ __global__ void jacobi32_kernel(const double *__restrict__ R, int c, double *__r
     if (tid == 0 && sweeps_out) *sweeps_out = sweep;
 }
 
-// Register-resident variant of the same Jacobi (c <= 144). The columns go in
-// blocks of two; each 8-thread group holds a pair of blocks in registers (E
-// elements per column and thread, as float2 chunks: element 16 q + 2 sub +
-// {0, 1}) and makes the four rotations between them, two at a time, before the
-// blocks move on through a shared exchange buffer. The rotations W are not
-// accumulated here: every rotation's (cos, sin) and column labels are recorded,
-// and jacobi_replay_kernel applies them to the identity afterwards, one row of W
-// per warp on many SMs (the rows of W evolve independently).
+// Register-resident variant of the same Jacobi (c <= 144). Each 8-thread
+// group holds its pair of columns of A in registers (E elements per column
+// and thread, as float2 chunks: element 16 q + 2 sub + {0, 1}), so a round
+// reads nothing from shared memory; columns move between groups through a
+// shared exchange buffer only when the pairing changes. The rotations W are
+// not accumulated here: every round's (cos, sin) and column labels are
+// recorded, and jacobi_replay_kernel applies them to the identity afterwards,
+// one row of W per warp on many SMs (the rows of W evolve independently).
 //
-// The order of the block pairs is chosen so that most rounds move one block of
-// each pair instead of both: a sweep over m = 2G blocks takes the blocks in slot
+// The pairing order is chosen so that most rounds move one column of each
+// pair instead of both: a sweep over m = 2G columns takes the columns in slot
 // 0 as a set X and those in slot 1 as Y, and pairs X[i] with Y[(i + r) mod G]
 // for r = 0..G-1 (only Y moves, one group along); then X and Y are each split
 // in halves and the same is done inside X and inside Y in parallel, and so on
 // while the set size is even. Sets of odd size s then finish with s rounds of
-// the circle method (one block of each set idle per round). Every pair of blocks
-// meets exactly once per sweep, the two columns of a block at its start; the
-// layout a sweep ends with is the next sweep's starting point, and a label per
-// column records which column of R^T it started as.
-//
-// One CTA, so a round is a chain: dot products, shuffles, the angle, the
-// update, the exchange. What shortens it: a rotation scales its columns lazily
-// (a0 <- a0 - t (d1 / d0) a1, a1 <- a1 + t (d0 / d1) a0, d <- cos d: one FMA an
-// entry) and keeps the squared norms up (only the dot product is formed: a
-// third of the sums and shuffles; both are refreshed at every level of a sweep,
-// two rounds' worth of work), and blocks of two halve the bytes that cross
-// shared memory per rotation, whose wavefronts (650 cycles a round of 72
-// columns of 144 entries, written and read) were the longest link with one
-// column a move. Straight-line code makes both rotations' chains overlap, with
-// one-instruction approximations where only the angle's quality depends on them.
-// Measured (start and replay of a random factor): c = 32 127 -> 90 us, c = 48
-// 211 -> 143, c = 128 990 -> 671, c = 144 1343 -> 1032 (0.25 us a round up to
-// c = 64, 0.68 at 144; the replay is 29 to 139 us of it).
+// the circle method (one column of each set idle per round). Every pair meets
+// exactly once per sweep; the layout a sweep ends with is the next sweep's
+// starting point, and a label per column records which column of R^T it
+// started as.
+// Blocks of two columns a move with lazily scaled rotations and kept norms took 0.6
+// (c = 32) to 0.8 (c = 144) of the time and were given up: the squares of squared
+// norms that their test formed underflow for columns below 3e-9 of the largest, which
+// then were not rotated, and another order of rotations moves tuning scores.
 constexpr int kJacRegMaxC = 144;
 constexpr int kJacMaxSweeps = 20;
 
-// blocks of two columns, padded to an even number
-__host__ __device__ constexpr int jreg_blocks(int c) { return ((c + 1) / 2 + 1) / 2 * 2; }
-// floats of an exchange entry (two columns and their labels, norms and scales);
-// = 16 mod 32, so that neighbouring groups' float2 accesses hit distinct banks
-__host__ __device__ constexpr int jreg_stride(int E) { return 16 * E + 16; }
-// rounds of disjoint rotations per sweep for m blocks, m rotations each
-__host__ __device__ inline int jreg_rounds(int m) { return 2 * jorder_rounds(m) + 1; }
-
-// Paired FP32 arithmetic (fma.rn.f32x2 / mul.rn.f32x2, sm_100 and later):
-// one instruction for two lanes of a float2, each rounded as the scalar op.
-__device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) {
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;"
-        : "=l"(d)
-        : "l"(*reinterpret_cast<const uint64_t *>(&a)), "l"(*reinterpret_cast<const uint64_t *>(&b)),
-          "l"(*reinterpret_cast<const uint64_t *>(&c)));
-    return *reinterpret_cast<const float2 *>(&d);
-}
-__device__ __forceinline__ float2 f2_mul(float2 a, float2 b) {
-    uint64_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;"
-        : "=l"(d)
-        : "l"(*reinterpret_cast<const uint64_t *>(&a)), "l"(*reinterpret_cast<const uint64_t *>(&b)));
-    return *reinterpret_cast<const float2 *>(&d);
-}
-
-// Approximate square root, reciprocal and reciprocal square root (2 ulp or so),
-// denormals taken as zero: one instruction each.
-__device__ __forceinline__ float fast_sqrt(float x) {
-    float y;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float fast_rcp(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float fast_rsqrt(float x) {
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// One column of a group's pair of blocks: the calling thread's entries of it,
-// the column being scale * v, its squared norm, and the column of R^T it
-// started as.
 template <int E>
-struct JacCol {
-    float2 v[E / 2];
-    float nrm, scl;
-    int lab;
-};
+__host__ __device__ constexpr int jreg_stride() { return ((8 * E + 31) / 32) * 32 + 16; }
+
+// rounds per sweep of the order above for m (even) columns
+__host__ __device__ inline int jreg_rounds(int m) { return jorder_rounds(m); }
 
 template <int E>
-__global__ void __launch_bounds__(16 * E, 1) jacobi_reg_kernel(const double *__restrict__ R, int c,
+__global__ void __launch_bounds__(32 * E, 1) jacobi_reg_kernel(const double *__restrict__ R, int c,
                                                                double *__restrict__ Vout,
                                                                float2 *__restrict__ rot,
                                                                uint32_t *__restrict__ rlab, int max_sweeps,
@@ -948,176 +865,106 @@ __global__ void __launch_bounds__(16 * E, 1) jacobi_reg_kernel(const double *__r
     constexpr int CP = 8 * E;            // padded column length
     constexpr int NQ = E / 2;            // float2 chunks per column and thread
     static_assert(E % 2 == 0, "columns are held as float2 chunks");
-    constexpr int ST = jreg_stride(E);   // floats per exchange entry: two columns, then their labels, norms, scales
-    extern __shared__ __align__(16) float xb[];   // 2 G entries
+    constexpr int ST = jreg_stride<E>(); // floats per exchange entry (= 16 mod 32: conflict-free float2)
+    extern __shared__ float xb[];        // 2 G entries: column [CP], label at CP
     __shared__ float red[32];
-    const int m = jreg_blocks(c), G = m / 2, SUB = jreg_rounds(m);
+    __shared__ int s_done;
+    const int m = c + (c & 1), G = m / 2, RD = jreg_rounds(m);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = tid >> 3, sub = tid & 7;
     const bool real = g < G;             // groups past G only fill the last warp
-    JacCol<E> A[2], B[2];                // the blocks in slots 0 and 1
-    float big = 0.f;
+    // element 2 q + t of a column is component t of chunk q (rows 16 q + 2 sub + t)
+    float2 a0[NQ], a1[NQ];
+    int lab0 = g, lab1 = g + G;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        JacCol<E> &x = k < 2 ? A[k & 1] : B[k & 1];
-        x.lab = 2 * (k < 2 ? g : g + G) + (k & 1);
-        x.nrm = 0.f;
-        const bool live = real && x.lab < c;   // column lab of R^T
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            const int i = 16 * q + 2 * sub;
-            x.v[q].x = live && i < c ? (float)R[(size_t)x.lab * c + i] : 0.f;
-            x.v[q].y = live && i + 1 < c ? (float)R[(size_t)x.lab * c + i + 1] : 0.f;
-            big = fmaxf(big, fmaxf(fabsf(x.v[q].x), fabsf(x.v[q].y)));
-        }
+    for (int q = 0; q < NQ; ++q) {
+        const int i = 16 * q + 2 * sub;
+        const bool r0 = real && lab0 < c, r1 = real && lab1 < c;   // column lab of R^T
+        a0[q].x = r0 && i < c ? (float)R[(size_t)lab0 * c + i] : 0.f;
+        a0[q].y = r0 && i + 1 < c ? (float)R[(size_t)lab0 * c + i + 1] : 0.f;
+        a1[q].x = r1 && i < c ? (float)R[(size_t)lab1 * c + i] : 0.f;
+        a1[q].y = r1 && i + 1 < c ? (float)R[(size_t)lab1 * c + i + 1] : 0.f;
     }
-    // scaled by a power of two so that the largest entry is in [1, 2): squares of
-    // squared norms stay in FP32's range, and nothing that is kept depends on it
-    big = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(big)));
-    if (lane == 0) red[warp] = big;
-    __syncthreads();
-    for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) big = fmaxf(big, red[w]);
-    const uint32_t bexp = __float_as_uint(big) >> 23;
-    const float unit = bexp >= 1 && bexp <= 253 ? __uint_as_float((254u - bexp) << 23) : 1.f;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) A[k].scl = B[k].scl = unit;   // multiplied in by the first renormalisation
     // stop at cosines of 0.4 c ulp (at least 8 ulp): the FP64 refinement's first-order
     // step needs the start's rotations this close where singular values are dense
     const float tol = fmaxf(0.4f * (float)c, 8.f) * 5.9604645e-8f;
     const int tz = jorder_levels(m);
     const int s_odd = m >> tz;           // set size the halving ends at
-    const float tol2 = tol * tol;
-    bool rotated = false;                // a pair above the tolerance in this sweep
-    size_t rec = 0;                      // this round's first record
+    float local_max = 0.f;
+    int rec = 0;                         // record index of this round's group 0
 
-    auto put = [&](int entry, const JacCol<E> (&x)[2]) {
+    auto put = [&](int entry, const float2 (&a)[NQ], int lab) {
         float *eb = xb + (size_t)entry * ST;
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) *reinterpret_cast<float2 *>(eb + k * CP + 16 * q + 2 * sub) = x[k].v[q];
-            if (sub == k)
-                *reinterpret_cast<float4 *>(eb + 2 * CP + 4 * k) =
-                    make_float4(__int_as_float(x[k].lab), x[k].nrm, x[k].scl, 0.f);
-        }
+        for (int q = 0; q < NQ; ++q) *reinterpret_cast<float2 *>(eb + 16 * q + 2 * sub) = a[q];
+        if (sub == 0) reinterpret_cast<int *>(eb)[CP] = lab;
     };
-    auto take = [&](int entry, JacCol<E> (&x)[2]) {
+    auto take = [&](int entry, float2 (&a)[NQ], int &lab) {
         const float *eb = xb + (size_t)entry * ST;
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) x[k].v[q] = *reinterpret_cast<const float2 *>(eb + k * CP + 16 * q + 2 * sub);
-            const float4 t = *reinterpret_cast<const float4 *>(eb + 2 * CP + 4 * k);
-            x[k].lab = __float_as_int(t.x);
-            x[k].nrm = t.y;
-            x[k].scl = t.z;
-        }
+        for (int q = 0; q < NQ; ++q) a[q] = *reinterpret_cast<const float2 *>(eb + 16 * q + 2 * sub);
+        lab = reinterpret_cast<const int *>(eb)[CP];
     };
-    // both blocks of every group move (sources as group * 2 + slot)
+    // both columns of every group move (sources as group * 2 + slot)
     auto move_both = [&](int src0, int src1) {
         __syncthreads();
         if (real) {
-            put(2 * g, A);
-            put(2 * g + 1, B);
+            put(2 * g, a0, lab0);
+            put(2 * g + 1, a1, lab1);
         }
         __syncthreads();
         if (real) {
-            take(src0, A);
-            take(src1, B);
+            take(src0, a0, lab0);
+            take(src1, a1, lab1);
         }
         __syncthreads();
     };
-    // scales multiplied in, squared norms from the entries
-    auto renorm = [&](JacCol<E> &x) {
-        float2 n2 = make_float2(0.f, 0.f);
-        const float2 d = make_float2(x.scl, x.scl);
+    // one rotation of the group's pair (every lane takes part in the shuffles),
+    // recorded as (cos, sin) = (1, 0) when the pair is left as it is
+    auto rotate = [&](bool active) {
+        float2 al2 = make_float2(0.f, 0.f), be2 = al2, ga2 = al2;
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
-            x.v[q] = f2_mul(d, x.v[q]);
-            n2 = f2_fma(x.v[q], x.v[q], n2);
+            al2 = f2_fma(a0[q], a0[q], al2);
+            be2 = f2_fma(a1[q], a1[q], be2);
+            ga2 = f2_fma(a0[q], a1[q], ga2);
         }
-        float n = n2.x + n2.y;
-#pragma unroll
-        for (int off = 1; off < 8; off <<= 1) n += __shfl_xor_sync(0xffffffffu, n, off);
-        x.nrm = n;
-        x.scl = 1.f;
-    };
-    auto renorm_all = [&]() {
-        renorm(A[0]);
-        renorm(A[1]);
-        renorm(B[0]);
-        renorm(B[1]);
-    };
-    // one round: the rotations of the pairs (x0, y0) and (x1, y1), recorded as
-    // (cos, sin) = (1, 0) where a pair is left as it is. Straight-line code for
-    // both pairs at once, so that their chains overlap; t = tan of the angle
-    // = 2 g / (d + sign(d) sqrt(d^2 + 4 g^2)) for the dot product g and the squared
-    // norms' difference d. It only steers the convergence (approximate sqrt and
-    // division); (cos, sin) is a unit vector.
-    auto rotate = [&](JacCol<E> &x0, JacCol<E> &y0, JacCol<E> &x1, JacCol<E> &y1, bool active) {
-        JacCol<E> *const xs[2] = {&x0, &x1}, *const ys[2] = {&y0, &y1};
-        float ga[2], t[2], cs[2], r[2], ri[2];
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            float2 a = make_float2(0.f, 0.f), b = a;
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                if (q & 1) b = f2_fma(xs[k]->v[q], ys[k]->v[q], b);
-                else a = f2_fma(xs[k]->v[q], ys[k]->v[q], a);
-            }
-            ga[k] = (a.x + a.y) + (b.x + b.y);
-            r[k] = ys[k]->scl * fast_rcp(xs[k]->scl);
-            ri[k] = xs[k]->scl * fast_rcp(ys[k]->scl);
-        }
+        float al = al2.x + al2.y, be = be2.x + be2.y, ga = ga2.x + ga2.y;
 #pragma unroll
         for (int off = 1; off < 8; off <<= 1) {
-            ga[0] += __shfl_xor_sync(0xffffffffu, ga[0], off);
-            ga[1] += __shfl_xor_sync(0xffffffffu, ga[1], off);
+            al += __shfl_xor_sync(0xffffffffu, al, off);
+            be += __shfl_xor_sync(0xffffffffu, be, off);
+            ga += __shfl_xor_sync(0xffffffffu, ga, off);
         }
+        float cs = 1.f, sn = 0.f;
+        if (active && ga != 0.f && al > 0.f && be > 0.f) {
+            const float rel = fabsf(ga) * rsqrtf(al * be);
+            local_max = fmaxf(local_max, rel);
+            if (rel > tol) {
+                const float zeta = (be - al) / (2.f * ga);
+                const float t = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
+                cs = rsqrtf(1.f + t * t);
+                sn = cs * t;
+                const float2 c2 = make_float2(cs, cs), s2 = make_float2(sn, sn), ms2 = make_float2(-sn, -sn);
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            JacCol<E> &x = *xs[k], &y = *ys[k];
-            const float g1 = ga[k] * (x.scl * y.scl), g2 = g1 + g1, d = y.nrm - x.nrm;
-            const float tk = (d < 0.f ? -g2 : g2) * fast_rcp(fabsf(d) + fast_sqrt(fmaf(d, d, g2 * g2)));
-            const bool go = active && g1 * g1 > tol2 * (x.nrm * y.nrm) && x.nrm > 0.f && y.nrm > 0.f;
-            rotated = rotated || go;
-            t[k] = go ? tk : 0.f;
-            cs[k] = go ? fast_rsqrt(fmaf(tk, tk, 1.f)) : 1.f;
-            ga[k] = g1;
-        }
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            JacCol<E> &x = *xs[k], &y = *ys[k];
-            const float2 k0 = make_float2(-t[k] * r[k], -t[k] * r[k]), k1 = make_float2(t[k] * ri[k], t[k] * ri[k]);
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                const float2 u = x.v[q];
-                x.v[q] = f2_fma(k0, y.v[q], u);
-                y.v[q] = f2_fma(k1, u, y.v[q]);
-            }
-            x.scl *= cs[k];
-            y.scl *= cs[k];
-            x.nrm = fmaxf(fmaf(-t[k], ga[k], x.nrm), 0.f);
-            y.nrm = fmaxf(fmaf(t[k], ga[k], y.nrm), 0.f);
-            if (real && sub == 4 * k) {
-                rot[rec + 2 * g + k] = make_float2(cs[k], cs[k] * t[k]);
-                rlab[rec + 2 * g + k] = (uint32_t)x.lab | ((uint32_t)y.lab << 16);
+                for (int q = 0; q < NQ; ++q) {
+                    const float2 x = a0[q], y = a1[q];
+                    a0[q] = f2_fma(c2, x, f2_mul(ms2, y));   // cs x - sn y
+                    a1[q] = f2_fma(c2, y, f2_mul(s2, x));    // sn x + cs y
+                }
             }
         }
-        rec += m;
-    };
-    // the four rotations between a group's two blocks
-    auto cross = [&](bool active) {
-        rotate(A[0], B[0], A[1], B[1], active);
-        rotate(A[0], B[1], A[1], B[0], active);
+        if (real && sub == 0) {
+            rot[(size_t)rec + g] = make_float2(cs, sn);
+            rlab[(size_t)rec + g] = (uint32_t)lab0 | ((uint32_t)lab1 << 16);
+        }
+        rec += G;
     };
 
     int sweep = 0, par = 0;
     for (; sweep < max_sweeps; ++sweep) {
-        rotated = false;
-        rec = (size_t)sweep * SUB * m;
-        renorm_all();
-        rotate(A[0], A[1], B[0], B[1], true);   // inside the blocks
+        local_max = 0.f;
+        rec = sweep * RD * G;
         for (int lev = 0; lev < tz; ++lev) {
             const int h = m >> (lev + 1);   // ring length: pairs per set and rounds of this level
             if (lev > 0) {
@@ -1125,54 +972,71 @@ __global__ void __launch_bounds__(16 * E, 1) jacobi_reg_kernel(const double *__r
                 int src0, src1;
                 jorder_split_sources(g, h, src0, src1);
                 move_both(src0, src1);   // every thread reaches the same barriers
-                renorm_all();
             }
-            const int ks = jorder_ring_source(g, h);   // slot-1 block comes from the next group
+            const int ks = jorder_ring_source(g, h);   // slot-1 column comes from the next group
             for (int r = 0; r < h; ++r) {
                 if (r > 0) {
                     // double-buffered halves: one barrier per round
-                    if (real) put(par * G + g, B);
+                    if (real) put(par * G + g, a1, lab1);
                     __syncthreads();
-                    if (real) take(par * G + ks, B);
+                    if (real) take(par * G + ks, a1, lab1);
                     par ^= 1;
                 }
-                cross(true);
+                rotate(true);
             }
         }
         if (s_odd > 1) {
             // circle method inside each set of odd size s: positions 1..k paired
             // with s-1..k+1 in k groups per set, position 0 idle (the two sets
-            // that share a parent put their idle blocks in one group)
+            // that share a parent put their idle columns in one group)
             const int s = s_odd;
             int e0, e1, r0, r1;
             bool idle;
             jorder_tail_sources(g, s, e0, e1, r0, r1, idle);
             for (int r = 0; r < s; ++r) {
                 move_both(r == 0 ? e0 : r0, r == 0 ? e1 : r1);
-                if (r == 0) renorm_all();
-                cross(!idle);
+                rotate(!idle);
             }
         }
-        if (!__syncthreads_or(rotated)) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) local_max = fmaxf(local_max, __shfl_xor_sync(0xffffffffu, local_max, off));
+        if (lane == 0) red[warp] = local_max;
+        __syncthreads();
+        if (tid == 0) {
+            float mx = 0.f;
+            for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) mx = fmaxf(mx, red[w]);
+            s_done = mx <= tol;
+        }
+        __syncthreads();
+        if (s_done) {
             ++sweep;
             break;
         }
     }
     // right singular vectors of R: normalised columns of R^T W, by label
-    renorm_all();
+    float2 n02 = make_float2(0.f, 0.f), n12 = n02;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        n02 = f2_fma(a0[q], a0[q], n02);
+        n12 = f2_fma(a1[q], a1[q], n12);
+    }
+    float n0 = n02.x + n02.y, n1 = n12.x + n12.y;
+#pragma unroll
+    for (int off = 1; off < 8; off <<= 1) {
+        n0 += __shfl_xor_sync(0xffffffffu, n0, off);
+        n1 += __shfl_xor_sync(0xffffffffu, n1, off);
+    }
+    const float q0 = n0 > 0.f ? rsqrtf(n0) : 0.f, q1 = n1 > 0.f ? rsqrtf(n1) : 0.f;
     if (real) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const JacCol<E> &x = k < 2 ? A[k & 1] : B[k & 1];
-            const float inv = x.nrm > 0.f ? rsqrtf(x.nrm) : 0.f;
-            if (x.lab >= c) continue;
+        for (int q = 0; q < NQ; ++q)
 #pragma unroll
-            for (int q = 0; q < NQ; ++q) {
-                const int i = 16 * q + 2 * sub;
-                if (i < c) Vout[(size_t)i * c + x.lab] = (double)(x.v[q].x * inv);
-                if (i + 1 < c) Vout[(size_t)(i + 1) * c + x.lab] = (double)(x.v[q].y * inv);
+            for (int t = 0; t < 2; ++t) {
+                const int i = 16 * q + 2 * sub + t;
+                const float x0 = t ? a0[q].y : a0[q].x, x1 = t ? a1[q].y : a1[q].x;
+                if (i < c && lab0 < c) Vout[(size_t)i * c + lab0] = (double)(x0 * q0);
+                if (i < c && lab1 < c) Vout[(size_t)i * c + lab1] = (double)(x1 * q1);
             }
-        }
     }
     if (tid == 0 && sweeps_out) *sweeps_out = sweep;
 }
@@ -1279,21 +1143,21 @@ __global__ void __launch_bounds__(kRpWarps * 32) jacobi_replay_kernel(const floa
 
 // records a Jacobi run on c <= kJacRegMaxC columns may write
 inline size_t jreg_records(int c) {
-    const int m = jreg_blocks(c);
-    return (size_t)kJacMaxSweeps * jreg_rounds(m) * m;
+    const int m = c + (c & 1);
+    return (size_t)kJacMaxSweeps * jreg_rounds(m) * (m / 2);
 }
 
 template <int E>
 int launch_jacobi_reg_e(const double *R, int c, double *U, double *V, float2 *rot, uint32_t *rlab, int *sweeps,
                         unsigned *sync, cudaStream_t st) {
-    const int m = jreg_blocks(c);
+    const int m = c + (c & 1);
     const int threads = ((m / 2) * 8 + 31) / 32 * 32;
-    const int smem = m * jreg_stride(E) * (int)sizeof(float);
+    const int smem = m * jreg_stride<E>() * (int)sizeof(float);
     if (smem > 48 * 1024) LNE_TRY(allow_dynamic_smem(jacobi_reg_kernel<E>));
     jacobi_reg_kernel<E><<<1, threads, smem, st>>>(R, c, V, rot, rlab, kJacMaxSweeps, sweeps);
     LNE_LAUNCH_CHECK();
-    jacobi_replay_kernel<<<(unsigned)ceil_div(c, kRpWarps), kRpWarps * 32, 0, st>>>(rot, rlab, m, jreg_rounds(m),
-                                                                                  sweeps, c, U, sync);
+    jacobi_replay_kernel<<<(unsigned)ceil_div(c, kRpWarps), kRpWarps * 32, 0, st>>>(
+        rot, rlab, m / 2, jreg_rounds(m), sweeps, c, U, sync);
     LNE_LAUNCH_CHECK();
     return 0;
 }
@@ -1337,16 +1201,14 @@ int launch_jacobi(const double *R, int c, double *U, double *V, float2 *rot, uin
 // delta = 2 (||offdiag T|| + max|s| (||P|| + ||Q||)). A itself is never squared,
 // so the accuracy does not depend on the condition number of A.
 //
-// Up to kOaSteps steps in one cooperative launch: quadratic convergence, but the
+// kOaSteps steps in one cooperative launch: quadratic convergence, but the
 // FP32 start may be loose in directions FP32 cannot resolve. A step is four
 // phases between grid barriers: P, Q (upper tiles, mirrored) and W = A V; T =
-// U^T W with sigma and the norms' partial sums; F and G; U + U F and V + V G. The
-// step whose corrections are all below 2^-43 is the last (the next one would be
-// below rounding, and T, which the cluster step reads, is U's to 2^-42); usually
-// the third. Bound by FP64 at large c (per step 6 c^3 multiply-adds at 2 a cycle
-// and SM: 29 us at c = 144) and by barriers and load latency at small c; as four
-// products and two element passes of their own launches a step took 38 us at
-// c = 32 and 84 us at 144.
+// U^T W with sigma and the norms' partial sums; F and G; U + U F and V + V G.
+// Bound by FP64 at large c (per step 6 c^3 multiply-adds at 2 a cycle and SM: 29 us
+// at c = 144) and by barriers and load latency at small c. Measured, all steps: c =
+// 32 83 us, c = 144 313; as four products and two element passes of their own
+// launches a step 190 and 335.
 // A 64-thread group takes an 8 x 8 tile: its 8 rows of op(A) and 8 columns of B
 // over the whole k range go to shared memory at once (one round of load
 // latency), then each thread runs its dot product.
@@ -1476,7 +1338,6 @@ __global__ void __launch_bounds__(kOaThreads) svd_refine_kernel(OaArgs A) {
         }
         __syncthreads();
         const double delta = s_delta;
-        float big = 0.f;
         for (int e = blockIdx.x * kOaThreads + tid; e < c * c; e += gridDim.x * kOaThreads) {
             const int i = e / c, j = e - i * c;
             const double pij = __ldcg(A.P + e), qij = __ldcg(A.Q + e);
@@ -1501,12 +1362,9 @@ __global__ void __launch_bounds__(kOaThreads) svd_refine_kernel(OaArgs A) {
             }
             A.F[e] = f;
             A.G[e] = g;
-            big = fmaxf(big, fmaxf(fabsf((float)f), fabsf((float)g)));
         }
-        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(big));
-        if (lane == 0 && m) atomicMax(A.sync + 1 + it, m);
         if (!grid_barrier(A.sync, target, A.status)) return;
-        const bool last = it + 1 == kOaSteps || __uint_as_float(__ldcg(A.sync + 1 + it)) <= 0x1p-43f;
+        const bool last = it + 1 == kOaSteps;
         // U + U F (the last step's goes to `out`), V + V G
         double *to = last ? A.out : U2;
         for (int q = g0; q < (last ? 1 : 2) * nt * nt; q += ng) {
@@ -1919,11 +1777,13 @@ static int gram(Workspace &ws, const float *Y, int64_t n, int c, int64_t ld, dou
     const int cp = (c + 7) & ~7;
     const int threads = kGramThreads;
     const bool vec = c % 4 == 0 && ld % 4 == 0 && reinterpret_cast<uintptr_t>(Y) % 16 == 0;
-    const int smem = (2 * kGramRows * cp + cp + 64 * kGramThreads) * 4;   // cp <= 240: 217 KB
+    const int smem = 2 * kGramRows * cp * 4;   // cp <= 240: 120 KB
     LNE_TRY(vec ? allow_dynamic_smem(gram_partial_kernel<true>) : allow_dynamic_smem(gram_partial_kernel<false>));
-    // whole waves of resident CTAs (one per SM at this kernel's register use)
+    // whole waves of resident CTAs (one per SM at this kernel's register use). The
+    // split of the rows is part of the result: sums of other blocks round differently
     const int64_t slots = num_sms();
-    int64_t nblk = std::min<int64_t>(slots, std::max<int64_t>(1, ceil_div(n, 32)));
+    int64_t nblk = std::min<int64_t>(2 * slots, std::max<int64_t>(1, ceil_div(n, 64)));
+    if (nblk > slots) nblk = (nblk / slots) * slots;
     const int64_t rows_per = ceil_div(std::max<int64_t>(n, 1), nblk);
     nblk = ceil_div(std::max<int64_t>(n, 1), rows_per);
     double *partial = nullptr;
@@ -1951,7 +1811,7 @@ static int gram(Workspace &ws, const float *Y, int64_t n, int c, int64_t ld, dou
 // G comes from gram() on the same stream, whose reduction zeroes the tile
 // counters. Measured (c = 32 / 48 / 144): one CTA with a rank-1 update and three
 // barriers a pivot took 27 / 44 us, one cooperative launch with grid barriers
-// between panels 159 us at c = 144; now 20 / 32 / 106 us.
+// between panels 159 us at c = 144; now 27 / 41 / 123 us (the pivot's chain).
 static int chol(Workspace &ws, const double *G, int c, double *R, cudaStream_t st) {
     int *status = nullptr;
     unsigned *cnt = nullptr;
@@ -2182,10 +2042,10 @@ namespace {
 
 constexpr int kNoAllocMaxC = 160;
 constexpr size_t kNoAllocMat = (size_t)kNoAllocMaxC * kNoAllocMaxC;
-constexpr size_t kNoAllocRec = (size_t)kJacMaxSweeps * (kJacRegMaxC + 2) * (kJacRegMaxC / 2);   // >= jreg_records(c)
+constexpr size_t kNoAllocRec = (size_t)kJacMaxSweeps * kJacRegMaxC * (kJacRegMaxC / 2);   // >= jreg_records(c)
 constexpr size_t kNoAllocSmall = 4 * kOaMaxCtas + 16;   // norm partials; sweep count and sync words
 constexpr size_t kNoAllocDoubles = 10 * kNoAllocMat + kNoAllocMaxC + kNoAllocSmall + kNoAllocRec + kNoAllocRec / 2;
-static_assert((kOaSync + 2) * sizeof(unsigned) <= 16 * sizeof(double) && kOaSteps + 3 <= kOaSync, "the words fit the reserve");
+static_assert((kOaSync + 2) * sizeof(unsigned) <= 16 * sizeof(double) && kOaSync >= 3, "the words fit the reserve");
 static __device__ __align__(256) double g_svd_scratch[kNoAllocDoubles];
 
 constexpr int kNoAllocMaxDevices = 64;

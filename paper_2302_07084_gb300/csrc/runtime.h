@@ -170,8 +170,11 @@ int sparsifier_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Csr
 
 // ---- dense and sparse linear algebra (dense.cu, spmm.cu) -------------------
 int gaussian_sketch(int64_t n, int c, uint64_t seed, float *out, int64_t ld, cudaStream_t st);
+// eight: products of up to 16 columns may take eight nonzeros a warp step, whose sums
+// have another order. For a product that is asked for as such: the randomized SVD's
+// keep the order of four, since tuning scores step where a last bit tips a near tie.
 int spmm(Workspace &ws, const CsrView &M, const float *X, int64_t ldx, int c, float *Y, int64_t ldy,
-         cudaStream_t st);
+         cudaStream_t st, bool eight = false);
 // Y := Q in place; R (optional, device FP64 [c][c]) receives the upper factor.
 int cholqr2(Workspace &ws, float *Y, int64_t n, int c, int64_t ld, double *R, cudaStream_t st);
 // One CholeskyQR pass: Q = Y chol(Y^T Y)^-1 (FP64 Gram and Cholesky, FP32 Q).
@@ -218,6 +221,7 @@ struct SpmmEpilogue {
     uint32_t *row_cnt = nullptr;
     const int32_t *slice_row = nullptr;
     int64_t max_row = 0;                // the longest row, if known: short rows take a lane group each
+    bool eight = false;                 // weighted products of up to 16 columns: eight nonzeros a warp step
 };
 // Device status words of the context (workspace "dev.status", zeroed when
 // created): [0] the first Cholesky breakdown, [1] a tensor-core pipeline wait
@@ -249,7 +253,7 @@ int graph_spmm(Workspace &ws, const GraphView &g, const float *X, int64_t ldx, i
                const SpmmEpilogue &ep, cudaStream_t st);
 // The same products with a BF16 dense operand (FP32 accumulation); c % 4 == 0.
 int spmm_bf16(Workspace &ws, const CsrView &M, const __nv_bfloat16 *X, int64_t ldx, int c, float *Y, int64_t ldy,
-              __nv_bfloat16 *Yb, cudaStream_t st);
+              __nv_bfloat16 *Yb, cudaStream_t st, bool eight = false);
 int graph_spmm_bf16(Workspace &ws, const GraphView &g, const __nv_bfloat16 *X, int64_t ldx, int c, float *Y,
                     int64_t ldy, const SpmmEpilogue &ep, cudaStream_t st);
 // out[i] = bf16(in[i]) for count elements.

@@ -733,11 +733,11 @@ int launch_merge(Workspace &ws, int64_t n, int64_t nnz, const int64_t *indptr, c
     }
     // weighted products with at most 16 float4 column groups: several nonzeros
     // per warp step (the graph products keep one, so batched propagation sums
-    // in the same order as a single candidate's). Up to 16 columns eight of them:
-    // 1.9e8 nonzeros, 16 columns 2.56 ms with four (half the lanes idle), 1.74 with
-    // eight, 1.61 with the next indices loaded ahead; 64 bytes of X a nonzero from
-    // L2 bound it
-    if (WEIGHTED && c4 <= 4) LNE_MERGE_GROUPED(4)
+    // in the same order as a single candidate's). Up to 16 columns eight of them
+    // where ep.eight allows that order of the sums: 1.9e8 nonzeros, 16 columns
+    // 2.56 ms with four (half the lanes idle), 1.74 with eight, 1.61 with the next
+    // indices loaded ahead; 64 bytes of X a nonzero from L2 bound it
+    if (WEIGHTED && c4 <= 4 && ep.eight) LNE_MERGE_GROUPED(4)
     else if (WEIGHTED && c4 <= 8) LNE_MERGE_GROUPED(8)
     else if (WEIGHTED && c4 <= 16) LNE_MERGE_GROUPED(16)
     else switch (nv) {
@@ -974,9 +974,10 @@ int merge_chain_prepare(const GraphView &g, uint32_t *row_cnt, int32_t *slice_ro
 }
 
 int spmm(Workspace &ws, const CsrView &M, const float *X, int64_t ldx, int c, float *Y, int64_t ldy,
-         cudaStream_t st) {
+         cudaStream_t st, bool eight) {
     SpmmEpilogue ep;
     ep.lde = ldy;
+    ep.eight = eight;
     if (M.vb && merge_ok(X, ldx, c, Y, ldy, ep)) return launch_merge_vb<float>(ws, M, X, ldx, c, Y, ldy, ep, st);
     if (merge_ok(X, ldx, c, Y, ldy, ep))
         return launch_merge<true, float>(ws, M.n, M.nnz, M.indptr, M.indices, M.data, X, ldx, c, Y, ldy, ep, st);
@@ -984,9 +985,10 @@ int spmm(Workspace &ws, const CsrView &M, const float *X, int64_t ldx, int c, fl
 }
 
 int spmm_bf16(Workspace &ws, const CsrView &M, const __nv_bfloat16 *X, int64_t ldx, int c, float *Y, int64_t ldy,
-              __nv_bfloat16 *Yb, cudaStream_t st) {
+              __nv_bfloat16 *Yb, cudaStream_t st, bool eight) {
     SpmmEpilogue ep;
     ep.lde = ldy;
+    ep.eight = eight;
     ep.Yb = Yb;
     if (!merge_ok(X, ldx, c, Y, ldy, ep)) return fail(LNE_ERR_UNSUPPORTED, "BF16 operands need c and ld multiples of 4");
     if (M.vb) return launch_merge_vb<__nv_bfloat16>(ws, M, X, ldx, c, Y, ldy, ep, st);
