@@ -115,7 +115,10 @@ __device__ __forceinline__ unsigned same_digit(uint32_t d) {
 
 // One pass. Tiles are taken in order from a counter, so the tiles a tile waits
 // for are running or done. A wait gives up after 2 s, sets status[1] and the CTA
-// ends without writing (as do those that find it set).
+// ends without writing its keys, as do CTAs that find it set while they wait. A CTA
+// that finds it set when it starts does nothing: after a pass that gave up its
+// output holds stale words, whose digits were never counted and would be placed
+// past the buffers' ends.
 template <bool VALS>
 __global__ void __launch_bounds__(kPassThreads, VALS ? 3 : 4) radix_pass_kernel(
     const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin, int64_t n, int shift, int pass,
@@ -131,10 +134,11 @@ __global__ void __launch_bounds__(kPassThreads, VALS ? 3 : 4) radix_pass_kernel(
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
         s_tile = atomicAdd(next_tile, 1u);
-        s_fail = 0;
+        s_fail = *reinterpret_cast<volatile int *>(status + 1);
     }
     for (int e = tid; e < kPassWarps * 256; e += kPassThreads) s_wc[e >> 8][e & 255] = 0;
     __syncthreads();
+    if (s_fail) return;
     const int64_t tile = s_tile, i0 = tile * kPassTile;
     const int nt = (int)imin64(kPassTile, n - i0);
     // the warp's 512 consecutive keys, all requested up front
