@@ -54,27 +54,33 @@ __device__ __forceinline__ void f2_add_prod(float2 &acc, float2 a, float2 b) {
         : "l"(reinterpret_cast<const uint64_t &>(a)), "l"(reinterpret_cast<const uint64_t &>(b)));
 }
 
-// A barrier over the grid of a cooperative launch (all CTAs resident). Gives
-// up after 2 s: status[1] is set and every CTA returns false, after which the
-// kernel ends.
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &target, int *status) {
+// A barrier over the grid of a cooperative launch (all CTAs resident); the word's low
+// 63 bits count arrivals, the top bit says that a CTA gave up. A CTA gives up after
+// limit_ns: it sets status[1] and the top bit and returns false, after which the kernel
+// ends. CTAs that wait then or arrive later find the bit and return false too; those
+// that had left the barrier before do so at their next one. What a launch has written
+// is valid only if status[1] is 0 afterwards.
+__device__ __forceinline__ bool grid_barrier(uint64_t *bar, uint64_t &target, int *status,
+                                             uint64_t limit_ns = 2000000000ull) {
     __shared__ int ok_s;
     __syncthreads();
     target += gridDim.x;
     if (threadIdx.x == 0) {
         int ok = 1;
-        unsigned v;
+        uint64_t v;
         __threadfence();
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(bar) : "memory");
         uint64_t t0 = 0;
         for (unsigned spin = 1;; ++spin) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if ((int)(v - target) >= 0) break;   // the count may wrap
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(bar) : "memory");
+            if ((int64_t)v < 0) ok = 0;
+            if ((int64_t)v < 0 || v >= target) break;
             if ((spin & 63u) == 0u) {
                 uint64_t t;
                 asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
                 if (t0 == 0) t0 = t;
-                if (t - t0 > 2000000000ull) {
+                if (t - t0 > limit_ns) {
+                    atomicOr(reinterpret_cast<unsigned long long *>(bar), 1ull << 63);
                     atomicExch(status + 1, 1);
                     ok = 0;
                     break;

@@ -291,7 +291,7 @@ __device__ __forceinline__ double pivot_rsqrt(double a) {
 
 constexpr int kMaxSmemC = 160;   // largest c of the small SVD
 constexpr int kOaSteps = 4;      // refinement steps
-constexpr int kOaSync = 8;       // words: grid barrier; two are lne_svd_small_noalloc's status, the others spare
+constexpr int kOaSync = 8;       // words: two of the grid barrier; two are lne_svd_small_noalloc's status, the others spare
 
 // ---------------------------------------------------------------------------
 // Cholesky (upper, G = R^T R) in FP64, 16 x 16 tiles, one CTA per block column.
@@ -1220,7 +1220,7 @@ struct OaArgs {
     const double *R;
     double *U, *U2, *V, *V2, *W, *T, *P, *Q, *F, *G, *out, *sig;
     double *part;       // 4 per CTA
-    unsigned *sync;     // kOaSync words, zeroed
+    unsigned *sync;     // kOaSync words, zeroed, 8-byte aligned
     int *status;        // [1] is set where a barrier gave up
     int c;
 };
@@ -1259,7 +1259,7 @@ __global__ void __launch_bounds__(kOaThreads) svd_refine_kernel(OaArgs A) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, grp = tid >> 6, gt = tid & 63;
     const int g0 = blockIdx.x * kOaGroups + grp, ng = gridDim.x * kOaGroups;
     const int tx = gt % kOaTile, ty = gt / kOaTile;
-    unsigned target = 0;
+    uint64_t target = 0, *const bar = reinterpret_cast<uint64_t *>(A.sync);   // the first two words
     double *U = A.U, *U2 = A.U2, *V = A.V, *V2 = A.V2;
     for (int it = 0; it < kOaSteps; ++it) {
         // P = I - U^T U, Q = I - V^T V, W = R V
@@ -1288,7 +1288,7 @@ __global__ void __launch_bounds__(kOaThreads) svd_refine_kernel(OaArgs A) {
                 to[col * c + row] = v;
             }
         }
-        if (!grid_barrier(A.sync, target, A.status)) return;
+        if (!grid_barrier(bar, target, A.status)) return;
         // T = U^T W; sigma; partial sums of |offdiag T|^2, |P|^2, |Q|^2 and max |sigma|
         double o2 = 0.0, p2 = 0.0, q2 = 0.0, smax = 0.0;
         for (int q = g0; q < nt * nt; q += ng) {
@@ -1321,7 +1321,7 @@ __global__ void __launch_bounds__(kOaThreads) svd_refine_kernel(OaArgs A) {
             for (int w = 1; w < kOaThreads / 32; ++w) v = tid < 3 ? v + red[tid][w] : fmax(v, red[tid][w]);
             A.part[4 * blockIdx.x + tid] = v;
         }
-        if (!grid_barrier(A.sync, target, A.status)) return;
+        if (!grid_barrier(bar, target, A.status)) return;
         // F and G, an element per thread
         if (warp == 0) {
             double s[4] = {0.0, 0.0, 0.0, 0.0};
@@ -1363,7 +1363,7 @@ __global__ void __launch_bounds__(kOaThreads) svd_refine_kernel(OaArgs A) {
             A.F[e] = f;
             A.G[e] = g;
         }
-        if (!grid_barrier(A.sync, target, A.status)) return;
+        if (!grid_barrier(bar, target, A.status)) return;
         const bool last = it + 1 == kOaSteps;
         // U + U F (the last step's goes to `out`), V + V G
         double *to = last ? A.out : U2;
@@ -1374,7 +1374,7 @@ __global__ void __launch_bounds__(kOaThreads) svd_refine_kernel(OaArgs A) {
             if (row < c && col < c) (v ? V2 : to)[row * c + col] = __ldcg((v ? V : U) + row * c + col) + acc;
         }
         if (last) return;
-        if (!grid_barrier(A.sync, target, A.status)) return;
+        if (!grid_barrier(bar, target, A.status)) return;
         double *x = U;
         U = U2;
         U2 = x;
@@ -2045,7 +2045,7 @@ constexpr size_t kNoAllocMat = (size_t)kNoAllocMaxC * kNoAllocMaxC;
 constexpr size_t kNoAllocRec = (size_t)kJacMaxSweeps * kJacRegMaxC * (kJacRegMaxC / 2);   // >= jreg_records(c)
 constexpr size_t kNoAllocSmall = 4 * kOaMaxCtas + 16;   // norm partials; sweep count and sync words
 constexpr size_t kNoAllocDoubles = 10 * kNoAllocMat + kNoAllocMaxC + kNoAllocSmall + kNoAllocRec + kNoAllocRec / 2;
-static_assert((kOaSync + 2) * sizeof(unsigned) <= 16 * sizeof(double) && kOaSync >= 3, "the words fit the reserve");
+static_assert((kOaSync + 2) * sizeof(unsigned) <= 16 * sizeof(double) && kOaSync >= 4, "the words fit the reserve");
 static __device__ __align__(256) double g_svd_scratch[kNoAllocDoubles];
 
 constexpr int kNoAllocMaxDevices = 64;

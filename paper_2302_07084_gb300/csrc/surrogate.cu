@@ -536,7 +536,7 @@ struct TrainArgs {
     int64_t n_rows, batch;
     int epochs;
     float *Xs2;
-    unsigned *bar;
+    uint64_t *bar;
     int *status;
 };
 
@@ -544,7 +544,7 @@ template <int R>
 __global__ void __launch_bounds__(kThreads, 1) sur_train_kernel(TrainArgs T) {
     extern __shared__ __align__(16) char sm[];
     const RowBufs<R> b(sm);
-    unsigned target = 0;
+    uint64_t target = 0;
     const int64_t nb = (T.n_rows + T.batch - 1) / T.batch, steps = nb * T.epochs;
     const int64_t first = (int64_t)blockIdx.x * R;
     auto batch_of = [&](int64_t s) {
@@ -846,7 +846,7 @@ int surrogate_train(Surrogate &S, Workspace &ws, const float *X, const float *t,
     int32_t *idx = nullptr;
     float2 *corr = nullptr;
     float *xs2 = nullptr;
-    unsigned *bar = nullptr;
+    uint64_t *bar = nullptr;
     int *status = nullptr;
     LNE_TRY(ws.get("sur.idx", (size_t)rows * most, &idx));
     LNE_TRY(ws.get("sur.corr", (size_t)nb * most, &corr));
@@ -889,7 +889,7 @@ int surrogate_train(Surrogate &S, Workspace &ws, const float *X, const float *t,
         if (e0 > 0) LNE_CUDA_TRY(cudaStreamSynchronize(st));
         LNE_CUDA_TRY(cudaMemcpyAsync(idx, perm.data(), sizeof(int32_t) * perm.size(), cudaMemcpyHostToDevice, st));
         LNE_CUDA_TRY(cudaMemcpyAsync(corr, hc.data(), sizeof(float2) * hc.size(), cudaMemcpyHostToDevice, st));
-        LNE_CUDA_TRY(cudaMemsetAsync(bar, 0, sizeof(unsigned), st));
+        LNE_CUDA_TRY(cudaMemsetAsync(bar, 0, sizeof(uint64_t), st));
         LNE_TRACE("sur_train", st);
         const int64_t per = ceil_div(B, num_sms());
         if (per <= 2) LNE_TRY(launch_train<2>(T, st));

@@ -24,3 +24,7 @@ def _run(tmp_path, name):
 
 def test_sort_after_an_expired_wait_writes_nothing(tmp_path):
     _run(tmp_path, "sort_after_timeout")
+
+
+def test_late_cta_leaves_a_given_up_barrier(tmp_path):
+    _run(tmp_path, "grid_barrier_late")
