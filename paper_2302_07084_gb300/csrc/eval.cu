@@ -9,12 +9,13 @@
 //   partials  r = C (sigma(yz) - 1) y, D = C sigma (1 - sigma); X^T r and
 //             X^T diag(D) X of a block of 128 rows and one label, FP32
 //   sums      G = W + sum of the X^T r blocks (FP64), H = I + sum of the
-//             X^T D X blocks (error-free float pairs)
+//             X^T D X blocks (three floats a sum, as good as FP64)
 //   update    W_l -= H_l^-1 G_l to FP64 accuracy: FP32 Cholesky, FP64 residuals
 #include <algorithm>
 #include <cmath>
 #include <vector>
 
+#include "float_sum.h"
 #include "runtime.h"
 
 namespace lne {
@@ -175,9 +176,11 @@ __device__ __forceinline__ void pair_add(float &hi, float &lo, float p) {
 }
 
 // H_l = I + sum_b hpart[b][l] (both triangles; FP64 in H, as a float pair in
-// Hp) and G = W + sum_b gpart[b] (FP64). The Hessian's sums over the row blocks are error-free float pairs
-// (two-sum; the pair holds about 46 bits): FP64 additions and conversions run
-// at 1/64 of the FP32 rate on this GPU and would bound this pass.
+// Hp) and G = W + sum_b gpart[b] (FP64). The Hessian's sums over the row blocks are
+// running sums in three floats (float_sum.h), as good as FP64 ones: FP64 additions and
+// conversions run at 1/64 of the FP32 rate on this GPU and would bound this pass. A sum
+// past FP32's range is taken in FP64. Measured (d = 128, 39 labels, 41 row blocks): 24.7
+// us a step; sums in two floats, 46 bits, 22.3.
 template <int TS>
 __global__ void __launch_bounds__(256) newton_reduce_kernel(const float *__restrict__ gpart,
                                                             const float *__restrict__ hpart, int nblk, int da, int L,
@@ -195,14 +198,20 @@ __global__ void __launch_bounds__(256) newton_reduce_kernel(const float *__restr
         const int a = ti * TS + q / TS, c = tj * TS + q % TS;
         if (a <= c && c < da) {
             const float *src = hpart + (int64_t)l * total + e;
-            float hi = a == c ? 1.f : 0.f, lo = 0.f;
+            FloatSum sum = {a == c ? 1.f : 0.f, 0.f, 0.f};
 #pragma unroll 16
-            for (int b = 0; b < nblk; ++b) pair_add(hi, lo, src[b * stride]);
-            const float s = __fadd_rn(hi, lo);
-            lo = __fsub_rn(lo, __fsub_rn(s, hi));   // |lo| <= |hi|: exact
+            for (int b = 0; b < nblk; ++b) float_sum_add(sum, src[b * stride]);
+            double h = float_sum_value(sum);
+            if (!(fabs(h) <= 3.0e38)) {   // past FP32's range, or not finite
+                h = a == c ? 1.0 : 0.0;
+                for (int b = 0; b < nblk; ++b) h += (double)src[b * stride];
+            }
             const int64_t at = (int64_t)l * da * da;
-            H[at + a * da + c] = H[at + c * da + a] = (double)s + (double)lo;
-            Hp[at + a * da + c] = Hp[at + c * da + a] = make_float2(s, lo);
+            H[at + a * da + c] = H[at + c * da + a] = h;
+            const float s = __fadd_rn(sum.hi, sum.lo);
+            float rest = __fsub_rn(sum.lo, __fsub_rn(s, sum.hi));   // |lo| <= |hi|: exact
+            rest = __fadd_rn(rest, sum.tail);
+            Hp[at + a * da + c] = Hp[at + c * da + a] = make_float2(s, rest);
         }
     } else if (e - total < da) {
         const int a = e - total;
