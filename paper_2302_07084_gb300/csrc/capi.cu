@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <set>
 #include <utility>
@@ -142,22 +143,81 @@ void trace_end(cudaStream_t st) {
     r.closed = true;
 }
 
-// Bytes of all workspaces' retired buffers.
-static std::atomic<int64_t> g_idle_bytes{0};
+namespace {
+// One pool of scratch memory per device. Allocations and frees go through a stream of
+// its own that is waited for, so that a buffer may be used on any stream between them.
+struct ScratchPool {
+    cudaMemPool_t pool = nullptr;
+    cudaStream_t st = nullptr;
+};
+std::mutex g_pool_mu;
+std::map<int, ScratchPool> g_pools;
 
+// The current device's pool; create: made if there is none yet.
+int scratch_pool(bool create, ScratchPool *out) {
+    int dev = 0;
+    LNE_CUDA_TRY(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    ScratchPool &sp = g_pools[dev];
+    if (!sp.pool && create) {
+        size_t unused = 0, total = 0;
+        LNE_CUDA_TRY(cudaMemGetInfo(&unused, &total));
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        if (!sp.st) LNE_CUDA_TRY(cudaStreamCreateWithFlags(&sp.st, cudaStreamNonBlocking));
+        cudaMemPool_t pool = nullptr;
+        LNE_CUDA_TRY(cudaMemPoolCreate(&pool, &props));
+        uint64_t keep = total / 8;
+        const cudaError_t e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(pool);
+            return cuda_fail("cudaMemPoolSetAttribute", e, __FILE__, __LINE__);
+        }
+        sp.pool = pool;
+    }
+    *out = sp;
+    return 0;
+}
+
+int out_of_memory(size_t want, const std::string &name, cudaError_t e) {
+    cudaGetLastError();
+    char buf[256];
+    std::snprintf(buf, sizeof(buf), "device allocation of %zu bytes for '%s' failed: %s", want, name.c_str(),
+                  cudaGetErrorString(e));
+    g_msg = buf;
+    return LNE_ERR_OOM;
+}
+}  // namespace
+
+void trim_scratch() {
+    ScratchPool sp;
+    if (scratch_pool(false, &sp) != 0 || !sp.pool) return;
+    if (cudaStreamSynchronize(sp.st) != cudaSuccess || cudaMemPoolTrimTo(sp.pool, 0) != cudaSuccess) cudaGetLastError();
+}
+
+// Work on a pooled buffer has ended (give_back and settle wait for it, and so do the
+// callers of release()).
 void Workspace::free_buf(Buf &b) {
-    if (b.idle) g_idle_bytes -= (int64_t)b.bytes;
-    if (b.p) cudaFree(b.p);
+    ScratchPool sp;
+    if (b.p && b.pooled && scratch_pool(false, &sp) == 0) cudaFreeAsync(b.p, sp.st);
+    else if (b.p) cudaFree(b.p);
     b = Buf();
+}
+
+// After an allocation failed: frees the retired buffers and the unused scratch memory.
+void Workspace::make_room() {
+    cudaGetLastError();
+    for (auto &kv : bufs_)
+        if (kv.second.idle) free_buf(kv.second);
+    trim_scratch();
 }
 
 int Workspace::get(const std::string &name, size_t bytes, void **ptr) {
     if (bytes == 0) bytes = 1;
     Buf &b = bufs_[name];
-    if (b.idle) {
-        g_idle_bytes -= (int64_t)b.bytes;
-        b.idle = false;
-    }
+    b.idle = false;
     if (b.bytes < bytes) {
         if (b.p) {
             cudaError_t e = cudaFree(b.p);
@@ -169,29 +229,66 @@ int Workspace::get(const std::string &name, size_t bytes, void **ptr) {
         size_t want = bytes + std::min(bytes / 8, (size_t)1 << 28);
         want = (want + 255) & ~(size_t)255;
         cudaError_t e = cudaMalloc(&b.p, want);
-        if (e == cudaErrorMemoryAllocation) {   // once more without the retired buffers
-            cudaGetLastError();
-            bool freed = false;
-            for (auto &kv : bufs_) {
-                if (!kv.second.idle) continue;
-                free_buf(kv.second);
-                freed = true;
-            }
-            if (freed) e = cudaMalloc(&b.p, want);
+        if (e == cudaErrorMemoryAllocation) {
+            make_room();
+            e = cudaMalloc(&b.p, want);
         }
         if (e != cudaSuccess) {
-            cudaGetLastError();
             b.p = nullptr;
-            char buf[256];
-            std::snprintf(buf, sizeof(buf), "device allocation of %zu bytes for '%s' failed: %s", want,
-                          name.c_str(), cudaGetErrorString(e));
-            g_msg = buf;
-            return LNE_ERR_OOM;
+            return out_of_memory(want, name, e);
         }
         b.bytes = want;
     }
     *ptr = b.p;
     return 0;
+}
+
+int Workspace::temp(const std::string &name, size_t bytes, void **ptr) {
+    if (bytes == 0) bytes = 1;
+    Buf &b = bufs_[name];
+    if (b.bytes < bytes) {
+        ScratchPool sp;
+        LNE_TRY(scratch_pool(true, &sp));
+        if (b.p) {   // taken before in this call
+            LNE_CUDA_TRY(cudaDeviceSynchronize());
+            free_buf(b);
+        }
+        const size_t want = (bytes + 255) & ~(size_t)255;
+        cudaError_t e = cudaMallocFromPoolAsync(&b.p, want, sp.pool, sp.st);
+        if (e == cudaErrorMemoryAllocation) {
+            make_room();
+            e = cudaMallocFromPoolAsync(&b.p, want, sp.pool, sp.st);
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(sp.st);
+        if (e != cudaSuccess) {
+            b.p = nullptr;
+            return out_of_memory(want, name, e);
+        }
+        b.bytes = want;
+        b.pooled = true;
+    }
+    *ptr = b.p;
+    return 0;
+}
+
+int Workspace::give_back(std::initializer_list<const char *> names, cudaStream_t st) {
+    LNE_CUDA_TRY(cudaStreamSynchronize(st));
+    for (const char *name : names) release(name);
+    return 0;
+}
+
+void Workspace::settle() {
+    bool waited = false;
+    for (auto it = bufs_.begin(); it != bufs_.end();) {
+        if (!it->second.pooled) {
+            ++it;
+            continue;
+        }
+        if (!waited) cudaDeviceSynchronize();
+        waited = true;
+        free_buf(it->second);
+        it = bufs_.erase(it);
+    }
 }
 
 void Workspace::release() {
@@ -207,23 +304,11 @@ void Workspace::release(const std::string &name) {
 }
 
 void Workspace::retire(const std::string &name) {
-    static const int64_t kKeep = [] {
-        int dev = 0;
-        cudaDeviceProp prop;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return (int64_t)0;
-        return (int64_t)(prop.totalGlobalMem / 8);
-    }();
     auto it = bufs_.find(name);
-    if (it == bufs_.end() || it->second.idle) return;
-    const int64_t size = (int64_t)it->second.bytes;
-    if (size > kKeep / 8) {
-        release(name);
-    } else if ((g_idle_bytes += size) > kKeep) {
-        g_idle_bytes -= size;
-        release(name);
-    } else {
-        it->second.idle = true;
-    }
+    if (it == bufs_.end()) return;
+    size_t unused = 0, total = 0;
+    if (cudaMemGetInfo(&unused, &total) == cudaSuccess && it->second.bytes <= total / 64) it->second.idle = true;
+    else release(name);
 }
 
 int64_t Workspace::bytes() const {
@@ -258,6 +343,8 @@ int finish(lne_ctx *ctx, int rc) {
     if (rc != 0) {
         ctx->err = lne::last_message();
         if (ctx->err.empty()) ctx->err = "unknown error";
+        ctx->ws.settle();
+        for (auto &w : ctx->workers) w->ws.settle();
     }
     return rc;
 }
@@ -421,6 +508,7 @@ void lne_destroy(lne_ctx *ctx) {
     if (ctx->prop_graph) lne::destroy_prop_cache(ctx->prop_graph);
     ctx->workers.clear();
     ctx->ws.release();
+    lne::trim_scratch();
     delete ctx;
 }
 
@@ -530,6 +618,7 @@ int lne_trim(lne_ctx *ctx) {
         ctx->prop_graph = nullptr;
         ctx->workers.clear();
         ctx->ws.release();
+        lne::trim_scratch();
     }
     return finish(ctx, rc);
 }

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
 #include <map>
 #include <memory>
 #include <string>
@@ -31,24 +32,43 @@ public:
     bool has(const std::string &name) const { return bufs_.count(name) != 0; }
     // Frees one named buffer (no-op if absent).
     void release(const std::string &name);
-    // Done with a named buffer until the next get() of it (no-op if absent). Kept,
-    // contents undefined, if it takes at most 1/64 of the device's memory and all
-    // workspaces together then keep at most 1/8 of it this way, else freed; a
-    // workspace's kept ones are freed when one of its allocations fails. Freeing and allocating the sort path's buffers on
-    // every call took 8 of 26 ms at 2e8 samples (7 GB); a run of tens of GB still
-    // hands them back as it goes.
+    // The contents of a buffer that the context holds between calls are not needed any
+    // more (no-op if absent): freed if it takes more than 1/64 of the device's memory, else
+    // reused by the next get(), or freed when an allocation of this workspace fails.
     void retire(const std::string &name);
+    // A buffer that a call hands back before it returns (give_back): taken from the
+    // device's scratch pool, one for all contexts of the process. What has been handed
+    // back stays mapped up to 1/8 of the device's memory, and the driver takes it for any
+    // other allocation of the process that would fail without it; trim_scratch unmaps it.
+    // At 2e8 samples (7 GB of buffers) a sparsifier takes 18.9 ms this way, 17.9 where
+    // each context kept its buffers mapped, 26 where they were freed and allocated on
+    // every call; a run of tens of GB still hands them back as it goes.
+    int temp(const std::string &name, size_t bytes, void **ptr);
+    template <typename T>
+    int temp(const std::string &name, size_t count, T **ptr) {
+        return temp(name, count * sizeof(T), reinterpret_cast<void **>(ptr));
+    }
+    // Waits for the stream that has used the buffers and hands them back (absent names
+    // are skipped).
+    int give_back(std::initializer_list<const char *> names, cudaStream_t st);
+    // After a call that failed: waits for the device and hands back what the call still
+    // had, so that no such buffer outlives the call that took it.
+    void settle();
     int64_t bytes() const;
 
 private:
     struct Buf {
         void *p = nullptr;
         size_t bytes = 0;
-        bool idle = false;   // retired
+        bool pooled = false;   // from the scratch pool
+        bool idle = false;     // retired
     };
     static void free_buf(Buf &b);
+    void make_room();
     std::map<std::string, Buf> bufs_;
 };
+// Unmaps what the current device's scratch pool holds and nobody uses.
+void trim_scratch();
 
 struct GraphView {
     int64_t n = 0;
@@ -447,7 +467,7 @@ int stratified_sample(Workspace &ws, const GraphView &g, const SamplerSpec &sp, 
 // The candidate sp's sparsifier (its s, b) from the strata.
 int stratified_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, const Strata &S, CsrResult *out,
                    cudaStream_t st);
-void stratified_release(Workspace &ws);
+int stratified_release(Workspace &ws, cudaStream_t st);
 
 // Number of keys of a sorted array below `key` (synchronises).
 int count_below(Workspace &ws, const uint64_t *keys, int64_t n, uint64_t key, int64_t *count, cudaStream_t st);

@@ -2656,7 +2656,7 @@ struct Table {
 
 // Samples of every arc as 64-bit keys, sorted, as unique keys with counts.
 // On return the unique keys are in *uk ("sort.k0" or "sort.k1"), counts in
-// "sort.cnt"; the other key buffer is retired. With edge
+// "sort.cnt"; the other key buffer is handed back. With edge
 // downsampling each key carries its arc, a dropped draw's key is all ones
 // (sorted past every pair: the sort takes one more bit when n = 2^B, where the
 // all-ones pair of B-bit halves is a real vertex pair), and *w gets the summed
@@ -2687,12 +2687,12 @@ int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *
     LNE_TRY(tile_offsets(ws, A, 0, g.nnz, tile_arcs, &tile_off, &total, st));
     R->total = total;
     uint64_t *k0 = nullptr, *k1 = nullptr;
-    LNE_TRY(ws.get("sort.k0", (size_t)std::max<int64_t>(total, 1), &k0));
-    LNE_TRY(ws.get("sort.k1", (size_t)std::max<int64_t>(total, 1), &k1));
+    LNE_TRY(ws.temp("sort.k0", (size_t)std::max<int64_t>(total, 1), &k0));
+    LNE_TRY(ws.temp("sort.k1", (size_t)std::max<int64_t>(total, 1), &k1));
     uint32_t *arc0 = nullptr, *arc1 = nullptr;
     if (ds) {
-        LNE_TRY(ws.get("sort.a0", (size_t)std::max<int64_t>(total, 1), &arc0));
-        LNE_TRY(ws.get("sort.a1", (size_t)std::max<int64_t>(total, 1), &arc1));
+        LNE_TRY(ws.temp("sort.a0", (size_t)std::max<int64_t>(total, 1), &arc0));
+        LNE_TRY(ws.temp("sort.a1", (size_t)std::max<int64_t>(total, 1), &arc1));
     }
     {
         LNE_TRACE("walk_keys", st);
@@ -2703,34 +2703,30 @@ int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *
     bool in_alt = false;
     LNE_TRY(radix_sort_u64(ws, k0, k1, arc0, arc1, total, 0, bits, &in_alt, st));
     uint64_t *sorted = in_alt ? k1 : k0, *spare = in_alt ? k0 : k1;
-    ws.retire("sort.words");
+    LNE_TRY(ws.give_back({"sort.words"}, st));
     if (ds) {
         // the dropped draws sort last: run lengths over the kept ones only
         int64_t kept = 0;
         LNE_TRY(count_below(ws, sorted, total, ~0ull, &kept, st));
-        LNE_TRY(ws.get("sort.w", (size_t)std::max<int64_t>(kept, 1), &R->w));
+        LNE_TRY(ws.temp("sort.w", (size_t)std::max<int64_t>(kept, 1), &R->w));
         LNE_TRY(run_length_weighted(ws, sorted, in_alt ? arc1 : arc0, A.ds_w, kept, spare, R->w, &R->U, st));
-        ws.retire("sort.a0");
-        ws.retire("sort.a1");
-        LNE_TRY(ws.get("sort.cnt", (size_t)std::max<int64_t>(R->U, 1), &R->cnt));
+        LNE_TRY(ws.give_back({"sort.a0", "sort.a1"}, st));
+        LNE_TRY(ws.temp("sort.cnt", (size_t)std::max<int64_t>(R->U, 1), &R->cnt));
     } else {
-        LNE_TRY(ws.get("sort.cnt", (size_t)std::max<int64_t>(total, 1), &R->cnt));
+        LNE_TRY(ws.temp("sort.cnt", (size_t)std::max<int64_t>(total, 1), &R->cnt));
         LNE_TRY(run_length(ws, sorted, total, spare, R->cnt, &R->U, st));
     }
-    LNE_CUDA_TRY(cudaStreamSynchronize(st));
     R->uk = spare;
     R->uk_name = in_alt ? "sort.k0" : "sort.k1";
     R->spare_name = in_alt ? "sort.k1" : "sort.k0";
-    ws.retire(R->spare_name);
-    return 0;
+    return ws.give_back({R->spare_name}, st);
 }
 
-void sort_release(Workspace &ws) {
-    for (const char *n : {"sort.k0", "sort.k1", "sort.cnt", "sort.w", "sort.a0", "sort.a1", "sort.bound", "sort.words",
-                          "sort.mk", "sort.mv",
-                          "path.dcol", "path.dval", "path.tk", "path.tm", "path.ko", "path.mo", "path.deg",
-                          "path.dend", "path.rowlen", "path.dstart", "path.first", "path.end"})
-        ws.retire(n);
+int sort_release(Workspace &ws, cudaStream_t st) {
+    return ws.give_back({"sort.k0", "sort.k1", "sort.cnt", "sort.w", "sort.a0", "sort.a1", "sort.bound", "sort.words",
+                         "sort.mk", "sort.mv", "path.dcol", "path.dval", "path.tk", "path.tm", "path.ko", "path.mo",
+                         "path.deg", "path.dend", "path.rowlen", "path.dstart", "path.first", "path.end"},
+                        st);
 }
 
 int sort_counts(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CountsResult *out, cudaStream_t st) {
@@ -2751,8 +2747,7 @@ int sort_counts(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Counts
         else
             LNE_CUDA_TRY(cudaMemcpyAsync(out->cnt, R.cnt, sizeof(uint32_t) * u, cudaMemcpyDeviceToDevice, st));
     }
-    LNE_CUDA_TRY(cudaStreamSynchronize(st));
-    sort_release(ws);
+    LNE_TRY(sort_release(ws, st));
     out->nnz = u;
     out->total_samples = R.total;
     return 0;
@@ -2761,7 +2756,7 @@ int sort_counts(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Counts
 // Symmetric CSR from U ascending unique pair keys uk and their Eq. 1 value
 // bits val (0 = dropped), with per-tile (kPathTile) kept / kept off-diagonal
 // counts tk / tm. uk and val (workspace buffers uk_name / val_name) serve as
-// spare buffers of the mirrored sort and are retired.
+// spare buffers of the mirrored sort and are handed back.
 int assemble_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, uint64_t *uk, uint32_t *val, int64_t U,
                  const uint32_t *tk, const uint32_t *tm, const char *uk_name, const char *val_name, CsrResult *out,
                  cudaStream_t st) {
@@ -2770,13 +2765,13 @@ int assemble_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, uint6
     const unsigned egrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256), num_sms() * 16));
     uint32_t *rowlen = nullptr;
     int64_t *ko = nullptr, *mo = nullptr, *first = nullptr, *end = nullptr, *dstart = nullptr, *dend = nullptr;
-    LNE_TRY(ws.get("path.ko", (size_t)ntiles + 1, &ko));
-    LNE_TRY(ws.get("path.mo", (size_t)ntiles + 1, &mo));
-    LNE_TRY(ws.get("path.dend", (size_t)n, &dend));
-    LNE_TRY(ws.get("path.rowlen", (size_t)n, &rowlen));
-    LNE_TRY(ws.get("path.dstart", (size_t)n, &dstart));
-    LNE_TRY(ws.get("path.first", (size_t)n, &first));
-    LNE_TRY(ws.get("path.end", (size_t)n, &end));
+    LNE_TRY(ws.temp("path.ko", (size_t)ntiles + 1, &ko));
+    LNE_TRY(ws.temp("path.mo", (size_t)ntiles + 1, &mo));
+    LNE_TRY(ws.temp("path.dend", (size_t)n, &dend));
+    LNE_TRY(ws.temp("path.rowlen", (size_t)n, &rowlen));
+    LNE_TRY(ws.temp("path.dstart", (size_t)n, &dstart));
+    LNE_TRY(ws.temp("path.first", (size_t)n, &first));
+    LNE_TRY(ws.temp("path.end", (size_t)n, &end));
     LNE_TRY(ws.get("csr.indptr", (size_t)n + 1, &out->indptr));
     LNE_CUDA_TRY(cudaMemsetAsync(dend, 0, sizeof(int64_t) * n, st));
     LNE_CUDA_TRY(cudaMemsetAsync(end, 0, sizeof(int64_t) * n, st));
@@ -2790,10 +2785,10 @@ int assemble_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, uint6
     int32_t *dcol = nullptr;
     uint32_t *dval = nullptr, *mv = nullptr;
     uint64_t *mk = nullptr;
-    LNE_TRY(ws.get("path.dcol", (size_t)std::max<int64_t>(nk, 1), &dcol));
-    LNE_TRY(ws.get("path.dval", (size_t)std::max<int64_t>(nk, 1), &dval));
-    LNE_TRY(ws.get("sort.mk", (size_t)std::max<int64_t>(nm, 1), &mk));
-    LNE_TRY(ws.get("sort.mv", (size_t)std::max<int64_t>(nm, 1), &mv));
+    LNE_TRY(ws.temp("path.dcol", (size_t)std::max<int64_t>(nk, 1), &dcol));
+    LNE_TRY(ws.temp("path.dval", (size_t)std::max<int64_t>(nk, 1), &dval));
+    LNE_TRY(ws.temp("sort.mk", (size_t)std::max<int64_t>(nm, 1), &mk));
+    LNE_TRY(ws.temp("sort.mv", (size_t)std::max<int64_t>(nm, 1), &mv));
     {
         LNE_TRACE("path_rows", st);
         path_rows_kernel<<<(unsigned)ntiles, kPathThreads, 0, st>>>(uk, val, U, sp.B, ko, mo, dstart, dend, dcol,
@@ -2823,11 +2818,9 @@ int assemble_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, uint6
     LNE_CUDA_TRY(cudaStreamSynchronize(st));
     // the buffers not holding the sorted mirrored entries are free now
     if (in_alt) {
-        ws.retire("sort.mk");
-        ws.retire("sort.mv");
+        LNE_TRY(ws.give_back({"sort.mk", "sort.mv"}, st));
     } else {
-        ws.retire(uk_name);
-        ws.retire(val_name);
+        LNE_TRY(ws.give_back({uk_name, val_name}, st));
     }
     LNE_TRY(ws.get("csr.indices", (size_t)std::max<int64_t>(nnz, 1), &out->indices));
     LNE_TRY(ws.get("csr.data", (size_t)std::max<int64_t>(nnz, 1), &out->data));
@@ -2842,18 +2835,16 @@ int assemble_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, uint6
             LNE_LAUNCH_CHECK();
         }
     }
-    LNE_CUDA_TRY(cudaStreamSynchronize(st));
-    sort_release(ws);
-    ws.retire(uk_name);
-    ws.retire(val_name);
+    LNE_TRY(sort_release(ws, st));
+    LNE_TRY(ws.give_back({uk_name, val_name}, st));
     out->n = n;
     out->nnz = nnz;
     return 0;
 }
 
 int sort_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CsrResult *out, cudaStream_t st) {
-    // a previous sparsifier's arrays are rebuilt below: retire them before the
-    // sort's peak (tens of GB for billions of samples)
+    // a previous sparsifier's arrays are rebuilt below: large ones are freed before
+    // the sort's peak (tens of GB for billions of samples)
     ws.retire("csr.indices");
     ws.retire("csr.data");
     SortRaw R;
@@ -2862,9 +2853,9 @@ int sort_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, CsrResult
     const int64_t ntiles = std::max<int64_t>(1, ceil_div(U, (int64_t)kPathTile));
     const unsigned egrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256), num_sms() * 16));
     uint32_t *tk = nullptr, *tm = nullptr, *deg = nullptr;
-    LNE_TRY(ws.get("path.tk", (size_t)ntiles, &tk));
-    LNE_TRY(ws.get("path.tm", (size_t)ntiles, &tm));
-    LNE_TRY(ws.get("path.deg", (size_t)n, &deg));
+    LNE_TRY(ws.temp("path.tk", (size_t)ntiles, &tk));
+    LNE_TRY(ws.temp("path.tm", (size_t)ntiles, &tm));
+    LNE_TRY(ws.temp("path.deg", (size_t)n, &deg));
     {
         LNE_TRACE("path_value", st);
         if (!g.wdeg) {
@@ -3180,8 +3171,8 @@ int strat_keys(Workspace &ws, const GraphView &g, const SamplerSpec &sp, int64_t
     int64_t total = 0;
     LNE_TRY(tile_offsets(ws, A, 0, g.nnz, tile_arcs, &tile_off, &total, st));
     uint64_t *k0 = nullptr, *k1 = nullptr;
-    LNE_TRY(ws.get("sort.k0", (size_t)std::max<int64_t>(total, 1), &k0));
-    LNE_TRY(ws.get("sort.k1", (size_t)std::max<int64_t>(total, 1), &k1));
+    LNE_TRY(ws.temp("sort.k0", (size_t)std::max<int64_t>(total, 1), &k0));
+    LNE_TRY(ws.temp("sort.k1", (size_t)std::max<int64_t>(total, 1), &k1));
     {
         LNE_TRACE("walk_keys", st);
         LNE_TRY(launch_walk_batch<kKeysGen>(A, tile_arcs, tile_off, k0, nullptr, nullptr, 0, st));
@@ -3189,8 +3180,8 @@ int strat_keys(Workspace &ws, const GraphView &g, const SamplerSpec &sp, int64_t
     bool in_alt = false;
     LNE_TRY(radix_sort_u64(ws, k0, k1, nullptr, nullptr, total, 0, 2 * su.B + 4, &in_alt, st));
     uint64_t *sorted = in_alt ? k1 : k0, *other = in_alt ? k0 : k1;
-    ws.retire("sort.words");
-    LNE_TRY(ws.get("sort.cnt", (size_t)std::max<int64_t>(total, 1), cnt));
+    LNE_TRY(ws.give_back({"sort.words"}, st));
+    LNE_TRY(ws.temp("sort.cnt", (size_t)std::max<int64_t>(total, 1), cnt));
     LNE_TRY(run_length(ws, sorted, total, other, *cnt, U, st));
     *total_out = total;
     *ukr = other;
@@ -3258,7 +3249,7 @@ int prepare_weighted(Workspace &ws, GraphView *g, cudaStream_t st) {
 }
 
 int stratified_sample(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Strata *out, cudaStream_t st) {
-    stratified_release(ws);
+    LNE_TRY(stratified_release(ws, st));
     int64_t total = 0, U = 0, P = 0;
     uint64_t *ukr = nullptr, *spare = nullptr;
     uint32_t *cnt = nullptr;
@@ -3267,8 +3258,8 @@ int stratified_sample(Workspace &ws, const GraphView &g, const SamplerSpec &sp, 
     uint32_t *scnt = nullptr, *seglen = nullptr;
     uint64_t *pair = nullptr;
     int64_t *seg = nullptr;
-    LNE_TRY(ws.get("strat.r", (size_t)std::max<int64_t>(U, 1), &r));
-    LNE_TRY(ws.get("strat.cnt", (size_t)std::max<int64_t>(U, 1), &scnt));
+    LNE_TRY(ws.temp("strat.r", (size_t)std::max<int64_t>(U, 1), &r));
+    LNE_TRY(ws.temp("strat.cnt", (size_t)std::max<int64_t>(U, 1), &scnt));
     if (U > 0) {
         LNE_TRACE("strat_split", st);
         strat_split_kernel<<<(unsigned)std::min<int64_t>(ceil_div(U, 256), num_sms() * 16), 256, 0, st>>>(ukr, U, spare,
@@ -3277,14 +3268,12 @@ int stratified_sample(Workspace &ws, const GraphView &g, const SamplerSpec &sp, 
         LNE_CUDA_TRY(cudaMemcpyAsync(scnt, cnt, sizeof(uint32_t) * U, cudaMemcpyDeviceToDevice, st));
     }
     // the pair keys are sorted with their windows: pairs are runs of them
-    LNE_TRY(ws.get("strat.pair", (size_t)std::max<int64_t>(U, 1), &pair));
-    LNE_TRY(ws.get("strat.seglen", (size_t)std::max<int64_t>(U, 1), &seglen));
+    LNE_TRY(ws.temp("strat.pair", (size_t)std::max<int64_t>(U, 1), &pair));
+    LNE_TRY(ws.temp("strat.seglen", (size_t)std::max<int64_t>(U, 1), &seglen));
     LNE_TRY(run_length(ws, spare, U, pair, seglen, &P, st));
-    LNE_TRY(ws.get("strat.seg", (size_t)P + 1, &seg));
+    LNE_TRY(ws.temp("strat.seg", (size_t)P + 1, &seg));
     LNE_TRY(scan_exclusive_u32_to_i64(seglen, seg, P, st));
-    LNE_CUDA_TRY(cudaStreamSynchronize(st));
-    for (const char *nm : {"sort.k0", "sort.k1", "sort.cnt", "strat.seglen", "rle.cnt", "rle.off"})
-        ws.retire(nm);
+    LNE_TRY(ws.give_back({"sort.k0", "sort.k1", "sort.cnt", "strat.seglen"}, st));
     out->total = total;
     out->U = U;
     out->P = P;
@@ -3315,11 +3304,11 @@ int stratified_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, con
     const unsigned egrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(n, 256), num_sms() * 16));
     uint32_t *tk = nullptr, *tm = nullptr, *deg = nullptr, *val = nullptr;
     uint64_t *uk = nullptr;
-    LNE_TRY(ws.get("path.tk", (size_t)ntiles, &tk));
-    LNE_TRY(ws.get("path.tm", (size_t)ntiles, &tm));
-    LNE_TRY(ws.get("path.deg", (size_t)n, &deg));
-    LNE_TRY(ws.get("strat.cuk", (size_t)std::max<int64_t>(P, 1), &uk));
-    LNE_TRY(ws.get("strat.cval", (size_t)std::max<int64_t>(P, 1), &val));
+    LNE_TRY(ws.temp("path.tk", (size_t)ntiles, &tk));
+    LNE_TRY(ws.temp("path.tm", (size_t)ntiles, &tm));
+    LNE_TRY(ws.temp("path.deg", (size_t)n, &deg));
+    LNE_TRY(ws.temp("strat.cuk", (size_t)std::max<int64_t>(P, 1), &uk));
+    LNE_TRY(ws.temp("strat.cval", (size_t)std::max<int64_t>(P, 1), &val));
     if (P > 0) LNE_CUDA_TRY(cudaMemcpyAsync(uk, S.pair, sizeof(uint64_t) * P, cudaMemcpyDeviceToDevice, st));
     {
         LNE_TRACE("path_value", st);
@@ -3335,10 +3324,9 @@ int stratified_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, con
     return assemble_csr(ws, g, sp, uk, val, P, tk, tm, "strat.cuk", "strat.cval", out, st);
 }
 
-void stratified_release(Workspace &ws) {
-    for (const char *nm : {"strat.r", "strat.cnt", "strat.pair", "strat.seglen", "strat.seg", "strat.cuk",
-                           "strat.cval"})
-        ws.retire(nm);
+int stratified_release(Workspace &ws, cudaStream_t st) {
+    return ws.give_back({"strat.r", "strat.cnt", "strat.pair", "strat.seglen", "strat.seg", "strat.cuk", "strat.cval"},
+                        st);
 }
 
 namespace {
@@ -3360,8 +3348,7 @@ int strat_counts(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Count
         LNE_LAUNCH_CHECK();
         LNE_CUDA_TRY(cudaMemcpyAsync(out->cnt, cnt, sizeof(uint32_t) * U, cudaMemcpyDeviceToDevice, st));
     }
-    LNE_CUDA_TRY(cudaStreamSynchronize(st));
-    sort_release(ws);
+    LNE_TRY(sort_release(ws, st));
     out->nnz = U;
     out->total_samples = total;
     return 0;
@@ -3386,9 +3373,8 @@ int sparsifier_csr(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Csr
     if (sp.stratified) {
         Strata S;
         LNE_TRY(stratified_sample(ws, g, sp, &S, st));
-        const int rc = stratified_csr(ws, g, sp, S, out, st);
-        stratified_release(ws);
-        return rc;
+        LNE_TRY(stratified_csr(ws, g, sp, S, out, st));
+        return stratified_release(ws, st);
     }
     if (sp.ds_C > 0.0 && !use_table(g, sp) && sp.aggregation == LNE_AGG_BUCKET)
         return fail(LNE_ERR_UNSUPPORTED, "edge downsampling needs the table or the sort aggregation");

@@ -355,7 +355,7 @@ __global__ void lower_bound_kernel(const uint64_t *__restrict__ keys, int64_t n,
 
 int count_below(Workspace &ws, const uint64_t *keys, int64_t n, uint64_t key, int64_t *count, cudaStream_t st) {
     int64_t *d = nullptr;
-    LNE_TRY(ws.get("sort.bound", 1, &d));
+    LNE_TRY(ws.temp("sort.bound", 1, &d));
     lower_bound_kernel<<<1, 1, 0, st>>>(keys, n, key, d);
     LNE_LAUNCH_CHECK();
     LNE_CUDA_TRY(cudaMemcpyAsync(count, d, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -378,7 +378,7 @@ int radix_sort_u64(Workspace &ws, uint64_t *keys, uint64_t *keys_alt, uint32_t *
     unsigned long long *hist = nullptr;
     unsigned *next = nullptr;
     int *status = nullptr;
-    LNE_TRY(ws.get("sort.words", (size_t)256 * ntiles, &words));
+    LNE_TRY(ws.temp("sort.words", (size_t)256 * ntiles, &words));
     LNE_TRY(ws.get("sort.hist", (size_t)256 * kMaxPasses, &hist));
     LNE_TRY(ws.get("sort.next", kMaxPasses, &next));
     LNE_TRY(device_status(ws, &status, st));

@@ -175,7 +175,7 @@ int tune_batch(Workspace &ws, PropBatchGraph *cache, SpmmTune &tc, int aggregati
         LNE_TRY(rsvd(ws, product_view(M, dense_mode, d + os_of(p)), d, os_of(p), p.q, p.seed, p.precision, nullptr, nullptr,
                      X0s + (size_t)q * n * d, st, sk));
     }
-    if (have_strata) stratified_release(ws);
+    if (have_strata) LNE_TRY(stratified_release(ws, st));
     float *X = nullptr, *U = nullptr;
     double *R = nullptr, *UR = nullptr, *sig = nullptr;
     LNE_TRY(ws.get("tune.x", (size_t)n * d, &X));
