@@ -261,7 +261,7 @@ int Workspace::temp(const std::string &name, size_t bytes, void **ptr) {
         }
         if (e == cudaSuccess) e = cudaStreamSynchronize(sp.st);
         if (e != cudaSuccess) {
-            b.p = nullptr;
+            bufs_.erase(name);
             return out_of_memory(want, name, e);
         }
         b.bytes = want;
@@ -271,9 +271,17 @@ int Workspace::temp(const std::string &name, size_t bytes, void **ptr) {
     return 0;
 }
 
-int Workspace::give_back(std::initializer_list<const char *> names, cudaStream_t st) {
-    LNE_CUDA_TRY(cudaStreamSynchronize(st));
-    for (const char *name : names) release(name);
+int Workspace::give_back(std::initializer_list<const char *> names, cudaStream_t st, bool wait) {
+    if (wait) LNE_CUDA_TRY(cudaStreamSynchronize(st));
+    for (const char *name : names) {
+        auto it = bufs_.find(name);
+        if (it == bufs_.end()) continue;
+        if (!wait && it->second.pooled) {   // the pool keeps later users of the memory behind st
+            LNE_CUDA_TRY(cudaFreeAsync(it->second.p, st));
+            it->second = Buf();
+        }
+        release(name);
+    }
     return 0;
 }
 

@@ -48,9 +48,9 @@ public:
     int temp(const std::string &name, size_t count, T **ptr) {
         return temp(name, count * sizeof(T), reinterpret_cast<void **>(ptr));
     }
-    // Waits for the stream that has used the buffers and hands them back (absent names
-    // are skipped).
-    int give_back(std::initializer_list<const char *> names, cudaStream_t st);
+    // Hands buffers back that st has used (absent names are skipped): waits for st
+    // first, or (wait = false) in the stream's order.
+    int give_back(std::initializer_list<const char *> names, cudaStream_t st, bool wait = true);
     // After a call that failed: waits for the device and hands back what the call still
     // had, so that no such buffer outlives the call that took it.
     void settle();

@@ -75,7 +75,7 @@ struct WalkArgs {
     // (first j with word < cum[off + j], cum = floor(2^32 prefix_j / d_x))
     const uint32_t *w;
     const uint32_t *cum;
-    const uint4 *wstep;           // per arc b of x: bracket and thresholds of bucket b (build_wstep_kernel)
+    const uint4 *wstep;           // per arc b of x: bracket and thresholds of bucket b (build_wstep_kernel); may be NULL
     double S, vol;
     uint32_t wmax;                // host copy of the largest weight (tile size bounds)
 };
@@ -296,6 +296,13 @@ __device__ __forceinline__ uint32_t weighted_arc(const WalkArgs &A, int64_t off,
     return lo;
 }
 
+// The record of word w's bracket; without records (no memory for them) the bracket is
+// all of the vertex's arcs.
+__device__ __forceinline__ uint4 weighted_record(const WalkArgs &A, int64_t off, uint32_t deg, uint32_t w) {
+    if (A.wstep) return __ldg(A.wstep + off + __umulhi(w, deg));
+    return make_uint4(0u, deg - 1u, __ldg(A.cum + off), deg > 1u ? __ldg(A.cum + off + 1) : 0xFFFFFFFFu);
+}
+
 // One walk step: x <- nbr(x)[w mod deg(x)] (Sec. 5.2), reading the taken
 // arc's record. GEN: the variant that also handles weighted graphs.
 template <bool GEN>
@@ -306,7 +313,7 @@ __device__ __forceinline__ void walk_step(const WalkArgs &A, WalkCur &c, uint32_
     uint32_t j;
     if (deg == 0xFFFFFFu) deg = (uint32_t)(__ldg(A.indptr + c.x + 1) - __ldg(A.indptr + c.x));
     if (GEN && A.cum) {
-        j = weighted_arc(A, off, __ldg(A.wstep + off + __umulhi(w, deg)), w);
+        j = weighted_arc(A, off, weighted_record(A, off, deg, w), w);
     } else if ((c.hidg >> 8) == 0xFFFFFFu) {
         j = w % deg;
     } else {
@@ -1052,8 +1059,8 @@ __device__ __forceinline__ void gen_step(const WalkArgs &A, KeyDraw &d0, KeyDraw
     uint32_t j0 = 0, j1 = 0;
     if (A.cum) {
         uint4 g0 = make_uint4(0u, 0u, 0u, 0u), g1 = g0;
-        if (deg0) g0 = __ldg(A.wstep + off0 + __umulhi(w0, deg0));
-        if (deg1) g1 = __ldg(A.wstep + off1 + __umulhi(w1, deg1));
+        if (deg0) g0 = weighted_record(A, off0, deg0, w0);
+        if (deg1) g1 = weighted_record(A, off1, deg1, w1);
         j0 = weighted_arc(A, off0, g0, w0);
         j1 = weighted_arc(A, off1, g1, w1);
     } else {
@@ -2280,14 +2287,28 @@ int attach_vinfo(Workspace &ws, const GraphView &g, WalkArgs *A, cudaStream_t st
         build_cum_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(g.n, 8), num_sms() * 16)), 256, 0,
                            st>>>(g.indptr, g.w, g.wdeg, g.n, cum);
         LNE_LAUNCH_CHECK();
-        uint4 *wstep = nullptr;
-        LNE_TRY(ws.get("walk.wstep", (size_t)std::max<int64_t>(g.nnz, 1), &wstep));
-        build_wstep_kernel<<<(unsigned)std::max<int64_t>(1, ceil_div(g.nnz, (int64_t)kStepTile)), 256, 0, st>>>(
-            g.indptr, cum, g.n, g.nnz, wstep);
-        LNE_LAUNCH_CHECK();
         A->cum = cum;
-        A->wstep = wstep;
     }
+    return 0;
+}
+
+// The weighted step's records for the walk that is launched next (16 bytes an arc, of
+// the scratch pool, handed back behind the walk). A graph so large that they do not fit
+// beside the rest walks without them: each step then searches the vertex's thresholds.
+int attach_wstep(Workspace &ws, WalkArgs *A, cudaStream_t st) {
+    if (!A->cum) return 0;
+    uint4 *wstep = nullptr;
+    const int rc = ws.temp("walk.wstep", (size_t)std::max<int64_t>(A->n_arcs, 1), &wstep);
+    if (rc == LNE_ERR_OOM) {
+        clear_message();
+        return 0;
+    }
+    LNE_TRY(rc);
+    LNE_TRACE("build_wstep", st);
+    build_wstep_kernel<<<(unsigned)std::max<int64_t>(1, ceil_div(A->n_arcs, (int64_t)kStepTile)), 256, 0, st>>>(
+        A->indptr, A->cum, A->n, A->n_arcs, wstep);
+    LNE_LAUNCH_CHECK();
+    A->wstep = wstep;
     return 0;
 }
 
@@ -2348,9 +2369,10 @@ int walk_smem_bytes(int tile_arcs, int nb_smem) {
 // Per-tile offsets of arcs [a0, a1): returns the total number of samples.
 // Launches the walk kernel variant the arguments need (see walk_emit_kernel).
 template <typename KeyT, int MODE>
-int launch_walk_emit(const WalkArgs &A, unsigned grid, int smem, cudaStream_t st, int64_t a_begin, int64_t a_end,
-                     int tile_arcs, const int64_t *tile_off, KeyT *keys, int32_t *u1, int32_t *v1,
+int launch_walk_emit(Workspace &ws, WalkArgs A, unsigned grid, int smem, cudaStream_t st, int64_t a_begin,
+                     int64_t a_end, int tile_arcs, const int64_t *tile_off, KeyT *keys, int32_t *u1, int32_t *v1,
                      uint32_t *bucket_cnt, int nb_smem) {
+    LNE_TRY(attach_wstep(ws, &A, st));
     if (A.ds_thr || A.cum || A.w) {
         LNE_TRY(allow_dynamic_smem(walk_emit_kernel<KeyT, MODE, true>));
         walk_emit_kernel<KeyT, MODE, true><<<grid, kWalkThreads, smem, st>>>(A, a_begin, a_end, tile_arcs, tile_off,
@@ -2361,16 +2383,17 @@ int launch_walk_emit(const WalkArgs &A, unsigned grid, int smem, cudaStream_t st
                                                                              keys, u1, v1, bucket_cnt, nb_smem);
     }
     LNE_LAUNCH_CHECK();
-    return 0;
+    return ws.give_back({"walk.wstep"}, st, false);
 }
 
 template <WalkOut OUT>
-int launch_walk_batch(const WalkArgs &A, int tile_arcs, const int64_t *tile_off, uint64_t *keys, uint32_t *arcs,
-                      uint32_t *cnt, uint32_t ld, cudaStream_t st) {
+int launch_walk_batch(Workspace &ws, WalkArgs A, int tile_arcs, const int64_t *tile_off, uint64_t *keys,
+                      uint32_t *arcs, uint32_t *cnt, uint32_t ld, cudaStream_t st) {
+    LNE_TRY(attach_wstep(ws, &A, st));
     walk_batch_kernel<OUT><<<(unsigned)ceil_div(A.n_arcs, tile_arcs), kTabThreads, walk_smem_bytes(tile_arcs, 0), st>>>(
         A, tile_arcs, tile_off, keys, arcs, cnt, ld);
     LNE_LAUNCH_CHECK();
-    return 0;
+    return ws.give_back({"walk.wstep"}, st, false);
 }
 
 int tile_offsets(Workspace &ws, const WalkArgs &A, int64_t a0, int64_t a1, int tile_arcs,
@@ -2466,7 +2489,7 @@ int sample_pairs(Workspace &ws, const GraphView &g, const SamplerSpec &sp, int64
     // dynamic shared memory comes on top of the kernel's static tables
     {
         LNE_TRACE("walk_emit", st);
-        LNE_TRY((launch_walk_emit<uint32_t, 0>(A, (unsigned)ntiles, smem, st, a0, a1, tile_arcs, tile_off, nullptr, u1,
+        LNE_TRY((launch_walk_emit<uint32_t, 0>(ws, A, (unsigned)ntiles, smem, st, a0, a1, tile_arcs, tile_off, nullptr, u1,
                                               v1, nullptr, 0)));
     }
     return 0;
@@ -2514,7 +2537,7 @@ int sample_and_reduce(Workspace &ws, const GraphView &g, const SamplerSpec &sp, 
     // dynamic shared memory comes on top of the kernel's static tables
     {
         LNE_TRACE("walk_emit", st);
-        LNE_TRY((launch_walk_emit<uint32_t, 1>(A, (unsigned)ntiles, smem, st, 0, g.nnz, tile_arcs, tile_off, keys0,
+        LNE_TRY((launch_walk_emit<uint32_t, 1>(ws, A, (unsigned)ntiles, smem, st, 0, g.nnz, tile_arcs, tile_off, keys0,
                                               nullptr, nullptr, bucket_cnt, nb_smem)));
     }
     LNE_TRY(scan_exclusive_u32_to_i64(bucket_cnt, R->bucket_off, nb, st));
@@ -2696,9 +2719,9 @@ int sort_raw(Workspace &ws, const GraphView &g, const SamplerSpec &sp, SortRaw *
     }
     {
         LNE_TRACE("walk_keys", st);
-        if (!lean) LNE_TRY(launch_walk_batch<kKeysGen>(A, tile_arcs, tile_off, k0, arc0, nullptr, 0, st));
-        else if (A.arcrec) LNE_TRY(launch_walk_batch<kKeysRec>(A, tile_arcs, tile_off, k0, nullptr, nullptr, 0, st));
-        else LNE_TRY(launch_walk_batch<kKeysNbr>(A, tile_arcs, tile_off, k0, nullptr, nullptr, 0, st));
+        if (!lean) LNE_TRY(launch_walk_batch<kKeysGen>(ws, A, tile_arcs, tile_off, k0, arc0, nullptr, 0, st));
+        else if (A.arcrec) LNE_TRY(launch_walk_batch<kKeysRec>(ws, A, tile_arcs, tile_off, k0, nullptr, nullptr, 0, st));
+        else LNE_TRY(launch_walk_batch<kKeysNbr>(ws, A, tile_arcs, tile_off, k0, nullptr, nullptr, 0, st));
     }
     bool in_alt = false;
     LNE_TRY(radix_sort_u64(ws, k0, k1, arc0, arc1, total, 0, bits, &in_alt, st));
@@ -2931,9 +2954,9 @@ int sample_table(Workspace &ws, const GraphView &g, const SamplerSpec &sp, Table
     if (A.ds_thr) {   // downsampled: 64-bit weight sums
         LNE_TRY(ws.get("table.W", (size_t)(ld * ld), &tb->W));
         LNE_CUDA_TRY(cudaMemsetAsync(tb->W, 0, sizeof(uint64_t) * (size_t)(ld * ld), st));
-        LNE_TRY(launch_walk_batch<kWeightsGen>(A, tile_arcs, nullptr, tb->W, nullptr, nullptr, (uint32_t)ld, st));
+        LNE_TRY(launch_walk_batch<kWeightsGen>(ws, A, tile_arcs, nullptr, tb->W, nullptr, nullptr, (uint32_t)ld, st));
     } else {
-        LNE_TRY(launch_walk_batch<kCountsGen>(A, tile_arcs, nullptr, nullptr, nullptr, tb->T, (uint32_t)ld, st));
+        LNE_TRY(launch_walk_batch<kCountsGen>(ws, A, tile_arcs, nullptr, nullptr, nullptr, tb->T, (uint32_t)ld, st));
     }
     return 0;
 }
@@ -3175,7 +3198,7 @@ int strat_keys(Workspace &ws, const GraphView &g, const SamplerSpec &sp, int64_t
     LNE_TRY(ws.temp("sort.k1", (size_t)std::max<int64_t>(total, 1), &k1));
     {
         LNE_TRACE("walk_keys", st);
-        LNE_TRY(launch_walk_batch<kKeysGen>(A, tile_arcs, tile_off, k0, nullptr, nullptr, 0, st));
+        LNE_TRY(launch_walk_batch<kKeysGen>(ws, A, tile_arcs, tile_off, k0, nullptr, nullptr, 0, st));
     }
     bool in_alt = false;
     LNE_TRY(radix_sort_u64(ws, k0, k1, nullptr, nullptr, total, 0, 2 * su.B + 4, &in_alt, st));

@@ -47,9 +47,11 @@ def test_other_allocators_get_the_scratch():
     assert scratch > 3 * GB
     # another allocator: all but 2 GB of what is free, then 2 GB more than that
     held = torch.empty(_free() - 2 * GB, dtype=torch.uint8, device="cuda")
-    more = torch.empty(4 * GB, dtype=torch.uint8, device="cuda")   # out of the scratch
-    del held, more
-    _free()
+    try:
+        torch.empty(4 * GB, dtype=torch.uint8, device="cuda")   # out of the scratch
+    finally:
+        del held
+        _free()
     m = a.sparsifier_csr(g, p)   # and the next call takes its scratch again
     assert m["nnz"] == nnz and float(m["data"].double().sum()) == total
     del m
@@ -86,3 +88,37 @@ def test_threads_share_the_scratch():
     for t in threads:
         t.join()
     assert not bad, bad
+
+
+def test_weighted_walk_without_memory_for_its_records():
+    """The weighted step's records (16 bytes an arc) are left out where they do not fit:
+    the walk searches the thresholds then, and draws the same pairs."""
+    indptr, indices = synth.chung_lu_device(300000, 6000000, 2.1, 5)   # 12M arcs: 192 MB of records
+    g = lne.DeviceGraph.from_tensors(indptr, indices)
+    src = torch.repeat_interleave(torch.arange(300000, device="cuda"), torch.diff(indptr))
+    g.weights = (1 + (src + indices.long()) % 9).to(torch.int32)       # equal on both arcs of an edge
+    del src
+    p = lne.Params(T=6, s=[1 / 6] * 6, samples=300000.0, d=32, seed=7)
+    a = lne.Context(0)
+    a.set_option(lne.OPT_AGGREGATION, lne.AGG_SORT)
+
+    def counts():
+        a.trace(True)
+        r = a.sparsifier_counts(g, p)
+        r = {k: r[k].cpu() for k in ("x", "y", "count")}   # nothing stays in the held memory's segment
+        names = {t["name"] for t in a.trace_read()}
+        a.trace(False)
+        return r, names
+
+    ref, names = counts()
+    assert "build_wstep" in names
+    lne.Context(0).close()   # unmaps the scratch
+    held = torch.empty(_free() - 128 * (1 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        got, names = counts()
+    finally:
+        del held
+        _free()
+    assert "build_wstep" not in names
+    assert all(torch.equal(ref[k], got[k]) for k in ref)
+    a.close()
