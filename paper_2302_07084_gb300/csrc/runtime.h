@@ -260,13 +260,16 @@ int dense_tc_prepare(Workspace &ws, const float *T, int64_t ld, const float **hi
                      cudaStream_t st);
 int dense_tc_spmm(Workspace &ws, const float *Ahi, const float *Alo, int64_t ld, int64_t n, const float *X,
                   int64_t ldx, int c, float *Y, int64_t ldy, cudaStream_t st);
-// Carry buffers of the merge SpMM for nnz nonzeros over n rows and c columns, under the
-// workspace names tag + ".c" / tag + ".r" (tag NULL = "spmm.carry").
+// Whether a graph product of c columns takes a lane group per row (which ignores the
+// merge kernel's CTA size and needs no chain buffers).
+bool short_rows(int64_t n, int64_t max_row, int c);
 // Buffers of a chain of products of g's matrix with c columns
 // (SpmmEpilogue::row_cnt, slice_row; NULL where none are needed), and the work
 // before the chain's first product.
 int merge_chain(Workspace &ws, const char *tag, const GraphView &g, int c, uint32_t **row_cnt, int32_t **slice_row);
 int merge_chain_prepare(const GraphView &g, uint32_t *row_cnt, int32_t *slice_row, cudaStream_t st);
+// Carry buffers of the merge SpMM for nnz nonzeros over n rows and c columns, under the
+// workspace names tag + ".c" / tag + ".r" (tag NULL = "spmm.carry").
 int merge_carry(Workspace &ws, const char *tag, int64_t nnz, int64_t n, int c, float4 **carry,
                 int64_t **carry_row);
 int graph_spmm(Workspace &ws, const GraphView &g, const float *X, int64_t ldx, int c, float *Y, int64_t ldy,
@@ -335,8 +338,8 @@ std::vector<double> chebyshev_coefficients(int k, double theta);
 
 // The batched merge SpMM's tile shape, picked by timing every candidate
 // (CTA size 64 / 128 / 256 x column blocks of 128 / 256 / 512 / all columns)
-// once per (row-length bucket, nnz bucket, width) and cached; `forced` fixes
-// the CTA size. Results do not depend on the choice.
+// once per (row-length bucket, nnz bucket, width, whether rows are short) and cached;
+// `forced` fixes the CTA size. Results do not depend on the choice.
 struct SpmmTune {
     int forced = 0;         // CTA size (0 = tuned)
     int forced_block = 0;   // column-block width (0 = tuned, -1 = all columns at once)

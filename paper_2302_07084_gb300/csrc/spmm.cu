@@ -23,6 +23,14 @@
 
 namespace lne {
 
+// Rows of at most 256 nonzeros and 256 columns, graphs of at most 16 rows per
+// resident warp of the GPU: beyond, the merge kernel's balanced slices keep more
+// gathers going.
+bool short_rows(int64_t n, int64_t max_row, int c) {
+    return max_row > 0 && max_row <= 256 && c <= 256 && n <= (int64_t)num_sms() * 64 * 16;
+}
+
+
 
 namespace {
 
@@ -467,7 +475,7 @@ __global__ void __launch_bounds__(256) spmm_fixup_kernel(int64_t n, const int64_
 }
 
 // The same product with a lane group per row, for small graphs whose rows are
-// short (rows_ok): nothing crosses groups, so no carry, no fix-up and no search;
+// short (short_rows): nothing crosses groups, so no carry, no fix-up and no search;
 // the group itself adds the row's slices in slice order, which gives the merge
 // kernel's sums. LG lanes (the float4 columns, rounded up to a power of two) take
 // a row. Latency-bound: the epilogue's operands and the next batch's indices are
@@ -588,13 +596,6 @@ __global__ void __launch_bounds__(128) spmm_rows_kernel(int64_t n, const int64_t
     }
 }
 
-// Rows of at most 256 nonzeros and 256 columns, graphs of at most 16 rows per
-// resident warp of the GPU: beyond, the merge kernel's balanced slices keep more
-// gathers going.
-bool rows_ok(int64_t n, int64_t max_row, int c) {
-    return max_row > 0 && max_row <= 256 && c <= 256 && n <= (int64_t)num_sms() * 64 * 16;
-}
-
 template <bool WEIGHTED>
 int launch_spmm(int64_t n, const int64_t *indptr, const int32_t *indices, const float *vals,
                 const float *X, int64_t ldx, int c, float *Y, int64_t ldy, const SpmmEpilogue &ep,
@@ -699,7 +700,7 @@ int launch_merge(Workspace &ws, int64_t n, int64_t nnz, const int64_t *indptr, c
     const unsigned fblocks = (unsigned)std::min<int64_t>(ceil_div(n, 8), num_sms() * 32);
     const bool fused = ep.row_cnt && ep.slice_row && nnz > 0 && !(WEIGHTED && c4 <= 16);
     LNE_TRACE(WEIGHTED ? "spmm" : "graph_spmm", st);
-    if (nnz > 0 && rows_ok(n, ep.max_row, c) && !(WEIGHTED && c4 <= 16)) {
+    if (nnz > 0 && short_rows(n, ep.max_row, c) && !(WEIGHTED && c4 <= 16)) {
 #define LNE_ROWS_CASE(LGV, K)                                                                               \
     spmm_rows_kernel<LGV, K, WEIGHTED, TX><<<(unsigned)ceil_div(n, 128 / LGV), 128, 0, st>>>(                \
         n, indptr, indices, vals, X, ldx, c4, Y, ldy, ep, (uint32_t)W)
@@ -954,7 +955,7 @@ int merge_chain(Workspace &ws, const char *tag, const GraphView &g, int c, uint3
                 int32_t **slice_row) {
     *row_cnt = nullptr;
     *slice_row = nullptr;
-    if (rows_ok(g.n, g.max_deg, c)) return 0;   // a lane group per row: no slices
+    if (short_rows(g.n, g.max_deg, c)) return 0;   // a lane group per row: no slices
     const int64_t W = merge_slice(g.nnz, g.n), nwarps = std::max<int64_t>(1, ceil_div(g.nnz, W));
     const std::string t = tag ? tag : "spmm.chain";
     LNE_TRY(ws.get(t + ".n", (size_t)g.n, row_cnt));

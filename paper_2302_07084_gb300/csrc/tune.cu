@@ -54,7 +54,9 @@ int spmm_tile_for(SpmmTune &tc, Workspace &ws, const GraphView &g, const float *
     while ((int64_t(1) << (dbucket + 1)) <= avg) ++dbucket;
     int nbucket = 0;
     while ((int64_t(1) << (nbucket + 1)) <= std::max<int64_t>(1, g.nnz)) ++nbucket;
-    const uint64_t key = (uint64_t)dbucket | ((uint64_t)nbucket << 8) | ((uint64_t)C << 16) |
+    // short rows take another kernel, whose times say nothing of the merge kernel's
+    const uint64_t brief = short_rows(g.n, g.max_deg, 4) ? 1 : 0;
+    const uint64_t key = (uint64_t)dbucket | ((uint64_t)nbucket << 8) | (brief << 15) | ((uint64_t)C << 16) |
                          ((uint64_t)tc.forced << 32) | ((uint64_t)(tc.forced_block + 1) << 44);
     auto it = tc.best.find(key);
     if (it != tc.best.end()) {
@@ -74,7 +76,13 @@ int spmm_tile_for(SpmmTune &tc, Workspace &ws, const GraphView &g, const float *
     }
     std::vector<SpmmTile> cands;
     for (int t : ts)
-        for (int b : bs) cands.push_back(SpmmTile{t, b});
+        for (int b : bs)   // where the lane groups take a width the CTA size is ignored
+            if (t == ts[0] || !short_rows(g.n, g.max_deg, b > 0 ? b : C)) cands.push_back(SpmmTile{t, b});
+    // timed as the chain runs its products
+    uint32_t *row_cnt = nullptr;
+    int32_t *slice_row = nullptr;
+    LNE_TRY(merge_chain(ws, "tile.chain", g, C, &row_cnt, &slice_row));
+    LNE_TRY(merge_chain_prepare(g, row_cnt, slice_row, st));
     cudaEvent_t e0, e1;
     LNE_CUDA_TRY(cudaEventCreate(&e0));
     LNE_CUDA_TRY(cudaEventCreate(&e1));
@@ -89,6 +97,8 @@ int spmm_tile_for(SpmmTune &tc, Workspace &ws, const GraphView &g, const float *
         ep.threads = cand.threads;
         ep.col_block = cand.col_block;
         ep.max_row = g.max_deg;
+        ep.row_cnt = row_cnt;
+        ep.slice_row = slice_row;
         if ((rc = graph_spmm(ws, g, X, C, C, Y, C, ep, st)) != 0) break;   // warm-up
         cudaEventRecord(e0, st);
         for (int r = 0; r < 3 && rc == 0; ++r) rc = graph_spmm(ws, g, X, C, C, Y, C, ep, st);
