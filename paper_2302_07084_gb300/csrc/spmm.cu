@@ -704,11 +704,13 @@ int launch_merge(Workspace &ws, int64_t n, int64_t nnz, const int64_t *indptr, c
 #define LNE_ROWS_CASE(LGV, K)                                                                               \
     spmm_rows_kernel<LGV, K, WEIGHTED, TX><<<(unsigned)ceil_div(n, 128 / LGV), 128, 0, st>>>(                \
         n, indptr, indices, vals, X, ldx, c4, Y, ldy, ep, (uint32_t)W)
-        if (c4 <= 4) LNE_ROWS_CASE(4, 1);
-        else if (c4 <= 8) LNE_ROWS_CASE(8, 1);
-        else if (c4 <= 16) LNE_ROWS_CASE(16, 1);
-        else if (c4 <= 32) LNE_ROWS_CASE(32, 1);
-        else LNE_ROWS_CASE(32, 2);
+        if constexpr (!WEIGHTED) {   // weighted products this narrow take the grouped kernels below
+            if (c4 <= 4) LNE_ROWS_CASE(4, 1);
+            else if (c4 <= 8) LNE_ROWS_CASE(8, 1);
+            else if (c4 <= 16) LNE_ROWS_CASE(16, 1);
+        }
+        if (c4 > 32) LNE_ROWS_CASE(32, 2);
+        else if (c4 > 16) LNE_ROWS_CASE(32, 1);
 #undef LNE_ROWS_CASE
         LNE_LAUNCH_CHECK();
         return 0;
