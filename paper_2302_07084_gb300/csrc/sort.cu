@@ -49,7 +49,7 @@ static_assert(kPassThreads == 256, "a thread per digit");
 constexpr int kPassWarps = kPassThreads / 32;
 constexpr int kPassItems = 16;
 constexpr int kPassTile = kPassThreads * kPassItems;   // 4096 keys per tile
-constexpr int kMaxPasses = 8;
+constexpr int kMaxPasses = 8;   // lo + 8 passes <= 64
 
 // hist[p][d] = keys whose digit of pass p is d (zeroed before).
 __global__ void __launch_bounds__(512) radix_count_kernel(const uint64_t *__restrict__ keys, int64_t n, int lo,
@@ -372,7 +372,8 @@ int radix_sort_u64(Workspace &ws, uint64_t *keys, uint64_t *keys_alt, uint32_t *
     *in_alt = false;
     if (n <= 1 || hi <= lo) return 0;
     const int passes = (hi - lo + 7) / 8;
-    if (lo < 0 || hi > 64 || passes > kMaxPasses) return fail(LNE_ERR_INVALID, "radix sort bits out of range");
+    // the last digit is whole: the padding of a last tile has to be the largest one
+    if (lo < 0 || hi > 64 || lo + 8 * passes > 64) return fail(LNE_ERR_INVALID, "radix sort bits out of range");
     const int64_t ntiles = ceil_div(n, (int64_t)kPassTile);
     uint64_t *words = nullptr;
     unsigned long long *hist = nullptr;
