@@ -175,11 +175,11 @@ int lne_create(lne_ctx **out, int device);
 void lne_destroy(lne_ctx *ctx);
 const char *lne_last_error(const lne_ctx *ctx);
 /* Bytes of device workspace the context currently holds. Scratch that a call hands
- * back before it returns (the key sort's buffers) is not counted: it comes from a pool
- * that all contexts of the process share on a device and that stays mapped between
- * calls, up to 1/8 of the device's memory. The CUDA driver takes unused pool memory
- * for any allocation of the process (cudaMalloc, other libraries) that would fail
- * without it; lne_trim and lne_destroy unmap it. */
+ * back before it returns (the key sort's buffers) is not counted. Such buffers of up to
+ * 1/64 of the device's memory come from a pool that all contexts of the process share on
+ * a device; it stays mapped between calls, up to 1/8 of the device's memory. The CUDA
+ * driver takes unused pool memory for any allocation of the process (cudaMalloc, other
+ * libraries) that would fail without it; lne_trim and lne_destroy unmap it. */
 int64_t lne_workspace_bytes(const lne_ctx *ctx);
 /* Release all workspace, and unmap the unused scratch pool of the context's device (the
  * next call re-allocates). */

@@ -149,6 +149,7 @@ namespace {
 struct ScratchPool {
     cudaMemPool_t pool = nullptr;
     cudaStream_t st = nullptr;
+    size_t largest = 0;   // bytes of a buffer that comes from it
 };
 std::mutex g_pool_mu;
 std::map<int, ScratchPool> g_pools;
@@ -176,6 +177,7 @@ int scratch_pool(bool create, ScratchPool *out) {
             return cuda_fail("cudaMemPoolSetAttribute", e, __FILE__, __LINE__);
         }
         sp.pool = pool;
+        sp.largest = total / 64;
     }
     *out = sp;
     return 0;
@@ -254,18 +256,24 @@ int Workspace::temp(const std::string &name, size_t bytes, void **ptr) {
             free_buf(b);
         }
         const size_t want = (bytes + 255) & ~(size_t)255;
-        cudaError_t e = cudaMallocFromPoolAsync(&b.p, want, sp.pool, sp.st);
+        const bool pooled = want <= sp.largest;
+        auto take = [&]() -> cudaError_t {
+            if (!pooled) return cudaMalloc(&b.p, want);
+            const cudaError_t e = cudaMallocFromPoolAsync(&b.p, want, sp.pool, sp.st);
+            return e == cudaSuccess ? cudaStreamSynchronize(sp.st) : e;
+        };
+        cudaError_t e = take();
         if (e == cudaErrorMemoryAllocation) {
             make_room();
-            e = cudaMallocFromPoolAsync(&b.p, want, sp.pool, sp.st);
+            e = take();
         }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(sp.st);
         if (e != cudaSuccess) {
             bufs_.erase(name);
             return out_of_memory(want, name, e);
         }
         b.bytes = want;
-        b.pooled = true;
+        b.pooled = pooled;
+        b.lent = true;
     }
     *ptr = b.p;
     return 0;
@@ -282,13 +290,17 @@ int Workspace::give_back(std::initializer_list<const char *> names, cudaStream_t
         }
         release(name);
     }
+    // the driver can take the memory elsewhere once it has seen the frees end
+    ScratchPool sp;
+    LNE_TRY(scratch_pool(false, &sp));
+    if (wait && sp.pool) LNE_CUDA_TRY(cudaStreamSynchronize(sp.st));
     return 0;
 }
 
 void Workspace::settle() {
     bool waited = false;
     for (auto it = bufs_.begin(); it != bufs_.end();) {
-        if (!it->second.pooled) {
+        if (!it->second.lent) {
             ++it;
             continue;
         }
@@ -297,6 +309,7 @@ void Workspace::settle() {
         free_buf(it->second);
         it = bufs_.erase(it);
     }
+    if (waited) cudaDeviceSynchronize();   // so that the driver sees the frees end
 }
 
 void Workspace::release() {

@@ -36,10 +36,12 @@ public:
     // more (no-op if absent): freed if it takes more than 1/64 of the device's memory, else
     // reused by the next get(), or freed when an allocation of this workspace fails.
     void retire(const std::string &name);
-    // A buffer that a call hands back before it returns (give_back): taken from the
-    // device's scratch pool, one for all contexts of the process. What has been handed
-    // back stays mapped up to 1/8 of the device's memory, and the driver takes it for any
-    // other allocation of the process that would fail without it; trim_scratch unmaps it.
+    // A buffer that a call hands back before it returns (give_back): up to 1/64 of the
+    // device's memory from the device's scratch pool, one for all contexts of the process
+    // (larger ones are allocated and freed: mapping 4 GB takes a pool 3.3 ms, cudaMalloc
+    // 0.2). What has been handed back stays mapped up to 1/8 of the device's memory, and
+    // the driver takes it for any other allocation of the process that would fail
+    // without it; trim_scratch unmaps it.
     // At 2e8 samples (7 GB of buffers) a sparsifier takes 18.9 ms this way, 17.9 where
     // each context kept its buffers mapped, 26 where they were freed and allocated on
     // every call; a run of tens of GB still hands them back as it goes.
@@ -60,6 +62,7 @@ private:
     struct Buf {
         void *p = nullptr;
         size_t bytes = 0;
+        bool lent = false;     // a temp() buffer
         bool pooled = false;   // from the scratch pool
         bool idle = false;     // retired
     };

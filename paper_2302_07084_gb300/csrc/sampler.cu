@@ -2250,7 +2250,6 @@ WalkArgs make_walk_args(const GraphView &g, const SamplerSpec &sp) {
     return A;
 }
 
-// Builds the per-vertex walk records into the workspace.
 // Most arcs for which a plain key walk (walk_batch_kernel) reads per-arc records: 64 MB of them, half
 // of L2. Measured (records / neighbour and vertex record, 8e7 to 1e8 draws): 2M
 // arcs 1.01 / 1.02 ms at T = 5 and 2.0 / 2.5 at T = 10, 8M arcs 2.1 / 1.7 and
@@ -2258,6 +2257,8 @@ WalkArgs make_walk_args(const GraphView &g, const SamplerSpec &sp) {
 // record of its own per arc, is better off with them at 16M arcs too (13.9 / 15.6).
 constexpr int64_t kRecordArcs = (int64_t)4 << 20;
 
+// Builds the per-vertex walk records into the workspace, the per-arc ones if asked for,
+// and a weighted graph's thresholds.
 int attach_vinfo(Workspace &ws, const GraphView &g, WalkArgs *A, cudaStream_t st, bool arc_records = true) {
     uint4 *vi = nullptr;
     LNE_TRY(ws.get("walk.vinfo", (size_t)std::max<int64_t>(g.n, 1), &vi));
@@ -2366,7 +2367,6 @@ int walk_smem_bytes(int tile_arcs, int nb_smem) {
     return (tile_arcs + 1) * 4 + 2 * tile_arcs * 4 + nb_smem * 4;
 }
 
-// Per-tile offsets of arcs [a0, a1): returns the total number of samples.
 // Launches the walk kernel variant the arguments need (see walk_emit_kernel).
 template <typename KeyT, int MODE>
 int launch_walk_emit(Workspace &ws, WalkArgs A, unsigned grid, int smem, cudaStream_t st, int64_t a_begin,
@@ -2396,6 +2396,7 @@ int launch_walk_batch(Workspace &ws, WalkArgs A, int tile_arcs, const int64_t *t
     return ws.give_back({"walk.wstep"}, st, false);
 }
 
+// Per-tile offsets of arcs [a0, a1): returns the total number of samples.
 int tile_offsets(Workspace &ws, const WalkArgs &A, int64_t a0, int64_t a1, int tile_arcs,
                  int64_t **tile_off, int64_t *total, cudaStream_t st) {
     if (A.w) {   // a tile's sample count is a 32-bit sum: bound it by the heaviest arc (and tiles of 4096 arcs)

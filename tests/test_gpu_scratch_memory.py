@@ -45,8 +45,10 @@ def test_other_allocators_get_the_scratch():
     assert second <= b.workspace_bytes() + GB // 4 and second < 0.6 * first
     scratch = first - a.workspace_bytes()
     assert scratch > 3 * GB
-    # another allocator: all but 2 GB of what is free, then 2 GB more than that
-    held = torch.empty(_free() - 2 * GB, dtype=torch.uint8, device="cuda")
+    # another allocator: all but 2 GB of what is free, then 2 GB more than that; the call's
+    # end is enough, without a synchronisation of the device
+    a.sparsifier_csr(g, p, copy=False)
+    held = torch.empty(torch.cuda.mem_get_info()[0] - 2 * GB, dtype=torch.uint8, device="cuda")
     try:
         torch.empty(4 * GB, dtype=torch.uint8, device="cuda")   # out of the scratch
     finally:
